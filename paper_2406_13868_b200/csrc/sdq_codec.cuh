@@ -29,6 +29,13 @@ __device__ __forceinline__ uint32_t e8m0_scale_code(float amax, int rule) {
   return (uint32_t)min(max(c, 0), 254);
 }
 
+// the same from the bit pattern of a non-negative finite bf16: with exponent field E the floor rule gives E - 2, and the
+// smallest E with amax <= 6 * 2^E is one more when the significand exceeds 1.5; zeros and subnormals end at code 0 either way
+__device__ __forceinline__ uint32_t e8m0_scale_code_bf16(uint32_t key, bool ceil_rule) {
+  const int c = (int)(key >> 7) - 2 + ((ceil_rule && (key & 127u) > 64u) ? 1 : 0);
+  return (uint32_t)max(c, 0);
+}
+
 // int8 operands (Section 5.1: W_o and A_o in int8): scale amax / 127 (1 for an all-zero vector) and code = the integer
 // nearest to x / s, ties to even, limited to +-127 -- both quotients in fp32, IEEE round-to-nearest divisions, the
 // precision in which the code is decided; returns the code's byte
@@ -72,6 +79,18 @@ __device__ __forceinline__ float ue4m3_scale_value(uint32_t c, int t) {
 // two floats -> two E2M1 codes in one byte (x in the low nibble)
 __device__ __forceinline__ uint32_t e2m1x2(float x, float y) {
   return (uint32_t)__nv_cvt_float2_to_fp4x2(make_float2(x, y), __NV_E2M1, cudaRoundNearest);
+}
+// eight floats -> eight E2M1 codes in one word (the first in the lowest nibble)
+__device__ __forceinline__ uint32_t e2m1x8(const float (&v)[8]) {
+  uint32_t d;
+  asm("{\n.reg .b8 a, b, c, d;\n"
+      "cvt.rn.satfinite.e2m1x2.f32 a, %2, %1;\n"
+      "cvt.rn.satfinite.e2m1x2.f32 b, %4, %3;\n"
+      "cvt.rn.satfinite.e2m1x2.f32 c, %6, %5;\n"
+      "cvt.rn.satfinite.e2m1x2.f32 d, %8, %7;\n"
+      "mov.b32 %0, {a, b, c, d};\n}"
+      : "=r"(d) : "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]));
+  return d;
 }
 // two floats -> two E4M3 codes in 16 bits (x in the low byte)
 __device__ __forceinline__ uint32_t e4m3x2(float x, float y) {

@@ -1,11 +1,19 @@
 // Offline weight decomposition + packing (Section 5, Stage 2 -> Stage 1 -> Stage 3) and its exporter.
 //
-// One CTA per weight row; one thread per S-Vector of 8 consecutive K (a single 16-byte load).
-// Pass 1 finds the row's largest outlier magnitude (the per-row power-of-two scale); pass 2 selects
-// outliers, prunes the rest pair-wise, derives the Q-Vector scales by an 8-lane shuffle reduction
-// (8 S-Vectors = 64 K), encodes, and scatters into the stage-tiled layout of sdq_layout.h.  Without Stage 1 (dense
-// inliers) every position that is not an outlier is encoded, with one scale per 32 K.
+// Two launches.  `row_scale_kernel` reads W once and leaves, per row, what needs the whole row: the exponent (or fp32 scale)
+// of the outliers, for two-level scaling the inlier factor, the scale atom, and the non-finite flag.  `pack_tile_kernel`
+// reads W again (a matrix up to ~100 MB is then still in L2) and writes the stage-tiled layout of sdq_layout.h: a CTA takes
+// 128 rows x 256 K, one record of the layout, and a thread 128 K of one row -- 16 S-Vectors, whole Q-Vectors, so that scales
+// need no exchange between threads and everything a thread produces is 4 to 16 contiguous bytes of the layout; the 32
+// lanes of a warp are 32 consecutive rows, whose pieces make whole 128-byte lines.  W comes in through shared memory, rows
+// 528 B apart (the 16-byte reads of 8 lanes then touch all banks once).
+//
+// What bounds it: the integer pipe (77 % busy at ~140 instructions per S-Vector; selections on packed keys instead of index
+// loops took it from ~350 over two passes), DRAM is at 30 %.  11008 x 4096, 1:8 + pair-wise 4:8: 189 us as one kernel with a
+// CTA per row and a thread per S-Vector scattering bytes -> 20 + 42 us.
 #include <cstring>
+#include <mutex>
+#include <condition_variable>
 
 #include "sdq_codec.cuh"
 #include "sdq_internal.h"
@@ -14,253 +22,488 @@
 
 namespace sdq {
 
-struct GroupSel {
-  uint32_t key[8];   // 15-bit magnitude keys
-  int o0, o1;        // outlier positions (ascending), -1 if absent
+// ---- selections on one S-Vector of 8 weights, r[j] = elements 2 j (low half) and 2 j + 1 -----------------------------
+// Ranking keys, larger = more significant.  By magnitude: magnitude bits << 16 | (7 - i), so that plain maxima resolve ties
+// to the lower index.  Weighted (c != nullptr, the product |w| * c[k], one fp32 multiply): the product's bit pattern;
+// comparisons resolve ties.
+template <bool WGT>
+__device__ __forceinline__ void rank_keys(const uint32_t (&r)[4], const float* __restrict__ c, int (&k)[8]) {
+  if constexpr (!WGT) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      k[2 * j] = (int)(((r[j] & 0x7FFFu) << 16) | (uint32_t)(7 - 2 * j));
+      k[2 * j + 1] = (int)((r[j] & 0x7FFF0000u) | (uint32_t)(6 - 2 * j));
+    }
+  } else {
+    const float4 c0 = __ldg(reinterpret_cast<const float4*>(c)), c1 = __ldg(reinterpret_cast<const float4*>(c) + 1);
+    const float cc[8] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      k[2 * j] = __float_as_int(__fmul_rn(__uint_as_float((r[j] & 0x7FFFu) << 16), cc[2 * j]));
+      k[2 * j + 1] = __float_as_int(__fmul_rn(__uint_as_float(r[j] & 0x7FFF0000u), cc[2 * j + 1]));
+    }
+  }
+}
+// position of the largest key of k[B .. B + n), ties to the lower index
+template <bool WGT, int B, int E>
+__device__ __forceinline__ int arg_max(const int (&k)[8]) {
+  int best = k[B], at = B;
+#pragma unroll
+  for (int i = B + 1; i < E; ++i) {
+    if constexpr (WGT) { if (k[i] > best) { best = k[i]; at = i; } }
+    else best = max(best, k[i]);
+  }
+  return WGT ? at : 7 - (best & 7);
+}
+// position of the smallest key, ties to the higher index (the last in rank order)
+template <bool WGT>
+__device__ __forceinline__ int arg_min(const int (&k)[8]) {
+  int best = k[0], at = 0;
+#pragma unroll
+  for (int i = 1; i < 8; ++i) {
+    if constexpr (WGT) { if (k[i] <= best) { best = k[i]; at = i; } }
+    else best = min(best, k[i]);
+  }
+  return WGT ? at : 7 - (best & 7);
+}
+// Stage 2: positions of the outliers, ascending (-1: none).  order_mask turns the ranking round when the least significant
+// values are taken (SDQ_ORDER_SMALL); sv4: S-Vectors of 4, one outlier in each half.
+template <bool WGT, int OUTN>
+__device__ __forceinline__ void pick_outliers(const int (&key)[8], int order_mask, bool sv4, int& o0, int& o1) {
+  o0 = o1 = -1;
+  if constexpr (OUTN > 0) {
+    int k[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) k[i] = key[i] ^ order_mask;
+    if (OUTN == 2 && sv4) {
+      o0 = arg_max<WGT, 0, 4>(k);
+      o1 = arg_max<WGT, 4, 8>(k);
+    } else {
+      o0 = arg_max<WGT, 0, 8>(k);
+      if constexpr (OUTN == 2) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) k[i] = i == o0 ? -1 : k[i];
+        o1 = arg_max<WGT, 0, 8>(k);
+        const int lo = min(o0, o1);
+        o1 = max(o0, o1);
+        o0 = lo;
+      }
+    }
+  }
+}
+// element `at` of the S-Vector as a float
+__device__ __forceinline__ float pick_value(const uint32_t (&r)[4], int at) {
+  const uint32_t w = (at & 4) ? ((at & 2) ? r[3] : r[2]) : ((at & 2) ? r[1] : r[0]);
+  return __uint_as_float((at & 1) ? (w & 0xFFFF0000u) : (w << 16));
+}
+// r with position `at` zeroed (at = -1: nothing)
+__device__ __forceinline__ void zero_at(uint32_t (&r)[4], int at) {
+  const uint32_t keep = (at & 1) ? 0x0000FFFFu : 0xFFFF0000u;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) r[j] &= (at >> 1) == j ? keep : 0xFFFFFFFFu;
+}
+// Stage 1, pair-wise 4:8: the 2 pairs (of 4) with the largest summed significance among the non-outliers (x: outliers
+// zeroed), largest first, ties to the lower index.  A pair stays if it comes before at least two of the other three.
+// Returns the two pairs in ascending order and the pattern nibble j0 | j1 << 2.
+template <bool WGT>
+__device__ __forceinline__ void pick_pairs(const uint32_t (&x)[4], const int (&key)[8], int o0, int o1, uint32_t& w0, uint32_t& w1, uint32_t& nibble) {
+  float s[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    if constexpr (WGT) {
+      const float a = (2 * j == o0 || 2 * j == o1) ? 0.0f : __int_as_float(key[2 * j]);
+      const float b = (2 * j + 1 == o0 || 2 * j + 1 == o1) ? 0.0f : __int_as_float(key[2 * j + 1]);
+      s[j] = __fadd_rn(a, b);
+    } else {
+      s[j] = __fadd_rn(fabsf(__uint_as_float(x[j] << 16)), fabsf(__uint_as_float(x[j] & 0xFFFF0000u)));
+    }
+  }
+  const bool b01 = s[0] >= s[1], b02 = s[0] >= s[2], b03 = s[0] >= s[3], b12 = s[1] >= s[2], b13 = s[1] >= s[3], b23 = s[2] >= s[3];
+  const bool k0 = (b01 && b02) || (b03 && (b01 || b02));
+  const bool k1 = (!b01 && b12) || (b13 && (!b01 || b12));
+  const bool k3 = (!b03 && !b13) || (!b23 && (!b03 || !b13));
+  const bool k2 = !((k0 && k1) || (k3 && (k0 || k1)));
+  w0 = k0 ? x[0] : (k1 ? x[1] : x[2]);
+  w1 = k3 ? x[3] : (k2 ? x[2] : x[1]);
+  nibble = (k0 ? 0u : (k1 ? 1u : 2u)) | (k3 ? 12u : (k2 ? 8u : 4u));
+}
+// Stage 1 for the patterns stored dense: nibble i of the result is 15 if position i holds +0 -- the outliers and, among the
+// others, all but the keep_in most significant (of every 8, or of every 4 with grp4).  k: ranking keys, -1 at the outliers.
+template <bool WGT, int OUTN>
+__device__ __forceinline__ uint32_t dropped_nibbles(int (&k)[8], int o0, int o1, int keep_in, bool grp4) {
+  uint32_t m = 0;                                   // bit 4 i: position i holds +0
+  if (!grp4 && keep_in + OUTN >= 7) {
+    if (OUTN > 0) m |= 1u << (4 * o0);
+    if (OUTN > 1) m |= 1u << (4 * o1);
+    if (keep_in + OUTN == 7) {                      // exactly one value more: the last in rank order
+#pragma unroll
+      for (int i = 0; i < 8; ++i) k[i] = k[i] < 0 ? 0x7FFFFFFF : k[i];
+      m |= 1u << (4 * arg_min<WGT>(k));
+    }
+  } else {
+    uint32_t rank = 0;                              // nibble i: how many come before position i
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+      for (int j = i + 1; j < 8; ++j) {
+        if ((i >> 2) == (j >> 2) || !grp4) rank += k[i] >= k[j] ? (1u << (4 * j)) : (1u << (4 * i));
+      }
+    m = ((rank + (uint32_t)(8 - keep_in) * 0x11111111u) >> 3) & 0x11111111u;
+  }
+  return m * 15u;
+}
+
+struct PackParams {
+  const __nv_bfloat16* W;
+  int64_t N, K, ldw;
+  const float* colw;           // per-channel weights of the product metric, or nullptr
+  uint8_t* blob;
+  PackedOffsets off;
+  uint32_t* nonfinite;         // host-visible word, set to 1 when a weight (or channel weight) is not finite
+  int out_n, keep_in, order_mask;
+  int sv4, elem, ue, i8, b32, ceil_rule;
 };
 
-// S-Vectors of 4: the most significant of positions 0..3 and of positions 4..7 (ties to the lower index)
-__device__ __forceinline__ void select_outliers_per_4(const uint32_t (&key)[8], bool small, int& o0, int& o1) {
-  o0 = 0; o1 = 4;
-#pragma unroll
-  for (int i = 1; i < 4; ++i) {
-    if (small ? key[i] < key[o0] : key[i] > key[o0]) o0 = i;
-    if (small ? key[4 + i] < key[o1] : key[4 + i] > key[o1]) o1 = 4 + i;
-  }
-}
-
-// Stage 1, pair-wise 4:8: the 2 pairs (of 4) with the largest summed significance among the non-outliers (one fp32 add
-// per pair, largest first, ties to the lower index), ascending
-__device__ __forceinline__ void select_pairs(const uint32_t (&key)[8], const uint32_t (&skey)[8], bool weighted, int o0, int o1,
-                                             int& j0, int& j1) {
-  float score[4];
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const float a0 = (2 * j == o0 || 2 * j == o1) ? 0.0f : key_value(key[2 * j], skey[2 * j], weighted);
-    const float a1 = (2 * j + 1 == o0 || 2 * j + 1 == o1) ? 0.0f : key_value(key[2 * j + 1], skey[2 * j + 1], weighted);
-    score[j] = __fadd_rn(a0, a1);
-  }
-  j0 = 0;
-#pragma unroll
-  for (int j = 1; j < 4; ++j)
-    if (score[j] > score[j0]) j0 = j;
-  j1 = -1;
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    if (j == j0) continue;
-    if (j1 < 0 || score[j] > score[j1]) j1 = j;
-  }
-  if (j0 > j1) { int t = j0; j0 = j1; j1 = t; }
-}
-
-__global__ void __launch_bounds__(128)
-pack_kernel(const __nv_bfloat16* __restrict__ W, int64_t N, int64_t K, int64_t ldw, sdq_config_t cfg, const float* __restrict__ colw,
-            uint8_t* __restrict__ blob, PackedOffsets off, uint32_t* __restrict__ flags)
+// ---- launch 1: per row the outlier scale, the inlier factor of two-level scaling, non-finite check.  One warp per row.
+// SELECT = false: the outliers hold the row's largest magnitude, so nothing has to be selected (magnitude metric, most
+// significant values first, no two-level scaling).
+template <bool SELECT, bool WGT, int OUTN>
+__global__ void __launch_bounds__(256)
+row_scale_kernel(const PackParams p, const BlobHeader hdr)
 {
-  const int64_t n = blockIdx.x;
-  const int tid = threadIdx.x;
-  const int G = (int)(K / 8);
-  const int out_n = cfg.out_n;
-  const __nv_bfloat16* wrow = W + n * ldw;
-  __shared__ uint32_t s_red[4], s_red_in[4];
-  __shared__ int s_e, s_t;
-  const bool sv4 = cfg.in_gran == SDQ_GRAN_3OF4;          // S-Vectors of 4: one outlier and two inliers per 4
-  const bool small = cfg.out_order == SDQ_ORDER_SMALL;   // Stage 2 takes the least significant values (study control)
-  const bool ue = cfg.scale_rule == SDQ_SCALE_UE4M3;     // two-level scaling with E4M3 Q-Vector scales (pair-wise, block 32)
-  const bool i8 = cfg.out_fmt == SDQ_OUT_INT8;           // int8 outliers with an fp32 row scale
-
-  // ---- pass 1: largest outlier magnitude of the row (and, for two-level scaling, largest kept inlier), non-finite check
-  uint32_t okey_max = 0, ikey_max = 0, bad = 0;
-  for (int g = tid; g < G; g += 128) {
-    uint32_t bits[8], key[8];
-    load_group(wrow + 8 * g, bits);
+  const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t n = (int64_t)blockIdx.x * 8 + warp;               // N is a multiple of 128
+  if (blockIdx.x == 0 && threadIdx.x < HEADER_BYTES / 4)          // the self-describing header, zero-filled to its reservation
+    reinterpret_cast<uint32_t*>(p.blob)[threadIdx.x] =
+        threadIdx.x < sizeof(BlobHeader) / 4 ? reinterpret_cast<const uint32_t*>(&hdr)[threadIdx.x] : 0u;
+  const uint4* row = reinterpret_cast<const uint4*>(p.W + n * p.ldw);
+  const int G = (int)(p.K / 8);
+  uint32_t all2 = 0, omax = 0, imax = 0, bad = 0;                 // all2: two packed running maxima of the magnitudes
+  if constexpr (!SELECT) {
+    int g = (int)lane;
+    for (; g + 96 < G; g += 128) {
+      uint4 v[4];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      key[i] = bits[i] & 0x7FFFu;
-      bad |= (key[i] >= 0x7F80u);
+      for (int u = 0; u < 4; ++u) v[u] = __ldg(row + g + 32 * u);
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        all2 = __vmaxu2(all2, __vmaxu2(__vmaxu2(v[u].x & 0x7FFF7FFFu, v[u].y & 0x7FFF7FFFu), __vmaxu2(v[u].z & 0x7FFF7FFFu, v[u].w & 0x7FFF7FFFu)));
     }
-    uint32_t skey[8];
-    bad |= selection_keys(key, colw, g, skey);
-    int o0, o1;
-    if (sv4 && out_n) select_outliers_per_4(skey, small, o0, o1); else select_outliers(skey, out_n, small, o0, o1);
-    if (o0 >= 0) okey_max = max(okey_max, key[o0]);
-    if (o1 >= 0) okey_max = max(okey_max, key[o1]);
-    if (ue) {
-      int j0, j1;
-      select_pairs(key, skey, colw != nullptr, o0, o1, j0, j1);
-      const int pos[4] = {2 * j0, 2 * j0 + 1, 2 * j1, 2 * j1 + 1};
-#pragma unroll
-      for (int s = 0; s < 4; ++s)
-        if (pos[s] != o0 && pos[s] != o1) ikey_max = max(ikey_max, key[pos[s]]);
+    for (; g < G; g += 32) {
+      const uint4 v = __ldg(row + g);
+      all2 = __vmaxu2(all2, __vmaxu2(__vmaxu2(v.x & 0x7FFF7FFFu, v.y & 0x7FFF7FFFu), __vmaxu2(v.z & 0x7FFF7FFFu, v.w & 0x7FFF7FFFu)));
     }
-  }
+    omax = max(all2 & 0xFFFFu, all2 >> 16);
+    bad = omax >= 0x7F80u;
+  } else {
+#pragma unroll 2
+    for (int g = (int)lane; g < G; g += 32) {
+      const uint4 v = __ldg(row + g);
+      uint32_t r[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-  for (int s = 16; s > 0; s >>= 1) {
-    okey_max = max(okey_max, __shfl_xor_sync(0xffffffffu, okey_max, s));
-    ikey_max = max(ikey_max, __shfl_xor_sync(0xffffffffu, ikey_max, s));
-    bad |= __shfl_xor_sync(0xffffffffu, bad, s);
+      for (int j = 0; j < 4; ++j) all2 = __vmaxu2(all2, r[j] & 0x7FFF7FFFu);
+      if constexpr (WGT) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) { const float c = __ldg(p.colw + 8 * (int64_t)g + i); bad |= !(c >= 0.0f && c <= 3.4028234663852886e38f); }
+      }
+      int k[8], o0, o1;
+      rank_keys<WGT>(r, WGT ? p.colw + 8 * (int64_t)g : nullptr, k);
+      pick_outliers<WGT, OUTN>(k, p.order_mask, p.sv4 != 0, o0, o1);
+      if constexpr (OUTN > 0) omax = max(omax, __float_as_uint(pick_value(r, o0)) << 1 >> 17);
+      if constexpr (OUTN > 1) omax = max(omax, __float_as_uint(pick_value(r, o1)) << 1 >> 17);
+      if (p.ue) {                                                 // pair-wise pattern: the largest inlier that stays
+        if constexpr (OUTN > 0) zero_at(r, o0);
+        if constexpr (OUTN > 1) zero_at(r, o1);
+        uint32_t w0, w1, nibble;
+        pick_pairs<WGT>(r, k, o0, o1, w0, w1, nibble);
+        const uint32_t m = __vmaxu2(w0 & 0x7FFF7FFFu, w1 & 0x7FFF7FFFu);
+        imax = max(imax, max(m & 0xFFFFu, m >> 16));
+      }
+    }
+    bad |= max(all2 & 0xFFFFu, all2 >> 16) >= 0x7F80u;
   }
-  if ((tid & 31) == 0) { s_red[tid >> 5] = okey_max; s_red_in[tid >> 5] = ikey_max; }
-  if (bad && (tid & 31) == 0) atomicOr(&flags[FLAG_NONFINITE], 1u);
-  __syncthreads();
-  if (tid == 0) {
-    uint32_t m = max(max(s_red[0], s_red[1]), max(s_red[2], s_red[3]));
+  omax = __reduce_max_sync(0xffffffffu, omax);
+  imax = __reduce_max_sync(0xffffffffu, imax);
+  bad = __any_sync(0xffffffffu, bad != 0);
+  if (lane == 0) {
+    if (bad) *reinterpret_cast<volatile uint32_t*>(p.nonfinite) = 1u;
+    const float a = bf16_bits_to_float(OUTN ? omax : 0u);
     // int8 outliers: the row's fp32 scale amax / 127 travels as its bit pattern in the place of the exponent
-    s_e = i8 ? __float_as_int(int8_scale(bf16_bits_to_float(m))) : fp8_scale_exp(bf16_bits_to_float(m));
-    const uint32_t mi = max(max(s_red_in[0], s_red_in[1]), max(s_red_in[2], s_red_in[3]));
-    s_t = ue ? fp8_scale_exp(bf16_bits_to_float(mi)) : 0;   // exponent of the row's inlier factor 2^t
-  }
-  __syncthreads();
-  const int e = s_e, tw = s_t;
-
-  const int64_t rt = n / TILE_ROWS;
-  const uint32_t r = (uint32_t)(n % TILE_ROWS);
-  const int T1 = (int)(K / K1), T2 = (int)(K / K2);
-  const bool b32 = cfg.in_block == 32, dense = is_dense_layout(cfg);
-  const bool elem = cfg.in_gran == SDQ_GRAN_ELEM;        // element-wise 2:4: the 2 most significant non-outliers of every 4
-  const bool grp4 = sv4 || elem;                         // Stage 1 ranks inside groups of 4
-  // dense family: inliers kept per group (8 - out_n without Stage 1; groups of 4: 3 minus the outlier, or 2 for 2:4)
-  const int keep_in = elem ? 2 : (sv4 ? (out_n ? 2 : 3) : 10 - cfg.in_gran - out_n);
-  const int wib = wi_bytes(b32, dense);
-  uint8_t* wi_base = blob + off.wi + (size_t)rt * T2 * wib;
-  uint8_t* wo_base = blob + off.wo + (size_t)rt * T1 * WO_BYTES;
-
-  if (tid == 0) {
-    reinterpret_cast<int32_t*>(blob + off.osexp)[n] = e;
-    reinterpret_cast<int32_t*>(blob + off.wtexp)[n] = tw;
+    const int e = p.i8 ? __float_as_int(int8_scale(a)) : fp8_scale_exp(a);
+    const int tw = p.ue ? fp8_scale_exp(bf16_bits_to_float(imax)) : 0;       // exponent of the row's inlier factor 2^t
+    reinterpret_cast<int32_t*>(p.blob + p.off.osexp)[n] = e;
+    reinterpret_cast<int32_t*>(p.blob + p.off.wtexp)[n] = tw;
     // the accumulator of a row is kept in units of 2^tw (the inlier scale codes leave that factor out), so the outlier
     // row scale is 2^(e - tw); the GEMM's epilogue multiplies the factor back in
-    const uint32_t c = i8 ? 127u : (uint32_t)min(max(e - tw + 127, 0), 254);    // (int8: the epilogue applies the scales)
-    *reinterpret_cast<uint32_t*>(blob + off.sfa_out + (size_t)rt * SF_ATOM_BYTES + sf_off(r, 0)) = c * 0x01010101u;
-  }
-
-  // ---- pass 2 (G is a multiple of 32, so whole warps iterate together)
-  for (int g = tid; g < G; g += 128) {
-    uint32_t bits[8], key[8];
-    load_group(wrow + 8 * g, bits);
-#pragma unroll
-    for (int i = 0; i < 8; ++i) key[i] = bits[i] & 0x7FFFu;
-    uint32_t skey[8];
-    selection_keys(key, colw, g, skey);
-    int o0, o1;
-    if (sv4 && out_n) select_outliers_per_4(skey, small, o0, o1); else select_outliers(skey, out_n, small, o0, o1);
-    const int k1 = g >> 4, k2 = g >> 5;
-    uint8_t* wi = wi_base + (size_t)k2 * wib;
-    uint8_t* wo = wo_base + (size_t)k1 * WO_BYTES;
-
-    if (dense) {
-      // all eight positions are inlier slots; an outlier position holds +0, and so does a value that Stage 1 drops: a
-      // non-outlier survives if fewer than keep_in non-outliers rank before it (more significant, or equal with a
-      // lower index).  Stage 3 with one scale per 32 K = 4 S-Vectors = 4 lanes
-      uint32_t gone = 0;        // bit i: position i holds +0
-      uint32_t ikey = 0;
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        int before = 0;
-#pragma unroll
-        for (int j = 0; j < 8; ++j)
-          before += (j != o0 && j != o1 && (!grp4 || (j >> 2) == (i >> 2)) && (skey[j] > skey[i] || (skey[j] == skey[i] && j < i))) ? 1 : 0;
-        if (i == o0 || i == o1 || before >= keep_in) gone |= 1u << i;
-        else ikey = max(ikey, key[i]);
-      }
-      ikey = max(ikey, __shfl_xor_sync(0xffffffffu, ikey, 1));
-      ikey = max(ikey, __shfl_xor_sync(0xffffffffu, ikey, 2));
-      const uint32_t c = e8m0_scale_code(bf16_bits_to_float(ikey), cfg.scale_rule);
-      uint32_t codes = 0;
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const float v0 = ((gone >> (2 * i)) & 1) ? 0.0f : bf16_bits_to_float(bits[2 * i]) * pow2_inv_e8m0(c);
-        const float v1 = ((gone >> (2 * i + 1)) & 1) ? 0.0f : bf16_bits_to_float(bits[2 * i + 1]) * pow2_inv_e8m0(c);
-        codes |= e2m1x2(v0, v1) << (8 * i);
-      }
-      // 32 S-Vectors per 256-K stage, 4 code bytes each: bytes 32 j .. 32 j + 31 = K-block j (64 K)
-      *reinterpret_cast<uint32_t*>(wi + a_off(r, (uint32_t)(g & 31) * 4)) = codes;
-      if ((g & 3) == 0) wi[a_in_bytes(true) + in_sf_off(true, r, (uint32_t)((g >> 2) & 7))] = (uint8_t)c;
-      if (elem) {
-        // the kept indices (two ascending 2-bit values per group of 4) are only needed by the exporter
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const uint32_t kept = (~(gone >> (4 * h))) & 15u;            // exactly two bits
-          const int i0 = __ffs((int)kept) - 1, i1 = 31 - __clz((int)kept);
-          blob[off.emeta + (size_t)n * (size_t)(K / 4) + 2 * g + h] = (uint8_t)(i0 | (i1 << 2));
-        }
-      }
-    } else {
-    // Stage 1 on the remaining values: keep the 2 pairs (of 4) with the largest summed significance
-    int j0, j1;
-    select_pairs(key, skey, colw != nullptr, o0, o1, j0, j1);
-    const int slot_pos[4] = {2 * j0, 2 * j0 + 1, 2 * j1, 2 * j1 + 1};
-
-    // Stage 3, inliers: Q-Vector (64 K = 8 S-Vectors = 8 lanes, or 32 K = 4 lanes) largest kept magnitude -> E8M0 scale
-    uint32_t ikey = 0;
-#pragma unroll
-    for (int s = 0; s < 4; ++s) {
-      const int p = slot_pos[s];
-      if (p != o0 && p != o1) ikey = max(ikey, key[p]);
-    }
-    ikey = max(ikey, __shfl_xor_sync(0xffffffffu, ikey, 1));
-    ikey = max(ikey, __shfl_xor_sync(0xffffffffu, ikey, 2));
-    if (!b32) ikey = max(ikey, __shfl_xor_sync(0xffffffffu, ikey, 4));
-    const uint32_t c = ue ? ue4m3_scale_code(bf16_bits_to_float(ikey), tw) : e8m0_scale_code(bf16_bits_to_float(ikey), cfg.scale_rule);
-    const float sv = ue ? ue4m3_scale_value(c, tw) : 0.0f;
-    float v[4];
-#pragma unroll
-    for (int s = 0; s < 4; ++s) {
-      const int p = slot_pos[s];
-      const float w = bf16_bits_to_float(bits[p]);
-      v[s] = (p == o0 || p == o1) ? 0.0f : (ue ? (c ? __fdiv_rn(w, sv) : 0.0f) : w * pow2_inv_e8m0(c));
-    }
-    const uint32_t codes = e2m1x2(v[0], v[1]) | (e2m1x2(v[2], v[3]) << 8);
-
-    // 32 S-Vectors per 256-K stage, 2 code bytes each: bytes 0..31 = K-block 0, 32..63 = K-block 1
-    *reinterpret_cast<uint16_t*>(wi + a_off(r, (uint32_t)(g & 31) * 2)) = (uint16_t)codes;
-    // metadata nibble j0 | j1<<2; two S-Vectors share a byte (even one in the low nibble)
-    uint32_t nib = (uint32_t)(j0 | (j1 << 2));
-    const uint32_t nib_hi = __shfl_down_sync(0xffffffffu, nib, 1);
-    if ((g & 1) == 0) wi[A_IN_BYTES + r * 16 + ((g & 31) >> 1)] = (uint8_t)(nib | (nib_hi << 4));
-    if (b32) { if ((g & 3) == 0) wi[A_IN_BYTES + E_IN_BYTES + in_sf_off(true, r, (uint32_t)((g >> 2) & 7))] = (uint8_t)c; }
-    else if ((g & 7) == 0) wi[A_IN_BYTES + E_IN_BYTES + in_sf_off(false, r, (uint32_t)((g >> 3) & 3))] = (uint8_t)c;
-    }
-
-    if (out_n > 0) {
-      // Stage 3, outliers: E4M3 codes of w / 2^e; compact arrays plus the 2:4 embedding the sparse
-      // FP8 tensor-core path consumes (per 4 K: two ascending slot indices, unused slots hold +0)
-      // (or int8 codes of w / s, Section 5.1)
-      const uint32_t c0 = i8 ? int8_code(bf16_bits_to_float(bits[o0]), __int_as_float(e)) : e4m3x1(bf16_bits_to_float(bits[o0]) * pow2_neg(e));
-      const uint32_t c1 = (o1 >= 0) ? (i8 ? int8_code(bf16_bits_to_float(bits[o1]), __int_as_float(e)) : e4m3x1(bf16_bits_to_float(bits[o1]) * pow2_neg(e))) : 0u;
-      // compact record of the 128-K stage: codes, then position nibbles (two S-Vectors share a byte when out_n = 1)
-      uint8_t* wc = blob + off.wc + ((size_t)rt * T1 + k1) * (size_t)wc_bytes(out_n);
-      const uint32_t gi = (uint32_t)(g & 15);
-      if (out_n == 1) {
-        wc[r * 16 + gi] = (uint8_t)c0;
-        const uint32_t pos_hi = __shfl_down_sync(0xffffffffu, (uint32_t)o0, 1);
-        if ((g & 1) == 0) wc[WC_CODE_BYTES + r * 8 + (gi >> 1)] = (uint8_t)((uint32_t)o0 | (pos_hi << 4));
-      } else {
-        *reinterpret_cast<uint16_t*>(wc + r * 32 + gi * 2) = (uint16_t)(c0 | (c1 << 8));
-        wc[2 * WC_CODE_BYTES + r * 16 + gi] = (uint8_t)((uint32_t)o0 | ((uint32_t)o1 << 4));
-      }
-      uint32_t stored = 0, meta = 0;
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int a = (o0 >= 4 * h && o0 < 4 * h + 4) ? (o0 - 4 * h) : -1;
-        const int b = (o1 >= 4 * h && o1 < 4 * h + 4) ? (o1 - 4 * h) : -1;
-        int i0, i1;
-        uint32_t s0 = 0, s1 = 0;
-        if (a >= 0 && b >= 0) { i0 = a; i1 = b; s0 = c0; s1 = c1; }
-        else if (a >= 0 || b >= 0) {
-          const int p = (a >= 0) ? a : b;
-          const uint32_t cc = (a >= 0) ? c0 : c1;
-          if (p < 3) { i0 = p; i1 = 3; s0 = cc; } else { i0 = 0; i1 = 3; s1 = cc; }
-        } else { i0 = 0; i1 = 1; }
-        stored |= (s0 | (s1 << 8)) << (16 * h);
-        meta |= (uint32_t)(i0 | (i1 << 2)) << (4 * h);
-      }
-      // 16 S-Vectors per 128-K stage, 4 stored bytes each: bytes 0..31 = K-block 0 (64 K), 32..63 = K-block 1
-      *reinterpret_cast<uint32_t*>(wo + a_off(r, (uint32_t)(g & 15) * 4)) = stored;
-      wo[A_OUT_BYTES + r * 16 + (g & 15)] = (uint8_t)meta;
-    }
+    const uint32_t c = p.i8 ? 127u : (uint32_t)min(max(e - tw + 127, 0), 254);    // (int8: the epilogue applies the scales)
+    *reinterpret_cast<uint32_t*>(p.blob + p.off.sfa_out + (size_t)(n / TILE_ROWS) * SF_ATOM_BYTES + sf_off((uint32_t)(n % TILE_ROWS), 0)) = c * 0x01010101u;
   }
 }
+
+// ---- launch 2
+constexpr int PK_THREADS = 256;
+constexpr int PK_PITCH = 512 + 16;                       // bytes between rows of the staged tile
+constexpr int PK_SMEM = TILE_ROWS * PK_PITCH;            // 67584: three CTAs per SM
+
+template <bool DENSE, bool WGT, int OUTN>
+__global__ void __launch_bounds__(PK_THREADS, 3)
+pack_tile_kernel(const PackParams p)
+{
+  extern __shared__ __align__(16) uint8_t tile[];
+  const uint32_t tid = threadIdx.x;
+  const int T2 = (int)(p.K / K2), T1 = 2 * T2;
+  const int rt = (int)(blockIdx.x / (uint32_t)T2), k2 = (int)(blockIdx.x % (uint32_t)T2);
+  {
+    // 256 threads: 8 rows per round, 32 lanes x 16 B = the 512 B of one row
+    const uint32_t row = tid >> 5, lane = tid & 31;
+    const uint8_t* src = reinterpret_cast<const uint8_t*>(p.W + ((int64_t)rt * TILE_ROWS + row) * p.ldw + (int64_t)k2 * K2) + lane * 16;
+    const uint32_t dst = (uint32_t)__cvta_generic_to_shared(tile) + row * PK_PITCH + lane * 16;
+#pragma unroll
+    for (int i = 0; i < TILE_ROWS / 8; ++i)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + i * 8 * PK_PITCH), "l"(src + (int64_t)i * 16 * p.ldw) : "memory");
+    asm volatile("cp.async.wait_all;" ::: "memory");
+  }
+  const uint32_t r = tid & 127u, h = tid >> 7;           // this thread's row and 128-K half
+  const int64_t n = (int64_t)rt * TILE_ROWS + r;
+  const int e = reinterpret_cast<const int32_t*>(p.blob + p.off.osexp)[n];
+  const int tw = p.ue ? reinterpret_cast<const int32_t*>(p.blob + p.off.wtexp)[n] : 0;
+  __syncthreads();
+
+  const bool b32 = DENSE || p.b32 != 0;
+  uint8_t* wi = p.blob + p.off.wi + ((size_t)rt * T2 + k2) * (size_t)wi_bytes(b32, DENSE);
+  uint8_t* wo = p.blob + p.off.wo + ((size_t)rt * T1 + 2 * k2 + h) * (size_t)WO_BYTES;
+  uint8_t* wc = p.blob + p.off.wc + ((size_t)rt * T1 + 2 * k2 + h) * (size_t)wc_bytes(OUTN);
+  const uint8_t* mine = tile + r * PK_PITCH + h * 256;
+  const float* colw = WGT ? p.colw + (int64_t)k2 * K2 + h * K1 : nullptr;
+  const float s8 = pow2_neg(e);
+  const uint32_t core = (r >> 3) * 256 + (r & 7) * 16;   // this row inside a K-block of an A operand
+
+  uint32_t in_word[2][2];                                // pair-wise inliers: the 64-K half's codes, two S-Vectors per word
+  uint32_t nib = 0, sc = 0;                              // its pattern nibbles; scale bytes of the 128 K
+  uint32_t kept[16];                                     // pair-wise inliers of a Q-Vector of 64 K, outlier positions zeroed
+  uint32_t qmax2 = 0;                                    // packed running maximum of the Q-Vector
+#pragma unroll
+  for (int b = 0; b < 4; ++b) {                          // blocks of 4 S-Vectors (32 K)
+    uint32_t ocode[4], ocode1[4], opos[4], opos1[4];
+    uint32_t dense_codes[4], dval[16];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const uint4 v = *reinterpret_cast<const uint4*>(mine + (4 * b + i) * 16);
+      uint32_t x[4] = {v.x, v.y, v.z, v.w};
+      int k[8], o0, o1;
+      rank_keys<WGT>(x, WGT ? colw + 8 * (4 * b + i) : nullptr, k);
+      pick_outliers<WGT, OUTN>(k, p.order_mask, p.sv4 != 0, o0, o1);
+      // Stage 3, outliers: E4M3 codes of w / 2^e, or int8 codes of w / s
+      if constexpr (OUTN > 0) {
+        const float f = pick_value(x, o0);
+        ocode[i] = p.i8 ? int8_code(f, __int_as_float(e)) : e4m3x1(f * s8);
+        opos[i] = (uint32_t)o0;
+      }
+      if constexpr (OUTN > 1) {
+        const float f = pick_value(x, o1);
+        ocode1[i] = p.i8 ? int8_code(f, __int_as_float(e)) : e4m3x1(f * s8);
+        opos1[i] = (uint32_t)o1;
+      }
+      if constexpr (!DENSE) {
+        // Stage 1: the two pairs that stay, outlier positions at +0
+        if constexpr (OUTN > 0) zero_at(x, o0);
+        if constexpr (OUTN > 1) zero_at(x, o1);
+        uint32_t w0, w1, nibble;
+        pick_pairs<WGT>(x, k, o0, o1, w0, w1, nibble);
+        kept[2 * (4 * (b & 1) + i)] = w0;
+        kept[2 * (4 * (b & 1) + i) + 1] = w1;
+        qmax2 = __vmaxu2(qmax2, __vmaxu2(w0 & 0x7FFF7FFFu, w1 & 0x7FFF7FFFu));
+        nib |= nibble << (4 * (4 * (b & 1) + i));
+      } else {
+        if constexpr (OUTN > 0) {
+#pragma unroll
+          for (int j = 0; j < 8; ++j) k[j] = (j == o0 || (OUTN > 1 && j == o1)) ? -1 : k[j];
+        }
+        uint32_t mag = 0;                                // largest magnitude of the inliers
+        if constexpr (!WGT) {
+#pragma unroll
+          for (int j = 0; j < 8; ++j) mag = (uint32_t)max((int)mag, k[j]);   // the most significant non-outlier always stays
+          mag >>= 16;
+        }
+        const uint32_t gone = dropped_nibbles<WGT, OUTN>(k, o0, o1, p.keep_in, p.sv4 || p.elem);
+        if constexpr (WGT) {
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            mag = max(mag, (gone >> (8 * j)) & 1u ? 0u : (x[j] & 0x7FFFu));
+            mag = max(mag, (gone >> (8 * j + 4)) & 1u ? 0u : ((x[j] >> 16) & 0x7FFFu));
+          }
+        }
+        qmax2 = max(qmax2, mag);
+        dense_codes[i] = ~gone;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) dval[4 * i + j] = x[j];
+        if (p.elem) {
+          // the kept indices (two ascending 2-bit values per group of 4) are only needed by the exporter
+          uint32_t mb = 0;
+#pragma unroll
+          for (int q = 0; q < 2; ++q) {
+            const uint32_t g4 = ~gone >> (16 * q);       // nibbles of the group's four positions, exactly two of them set
+            const uint32_t bits = (g4 & 1u) | ((g4 >> 3) & 2u) | ((g4 >> 6) & 4u) | ((g4 >> 9) & 8u);
+            mb |= (uint32_t)((__ffs((int)bits) - 1) | ((31 - __clz((int)bits)) << 2)) << (8 * q);
+          }
+          reinterpret_cast<uint16_t*>(p.blob + p.off.emeta + (size_t)n * (size_t)(p.K / 4))[(k2 * 2 + (int)h) * 16 + 4 * b + i] = (uint16_t)mb;
+        }
+      }
+    }
+
+    // ---- Stage 3, inliers
+    if constexpr (DENSE) {
+      const uint32_t c = e8m0_scale_code_bf16(qmax2, p.ceil_rule != 0);
+      const float inv = pow2_inv_e8m0(c);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        float f[8];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          f[2 * j] = __uint_as_float(dval[4 * i + j] << 16) * inv;
+          f[2 * j + 1] = __uint_as_float(dval[4 * i + j] & 0xFFFF0000u) * inv;
+        }
+        dense_codes[i] &= e2m1x8(f);
+      }
+      // 16 code bytes per 32 K: K-block (64 K) 2 h + b / 2 of the record, chunk b & 1
+      *reinterpret_cast<uint4*>(wi + (2 * h + (b >> 1)) * 4096 + core + (b & 1) * 128) = make_uint4(dense_codes[0], dense_codes[1], dense_codes[2], dense_codes[3]);
+      sc |= c << (8 * b);
+      qmax2 = 0;
+    } else if ((b & 1) || b32) {
+      // a Q-Vector is complete: 64 K (both blocks of the half) or 32 K (this one)
+      const uint32_t key = max(qmax2 & 0xFFFFu, qmax2 >> 16);
+      const uint32_t c = p.ue ? ue4m3_scale_code(bf16_bits_to_float(key), tw) : e8m0_scale_code_bf16(key, p.ceil_rule != 0);
+      const float sv = p.ue ? ue4m3_scale_value(c, tw) : 0.0f, inv = pow2_inv_e8m0(c);
+#pragma unroll
+      for (int hb = 0; hb < 2; ++hb) {                   // 32-K block of the half
+        if (hb != (b & 1) && b32) continue;              // (one scale per 64 K: both now)
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {                    // two S-Vectors per code word
+          float f[8];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const uint32_t w = kept[8 * hb + 4 * i + j];
+            const float lo = __uint_as_float(w << 16), hi = __uint_as_float(w & 0xFFFF0000u);
+            if (p.ue) {
+              // (an outlier's position stays +0; the quotient of a dropped one is +0 as well)
+              f[2 * j] = c ? __fdiv_rn(lo, sv) : 0.0f;
+              f[2 * j + 1] = c ? __fdiv_rn(hi, sv) : 0.0f;
+            } else {
+              f[2 * j] = lo * inv;
+              f[2 * j + 1] = hi * inv;
+            }
+          }
+          in_word[hb][i] = e2m1x8(f);
+        }
+      }
+      if (b32) { sc |= c << (8 * b); }
+      else sc |= c << (8 * (b >> 1));
+      qmax2 = 0;
+    }
+    if constexpr (!DENSE) {
+      if (b & 1) {
+        // 16 code bytes per 64 K (K-block h, chunk b / 2) and 4 bytes of pattern nibbles
+        *reinterpret_cast<uint4*>(wi + h * 4096 + core + (b >> 1) * 128) = make_uint4(in_word[0][0], in_word[0][1], in_word[1][0], in_word[1][1]);
+        *reinterpret_cast<uint32_t*>(wi + A_IN_BYTES + r * 16 + h * 8 + (b >> 1) * 4) = nib;
+        nib = 0;
+      }
+    }
+
+    // ---- outliers of the 4 S-Vectors: compact record, and the 2:4 embedding the sparse FP8 path consumes (per 4 K two
+    // ascending slot indices, unused slots hold +0)
+    if constexpr (OUTN == 1) {
+      // per S-Vector: position ps (0..7) sits in group of 4 number ps >> 2 at p = ps & 3, whose slots are (p, 3), the value
+      // first, or (0, 3), the value second, when p = 3; the other group has slots (0, 1).  Metadata bytes and byte shifts
+      // come from 8-entry tables looked up by byte-permutes, the four position nibbles being the selector.
+      const uint32_t codes = ocode[0] | (ocode[1] << 8) | (ocode[2] << 16) | (ocode[3] << 24);
+      const uint32_t sel = opos[0] | (opos[1] << 4) | (opos[2] << 8) | (opos[3] << 12);
+      const uint32_t meta = __byte_perm(0x4C4E4D4Cu, 0xC4E4D4C4u, sel), sh = __byte_perm(0x08000000u, 0x18101010u, sel);
+      *reinterpret_cast<uint4*>(wo + (b >> 1) * 4096 + core + (b & 1) * 128) =
+          make_uint4(ocode[0] << (sh & 31u), ocode[1] << ((sh >> 8) & 31u), ocode[2] << ((sh >> 16) & 31u), ocode[3] << (sh >> 24));
+      *reinterpret_cast<uint32_t*>(wo + A_OUT_BYTES + r * 16 + 4 * b) = meta;
+      *reinterpret_cast<uint32_t*>(wc + r * 16 + 4 * b) = codes;
+      *reinterpret_cast<uint16_t*>(wc + WC_CODE_BYTES + r * 8 + 2 * b) = (uint16_t)sel;
+    } else if constexpr (OUTN == 2) {
+      uint32_t st[4], meta = 0;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int o0 = (int)opos[i], o1 = (int)opos1[i];
+        st[i] = 0;
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          const bool in0 = (o0 >> 2) == q, in1 = (o1 >> 2) == q;
+          uint32_t s, m;
+          if (in0 && in1) { s = ocode[i] | (ocode1[i] << 8); m = (uint32_t)((o0 & 3) | ((o1 & 3) << 2)); }
+          else if (in0 || in1) {
+            const uint32_t pp = (uint32_t)((in0 ? o0 : o1) & 3), cc = in0 ? ocode[i] : ocode1[i];
+            s = pp == 3u ? cc << 8 : cc;
+            m = (pp == 3u ? 0u : pp) | 12u;
+          } else { s = 0; m = 4u; }
+          st[i] |= s << (16 * q);
+          meta |= m << (8 * i + 4 * q);
+        }
+      }
+      *reinterpret_cast<uint4*>(wo + (b >> 1) * 4096 + core + (b & 1) * 128) = make_uint4(st[0], st[1], st[2], st[3]);
+      *reinterpret_cast<uint32_t*>(wo + A_OUT_BYTES + r * 16 + 4 * b) = meta;
+      *reinterpret_cast<uint2*>(wc + r * 32 + 8 * b) =
+          make_uint2(ocode[0] | (ocode1[0] << 8) | (ocode[1] << 16) | (ocode1[1] << 24), ocode[2] | (ocode1[2] << 8) | (ocode[3] << 16) | (ocode1[3] << 24));
+      *reinterpret_cast<uint32_t*>(wc + 2 * WC_CODE_BYTES + r * 16 + 4 * b) =
+          opos[0] | (opos1[0] << 4) | (opos[1] << 8) | (opos1[1] << 12) | (opos[2] << 16) | (opos1[2] << 20) | (opos[3] << 24) | (opos1[3] << 28);
+    }
+  }
+  // ---- inlier scales: one atom per 128-K half with four scales of 32 K, or two scales of 64 K of the one atom
+  uint8_t* sf = wi + a_in_bytes(DENSE) + e_in_bytes(DENSE) + (r & 31) * 16 + (r >> 5) * 4;
+  if (b32) *reinterpret_cast<uint32_t*>(sf + h * SF_ATOM_BYTES) = sc;
+  else *reinterpret_cast<uint16_t*>(sf + 2 * h) = (uint16_t)sc;
+}
+
+template <bool WGT, int OUTN>
+static void launch_pack(const PackParams& p, const BlobHeader& hdr, bool dense, cudaStream_t st)
+{
+  const unsigned rows = (unsigned)(p.N / 8), tiles = (unsigned)((p.N / TILE_ROWS) * (p.K / K2));
+  if (WGT || p.order_mask || p.ue) row_scale_kernel<true, WGT, OUTN><<<rows, 256, 0, st>>>(p, hdr);
+  else row_scale_kernel<false, WGT, OUTN><<<rows, 256, 0, st>>>(p, hdr);
+  if (dense) {
+    cudaFuncSetAttribute(pack_tile_kernel<true, WGT, OUTN>, cudaFuncAttributeMaxDynamicSharedMemorySize, PK_SMEM);
+    pack_tile_kernel<true, WGT, OUTN><<<tiles, PK_THREADS, PK_SMEM, st>>>(p);
+  } else {
+    cudaFuncSetAttribute(pack_tile_kernel<false, WGT, OUTN>, cudaFuncAttributeMaxDynamicSharedMemorySize, PK_SMEM);
+    pack_tile_kernel<false, WGT, OUTN><<<tiles, PK_THREADS, PK_SMEM, st>>>(p);
+  }
+}
+
+// One host-visible word per call in flight, where the kernels report a non-finite weight: a page of pinned memory, taken
+// once per process and kept; a call holds its word until its stream has been synchronised, so calls of other threads and
+// streams never share one.  More calls at once than words wait for one to be given back.
+class ReportWords {
+ public:
+  uint32_t* take() {
+    std::unique_lock<std::mutex> lock(m_);
+    if (!base_) {
+      void* ptr = nullptr;
+      if (cudaHostAlloc(&ptr, COUNT * sizeof(uint32_t), cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) return nullptr;
+      base_ = (uint32_t*)ptr;
+      for (int i = 0; i < COUNT; ++i) free_[i] = i;
+      n_free_ = COUNT;
+    }
+    cv_.wait(lock, [this] { return n_free_ > 0; });
+    uint32_t* w = base_ + free_[--n_free_];
+    *reinterpret_cast<volatile uint32_t*>(w) = 0u;
+    return w;
+  }
+  void give_back(uint32_t* w) {
+    { std::lock_guard<std::mutex> lock(m_); free_[n_free_++] = (int)(w - base_); }
+    cv_.notify_one();
+  }
+ private:
+  static constexpr int COUNT = 64;
+  std::mutex m_;
+  std::condition_variable cv_;
+  uint32_t* base_ = nullptr;
+  int free_[COUNT];
+  int n_free_ = 0;
+};
+static ReportWords g_report;
 
 // outlier t of S-Vector g of row r in row tile rt, from the compact records: code and position
 __device__ __forceinline__ uint8_t wc_code(const uint8_t* blob, const PackedOffsets& off, int64_t rt, int T1, uint32_t r, int g, int out_n, int t) {
@@ -395,14 +638,6 @@ extern "C" sdq_status_t sdq_decompose_metric(const void* W, int64_t N, int64_t K
   const PlainPackedOffsets poff = plain_packed_offsets(N, K, *cfg);
   if (packed_bytes < (tc ? off.total : poff.total)) return SDQ_ERR_BUFFER_TOO_SMALL;
   cudaStream_t st = (cudaStream_t)stream;
-  uint32_t* flags = device_flags();
-  if (!flags) return SDQ_ERR_CUDA;
-  if (cudaMemsetAsync(flags + FLAG_NONFINITE, 0, sizeof(uint32_t), st) != cudaSuccess) return SDQ_ERR_CUDA;
-  if (tc) pack_kernel<<<(unsigned)N, 128, 0, st>>>((const __nv_bfloat16*)W, N, K, ldw, *cfg, col_weight, (uint8_t*)packed_buf, off, flags);
-  else launch_pack_plain(W, N, K, ldw, *cfg, col_weight, packed_buf, flags, st);
-  if (cudaGetLastError() != cudaSuccess) return SDQ_ERR_CUDA;
-  uint32_t nonfinite = 0;
-  if (cudaMemcpyAsync(&nonfinite, flags + FLAG_NONFINITE, sizeof(uint32_t), cudaMemcpyDeviceToHost, st) != cudaSuccess) return SDQ_ERR_CUDA;
   out->dev = packed_buf;
   out->bytes = tc ? off.total : poff.total;
   out->N = N;
@@ -416,12 +651,46 @@ extern "C" sdq_status_t sdq_decompose_metric(const void* W, int64_t N, int64_t K
     out->off[0] = poff.in_code; out->off[1] = poff.in_meta; out->off[2] = poff.in_scale;
     out->off[3] = poff.out_code; out->off[4] = poff.out_idx; out->off[5] = poff.osexp;
   }
-  // the self-describing header (read back by sdq_packed_attach); the copy is complete before `hdr` goes out of scope
-  // because the stream is synchronised below
-  alignas(16) unsigned char hdr[HEADER_BYTES] = {0};
-  fill_header(reinterpret_cast<BlobHeader*>(hdr), *out, tc);
-  if (cudaMemcpyAsync(packed_buf, hdr, HEADER_BYTES, cudaMemcpyHostToDevice, st) != cudaSuccess) return SDQ_ERR_CUDA;
-  if (cudaStreamSynchronize(st) != cudaSuccess) return SDQ_ERR_CUDA;
+  // the self-describing header (read back by sdq_packed_attach)
+  alignas(16) unsigned char raw[HEADER_BYTES] = {0};
+  BlobHeader* hdr = reinterpret_cast<BlobHeader*>(raw);
+  fill_header(hdr, *out, tc);
+  uint32_t* report = g_report.take();
+  if (!report) return SDQ_ERR_CUDA;
+  uint32_t* report_dev = nullptr;
+  bool ok = cudaHostGetDevicePointer((void**)&report_dev, report, 0) == cudaSuccess;
+  if (ok && tc) {
+    PackParams p;
+    p.W = (const __nv_bfloat16*)W; p.N = N; p.K = K; p.ldw = ldw; p.colw = col_weight;
+    p.blob = (uint8_t*)packed_buf; p.off = off; p.nonfinite = report_dev;
+    p.out_n = cfg->out_n;
+    p.sv4 = cfg->in_gran == SDQ_GRAN_3OF4;          // S-Vectors of 4: one outlier and two inliers per 4
+    p.elem = cfg->in_gran == SDQ_GRAN_ELEM;         // element-wise 2:4: the 2 most significant non-outliers of every 4
+    // dense family: inliers kept per group (8 - out_n without Stage 1; groups of 4: 3 minus the outlier, or 2 for 2:4)
+    p.keep_in = p.elem ? 2 : (p.sv4 ? (cfg->out_n ? 2 : 3) : 10 - cfg->in_gran - cfg->out_n);
+    p.order_mask = cfg->out_order == SDQ_ORDER_SMALL ? (col_weight ? 0x7FFFFFFF : 0x7FFF0000) : 0;
+    p.ue = cfg->scale_rule == SDQ_SCALE_UE4M3;
+    p.i8 = cfg->out_fmt == SDQ_OUT_INT8;
+    p.b32 = cfg->in_block == 32;
+    p.ceil_rule = cfg->scale_rule == SDQ_SCALE_CEIL_NOSAT;
+    const bool dense = is_dense_layout(*cfg);
+    switch ((col_weight ? 3 : 0) + cfg->out_n) {
+      case 0: launch_pack<false, 0>(p, *hdr, dense, st); break;
+      case 1: launch_pack<false, 1>(p, *hdr, dense, st); break;
+      case 2: launch_pack<false, 2>(p, *hdr, dense, st); break;
+      case 3: launch_pack<true, 0>(p, *hdr, dense, st); break;
+      case 4: launch_pack<true, 1>(p, *hdr, dense, st); break;
+      default: launch_pack<true, 2>(p, *hdr, dense, st); break;
+    }
+  } else if (ok) {
+    launch_pack_plain(W, N, K, ldw, *cfg, col_weight, packed_buf, report_dev, st);
+    ok = cudaMemcpyAsync(packed_buf, raw, HEADER_BYTES, cudaMemcpyHostToDevice, st) == cudaSuccess;
+  }
+  ok = (cudaGetLastError() == cudaSuccess) && ok;
+  ok = (cudaStreamSynchronize(st) == cudaSuccess) && ok;      // also before the word goes back: no kernel writes it afterwards
+  const uint32_t nonfinite = *reinterpret_cast<volatile uint32_t*>(report);
+  g_report.give_back(report);
+  if (!ok) return SDQ_ERR_CUDA;
   return nonfinite ? SDQ_ERR_NONFINITE : SDQ_OK;
 }
 

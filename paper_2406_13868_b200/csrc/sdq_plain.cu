@@ -12,7 +12,7 @@ namespace sdq {
 
 __global__ void __launch_bounds__(128)
 pack_plain_kernel(const __nv_bfloat16* __restrict__ W, int64_t N, int64_t K, int64_t ldw, sdq_config_t cfg, const float* __restrict__ colw,
-                  uint8_t* __restrict__ blob, PlainPackedOffsets off, uint32_t* __restrict__ flags)
+                  uint8_t* __restrict__ blob, PlainPackedOffsets off, uint32_t* __restrict__ nonfinite)
 {
   const int64_t n = blockIdx.x;
   const int tid = threadIdx.x;
@@ -44,7 +44,7 @@ pack_plain_kernel(const __nv_bfloat16* __restrict__ W, int64_t N, int64_t K, int
     bad |= __shfl_xor_sync(0xffffffffu, bad, s);
   }
   if ((tid & 31) == 0) s_red[tid >> 5] = okey_max;
-  if (bad && (tid & 31) == 0) atomicOr(&flags[FLAG_NONFINITE], 1u);
+  if (bad && (tid & 31) == 0) *reinterpret_cast<volatile uint32_t*>(nonfinite) = 1u;
   __syncthreads();
   if (tid == 0) s_e = fp8_scale_exp(bf16_bits_to_float(max(max(s_red[0], s_red[1]), max(s_red[2], s_red[3]))));
   __syncthreads();
@@ -141,9 +141,9 @@ pack_plain_kernel(const __nv_bfloat16* __restrict__ W, int64_t N, int64_t K, int
 }
 
 void launch_pack_plain(const void* W, int64_t N, int64_t K, int64_t ldw, const sdq_config_t& cfg, const float* col_weight, void* buf,
-                       uint32_t* flags, cudaStream_t st)
+                       uint32_t* nonfinite, cudaStream_t st)
 {
   pack_plain_kernel<<<(unsigned)N, 128, 0, st>>>((const __nv_bfloat16*)W, N, K, ldw, cfg, col_weight, (uint8_t*)buf,
-                                                 plain_packed_offsets(N, K, cfg), flags);
+                                                 plain_packed_offsets(N, K, cfg), nonfinite);
 }
 }  // namespace sdq

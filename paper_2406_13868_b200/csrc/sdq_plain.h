@@ -43,6 +43,7 @@ inline PlainPackedOffsets plain_packed_offsets(int64_t N, int64_t K, const sdq_c
   o.total = al(o.osexp + n * 4);
   return o;
 }
+// nonfinite: host-visible word, set to 1 when a weight (or channel weight) is not finite
 void launch_pack_plain(const void* W, int64_t N, int64_t K, int64_t ldw, const sdq_config_t& cfg, const float* col_weight, void* buf,
-                       uint32_t* flags, cudaStream_t st);
+                       uint32_t* nonfinite, cudaStream_t st);
 }  // namespace sdq
