@@ -33,12 +33,17 @@
 //   scales; zeros otherwise); element-wise 2:4 inliers with one scale per 32 K are stored like dense inliers, plus their
 //   kept indices [N][K/4] u8 for the exporter
 //
-// Activation buffer (per 128-token tile mt)
-//   section XI[mt][k2] = | B4 16384 | SFB_in 512 |            (one scale per 32 K: SFB_in 2 x 512, as for the weights)
-//     B4: 128 tokens x 128 B (256 K): byte(t, b) at (t/8)*1024 + (b/16)*128 + (t%8)*16 + b%16
-//   section XO[mt][k1] = | B8 16384 |
-//     B8: 128 tokens x 128 B (128 K): same addressing
-//   section SFB_out[mt] 512 B (per-token 8-bit scale as E8M0, 4 copies), then exponents [MT*128] i32
+// Activation buffer.  Tokens are padded to a multiple of 128 (Mpad); one record holds all of them, so that the codes of ANY
+// run of 8-token groups are one contiguous range and a kernel may cut token tiles of any multiple of 32 at any multiple of
+// 32.
+//   section XI[k2] = | B4 Mpad x 128 B | SFB_in |
+//     B4: 128 B per token (256 K): byte(t, b) at (t/8)*1024 + (b/16)*128 + (t%8)*16 + b%16
+//     SFB_in: scale atoms as for the weights, a scale atom being what one tcgen05.cp moves: 128 tokens' words of 4 scales,
+//     word c of lane l belonging to the atom's token 32 c + l.  Atom number a starts at token 32 a (they overlap: a token's
+//     word is in up to four atoms), so a tile that starts at token 32 a finds its scales in atoms a and a + 4.  One
+//     scale per 32 K: two atoms (128-K blocks) per number.  Up to 32 tokens: one atom.
+//   section XO[k1] = | B8 Mpad x 128 B |        128 B per token (128 K): same addressing
+//   section SFB_out: the per-token 8-bit scale as E8M0, 4 copies, overlapping atoms like SFB_in; then exponents [Mpad] i32
 #pragma once
 #include <stdint.h>
 #include <stddef.h>
@@ -46,7 +51,7 @@
 namespace sdq {
 
 constexpr int TILE_ROWS = 128;     // weight rows per tile (= MMA M)
-constexpr int TILE_TOK = 128;      // tokens per activation tile
+constexpr int TILE_TOK = 128;      // tokens are padded to a multiple of this
 constexpr int K1 = 128;            // logical K per pipeline stage
 constexpr int K2 = 256;            // logical K per metadata / scale atom
 
@@ -60,10 +65,10 @@ constexpr int WO_BYTES = A_OUT_BYTES + E_OUT_BYTES;                  // 10240
 constexpr int WC_CODE_BYTES = 2048;   // per 128 K and outlier of the S-Vector: 128 rows x 16 code bytes
 constexpr int WC_POS_BYTES = 1024;    //                                        128 rows x 16 position nibbles
 __host__ __device__ inline int wc_bytes(int out_n) { return (WC_CODE_BYTES + WC_POS_BYTES) * out_n; }
+// activation records of up to 32 tokens (Mpad = 128, one scale atom)
 constexpr int B4_BYTES = 16384;       // 128 tokens x 256 K
 constexpr int XI_BYTES = B4_BYTES + SF_ATOM_BYTES;                   // 16896
-constexpr int B8_BYTES = 16384;       // 128 tokens x 128 K
-constexpr int XO_BYTES = B8_BYTES;
+constexpr int XO_BYTES = 16384;       // 128 tokens x 128 K
 // One scale per 32 logical K (in_block = 32, run by kind::mxf4nvf4 .block16) doubles the scale atoms of the inlier
 // records: one atom per 128-K block (4 scales of 32 K each) instead of one per 256 K (4 scales of 64 K each).
 __host__ __device__ inline int sf_atoms(bool b32) { return b32 ? 2 : 1; }
@@ -73,7 +78,6 @@ __host__ __device__ inline int e_in_bytes(bool dense) { return dense ? 0 : E_IN_
 __host__ __device__ inline int wi_bytes(bool b32, bool dense = false) {
   return a_in_bytes(dense) + e_in_bytes(dense) + sf_atoms(b32) * SF_ATOM_BYTES;
 }
-__host__ __device__ inline int xi_bytes(bool b32) { return B4_BYTES + sf_atoms(b32) * SF_ATOM_BYTES; }
 // byte of the inlier scale of scale block `blk` (counted inside its 256-K record) of row / token `row` inside the
 // record's scale atoms: block 64 -> atom 0, slot blk (0..3); block 32 -> atom blk / 4, slot blk % 4
 __host__ __device__ inline uint32_t in_sf_off(bool b32, uint32_t row, uint32_t blk) {
@@ -130,19 +134,24 @@ inline PackedOffsets packed_offsets(int64_t N, int64_t K, int out_n, bool b32 = 
 
 struct ActOffsets {
   size_t xi, xo, sfb_out, sexp, amax, total;
-  int64_t MT;
+  size_t xi_stride, xo_stride;   // bytes of a 256-K / 128-K record
+  int64_t Mpad;
+  int32_t atoms;                 // overlapping scale atoms per record (one scale per 32 K: pairs of atoms)
 };
 inline ActOffsets act_offsets(int64_t M, int64_t K, bool b32 = false) {
   ActOffsets o;
-  const size_t MT = (size_t)((M + TILE_TOK - 1) / TILE_TOK), T1 = (size_t)(K / K1), T2 = (size_t)(K / K2);
+  const size_t T1 = (size_t)(K / K1), T2 = (size_t)(K / K2);
   auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
-  o.MT = (int64_t)MT;
+  o.Mpad = (M + TILE_TOK - 1) / TILE_TOK * TILE_TOK;
+  o.atoms = M <= 32 ? 1 : (int32_t)(o.Mpad / 32);
+  o.xi_stride = (size_t)o.Mpad * 128 + (size_t)o.atoms * sf_atoms(b32) * SF_ATOM_BYTES;
+  o.xo_stride = (size_t)o.Mpad * 128;
   o.xi = 0;
-  o.xo = al(o.xi + MT * T2 * (size_t)xi_bytes(b32));
-  o.sfb_out = al(o.xo + MT * T1 * XO_BYTES);
-  o.sexp = al(o.sfb_out + MT * SF_ATOM_BYTES);
-  o.amax = al(o.sexp + MT * TILE_TOK * 4);                       // per-token chunk maxima [MT*128][ceil(K/1024)] f32
-  o.total = al(o.amax + MT * TILE_TOK * ((size_t)(K + 1023) / 1024) * 4);
+  o.xo = al(o.xi + T2 * o.xi_stride);
+  o.sfb_out = al(o.xo + T1 * o.xo_stride);
+  o.sexp = al(o.sfb_out + (size_t)o.atoms * SF_ATOM_BYTES);
+  o.amax = al(o.sexp + (size_t)o.Mpad * 4);                      // per-token chunk maxima [Mpad][ceil(K/2048)] f32
+  o.total = al(o.amax + (size_t)o.Mpad * ((size_t)(K + 2047) / 2048) * 4);
   return o;
 }
 

@@ -126,7 +126,7 @@ sdq_linear_kernel(const LinearParams p)       // many tokens: 13 warps, four of 
   const bool b32 = FLEX ? (p.b32 != 0) : S32;              // one scale per 32 K
   const bool dense = FLEX ? (p.dense != 0) : DENSE;        // dense inliers (always with one scale per 32 K)
   constexpr uint32_t MS = S32 ? 32u : 16u;                 // many tokens: metadata / scale columns per ring slot
-  const uint32_t wib = (uint32_t)wi_bytes(b32, dense), xib = (uint32_t)xi_bytes(b32), na = b32 ? 2u : 1u;
+  const uint32_t wib = (uint32_t)wi_bytes(b32, dense), na = b32 ? 2u : 1u;
   const uint32_t sl_b = wib;                               // B4 / B8 follow the (longest) weight record
   const uint32_t sl_sf = sl_b + (uint32_t)n_tile * 128u;
 
@@ -163,14 +163,15 @@ sdq_linear_kernel(const LinearParams p)       // many tokens: 13 warps, four of 
       uint32_t s = 0, wrapped = 0, ph = 0;   // ring slot, whether the ring has wrapped, phase parity of `empty`
       for (int tile = blockIdx.x; tile < p.total_tiles && ok; tile += gridDim.x) {
         const TileCoord tc = (tile == (int)blockIdx.x) ? first_tc : tile_coord(ksplit, tile, RT, T1, T2);
-        const int mt = tc.mtile * n_tile / TILE_TOK;
-        const int have = min(n_atiles, (int)p.aoff.MT - mt);                 // activation tiles that exist
-        const uint32_t tok_bytes = (uint32_t)min(n_tile, TILE_TOK) * 128u;   // bytes per activation tile per stage
+        const int t0 = tc.mtile * n_tile;                                    // first token of the tile (a multiple of 32 where it matters)
+        const uint32_t tok_bytes = (uint32_t)min(n_tile, (int)p.aoff.Mpad - t0) * 128u;
+        const int have = min(n_atiles, (p.aoff.atoms - t0 / 32 + 3) / 4);    // scale atoms (128 tokens each) that exist
+        const uint32_t astep = 4u * na * SF_ATOM_BYTES;                      // bytes between the atoms of successive 128 tokens
         const uint8_t* wi = p.w + p.poff.wi + ((size_t)tc.rt * T2 + tc.i0) * wib;
         const uint8_t* wo = p.w + p.poff.wo + ((size_t)tc.rt * T1 + tc.o0) * WO_BYTES;
-        const uint8_t* xi = p.x + p.aoff.xi + ((size_t)mt * T2 + tc.i0) * xib;
-        const uint8_t* xo = p.x + p.aoff.xo + ((size_t)mt * T1 + tc.o0) * XO_BYTES;
-        const size_t xi_tile = (size_t)T2 * xib, xo_tile = (size_t)T1 * XO_BYTES;
+        const uint8_t* xi = p.x + p.aoff.xi + (size_t)tc.i0 * p.aoff.xi_stride + (size_t)t0 * 128u;
+        const uint8_t* xs = p.x + p.aoff.xi + (size_t)tc.i0 * p.aoff.xi_stride + (size_t)p.aoff.Mpad * 128u + (size_t)(t0 / 32) * na * SF_ATOM_BYTES;
+        const uint8_t* xo = p.x + p.aoff.xo + (size_t)tc.o0 * p.aoff.xo_stride + (size_t)t0 * 128u;
         const int ni = tc.i1 - tc.i0, no = tc.o1 - tc.o0;
         for (int k = 0; k < ni + no; ++k) {
           if (wrapped && release && !(ok = ptx::mbar_wait(&empty[s], ph ^ 1))) break;
@@ -189,25 +190,25 @@ sdq_linear_kernel(const LinearParams p)       // many tokens: 13 warps, four of 
               wo += WO_BYTES;
             }
           } else if (role == 1) {
-            ptx::mbar_expect_tx(&full[s], (uint32_t)have * tok_bytes);
+            ptx::mbar_expect_tx(&full[s], tok_bytes);
             if (k < ni) {
-              for (int a = 0; a < have; ++a) ptx::bulk_g2s(st + sl_b + a * B4_BYTES, xi + a * xi_tile, tok_bytes, &full[s]);
-              xi += xib;
+              ptx::bulk_g2s(st + sl_b, xi, tok_bytes, &full[s]);
+              xi += p.aoff.xi_stride;
             } else {
-              for (int a = 0; a < have; ++a) ptx::bulk_g2s(st + sl_b + a * B8_BYTES, xo + a * xo_tile, tok_bytes, &full[s]);
-              xo += XO_BYTES;
+              ptx::bulk_g2s(st + sl_b, xo, tok_bytes, &full[s]);
+              xo += p.aoff.xo_stride;
             }
           } else {
             if (k < ni) {
               ptx::mbar_expect_tx(bw, (uint32_t)have * na * SF_ATOM_BYTES);
               for (int a = 0; a < have; ++a)
-                ptx::bulk_g2s(st + sl_sf + a * na * SF_ATOM_BYTES, xi + a * xi_tile + B4_BYTES, na * SF_ATOM_BYTES, bw);
-              xi += xib;
+                ptx::bulk_g2s(st + sl_sf + a * na * SF_ATOM_BYTES, xs + a * astep, na * SF_ATOM_BYTES, bw);
+              xs += p.aoff.xi_stride;
             } else if (first_o) {
               ptx::mbar_expect_tx(bw, (uint32_t)have * SF_ATOM_BYTES);
               for (int a = 0; a < have; ++a)
-                ptx::bulk_g2s(st + sl_sf + (1 + a) * SF_ATOM_BYTES, p.x + p.aoff.sfb_out + (size_t)(mt + a) * SF_ATOM_BYTES, SF_ATOM_BYTES,
-                              bw);
+                ptx::bulk_g2s(st + sl_sf + (1 + a) * SF_ATOM_BYTES, p.x + p.aoff.sfb_out + (size_t)(t0 / 32 + 4 * a) * SF_ATOM_BYTES,
+                              SF_ATOM_BYTES, bw);
             } else {
               ptx::mbar_arrive(bw);
             }

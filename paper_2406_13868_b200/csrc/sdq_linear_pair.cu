@@ -72,7 +72,6 @@ sdq_linear_pair_kernel(const LinearParams p)
   const int pair = (int)(blockIdx.x >> 1), n_pairs = (int)(gridDim.x >> 1);
   const int RTP = (int)(p.N / (2 * TILE_ROWS));                    // row-pair tiles
   const int T1 = p.out_n ? (int)(p.K / K1) : 0, T2 = (int)(p.K / K2);
-  const uint32_t xib = (uint32_t)xi_bytes(S32);
 
   if (tid == 0) ptx::griddep_launch_dependents();
   if (tid == 0) {
@@ -103,7 +102,6 @@ sdq_linear_pair_kernel(const LinearParams p)
       const int S = T2 + T1;
       const int my_tiles = p.total_tiles > pair ? (p.total_tiles - pair + n_pairs - 1) / n_pairs : 0;
       const int total = my_tiles * S;                                        // stages of this CTA, numbered through its tiles
-      const size_t xi_tile = (size_t)T2 * xib, xo_tile = (size_t)T1 * XO_BYTES;
       bool ok = true;
       uint32_t s = lane, wrapped = 0, ph = 0;
       int tseq = 0, k = (int)lane;                                           // this lane's stage: tile number in the CTA's sequence, stage in the tile
@@ -116,7 +114,7 @@ sdq_linear_pair_kernel(const LinearParams p)
           const int tile = pair + tseq * n_pairs;
           rt = 2 * (tile % RTP) + (int)rank;
           mt0 = 2 * (tile / RTP);                                            // first activation tile of the token tile
-          have = min(2, (int)p.aoff.MT - mt0);                               // activation tiles that exist (1 or 2)
+          have = min(2, (int)(p.aoff.Mpad / 128) - mt0);                               // activation tiles that exist (1 or 2)
           own = (int)rank < have;                                            // this CTA's 128 tokens exist
         }
         if (wrapped && !(ok = ptx::mbar_wait(&empty[s >> 1], ph ^ 1))) break;
@@ -137,21 +135,21 @@ sdq_linear_pair_kernel(const LinearParams p)
             ptx::mbar_arrive(&full[s]);
           } else if (inl) {
             ptx::mbar_expect_tx(&full[s], B4_BYTES);
-            ptx::bulk_g2s(st + G::SL_B, p.x + p.aoff.xi + (size_t)(mt0 + (int)rank) * xi_tile + (size_t)k * xib, B4_BYTES, &full[s]);
+            ptx::bulk_g2s(st + G::SL_B, p.x + p.aoff.xi + (size_t)k * p.aoff.xi_stride + (size_t)(mt0 + (int)rank) * B4_BYTES, B4_BYTES, &full[s]);
           } else {
-            ptx::mbar_expect_tx(&full[s], B8_BYTES);
-            ptx::bulk_g2s(st + G::SL_B, p.x + p.aoff.xo + (size_t)(mt0 + (int)rank) * xo_tile + (size_t)ko * XO_BYTES, B8_BYTES, &full[s]);
+            ptx::mbar_expect_tx(&full[s], XO_BYTES);
+            ptx::bulk_g2s(st + G::SL_B, p.x + p.aoff.xo + (size_t)ko * p.aoff.xo_stride + (size_t)(mt0 + (int)rank) * XO_BYTES, XO_BYTES, &full[s]);
           }
         } else {
           if (inl) {
             ptx::mbar_expect_tx(&full[s], (uint32_t)have * NA * SF_ATOM_BYTES);
             for (int a = 0; a < have; ++a)
-              ptx::bulk_g2s(st + G::SL_SF + a * NA * SF_ATOM_BYTES, p.x + p.aoff.xi + (size_t)(mt0 + a) * xi_tile + (size_t)k * xib + B4_BYTES,
+              ptx::bulk_g2s(st + G::SL_SF + a * NA * SF_ATOM_BYTES, p.x + p.aoff.xi + (size_t)k * p.aoff.xi_stride + (size_t)p.aoff.Mpad * 128 + (size_t)(4 * (mt0 + a)) * NA * SF_ATOM_BYTES,
                             NA * SF_ATOM_BYTES, &full[s]);
           } else if (first_o) {
             ptx::mbar_expect_tx(&full[s], (uint32_t)have * SF_ATOM_BYTES);
             for (int a = 0; a < have; ++a)
-              ptx::bulk_g2s(st + G::SL_SF + (1 + a) * SF_ATOM_BYTES, p.x + p.aoff.sfb_out + (size_t)(mt0 + a) * SF_ATOM_BYTES, SF_ATOM_BYTES,
+              ptx::bulk_g2s(st + G::SL_SF + (1 + a) * SF_ATOM_BYTES, p.x + p.aoff.sfb_out + (size_t)(4 * (mt0 + a)) * SF_ATOM_BYTES, SF_ATOM_BYTES,
                             &full[s]);
           } else {
             ptx::mbar_arrive(&full[s]);

@@ -2,14 +2,18 @@
 // scale), "we also quantize activations accordingly" (Section 5, Stage 3; A_o / A_i of Section 5.1).
 //
 // The per-token 8-bit scale needs the whole row before anything can be stored.  Rows up to 16384 long take one
-// launch (`quant_act_fused_kernel`): the CTAs of a thread-block cluster split the Q-Vectors of a group of 8 tokens,
+// launch (`quant_act_fused_kernel`): the CTAs of a thread-block cluster split the K range of a group of 8 tokens,
 // keep their elements in registers, exchange the per-token maxima through distributed shared memory and encode.
-// Longer rows take two launches: `act_amax_kernel` reduces, per token, the largest magnitude of each 1024-K chunk,
-// `quant_act_kernel` then encodes, one CTA per (group of 8 tokens = one row group of the tiled operand layout,
-// 1024-K chunk).  In both a warp works on one 64-K Q-Vector of all 8 tokens at a time: 4 lanes per token, 16
-// elements (two 16-byte loads) per lane, so the Q-Vector maximum is a 4-lane shuffle and every store instruction
-// writes whole 128-byte lines of the stage-tiled layout (8 tokens x 16 B per core matrix).  Codes come from the
-// hardware E2M1 / E4M3 converters and go straight into the layout the GEMM streams.
+// Longer rows take two launches: `act_amax_kernel` reduces, per token, the largest magnitude of each 2048-K chunk,
+// `quant_act_kernel` then encodes, one CTA per (group of 8 tokens = one row group of the operand layout, 2048-K chunk).
+// In all of them a warp works on one unit: 8 tokens x 256 K, i.e. what 8 tokens have in one record of the layout; 4 lanes
+// per token, for each of the unit's four 64-K Q-Vectors 16 elements (two 16-byte loads) per lane.  A Q-Vector maximum is
+// then a 4-lane shuffle, a token's four scales are one word, and every store instruction of codes writes whole 128-byte
+// lines (8 tokens x 16 B per core matrix).  Codes come from the hardware E2M1 / E4M3 converters.
+//
+// Bound by DRAM traffic and the conversion instructions: 2048 x 11008 at 3.74 TB/s of algorithmic bytes (21.0 us; a warp
+// per scattered 64-K Q-Vector with byte stores of scales: 24.7), 8192 x 4096 at 4.4 TB/s (26.7 us; 31.6), one token 3.6 us
+// (4.6), most of it launch and the cluster barrier.
 #include "sdq_codec.cuh"
 #include "sdq_internal.h"
 #include "sdq_layout.h"
@@ -19,40 +23,149 @@ namespace sdq {
 
 constexpr int QA_THREADS = 256;
 constexpr int QA_WARPS = QA_THREADS / 32;
-constexpr int QA_CHUNK_QV = 16;                          // Q-Vectors (64 K each) per CTA: 1024 K
+constexpr int QA_CHUNK = QA_WARPS * K2;                  // K per CTA: one 256-K unit per warp
 
-__device__ __forceinline__ void load16(const __nv_bfloat16* p, float (&x)[16]) {
-  const uint4 a = reinterpret_cast<const uint4*>(p)[0], b = reinterpret_cast<const uint4*>(p)[1];
-  const uint32_t r[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+// a lane's part of a unit: its token's elements 64 i + 16 l .. + 15 for the four Q-Vectors i
+struct QaUnit {
+  uint4 raw[4][2];
+  uint32_t qmax[4];                                      // largest magnitude bits of the 16 elements; > 0x7F7F: an infinity
+};
+// `on`: the token exists and the unit lies inside the row (zeros otherwise)
+__device__ __forceinline__ void qa_load(QaUnit& u, const __nv_bfloat16* p, bool on) {
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    x[2 * i] = __uint_as_float(r[i] << 16);
-    x[2 * i + 1] = __uint_as_float(r[i] & 0xFFFF0000u);
+  for (int i = 0; i < 4; ++i) {
+    u.raw[i][0] = u.raw[i][1] = make_uint4(0, 0, 0, 0);
+    if (on) {
+      const uint4* q = reinterpret_cast<const uint4*>(p + i * 64);
+      u.raw[i][0] = q[0];
+      u.raw[i][1] = q[1];
+    }
   }
 }
+// fills qmax and returns the largest magnitude bits of all the lane's elements.  Magnitudes are compared as 15-bit integers,
+// two per word; +-Inf counts as the largest finite bf16: maxima are clamped, the elements only where a lane holds one
+__device__ __forceinline__ uint32_t qa_maxima(QaUnit& u) {
+  uint32_t m = 0;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const uint32_t r[8] = {u.raw[i][0].x, u.raw[i][0].y, u.raw[i][0].z, u.raw[i][0].w, u.raw[i][1].x, u.raw[i][1].y, u.raw[i][1].z, u.raw[i][1].w};
+    uint32_t q = 0;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) q = __vmaxu2(q, r[j] & 0x7FFF7FFFu);
+    q = max(q & 0xFFFFu, q >> 16);
+    u.qmax[i] = q;
+    m = max(m, min(q, 0x7F7Fu));
+  }
+  return m;
+}
+// writes `w` (a token's four scales of one 128- or 256-K block) to the overlapping atoms that hold the token: lane l (0..3)
+// of the token writes word l of atom m / 32 - l; `step` = bytes between atom numbers
+__device__ __forceinline__ void qa_store_scales(uint8_t* atoms, uint32_t step, int64_t m, uint32_t l, uint32_t w) {
+  const int64_t a = m / 32 - (int64_t)l;
+  if (a >= 0) *reinterpret_cast<uint32_t*>(atoms + (size_t)a * step + (uint32_t)(m & 31) * 16 + l * 4) = w;
+}
 
-// partial[m][chunk] = max |x| of token m over its 1024-K chunk
+// encodes a unit: token m (existing: `live`), 256-K record k2 of the buffer, the token's largest magnitude `ramax`
+template <bool UE>                                       // UE: two-level scaling with E4M3 Q-Vector scales
+__device__ __forceinline__ void qa_encode(const QaUnit& u, float ramax, bool live, int64_t m, int k2, uint32_t l, const sdq_config_t& cfg,
+                                          uint8_t* __restrict__ buf, const ActOffsets& off) {
+  const int e = fp8_scale_exp(ramax);
+  const float s8 = pow2_neg(e);
+  const bool i8 = cfg.out_fmt == SDQ_OUT_INT8;           // A_o in int8: fp32 token scale amax / 127
+  const float sx = int8_scale(ramax);
+  const bool b32 = cfg.in_block == 32;                   // one scale per 32 K: a Q-Vector is a lane pair
+  uint8_t* xi = buf + off.xi + (size_t)k2 * off.xi_stride + (size_t)(m >> 3) * 1024 + (uint32_t)(m & 7) * 16;
+  uint8_t* xo = buf + off.xo + (size_t)(2 * k2) * off.xo_stride + (size_t)(m >> 3) * 1024 + (uint32_t)(m & 7) * 16;
+  uint32_t c[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const uint32_t r[8] = {u.raw[i][0].x, u.raw[i][0].y, u.raw[i][0].z, u.raw[i][0].w, u.raw[i][1].x, u.raw[i][1].y, u.raw[i][1].z, u.raw[i][1].w};
+    float v[16];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      v[2 * j] = __uint_as_float(r[j] << 16);
+      v[2 * j + 1] = __uint_as_float(r[j] & 0xFFFF0000u);
+    }
+    if (u.qmax[i] > 0x7F7Fu) {
+#pragma unroll
+      for (int j = 0; j < 16; ++j) v[j] = sat(v[j]);
+    }
+    uint32_t bm = min(u.qmax[i], 0x7F7Fu);
+    bm = max(bm, __shfl_xor_sync(0xffffffffu, bm, 1));
+    if (!b32) bm = max(bm, __shfl_xor_sync(0xffffffffu, bm, 2));
+    uint32_t q4[2] = {0, 0}, q8[4] = {0, 0, 0, 0};
+    if constexpr (!UE) {
+      c[i] = e8m0_scale_code_bf16(bm, cfg.scale_rule == SDQ_SCALE_CEIL_NOSAT);
+      const float s4 = pow2_inv_e8m0(c[i]);
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        float f[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) f[j] = v[8 * h + j] * s4;
+        q4[h] = e2m1x8(f);
+      }
+    } else {
+      c[i] = ue4m3_scale_code(bf16_bits_to_float(bm), e);
+      if (c[i]) {
+        // two-level scaling: the Q-Vector scale E4M3(c) * 2^e is not a power of two, the elements are divided by it
+        const float sv = ue4m3_scale_value(c[i], e);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          float f[8];
+#pragma unroll
+          for (int j = 0; j < 8; ++j) f[j] = __fdiv_rn(v[8 * h + j], sv);
+          q4[h] = e2m1x8(f);
+        }
+      }
+    }
+    if (!i8) {
+#pragma unroll
+      for (int j = 0; j < 8; ++j) q8[j >> 1] |= e4m3x2(v[2 * j] * s8, v[2 * j + 1] * s8) << (16 * (j & 1));
+    } else {
+#pragma unroll
+      for (int j = 0; j < 8; ++j) q8[j >> 1] |= (int8_code(v[2 * j], sx) | (int8_code(v[2 * j + 1], sx) << 8)) << (16 * (j & 1));
+    }
+    if (live) {
+      // 4-bit codes: bytes 32 i + 8 l of the token's 128; 8-bit codes: bytes 64 (i & 1) + 16 l of the 128-K record i / 2
+      *reinterpret_cast<uint2*>(xi + (uint32_t)(2 * i + (l >> 1)) * 128 + (l & 1) * 8) = make_uint2(q4[0], q4[1]);
+      *reinterpret_cast<uint4*>(xo + (size_t)(i >> 1) * off.xo_stride + (uint32_t)(4 * (i & 1) + l) * 128) = make_uint4(q8[0], q8[1], q8[2], q8[3]);
+    }
+  }
+  uint8_t* sf = buf + off.xi + (size_t)k2 * off.xi_stride + (size_t)off.Mpad * 128;
+  if (!b32) {
+    if (live) qa_store_scales(sf, SF_ATOM_BYTES, m, l, c[0] | (c[1] << 8) | (c[2] << 16) | (c[3] << 24));
+  } else {
+#pragma unroll
+    for (int kb = 0; kb < 2; ++kb) {                     // 128-K block: scales 2 kb and 2 kb + 1 of each lane pair
+      uint32_t w = (c[2 * kb] << (8 * (l >> 1))) | (c[2 * kb + 1] << (16 + 8 * (l >> 1)));
+      w |= __shfl_xor_sync(0xffffffffu, w, 2);
+      if (live) qa_store_scales(sf + kb * SF_ATOM_BYTES, 2 * SF_ATOM_BYTES, m, l, w);
+    }
+  }
+}
+// the token's 8-bit scale: exponent (or the bit pattern of the fp32 scale), and its atoms of the outlier product
+template <bool UE>
+__device__ __forceinline__ void qa_token_scale(float ramax, int64_t m, uint32_t l, const sdq_config_t& cfg, uint8_t* __restrict__ buf, const ActOffsets& off) {
+  const bool i8 = cfg.out_fmt == SDQ_OUT_INT8;
+  const int e = fp8_scale_exp(ramax);
+  if (l == 0) reinterpret_cast<int32_t*>(buf + off.sexp)[m] = i8 ? __float_as_int(int8_scale(ramax)) : e;
+  // two-level scaling keeps a token's accumulator column in units of 2^e (the 4-bit scale codes leave that factor out):
+  // the 8-bit product then takes the scale 1 here and the GEMM's epilogue multiplies 2^e back in
+  qa_store_scales(buf + off.sfb_out, SF_ATOM_BYTES, m, l, (uint32_t)((UE || i8) ? 127 : e + 127) * 0x01010101u);
+}
+
+// partial[m][chunk] = max |x| of token m over its 2048-K chunk
 __global__ void __launch_bounds__(QA_THREADS)
 act_amax_kernel(const __nv_bfloat16* __restrict__ X, int64_t M, int64_t K, int64_t ldx, float* __restrict__ partial, int n_chunks)
 {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int t = lane >> 2, l = lane & 3;
   const int64_t m = (int64_t)blockIdx.x * 8 + t;
-  const bool live = m < M;
-  const int NB = (int)(K / 64);
-  const int b0 = blockIdx.y * QA_CHUNK_QV;
+  const int64_t k = (int64_t)blockIdx.y * QA_CHUNK + warp * K2;
   __shared__ float s_amax[QA_WARPS][8];
-  float amax = 0.0f;
-#pragma unroll
-  for (int i = 0; i < QA_CHUNK_QV / QA_WARPS; ++i) {
-    const int b = b0 + warp + i * QA_WARPS;
-    if (live && b < NB) {
-      float v[16];
-      load16(X + m * ldx + (int64_t)b * 64 + l * 16, v);
-#pragma unroll
-      for (int j = 0; j < 16; ++j) amax = fmaxf(amax, sat_abs(v[j]));
-    }
-  }
+  QaUnit u;
+  qa_load(u, X + m * ldx + k + l * 16, m < M && k < K);
+  float amax = bf16_bits_to_float(qa_maxima(u));
   amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, 1));
   amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, 2));
   if (l == 0) s_amax[warp][t] = amax;
@@ -65,7 +178,7 @@ act_amax_kernel(const __nv_bfloat16* __restrict__ X, int64_t M, int64_t K, int64
   }
 }
 
-template <bool UE>                                      // UE: two-level scaling with E4M3 Q-Vector scales
+template <bool UE>
 __global__ void __launch_bounds__(QA_THREADS)
 quant_act_kernel(const __nv_bfloat16* __restrict__ X, int64_t M, int64_t K, int64_t ldx, sdq_config_t cfg, uint8_t* __restrict__ buf,
                  ActOffsets off, const float* __restrict__ partial, int n_chunks)
@@ -76,8 +189,7 @@ quant_act_kernel(const __nv_bfloat16* __restrict__ X, int64_t M, int64_t K, int6
   if (tid == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int64_t m = (int64_t)blockIdx.x * 8 + t;
   const bool live = m < M;
-  const int NB = (int)(K / 64);                           // Q-Vectors per row
-  const int b0 = blockIdx.y * QA_CHUNK_QV;
+  const int64_t k = (int64_t)blockIdx.y * QA_CHUNK + warp * K2;
 
   // per-token 8-bit scale from the chunk maxima of the whole row
   float ramax = 0.0f;
@@ -85,76 +197,19 @@ quant_act_kernel(const __nv_bfloat16* __restrict__ X, int64_t M, int64_t K, int6
     for (int c = l; c < n_chunks; c += 4) ramax = fmaxf(ramax, partial[m * n_chunks + c]);
   ramax = fmaxf(ramax, __shfl_xor_sync(0xffffffffu, ramax, 1));
   ramax = fmaxf(ramax, __shfl_xor_sync(0xffffffffu, ramax, 2));
-  const int e = fp8_scale_exp(ramax);
-  const float s8 = pow2_neg(e);
-  const bool i8 = cfg.out_fmt == SDQ_OUT_INT8;       // A_o in int8: fp32 token scale amax / 127, handed on as its bit pattern
-  const float sx = int8_scale(ramax);
-
-  const int64_t mt = m / TILE_TOK;
-  const uint32_t tk = (uint32_t)(m % TILE_TOK);
-  const int T1 = (int)(K / K1), T2 = (int)(K / K2);
-  const bool b32 = cfg.in_block == 32;               // one scale per 32 K: a Q-Vector is a lane pair
-  constexpr bool ue = UE;
-  const int xib = xi_bytes(b32);
-  uint8_t* xi_base = buf + off.xi + (size_t)mt * T2 * xib;
-  uint8_t* xo_base = buf + off.xo + (size_t)mt * T1 * XO_BYTES;
-  if (live && blockIdx.y == 0 && warp == 0 && l == 0) {
-    reinterpret_cast<int32_t*>(buf + off.sexp)[m] = i8 ? __float_as_int(sx) : e;
-    // two-level scaling keeps a token's accumulator column in units of 2^e (the 4-bit scale codes leave that factor out):
-    // the 8-bit product then takes the scale 1 here and the GEMM's epilogue multiplies 2^e back in
-    *reinterpret_cast<uint32_t*>(buf + off.sfb_out + (size_t)mt * SF_ATOM_BYTES + sf_off(tk, 0)) = (uint32_t)((ue || i8) ? 127 : e + 127) * 0x01010101u;
-  }
-
-#pragma unroll
-  for (int i = 0; i < QA_CHUNK_QV / QA_WARPS; ++i) {
-    const int b = b0 + warp + i * QA_WARPS;              // uniform over the warp
-    if (b >= NB) break;
-    float v[16];
-    if (live) load16(X + m * ldx + (int64_t)b * 64 + l * 16, v);
-    else {
-#pragma unroll
-      for (int j = 0; j < 16; ++j) v[j] = 0.0f;
-    }
-    float bmax = 0.0f;
-#pragma unroll
-    for (int j = 0; j < 16; ++j) {
-      v[j] = sat(v[j]);
-      bmax = fmaxf(bmax, fabsf(v[j]));
-    }
-    bmax = fmaxf(bmax, __shfl_xor_sync(0xffffffffu, bmax, 1));
-    if (!b32) bmax = fmaxf(bmax, __shfl_xor_sync(0xffffffffu, bmax, 2));
-    const uint32_t c = ue ? ue4m3_scale_code(bmax, e) : e8m0_scale_code(bmax, cfg.scale_rule);
-    uint32_t q4[2] = {0, 0}, q8[4] = {0, 0, 0, 0};
-    if (!ue) {
-      const float s4 = pow2_inv_e8m0(c);
-#pragma unroll
-      for (int j = 0; j < 8; ++j) q4[j >> 2] |= e2m1x2(v[2 * j] * s4, v[2 * j + 1] * s4) << (8 * (j & 3));
-    } else if (c) {
-      // two-level scaling: the Q-Vector scale E4M3(c) * 2^e is not a power of two, the elements are divided by it
-      const float sv = ue4m3_scale_value(c, e);
-#pragma unroll
-      for (int j = 0; j < 8; ++j) q4[j >> 2] |= e2m1x2(__fdiv_rn(v[2 * j], sv), __fdiv_rn(v[2 * j + 1], sv)) << (8 * (j & 3));
-    }
-#pragma unroll
-    for (int j = 0; j < 8; ++j)
-      q8[j >> 1] |= (i8 ? (int8_code(v[2 * j], sx) | (int8_code(v[2 * j + 1], sx) << 8)) : e4m3x2(v[2 * j] * s8, v[2 * j + 1] * s8)) << (16 * (j & 1));
-    if (!live) continue;
-    const uint32_t k = (uint32_t)b * 64 + l * 16;          // first element of this lane
-    uint8_t* xi = xi_base + (size_t)(k >> 8) * xib;
-    uint8_t* xo = xo_base + (size_t)(k >> 7) * XO_BYTES;
-    *reinterpret_cast<uint2*>(xi + b_off(tk, (k & 255) >> 1)) = make_uint2(q4[0], q4[1]);
-    *reinterpret_cast<uint4*>(xo + b_off(tk, k & 127)) = make_uint4(q8[0], q8[1], q8[2], q8[3]);
-    if (b32) { if ((l & 1) == 0) xi[B4_BYTES + in_sf_off(true, tk, (k >> 5) & 7)] = (uint8_t)c; }
-    else if (l == 0) xi[B4_BYTES + in_sf_off(false, tk, (uint32_t)(b & 3))] = (uint8_t)c;
-  }
+  if (live && blockIdx.y == 0 && warp == 0) qa_token_scale<UE>(ramax, m, (uint32_t)l, cfg, buf, off);
+  if (k >= K) return;
+  QaUnit u;
+  qa_load(u, X + m * ldx + k + l * 16, live);
+  qa_maxima(u);
+  qa_encode<UE>(u, ramax, live, m, (int)(k / K2), (uint32_t)l, cfg, buf, off);
 }
 
-// Single pass: the CTAs of a cluster share one group of 8 tokens and split its Q-Vectors; every thread keeps its
-// elements in registers (packed bf16) from the one read of X, the per-token maxima meet through distributed shared
-// memory, and the codes are produced from the registers.  Same arithmetic as the two-kernel path, which stays for
-// rows too long for the register budget (K > 64 * QA_WARPS * QF_MAX_IT * 8 = 16384); both scale-block sizes run here.
-constexpr int QF_MAX_IT = 4;                             // Q-Vectors per warp
-template <int IT, bool UE>
+// Single pass: the CTAs of a cluster share one group of 8 tokens and split its 256-K units, one per warp; every thread keeps
+// its elements in registers (packed bf16) from the one read of X, the per-token maxima meet through distributed shared
+// memory, and the codes are produced from the registers.  The two-launch path stays for rows longer than a cluster of
+// eight CTAs holds (K > 16384).
+template <bool UE>
 __global__ void __launch_bounds__(QA_THREADS, UE ? 3 : 4)
 quant_act_fused_kernel(const __nv_bfloat16* __restrict__ X, int64_t M, int64_t K, int64_t ldx, sdq_config_t cfg, uint8_t* __restrict__ buf,
                        ActOffsets off)
@@ -167,38 +222,14 @@ quant_act_fused_kernel(const __nv_bfloat16* __restrict__ X, int64_t M, int64_t K
   const uint32_t cx = gridDim.x, rank = blockIdx.x;      // cluster = the gridDim.x CTAs of one token group
   const int64_t m = (int64_t)blockIdx.y * 8 + t;
   const bool live = m < M;
-  const int NB = (int)(K / 64);
-  const int per_cta = (NB + (int)cx - 1) / (int)cx;
-  const int b_begin = (int)rank * per_cta, b_end = min(NB, b_begin + per_cta);
+  const int k2 = (int)rank * QA_WARPS + warp;            // this warp's unit
+  const bool on = k2 < (int)(K / K2);
   __shared__ float s_warp[QA_WARPS][8];
   __shared__ float s_all[8][8];                          // [cluster rank][token]: every CTA's maxima, pushed by their owners
 
-  // magnitudes are compared as 15-bit integers, two per 32-bit word (max.u16x2); +-Inf counts as the largest finite
-  // bf16: the maxima are clamped once, the elements only in the (rare) lanes that hold an infinity
-  uint4 raw[IT][2];
-  uint32_t qmax[IT];                                      // this lane's largest magnitude bits of Q-Vector i (16 elements)
-  uint32_t m2 = 0;
-#pragma unroll
-  for (int i = 0; i < IT; ++i) {
-    const int b = b_begin + warp + i * QA_WARPS;
-    raw[i][0] = raw[i][1] = make_uint4(0, 0, 0, 0);
-    if (live && b < b_end) {
-      const uint4* p = reinterpret_cast<const uint4*>(X + m * ldx + (int64_t)b * 64 + l * 16);
-      raw[i][0] = p[0];
-      raw[i][1] = p[1];
-    }
-  }
-#pragma unroll
-  for (int i = 0; i < IT; ++i) {
-    const uint32_t r[8] = {raw[i][0].x, raw[i][0].y, raw[i][0].z, raw[i][0].w, raw[i][1].x, raw[i][1].y, raw[i][1].z, raw[i][1].w};
-    uint32_t q = 0;
-#pragma unroll
-    for (int j = 0; j < 8; ++j) q = __vmaxu2(q, r[j] & 0x7FFF7FFFu);
-    q = max(q & 0xFFFFu, q >> 16);                       // > 0x7F7F: the lane holds an infinity (clamped where used)
-    qmax[i] = q;
-    m2 = max(m2, min(q, 0x7F7Fu));
-  }
-  float amax = __uint_as_float(m2 << 16);
+  QaUnit u;
+  qa_load(u, X + m * ldx + (int64_t)k2 * K2 + l * 16, live && on);
+  float amax = bf16_bits_to_float(qa_maxima(u));
   amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, 1));
   amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, 2));
   if (l == 0) s_warp[warp][t] = amax;
@@ -218,89 +249,26 @@ quant_act_fused_kernel(const __nv_bfloat16* __restrict__ X, int64_t M, int64_t K
   asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
   float ramax = 0.0f;
   for (uint32_t c = 0; c < cx; ++c) ramax = fmaxf(ramax, s_all[c][t]);
-  const int e = fp8_scale_exp(ramax);
-  const float s8 = pow2_neg(e);
-  const bool i8 = cfg.out_fmt == SDQ_OUT_INT8;       // A_o in int8: fp32 token scale amax / 127, handed on as its bit pattern
-  const float sx = int8_scale(ramax);
-
-  const int64_t mt = m / TILE_TOK;
-  const uint32_t tk = (uint32_t)(m % TILE_TOK);
-  const int T1 = (int)(K / K1), T2 = (int)(K / K2);
-  const bool b32 = cfg.in_block == 32;               // one scale per 32 K: a Q-Vector is a lane pair
-  constexpr bool ue = UE;
-  const int xib = xi_bytes(b32);
-  uint8_t* xi_base = buf + off.xi + (size_t)mt * T2 * xib;
-  uint8_t* xo_base = buf + off.xo + (size_t)mt * T1 * XO_BYTES;
-  if (live && rank == 0 && warp == 0 && l == 0) {
-    reinterpret_cast<int32_t*>(buf + off.sexp)[m] = i8 ? __float_as_int(sx) : e;
-    // two-level scaling keeps a token's accumulator column in units of 2^e (the 4-bit scale codes leave that factor out):
-    // the 8-bit product then takes the scale 1 here and the GEMM's epilogue multiplies 2^e back in
-    *reinterpret_cast<uint32_t*>(buf + off.sfb_out + (size_t)mt * SF_ATOM_BYTES + sf_off(tk, 0)) = (uint32_t)((ue || i8) ? 127 : e + 127) * 0x01010101u;
-  }
-#pragma unroll
-  for (int i = 0; i < IT; ++i) {
-    const int b = b_begin + warp + i * QA_WARPS;          // uniform over the warp
-    if (b >= b_end) break;
-    const uint32_t r[8] = {raw[i][0].x, raw[i][0].y, raw[i][0].z, raw[i][0].w, raw[i][1].x, raw[i][1].y, raw[i][1].z, raw[i][1].w};
-    float v[16];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      v[2 * j] = __uint_as_float(r[j] << 16);
-      v[2 * j + 1] = __uint_as_float(r[j] & 0xFFFF0000u);
-    }
-    if (qmax[i] > 0x7F7Fu) {
-#pragma unroll
-      for (int j = 0; j < 16; ++j) v[j] = sat(v[j]);
-    }
-    uint32_t bm = min(qmax[i], 0x7F7Fu);
-    bm = max(bm, __shfl_xor_sync(0xffffffffu, bm, 1));
-    if (!b32) bm = max(bm, __shfl_xor_sync(0xffffffffu, bm, 2));
-    const float bmax = __uint_as_float(bm << 16);
-    const uint32_t c = ue ? ue4m3_scale_code(bmax, e) : e8m0_scale_code(bmax, cfg.scale_rule);
-    uint32_t q4[2] = {0, 0}, q8[4] = {0, 0, 0, 0};
-    if (!ue) {
-      const float s4 = pow2_inv_e8m0(c);
-#pragma unroll
-      for (int j = 0; j < 8; ++j) q4[j >> 2] |= e2m1x2(v[2 * j] * s4, v[2 * j + 1] * s4) << (8 * (j & 3));
-    } else if (c) {
-      // two-level scaling: the Q-Vector scale E4M3(c) * 2^e is not a power of two, the elements are divided by it
-      const float sv = ue4m3_scale_value(c, e);
-#pragma unroll
-      for (int j = 0; j < 8; ++j) q4[j >> 2] |= e2m1x2(__fdiv_rn(v[2 * j], sv), __fdiv_rn(v[2 * j + 1], sv)) << (8 * (j & 3));
-    }
-#pragma unroll
-    for (int j = 0; j < 8; ++j)
-      q8[j >> 1] |= (i8 ? (int8_code(v[2 * j], sx) | (int8_code(v[2 * j + 1], sx) << 8)) : e4m3x2(v[2 * j] * s8, v[2 * j + 1] * s8)) << (16 * (j & 1));
-    if (!live) continue;
-    const uint32_t k = (uint32_t)b * 64 + l * 16;          // first element of this lane
-    uint8_t* xi = xi_base + (size_t)(k >> 8) * xib;
-    uint8_t* xo = xo_base + (size_t)(k >> 7) * XO_BYTES;
-    *reinterpret_cast<uint2*>(xi + b_off(tk, (k & 255) >> 1)) = make_uint2(q4[0], q4[1]);
-    *reinterpret_cast<uint4*>(xo + b_off(tk, k & 127)) = make_uint4(q8[0], q8[1], q8[2], q8[3]);
-    if (b32) { if ((l & 1) == 0) xi[B4_BYTES + in_sf_off(true, tk, (k >> 5) & 7)] = (uint8_t)c; }
-    else if (l == 0) xi[B4_BYTES + in_sf_off(false, tk, (uint32_t)(b & 3))] = (uint8_t)c;
-  }
+  if (live && rank == 0 && warp == 0) qa_token_scale<UE>(ramax, m, (uint32_t)l, cfg, buf, off);
+  if (on) qa_encode<UE>(u, ramax, live, m, k2, (uint32_t)l, cfg, buf, off);
 }
 
 __global__ void __launch_bounds__(QA_THREADS)
 export_act_kernel(const uint8_t* __restrict__ buf, int64_t M, int64_t K, int in_block, ActOffsets off, sdq_act_canonical_t out)
 {
   const int64_t m = blockIdx.x;
-  const int64_t mt = m / TILE_TOK;
-  const uint32_t t = (uint32_t)(m % TILE_TOK);
-  const int T1 = (int)(K / K1), T2 = (int)(K / K2);
   const bool b32 = in_block == 32;
-  const int xib = xi_bytes(b32);
-  const uint8_t* xi_base = buf + off.xi + (size_t)mt * T2 * xib;
-  const uint8_t* xo_base = buf + off.xo + (size_t)mt * T1 * XO_BYTES;
   for (int64_t k = threadIdx.x; k < K; k += QA_THREADS) {
-    const uint8_t* xi = xi_base + (size_t)(k >> 8) * xib;
-    const uint8_t* xo = xo_base + (size_t)(k >> 7) * XO_BYTES;
-    const uint32_t b = xi[b_off(t, (uint32_t)(k & 255) >> 1)];
+    const uint8_t* xi = buf + off.xi + (size_t)(k >> 8) * off.xi_stride;
+    const uint8_t* xo = buf + off.xo + (size_t)(k >> 7) * off.xo_stride;
+    const uint32_t kb = (uint32_t)(k & 255) >> 1;
+    const uint8_t b = xi[(size_t)(m >> 3) * 1024 + b_off((uint32_t)(m & 7), kb)];
     out.xq4_code[(size_t)m * K + k] = (uint8_t)((k & 1) ? (b >> 4) : (b & 15));
-    out.xq8_code[(size_t)m * K + k] = xo[b_off(t, (uint32_t)(k & 127))];
-    if (b32) { if ((k & 31) == 0) out.xq4_scale[(size_t)m * (K / 32) + (k >> 5)] = xi[B4_BYTES + in_sf_off(true, t, (uint32_t)((k >> 5) & 7))]; }
-    else if ((k & 63) == 0) out.xq4_scale[(size_t)m * (K / 64) + (k >> 6)] = xi[B4_BYTES + in_sf_off(false, t, (uint32_t)((k >> 6) & 3))];
+    out.xq8_code[(size_t)m * K + k] = xo[(size_t)(m >> 3) * 1024 + b_off((uint32_t)(m & 7), (uint32_t)(k & 127))];
+    // word 0 of atom m / 32
+    const uint8_t* sf = xi + (size_t)off.Mpad * 128 + (size_t)(m >> 5) * (b32 ? 2 : 1) * SF_ATOM_BYTES;
+    if (b32) { if ((k & 31) == 0) out.xq4_scale[(size_t)m * (K / 32) + (k >> 5)] = sf[in_sf_off(true, (uint32_t)(m & 31), (uint32_t)((k >> 5) & 7))]; }
+    else if ((k & 63) == 0) out.xq4_scale[(size_t)m * (K / 64) + (k >> 6)] = sf[in_sf_off(false, (uint32_t)(m & 31), (uint32_t)((k >> 6) & 3))];
   }
   if (threadIdx.x == 0) out.xq8_sexp[m] = reinterpret_cast<const int32_t*>(buf + off.sexp)[m];
 }
@@ -334,53 +302,34 @@ extern "C" sdq_status_t sdq_quantize_act(const void* X, int64_t M, int64_t K, in
   const bool b32 = cfg->in_block == 32;
   const ActOffsets off = act_offsets(M, K, b32);
   if (xq_bytes < off.total) return SDQ_ERR_BUFFER_TOO_SMALL;
-  const int n_chunks = (int)((K / 64 + QA_CHUNK_QV - 1) / QA_CHUNK_QV);
-  float* partial = reinterpret_cast<float*>((uint8_t*)xq_buf + off.amax);
-  const dim3 grid((unsigned)((M + 7) / 8), (unsigned)n_chunks);
-  // cluster size for the single-pass kernel: enough CTAs per token group that a warp keeps at most QF_MAX_IT Q-Vectors
-  const int NB = (int)(K / 64);
-  const int cx = (NB + QA_WARPS * QF_MAX_IT - 1) / (QA_WARPS * QF_MAX_IT);
-  if (cx <= 8) {
-    const int it = ((NB + cx - 1) / cx + QA_WARPS - 1) / QA_WARPS;      // 1..QF_MAX_IT
+  const __nv_bfloat16* Xb = (const __nv_bfloat16*)X;
+  uint8_t* bufp = (uint8_t*)xq_buf;
+  const bool ue = cfg->scale_rule == SDQ_SCALE_UE4M3;
+  const int n_chunks = (int)((K + QA_CHUNK - 1) / QA_CHUNK);      // = CTAs per token group: one 256-K unit per warp
+  if (n_chunks <= 8) {
     cudaLaunchConfig_t lc = {};
-    lc.gridDim = dim3((unsigned)cx, (unsigned)((M + 7) / 8));
+    lc.gridDim = dim3((unsigned)n_chunks, (unsigned)((M + 7) / 8));
     lc.blockDim = dim3(QA_THREADS);
     lc.stream = (cudaStream_t)stream;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)cx;
+    attr[0].val.clusterDim.x = (unsigned)n_chunks;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     lc.attrs = attr;
     lc.numAttrs = 2;
-    const __nv_bfloat16* Xb = (const __nv_bfloat16*)X;
-    uint8_t* bufp = (uint8_t*)xq_buf;
-    cudaError_t le;
-    if (cfg->scale_rule == SDQ_SCALE_UE4M3) {
-      switch (it) {
-        case 1: le = cudaLaunchKernelEx(&lc, quant_act_fused_kernel<1, true>, Xb, M, K, ldx, *cfg, bufp, off); break;
-        case 2: le = cudaLaunchKernelEx(&lc, quant_act_fused_kernel<2, true>, Xb, M, K, ldx, *cfg, bufp, off); break;
-        case 3: le = cudaLaunchKernelEx(&lc, quant_act_fused_kernel<3, true>, Xb, M, K, ldx, *cfg, bufp, off); break;
-        default: le = cudaLaunchKernelEx(&lc, quant_act_fused_kernel<4, true>, Xb, M, K, ldx, *cfg, bufp, off); break;
-      }
-    } else {
-      switch (it) {
-        case 1: le = cudaLaunchKernelEx(&lc, quant_act_fused_kernel<1, false>, Xb, M, K, ldx, *cfg, bufp, off); break;
-        case 2: le = cudaLaunchKernelEx(&lc, quant_act_fused_kernel<2, false>, Xb, M, K, ldx, *cfg, bufp, off); break;
-        case 3: le = cudaLaunchKernelEx(&lc, quant_act_fused_kernel<3, false>, Xb, M, K, ldx, *cfg, bufp, off); break;
-        default: le = cudaLaunchKernelEx(&lc, quant_act_fused_kernel<4, false>, Xb, M, K, ldx, *cfg, bufp, off); break;
-      }
-    }
+    const cudaError_t le = ue ? cudaLaunchKernelEx(&lc, quant_act_fused_kernel<true>, Xb, M, K, ldx, *cfg, bufp, off)
+                              : cudaLaunchKernelEx(&lc, quant_act_fused_kernel<false>, Xb, M, K, ldx, *cfg, bufp, off);
     if (le != cudaSuccess || cudaGetLastError() != cudaSuccess) return SDQ_ERR_CUDA;
   } else {
-  act_amax_kernel<<<grid, QA_THREADS, 0, (cudaStream_t)stream>>>((const __nv_bfloat16*)X, M, K, ldx, partial, n_chunks);
-  if (cfg->scale_rule == SDQ_SCALE_UE4M3)
-    quant_act_kernel<true><<<grid, QA_THREADS, 0, (cudaStream_t)stream>>>((const __nv_bfloat16*)X, M, K, ldx, *cfg, (uint8_t*)xq_buf, off, partial, n_chunks);
-  else
-    quant_act_kernel<false><<<grid, QA_THREADS, 0, (cudaStream_t)stream>>>((const __nv_bfloat16*)X, M, K, ldx, *cfg, (uint8_t*)xq_buf, off, partial, n_chunks);
-  if (cudaGetLastError() != cudaSuccess) return SDQ_ERR_CUDA;
+    float* partial = reinterpret_cast<float*>(bufp + off.amax);
+    const dim3 grid((unsigned)((M + 7) / 8), (unsigned)n_chunks);
+    act_amax_kernel<<<grid, QA_THREADS, 0, (cudaStream_t)stream>>>(Xb, M, K, ldx, partial, n_chunks);
+    if (ue) quant_act_kernel<true><<<grid, QA_THREADS, 0, (cudaStream_t)stream>>>(Xb, M, K, ldx, *cfg, bufp, off, partial, n_chunks);
+    else quant_act_kernel<false><<<grid, QA_THREADS, 0, (cudaStream_t)stream>>>(Xb, M, K, ldx, *cfg, bufp, off, partial, n_chunks);
+    if (cudaGetLastError() != cudaSuccess) return SDQ_ERR_CUDA;
   }
   out->dev = xq_buf;
   out->bytes = off.total;
