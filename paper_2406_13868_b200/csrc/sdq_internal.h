@@ -21,6 +21,7 @@ struct DeviceInfo {
   uint32_t pair_attr;      // bit per CTA-pair GEMM instantiation
   uint32_t diag_attr;      // the copy-rate diagnostic
   uint32_t group_attr;     // the grouped few-token GEMM
+  int pair_clusters[5];    // CTA-pair GEMM: clusters of k pairs that run at once (entry 1 set: filled in)
 };
 constexpr int MAX_DEVICES = 64;
 // entry of device `dev` (0 <= dev < MAX_DEVICES) in the table; nullptr outside that range

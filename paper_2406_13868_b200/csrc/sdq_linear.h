@@ -15,9 +15,8 @@ struct LinearParams {
   ActOffsets aoff;
   int64_t M, N, K;
   int out_n;
-  int n_tile;            // tokens per tile: 16, 32, 64, 128 or 256
-  int n_mtiles;          // ceil(M / n_tile)
-  int total_tiles;       // (N / 128) * n_mtiles * ksplit
+  int n_tile;            // few tokens: 16, 32, 64 or 128, the one token tile; pairs: tokens of the widest tile
+  int total_tiles;       // (N / 128) * ksplit
   int nslot, slot_bytes; // shared-memory ring geometry (depends on n_tile)
   int ring_bytes;        // nslot * slot_bytes; the transpose buffer and the barriers follow
   int release;           // 1: ring slots are reused (producer waits on `empty`, MMA issuer commits to it)
@@ -29,6 +28,13 @@ struct LinearParams {
   const int32_t* tw;     // [N] exponents of the rows' inlier factors (packed weights)
   const int32_t* tx;     // [tokens] exponents of the tokens' 8-bit scales (quantized activations)
   int dense;             // 1: dense inliers (no Stage 1): 4 dense kind::mxf4 MMAs of 64 K per stage, runtime geometry only
+  // CTA-pair kernel: a task is one token tile and one or two row units (a unit = 256 weight rows = 128 per CTA).  Token tile i
+  // of pt_mtiles covers the 32-token groups [i G / pt_mtiles, (i + 1) G / pt_mtiles) of the G there are; n_tile is the widest.
+  int pt_units, pt_mtiles, pt_groups;
+  int pt_doubles, pt_split;       // the first tasks, of two units; of the one-unit tasks behind them, the first pt_split are halves of two-unit ones
+  int pt_tasks;                   // all tasks
+  int pt_ks;                      // pairs that share the K range of a task, in a cluster of 2 pt_ks CTAs (then one task per cluster)
+  int pt_acc2;                    // 1: the accumulator alternates between two sets of columns (one-unit tasks only)
   int ksplit;            // CTAs sharing the K range of one row tile (1 = no split)
   int cluster_ks;        // > 1: those CTAs form a cluster and reduce through distributed shared memory
   uint32_t* ws_counter;  // split-K workspace: arrival counters [row tile], zero between calls
@@ -67,9 +73,9 @@ struct GroupParams {
 cudaError_t launch_linear_group(GroupParams p, bool f32_out, int sm_count, cudaStream_t stream, uint32_t* attr_done);
 bool group_xres_fits(int T2, int out_n);   // the activation-resident variant's shared-memory budget for K = 256 T2
 
-// CTA-pair (tcgen05 cta_group::2) many-token kernel: tiles of 256 weight rows x 256 tokens (sdq_linear_pair.cu).
-// `attr_mask` is the calling device's record of which instantiations already carry their shared-memory attribute.
-bool pair_kernel_applies(int64_t M, int64_t N, int64_t K, int out_n);
-cudaError_t launch_linear_pair(LinearParams p, bool f32_out, int sm_count, cudaStream_t stream, uint32_t* attr_mask);
+// CTA-pair (tcgen05 cta_group::2) many-token kernel (sdq_linear_pair.cu).
+// estimated time of a call in us, to choose between the kernels
+double pair_kernel_us(int64_t M, int64_t N, int64_t K, int out_n, bool b32, bool dense, DeviceInfo* d);
+cudaError_t launch_linear_pair(LinearParams p, bool f32_out, DeviceInfo* d, cudaStream_t stream);
 
 }  // namespace sdq

@@ -1,26 +1,43 @@
 // Fused decomposed GEMM for many tokens, CTA-pair form  Y = A_i W_i^T + A_o W_o^T   (Section 5.1: O = O_i + O_o)
 //
-// The many-token layer is bound by the bytes a tile pulls from L2 into shared memory, and three quarters of those are
-// activation codes that every row tile fetches again.  Here the two CTAs of a cluster work as one tensor-core unit
-// (tcgen05 cta_group::2) on a tile of 256 weight rows x 256 tokens: CTA r stages weight rows 128 r .. 128 r + 127 and
-// the codes of tokens 128 r .. 128 r + 127 only, and the pair-wide MMA takes half of its B operand from each CTA's
-// shared memory -- 27 KB per CTA and stage instead of 43 KB for the same MMA time.  The stage sequence of a tile is
-// that of the single-CTA kernel (all inlier stages of 256 K, then all outlier stages of 128 K, one fp32 accumulator).
+// The two CTAs of a cluster work as one tensor-core unit (tcgen05 cta_group::2).  A task is one token tile of T tokens and
+// one or two row units of 256 weight rows: CTA r stages weight rows 128 r .. 128 r + 127 of each unit and the codes of
+// tokens r T/2 .. only, and the pair-wide MMA takes half of its B operand from each CTA's shared memory.  All inlier stages
+// (256 K) run first, then all outlier stages (128 K), into one fp32 accumulator per unit.
 //
-// Per CTA: warps 0 / 6 / 7 bulk-copy producers (own weight records / own activation codes / scale atoms of both token
-// halves; two lanes each, see there), warps 2..5 and 9..12 epilogue (own 128 rows x 256 tokens: TMEM -> registers as
-// packed bf16, TMEM handed back, transposed stores under the next tile's K loop).  Even CTA (leader): warp 1 copies
-// metadata and scales of both CTAs to TMEM (pair-wide tcgen05.cp) and issues the pair-wide MMAs; its tcgen05.commit
-// signals "slots consumed" / "accumulator complete" to the barriers of both CTAs.  Odd CTA: two lanes of warp 1
-// forward "my part of the slot has landed" to the leader's barriers.  Every wait is bounded.
+// What bounds the layer is the bytes a task pulls from L2 into shared memory: with every SM pulling, an SM receives ~90 of
+// the ~117 B/ns that the copy-only kernel reaches, since the ring (all the shared memory there is) over the loaded L2 latency
+// is what can be in flight.  Per 256 K an SM stages 31 KB of weights per unit and 384 B per token of its half:
+//   one unit  x 256 tokens   80 KB for 6 MMAs of 80 ns    (167 B per ns of tensor time)
+//   two units x 224 tokens  105 KB for 12 MMAs of 76 ns   (116)
+// so two units share every staged activation byte, which T = 224 tokens leave room for in tensor memory: 2 x 224
+// accumulator columns, two alternating sets of metadata and scales (24 each) and the outlier scales (16) are 512.  Token
+// tiles are cut at any multiple of 32, so that they are equally wide and nothing is multiplied for padding.
+// Under a sustained load the GPU's power limit holds the clock at 1.3 to 1.45 GHz (1.97 otherwise); two-unit tasks then run
+// their four MMAs of a stage in 640 cycles (the pipe needs ~600), one-unit tasks their two in 427 (300).
 //
-// What was measured on the way (B200, 2048 tokens, 4096 -> 11008, 1:8 outliers; the single-CTA kernel takes 84 us):
-// a first version with one release per slot, a separate TMEM-mover thread and cluster-scope release / acquire on the
-// forwarding hop took 213 us -- a remote mbarrier arrive with .release.cluster costs ~0.8 us under load (the default
-// semantics suffice: the data was written by the bulk-copy engine and is read by the tensor core, both outside the
-// forwarding thread's view of memory) -> 94 us; warp-uniform issue loops, the copies to TMEM folded into the MMA issuer,
-// one barrier per slot and batches of landed slots -> 78 us; two lanes per producer -> 67 us (2.75 PFLOP/s).
+// Sustained (0.3 s of calls), one unit x 256 tokens before -> now: 2048 x 4096 -> 11008 80.2 -> 77.5 us, 8192 x 11008 -> 4096
+// 278 -> 259 us, with E4M3 scales 4096 x 16384 -> 4096 265 -> 232 us, dense inliers 1500 x 11008 -> 4096 90 -> 78 us; K over
+// several pairs 130 x 16384 -> 4096 27 -> 21 us, 400 x 16384 -> 1024 35 -> 17 us; 500 x 4096 -> 4096 21.1 -> 14.3 us.
+//
+// Few tasks (narrow matrices, few tokens): a task is one chain of stages at ~0.16 us each however few tokens it has, so its K
+// range is split over 2 to 4 pairs of a larger cluster; their fp32 partial tiles meet in shared memory and every CTA adds
+// one slice of rows over the splits, in order (no global scratch, reproducible).
+//
+// Per CTA: warps 0 / 2 / 3 bulk-copy producers (weight records / activation codes / scale atoms; two lanes each), warps
+// 4..19 epilogue in four groups (TMEM -> registers as packed bf16, TMEM handed back, transposed stores under the next
+// task's K loop).  Even CTA (leader): warp 1 copies metadata and scales of both CTAs to TMEM (pair-wide tcgen05.cp) and
+// issues the pair-wide MMAs; its tcgen05.commit signals "slots consumed" / "accumulator complete" to the barriers of both
+// CTAs.  Odd CTA: two lanes of warp 1 forward "my part of the slot has landed" to the leader's barriers.  Every wait is
+// bounded.
+//
+// Facts behind the form of the loops (measured on B200): a remote mbarrier arrive with .release.cluster costs ~0.8 us under
+// load (the default semantics suffice: the data was written by the bulk-copy engine and is read by the tensor core, both
+// outside the forwarding thread's view of memory); descriptors and TMEM addresses of tcgen05 instructions are
+// uniform-register operands, so the issue loop is warp-uniform with one elected lane; a trip of a single-thread loop costs
+// 0.3 us, hence two lanes per producer and runs of landed slots in the issuer; a pair-wide commit costs the pipe ~80 ns.
 #include <cuda_bf16.h>
+#include <type_traits>
 
 #include "sdq_internal.h"
 #include "sdq_layout.h"
@@ -29,49 +46,94 @@
 
 namespace sdq {
 
-constexpr int PAIR_THREADS = 416;            // 13 warps
-constexpr int PAIR_MAX_SLOTS = 8;
-constexpr int PAIR_TAIL = 2048 + 384 + 128;  // transpose buffer (2 groups x 4 tokens x 128 features bf16) + barriers + alignment slack
+constexpr int PAIR_THREADS = 640;            // 20 warps
+constexpr int PAIR_MAX_SLOTS = 12;
+constexpr int PAIR_STG = 4096;               // transpose buffer: 4 groups x 4 tokens x 128 features bf16
+constexpr int PAIR_TAIL = PAIR_STG + (2 * PAIR_MAX_SLOTS + 4) * 8 + 16 + 128;   // + barriers + alignment slack
+
+// Geometry of a launch.  TWO: tasks of two units (and one), FULL: of one unit with token tiles of up to 256, both with the
+// ring's and tensor memory's geometry known at compile time (the issue loop pays for every runtime parameter: 474 against
+// 427 cycles per stage of two 256-token MMAs); FLEX: one unit, narrower tiles, geometry from the launch parameters.
+enum { PAIR_TWO = 0, PAIR_FULL = 1, PAIR_FLEX = 2 };
 
 template <bool B32, bool DENSE>
 struct PairGeom {
   static constexpr bool S32 = B32 || DENSE;                       // one scale per 32 K
-  static constexpr uint32_t WIB = DENSE ? 17408u : (B32 ? 11264u : 10752u);   // inlier weight record (>= the outlier record)
-  static constexpr uint32_t NA = S32 ? 2u : 1u;                   // scale atoms per token tile and inlier stage
-  static constexpr uint32_t ATOMS = S32 ? 4u : 3u;                // inlier: NA per token half; first outlier stage: SFA_out + 2 SFB_out
-  static constexpr uint32_t SL_B = WIB;                           // own 128 tokens: B4 (256 K) or B8 (128 K)
-  static constexpr uint32_t SL_SF = WIB + 16384u;
-  static constexpr uint32_t SLOT = SL_SF + ATOMS * SF_ATOM_BYTES; // 28672 / 29696 / 35840
-  static constexpr uint32_t NSLOT = S32 ? 6u : 8u;                // ring slots, released two at a time (see the MMA issuer)
-  static constexpr uint32_t MS = S32 ? 32u : 16u;                 // TMEM columns of metadata / scales per ring slot
-  static constexpr uint32_t SM_STG = NSLOT * SLOT;                // transpose buffer, then the barriers
-  static constexpr uint32_t SM_BARS = SM_STG + 2048u;
-  static constexpr uint32_t SMEM = SM_STG + PAIR_TAIL;
-  static_assert(256u + MS * NSLOT + 24u <= 512u, "TMEM columns");
-  static_assert(SMEM <= 232448u, "shared memory");
+  static constexpr uint32_t WIB = DENSE ? 17408u : (B32 ? 11264u : 10752u);   // inlier weight record (>= the outlier record + one atom)
+  static constexpr uint32_t NA = S32 ? 2u : 1u;                   // scale atoms per 128 rows / tokens and inlier stage
+  // TMEM columns of one set of metadata / scales: E 2 x 4 | SFA 2 x 4 NA | SFB 8 NA; two sets alternate; then SFA_out 2 x 4 | SFB_out 8
+  static constexpr uint32_t SFA = 8u, SFB = 8u + 8u * NA, SET = 8u + 16u * NA, COLS = 2u * SET + 16u;
 };
+__host__ __device__ constexpr int pair_tmax(int form, bool s32) { return form == PAIR_TWO ? (s32 ? 192 : 224) : 256; }
+// slot = | weight record of each unit | codes of T / 2 tokens | scale atoms of the tokens, [128 tokens][K-block] |
+// (first outlier stage: the units' row-scale atoms directly behind their outlier records, the token-scale atoms like SFB)
+__host__ __device__ constexpr uint32_t pair_slot_bytes(uint32_t wib, bool s32, int units, int T) {
+  return (uint32_t)units * wib + (uint32_t)T * 64u + (s32 ? 4u : 2u) * SF_ATOM_BYTES;
+}
+__host__ __device__ constexpr int pair_slots(uint32_t slot) {      // released two at a time: an even number
+  const int n = (int)((232448u - PAIR_TAIL) / slot) / 2 * 2;
+  return n < PAIR_MAX_SLOTS ? n : PAIR_MAX_SLOTS;
+}
 
-template <bool F32_OUT, bool B32, bool DENSE>
-__global__ void __cluster_dims__(2, 1, 1) __maxnreg__(128)
-sdq_linear_pair_kernel(const LinearParams p)
+struct PairTask { int u0, nu, mt; };
+template <int FORM>
+__device__ __forceinline__ PairTask pair_task(const LinearParams& p, int task) {
+  PairTask t;
+  if (FORM != PAIR_TWO) {
+    t.mt = task / p.pt_units; t.u0 = task - t.mt * p.pt_units; t.nu = 1;
+    return t;
+  }
+  const int rp = p.pt_units >> 1;                                 // unit pairs per token tile
+  if (task < p.pt_doubles) {
+    t.mt = task / rp; t.u0 = 2 * (task - t.mt * rp); t.nu = 2;
+    return t;
+  }
+  const int s = task - p.pt_doubles;
+  t.nu = 1;
+  if (s < p.pt_split) {
+    const int d = p.pt_doubles + (s >> 1);
+    t.mt = d / rp; t.u0 = 2 * (d - t.mt * rp) + (s & 1);
+  } else {
+    t.mt = s - p.pt_split; t.u0 = p.pt_units - 1;                 // the odd unit of every token tile
+  }
+  return t;
+}
+// first 32-token group of token tile `mt`
+__device__ __forceinline__ int pair_group0(const LinearParams& p, int mt) { return (int)((int64_t)mt * p.pt_groups / p.pt_mtiles); }
+
+template <bool F32_OUT, bool B32, bool DENSE, int FORM>
+__global__ void __maxnreg__(96)
+sdq_linear_pair_kernel(const __grid_constant__ LinearParams p)
 {
   using G = PairGeom<B32, DENSE>;
   constexpr bool S32 = G::S32;
-  constexpr uint32_t NSLOT = G::NSLOT, SLOT = G::SLOT, MS = G::MS, NA = G::NA;
+  constexpr uint32_t NA = G::NA;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   uint8_t* sm = smem_raw + ((128 - (ptx::smem_u32(smem_raw) & 127)) & 127);
-  uint64_t* full = reinterpret_cast<uint64_t*>(sm + G::SM_BARS);   // the three producers' parts of slot s have landed (leader: + the peer's)
+  constexpr uint32_t SL_B = FORM == PAIR_TWO ? 2u * G::WIB : G::WIB, FIXED_T = (uint32_t)pair_tmax(FORM, S32);
+  constexpr uint32_t FIXED_SLOT = pair_slot_bytes(G::WIB, S32, FORM == PAIR_TWO ? 2 : 1, (int)FIXED_T);
+  const uint32_t TMAX = FORM == PAIR_FLEX ? (uint32_t)p.n_tile : FIXED_T, SLOT = FORM == PAIR_FLEX ? (uint32_t)p.slot_bytes : FIXED_SLOT;
+  const uint32_t NSLOT = FORM == PAIR_FLEX ? (uint32_t)p.nslot : (uint32_t)pair_slots(FIXED_SLOT), SL_SF = SL_B + TMAX * 64u;
+  const bool acc2 = FORM == PAIR_FLEX && p.pt_acc2;
+  uint8_t* stg_base = sm + NSLOT * SLOT;
+  uint64_t* full = reinterpret_cast<uint64_t*>(stg_base + PAIR_STG);   // the three producers' parts of slot s have landed (leader: + the peer's)
   uint64_t* empty = full + PAIR_MAX_SLOTS;                         // [s / 2]: the MMAs that read slots s and s ^ 1 have completed
-  uint64_t* acc_full = empty + PAIR_MAX_SLOTS;
-  uint64_t* acc_empty = acc_full + 1;                              // leader: all 16 epilogue warps of the pair have drained TMEM
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 1);
+  uint64_t* acc_full = empty + PAIR_MAX_SLOTS;                     // [2]
+  uint64_t* acc_empty = acc_full + 2;                              // [2] leader: all epilogue warps of the pair have drained the accumulator
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 2);
   volatile uint32_t* timed_out = tmem_slot + 1;                    // an epilogue group's wait gave up
 
-  const uint32_t rank = ptx::cluster_ctarank();                    // 0 = leader
-  const int pair = (int)(blockIdx.x >> 1), n_pairs = (int)(gridDim.x >> 1);
-  const int RTP = (int)(p.N / (2 * TILE_ROWS));                    // row-pair tiles
+  const uint32_t crank = ptx::cluster_ctarank(), rank = crank & 1u, lead = crank & ~1u;   // rank 0 = leader of the pair
+  const int ks = FORM == PAIR_FLEX ? p.pt_ks : 1, split = (int)(crank >> 1);   // pairs that share the K range of a task
+  const int pair = (int)blockIdx.x / (2 * ks), n_pairs = (int)gridDim.x / (2 * ks);
+  const uint16_t both = (uint16_t)(3u << lead);
+  const int RT = (int)(p.N / TILE_ROWS);
   const int T1 = p.out_n ? (int)(p.K / K1) : 0, T2 = (int)(p.K / K2);
+  const int i0 = ks == 1 ? 0 : split * T2 / ks, o0 = ks == 1 ? 0 : split * T1 / ks;       // first inlier / outlier stage of this pair
+  const int NI = ks == 1 ? T2 : (split + 1) * T2 / ks - i0, S = NI + (ks == 1 ? T1 : (split + 1) * T1 / ks - o0);
+  const int my_tasks = p.pt_tasks > pair ? (p.pt_tasks - pair + n_pairs - 1) / n_pairs : 0;
+  const int total = my_tasks * S;                                  // stages of this CTA, numbered through its tasks
 
   if (tid == 0) ptx::griddep_launch_dependents();
   if (tid == 0) {
@@ -80,8 +142,7 @@ sdq_linear_pair_kernel(const LinearParams p)
       ptx::mbar_init(&full[s], rank == 0 ? 4 : 3);
       if (!(s & 1)) ptx::mbar_init(&empty[s >> 1], 1);
     }
-    ptx::mbar_init(acc_full, 1);
-    ptx::mbar_init(acc_empty, 16);
+    for (int a = 0; a < 2; ++a) { ptx::mbar_init(&acc_full[a], 1); ptx::mbar_init(&acc_empty[a], 32); }
     ptx::fence_barrier_init();
   }
   if (warp == 1) ptx::tmem_alloc_pair(tmem_slot, 512);
@@ -90,67 +151,69 @@ sdq_linear_pair_kernel(const LinearParams p)
   ptx::cluster_sync();                                             // both CTAs' barriers exist before any remote arrival
   ptx::tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  const uint32_t meta = tmem + (FORM == PAIR_TWO || acc2 ? 2u * TMAX : TMAX);   // metadata and scales follow the accumulator columns
 
-  if (warp == 0 || warp == 6 || warp == 7) {
+  if (warp == 0 || warp == 2 || warp == 3) {
     if (lane < 2) {
       // ---------------- producers (both CTAs): role 0 = own weight records, 1 = own activation codes, 2 = scale atoms.
-      // One trip of a producer's loop (barrier wait, address arithmetic, expect-tx, copy) takes ~0.3 us, which one thread
-      // per role cannot hide at two MMAs per stage; ring slots are released in pairs, so lanes 0 and 1 of the warp run the
-      // loop in lockstep, lane l filling the slots of parity l: two stages per trip.
-      const int role = warp == 0 ? 0 : (int)warp - 5;
+      // Ring slots are released in pairs, so lanes 0 and 1 of the warp run the loop in lockstep, lane l filling the slots of
+      // parity l: two stages per trip.
+      const int role = warp == 0 ? 0 : (int)warp - 1;
       if (role != 0) ptx::griddep_wait();    // activations come from an earlier kernel; weights do not
-      const int S = T2 + T1;
-      const int my_tiles = p.total_tiles > pair ? (p.total_tiles - pair + n_pairs - 1) / n_pairs : 0;
-      const int total = my_tiles * S;                                        // stages of this CTA, numbered through its tiles
       bool ok = true;
       uint32_t s = lane, wrapped = 0, ph = 0;
-      int tseq = 0, k = (int)lane;                                           // this lane's stage: tile number in the CTA's sequence, stage in the tile
-      if (k >= S) { k -= S; ++tseq; }                                        // (S >= 2)
-      int cur = -1, rt = 0, mt0 = 0, have = 0;
-      bool own = false;
+      int tseq = 0, k = (int)lane;                                           // this lane's stage: task number in the CTA's sequence, stage in the task
+      while (k >= S) { k -= S; ++tseq; }
+      int cur = -1, rt0 = 0, rt1 = 0, nu = 1, have = 0;
+      int64_t t0 = 0;
+      size_t a0 = 0;
+      uint32_t own = 0;
       for (int i = (int)lane; i < total && ok; i += 2) {
         if (tseq != cur) {
           cur = tseq;
-          const int tile = pair + tseq * n_pairs;
-          rt = 2 * (tile % RTP) + (int)rank;
-          mt0 = 2 * (tile / RTP);                                            // first activation tile of the token tile
-          have = min(2, (int)(p.aoff.Mpad / 128) - mt0);                               // activation tiles that exist (1 or 2)
-          own = (int)rank < have;                                            // this CTA's 128 tokens exist
+          const PairTask t = pair_task<FORM>(p, pair + tseq * n_pairs);
+          nu = t.nu;
+          rt0 = min(2 * t.u0 + (int)rank, RT - 1);                           // (an odd number of row tiles: the last unit's second half
+          rt1 = min(2 * t.u0 + 2 + (int)rank, RT - 1);                       //  repeats the last tile and is not stored)
+          a0 = (size_t)pair_group0(p, t.mt);                                 // the tile's first scale atom
+          const int T = 32 * (pair_group0(p, t.mt + 1) - (int)a0);
+          t0 = (int64_t)a0 * 32 + rank * (T / 2);
+          own = (uint32_t)max((int64_t)0, min((int64_t)(T / 2), p.aoff.Mpad - t0)) * 128u;   // this CTA's code bytes that exist
+          have = T > 128 && (int)a0 + 4 < p.aoff.atoms ? 2 : 1;
         }
         if (wrapped && !(ok = ptx::mbar_wait(&empty[s >> 1], ph ^ 1))) break;
         uint8_t* st = sm + (size_t)s * SLOT;
-        const bool inl = k < T2, first_o = (k == T2);
-        const int ko = k - T2;                                               // outlier stage number
+        const bool inl = k < NI, first_o = (k == NI);
+        const int ki = i0 + k, ko = o0 + k - NI;                             // inlier / outlier stage number
         if (role == 0) {
-          if (inl) {
-            ptx::mbar_expect_tx(&full[s], G::WIB);
-            ptx::bulk_g2s(st, p.w + p.poff.wi + ((size_t)rt * T2 + k) * G::WIB, G::WIB, &full[s]);
-          } else {
-            ptx::mbar_expect_tx(&full[s], WO_BYTES + (first_o ? SF_ATOM_BYTES : 0u));
-            ptx::bulk_g2s(st, p.w + p.poff.wo + ((size_t)rt * T1 + ko) * WO_BYTES, WO_BYTES, &full[s]);
-            if (first_o) ptx::bulk_g2s(st + G::SL_SF, p.w + p.poff.sfa_out + (size_t)rt * SF_ATOM_BYTES, SF_ATOM_BYTES, &full[s]);
+          const uint32_t nb = inl ? G::WIB : (uint32_t)WO_BYTES;
+          const uint8_t* base = inl ? p.w + p.poff.wi + (size_t)ki * G::WIB : p.w + p.poff.wo + (size_t)ko * WO_BYTES;
+          const size_t step = inl ? (size_t)T2 * G::WIB : (size_t)T1 * WO_BYTES;   // bytes between row tiles
+          ptx::mbar_expect_tx(&full[s], (uint32_t)nu * (nb + (first_o ? SF_ATOM_BYTES : 0u)));
+          ptx::bulk_g2s(st, base + (size_t)rt0 * step, nb, &full[s]);
+          if (FORM == PAIR_TWO && nu == 2) ptx::bulk_g2s(st + G::WIB, base + (size_t)rt1 * step, nb, &full[s]);
+          if (first_o) {
+            ptx::bulk_g2s(st + WO_BYTES, p.w + p.poff.sfa_out + (size_t)rt0 * SF_ATOM_BYTES, SF_ATOM_BYTES, &full[s]);
+            if (FORM == PAIR_TWO && nu == 2) ptx::bulk_g2s(st + G::WIB + WO_BYTES, p.w + p.poff.sfa_out + (size_t)rt1 * SF_ATOM_BYTES, SF_ATOM_BYTES, &full[s]);
           }
         } else if (role == 1) {
           if (!own) {
             ptx::mbar_arrive(&full[s]);
-          } else if (inl) {
-            ptx::mbar_expect_tx(&full[s], B4_BYTES);
-            ptx::bulk_g2s(st + G::SL_B, p.x + p.aoff.xi + (size_t)k * p.aoff.xi_stride + (size_t)(mt0 + (int)rank) * B4_BYTES, B4_BYTES, &full[s]);
           } else {
-            ptx::mbar_expect_tx(&full[s], XO_BYTES);
-            ptx::bulk_g2s(st + G::SL_B, p.x + p.aoff.xo + (size_t)ko * p.aoff.xo_stride + (size_t)(mt0 + (int)rank) * XO_BYTES, XO_BYTES, &full[s]);
+            ptx::mbar_expect_tx(&full[s], own);
+            ptx::bulk_g2s(st + SL_B, (inl ? p.x + p.aoff.xi + (size_t)ki * p.aoff.xi_stride : p.x + p.aoff.xo + (size_t)ko * p.aoff.xo_stride) + (size_t)t0 * 128u,
+                          own, &full[s]);
           }
         } else {
           if (inl) {
+            const uint8_t* xs = p.x + p.aoff.xi + (size_t)ki * p.aoff.xi_stride + (size_t)p.aoff.Mpad * 128u + a0 * (NA * SF_ATOM_BYTES);
             ptx::mbar_expect_tx(&full[s], (uint32_t)have * NA * SF_ATOM_BYTES);
             for (int a = 0; a < have; ++a)
-              ptx::bulk_g2s(st + G::SL_SF + a * NA * SF_ATOM_BYTES, p.x + p.aoff.xi + (size_t)k * p.aoff.xi_stride + (size_t)p.aoff.Mpad * 128 + (size_t)(4 * (mt0 + a)) * NA * SF_ATOM_BYTES,
-                            NA * SF_ATOM_BYTES, &full[s]);
+              ptx::bulk_g2s(st + SL_SF + a * NA * SF_ATOM_BYTES, xs + a * (4 * NA * SF_ATOM_BYTES), NA * SF_ATOM_BYTES, &full[s]);
           } else if (first_o) {
             ptx::mbar_expect_tx(&full[s], (uint32_t)have * SF_ATOM_BYTES);
             for (int a = 0; a < have; ++a)
-              ptx::bulk_g2s(st + G::SL_SF + (1 + a) * SF_ATOM_BYTES, p.x + p.aoff.sfb_out + (size_t)(4 * (mt0 + a)) * SF_ATOM_BYTES, SF_ATOM_BYTES,
-                            &full[s]);
+              ptx::bulk_g2s(st + SL_SF + a * SF_ATOM_BYTES, p.x + p.aoff.sfb_out + (a0 + 4 * (size_t)a) * SF_ATOM_BYTES, SF_ATOM_BYTES, &full[s]);
           } else {
             ptx::mbar_arrive(&full[s]);
           }
@@ -158,229 +221,247 @@ sdq_linear_pair_kernel(const LinearParams p)
         s += 2;
         if (s >= NSLOT) { s -= NSLOT; wrapped = 1; ph ^= 1; }
         k += 2;
-        if (k >= S) { k -= S; ++tseq; }
+        while (k >= S) { k -= S; ++tseq; }
       }
       if (!ok) atomicOr(&p.flags[FLAG_TIMEOUT], 1u);
     }
   } else if (warp == 1 && rank == 1) {
     if (lane < 2) {
       // ---------------- odd CTA: forward "my part of the slot has landed" to the leader's barrier (lane l: slots of parity l)
-      const int S = T2 + T1;
-      const int my_tiles = p.total_tiles > pair ? (p.total_tiles - pair + n_pairs - 1) / n_pairs : 0;
-      const int total = my_tiles * S;
       bool ok = true;
       uint32_t s = lane, ph = 0;
       for (int i = (int)lane; i < total; i += 2) {
         if (!(ok = ptx::mbar_wait(&full[s], ph))) break;
-        ptx::mbar_arrive_remote(&full[s], 0);
+        ptx::mbar_arrive_remote(&full[s], lead);
         s += 2;
         if (s >= NSLOT) { s -= NSLOT; ph ^= 1; }
       }
       if (!ok) atomicOr(&p.flags[FLAG_TIMEOUT], 1u);
     }
   } else if (warp == 1) {
-    {
-      // ---------------- MMA issuer (leader): per slot the copies of metadata and scales to TMEM (both CTAs), then the
-      // pair-wide MMAs; tcgen05.cp and tcgen05.mma of one thread execute in issue order, so nothing waits in between, and
-      // TMEM buffer s (metadata, scales) simply belongs to ring slot s.
-      // The whole warp runs the loop and one elected lane issues: descriptors and TMEM addresses of tcgen05 instructions
-      // are uniform-register operands, and only warp-uniform control flow keeps the loop's arithmetic on the uniform
-      // datapath.  Even so one trip of the loop (barrier test, vote, election) costs more than the tensor pipe needs for
-      // the two MMAs of a slot, so a trip takes every slot that has landed: lane i tests slot s + i, one ballot gives the
-      // run of ready slots, and their instructions go out back to back.  When the pipe is the bottleneck the batches grow
-      // and the loop cost is spread; when the copies are, a batch is one slot and the loop is idle anyway.
-      // A pair-wide commit costs the pipe a bubble of ~80 ns (measured), hence one release per two slots.
-      bool ok = true;
-      const uint32_t smb = ptx::smem_u32(sm);
-      uint32_t s = 0, ph = 0, tcount = 0;
+    // ---------------- MMA issuer (leader): per slot the copies of metadata and scales to TMEM (both CTAs), then the
+    // pair-wide MMAs of its one or two units; tcgen05.cp and tcgen05.mma of one thread execute in issue order, so nothing
+    // waits in between and two alternating TMEM sets serve all slots.
+    // The whole warp runs the loop and one elected lane issues.  One trip of the loop (barrier test, vote, election) costs
+    // more than the tensor pipe needs for two MMAs, so a trip takes every slot that has landed: lane i tests slot s + i, one
+    // ballot gives the run of ready slots, and their instructions go out back to back.  (Testing the slots behind a run
+    // while the run is being issued hides that latency, but the answers are stale: 690 against 640 cycles per stage.)
+    // A pair-wide commit costs the pipe a bubble of ~80 ns, hence one release per two slots.
+    bool ok = true;
+    const uint32_t smb = ptx::smem_u32(sm);
+    uint32_t s = 0, ph = 0, par = 0;                                // ring slot, its lap parity, parity of the TMEM set
+    const uint64_t d_a = ptx::smem_desc(smb, 128, 256), d_b = ptx::smem_desc(smb + SL_B, 128, 1024);
+    const uint64_t d_cp = ptx::smem_desc(smb, 0, 128), d_sf = ptx::smem_desc(smb + SL_SF, 0, 128);   // copies to TMEM: weight record, scale atoms
+    constexpr uint32_t wib16 = G::WIB >> 4, atom16 = SF_ATOM_BYTES >> 4;
+    const uint32_t slot16 = SLOT >> 4;
+    const uint32_t sfo = meta + 2u * G::SET;                        // outlier scales of the task: SFA_out 2 x 4 | SFB_out 8
+    uint32_t tcount = 0;
+    for (int task = pair; task < p.pt_tasks && ok; task += n_pairs, ++tcount) {
+      const PairTask t = pair_task<FORM>(p, task);
+      const int nu = t.nu;
+      const uint32_t T = 32u * (uint32_t)(pair_group0(p, t.mt + 1) - pair_group0(p, t.mt));
       // (two-level scaling: the .block16 kind reads its scale codes as unsigned E4M3 when bit 23 is clear)
-      const uint32_t id4[2] = {ptx::idesc_block_scaled(256, 256, 1, true, 0, 0) ^ (p.tw ? (1u << 23) : 0u),
-                               ptx::idesc_block_scaled(256, 256, 1, true, 2, 2)};
-      const uint32_t id8 = ptx::idesc_block_scaled(256, 256, 0, true, 0, 0);
-      const uint32_t idd[2] = {ptx::idesc_block_scaled(256, 256, 1, false, 0, 0), ptx::idesc_block_scaled(256, 256, 1, false, 2, 2)};
-      const uint64_t d_a = ptx::smem_desc(smb, 128, 256), d_b = ptx::smem_desc(smb + G::SL_B, 128, 1024);
-      const uint64_t d_e_in = ptx::smem_desc(smb + A_IN_BYTES, 0, 128);
-      const uint64_t d_sfa_in = ptx::smem_desc(smb + (DENSE ? 2 * A_IN_BYTES : A_IN_BYTES + E_IN_BYTES), 0, 128);
-      const uint64_t d_e_out = ptx::smem_desc(smb + A_OUT_BYTES, 0, 128);
-      const uint64_t d_sf0 = ptx::smem_desc(smb + G::SL_SF, 0, 128), d_sf1 = ptx::smem_desc(smb + G::SL_SF + SF_ATOM_BYTES, 0, 128);
-      const uint64_t d_sf2 = ptx::smem_desc(smb + G::SL_SF + 2 * SF_ATOM_BYTES, 0, 128);
-      constexpr uint32_t slot16 = SLOT >> 4;
-      const int S = T2 + T1;
-      for (int tile = pair; tile < p.total_tiles && ok; tile += n_pairs, ++tcount) {
-        const uint32_t sfo = tmem + 256u + MS * NSLOT + 12u * (tcount & 1);   // outlier row / token scales: two alternating buffers
-        int k = 0;
-        while (k < S) {
-          // lane i: has slot s + i (the i-th next stage of this tile) landed in both CTAs?
-          const uint32_t idx = s + lane, sl = idx >= NSLOT ? idx - NSLOT : idx;
-          // (four slots ahead at most: testing all eight costs more per trip than the longer runs save, measured 1 %)
-          const bool r = (int)lane < min(4, S - k) && ptx::mbar_test(&full[sl], idx >= NSLOT ? ph ^ 1 : ph);
-          int n = __ffs(~__ballot_sync(0xffffffffu, r)) - 1;     // length of the run of ready slots
-          if (n == 0) {   // nothing yet: wait for the next slot, then look again (its neighbours tend to land with it)
-            ok = __all_sync(0xffffffffu, ptx::mbar_wait(&full[s], ph));
-            if (!ok) break;
-            continue;
-          }
-          if (k == 0 && tcount > 0) {   // the epilogues of both CTAs must have drained the accumulator of the previous tile
-            ok = __all_sync(0xffffffffu, ptx::mbar_wait(acc_empty, (tcount - 1) & 1));
-            if (!ok) break;
-          }
-          ptx::tc_fence_after();
-          if (ptx::elect_one()) {
-            uint32_t ss = s;
-            for (int kk = k; kk < k + n; ++kk) {
-              const uint64_t so = (uint64_t)(ss * slot16);
-              const uint32_t mb = tmem + 256u + MS * ss;
-              const uint32_t acc = kk ? 1u : 0u;   // the first MMA of the tile overwrites the accumulator
-              if (kk < T2) {
-                if constexpr (!DENSE) ptx::tc2_cp_128x128b(mb + 0, d_e_in + so);
-                ptx::tc2_cp_32x128b_warpx4(mb + 4, d_sfa_in + so);
-                if constexpr (S32) {
-                  // scale words: weights K-block 0 / 1 at +4 / +8; tokens K-block kb, token tile a at +12 + 4 (2 kb + a), staged
-                  // as [token tile][K-block]
-                  ptx::tc2_cp_32x128b_warpx4(mb + 8, d_sfa_in + so + (SF_ATOM_BYTES >> 4));
-                  ptx::tc2_cp_32x128b_warpx4(mb + 12, d_sf0 + so);
-                  ptx::tc2_cp_32x128b_warpx4(mb + 20, d_sf1 + so);
-                  ptx::tc2_cp_32x128b_warpx4(mb + 16, d_sf2 + so);
-                  ptx::tc2_cp_32x128b_warpx4(mb + 24, d_sf2 + so + (SF_ATOM_BYTES >> 4));
-                } else {
-                  ptx::tc2_cp_32x128b_warpx4(mb + 8, d_sf0 + so);
-                  ptx::tc2_cp_32x128b_warpx4(mb + 12, d_sf1 + so);
-                }
-                if constexpr (DENSE) {
+      const uint32_t id4[2] = {ptx::idesc_block_scaled(256, T, 1, true, 0, 0) ^ (p.tw ? (1u << 23) : 0u),
+                               ptx::idesc_block_scaled(256, T, 1, true, 2, 2)};
+      const uint32_t id8 = ptx::idesc_block_scaled(256, T, 0, true, 0, 0);
+      const uint32_t idd[2] = {ptx::idesc_block_scaled(256, T, 1, false, 0, 0), ptx::idesc_block_scaled(256, T, 1, false, 2, 2)};
+      const bool wide = T > 128u;
+      const uint32_t ab = acc2 ? tcount & 1u : 0u, use = acc2 ? tcount >> 1 : tcount;
+      const uint32_t acc0 = tmem + ab * TMAX, acc1 = acc0 + TMAX;
+      // instructions of the stages k .. k + n - 1 of the task in ring slots s ..., by one elected lane
+      auto issue = [&](auto units, int k, int n) {
+        constexpr int NU = decltype(units)::value;
+        uint32_t ss = s, pp = par;
+        for (int kk = k; kk < k + n; ++kk) {
+          const uint64_t so = (uint64_t)(ss * slot16);
+          const uint32_t mb = meta + (pp ? G::SET : 0u);
+          pp ^= 1u;
+          const uint32_t acc = kk ? 1u : 0u;   // the first MMA of the task overwrites the accumulator
+          if (kk < NI) {
+            // scale words of the tokens: K-block kb, 128 tokens a at SFB + 8 kb + 4 a, staged as [128 tokens][K-block]
+            ptx::tc2_cp_32x128b_warpx4(mb + G::SFB, d_sf + so);
+            if constexpr (S32) ptx::tc2_cp_32x128b_warpx4(mb + G::SFB + 8, d_sf + so + atom16);
+            if (wide) {
+              ptx::tc2_cp_32x128b_warpx4(mb + G::SFB + 4, d_sf + so + NA * atom16);
+              if constexpr (S32) ptx::tc2_cp_32x128b_warpx4(mb + G::SFB + 12, d_sf + so + 3 * atom16);
+            }
 #pragma unroll
-                  for (uint32_t j = 0; j < 4; ++j)
-                    ptx::mma2_mxf4(tmem, d_a + so + ((4096 * j) >> 4), d_b + so + ((256 * j) >> 4), idd[j & 1], mb + 4 + 4 * (j >> 1),
-                                   mb + 12 + 8 * (j >> 1), j ? 1u : acc);
-                } else if constexpr (B32) {
-                  ptx::mma2_sp_nvf4(tmem, d_a + so, d_b + so, id4[0], mb, mb + 4, mb + 12, acc);
-                  ptx::mma2_sp_nvf4(tmem, d_a + so + (4096 >> 4), d_b + so + (512 >> 4), id4[0], mb + 2, mb + 8, mb + 20, 1u);
-                } else {
-                  ptx::mma2_sp_mxf4(tmem, d_a + so, d_b + so, id4[0], mb, mb + 4, mb + 8, acc);
-                  ptx::mma2_sp_mxf4(tmem, d_a + so + (4096 >> 4), d_b + so + (512 >> 4), id4[1], mb + 2, mb + 4, mb + 8, 1u);
-                }
+            for (int u = 0; u < NU; ++u) {
+              const uint64_t wo = so + (u ? wib16 : 0u);
+              const uint32_t sfa = mb + G::SFA + (u ? 4u * NA : 0u), d = u ? acc1 : acc0;
+              [[maybe_unused]] const uint32_t e = mb + (u ? 4u : 0u);
+              constexpr uint32_t SFA_OFF = (DENSE ? 2 * A_IN_BYTES : A_IN_BYTES + E_IN_BYTES) >> 4;
+              if constexpr (!DENSE) ptx::tc2_cp_128x128b(e, d_cp + wo + (A_IN_BYTES >> 4));
+              ptx::tc2_cp_32x128b_warpx4(sfa, d_cp + wo + SFA_OFF);
+              if constexpr (S32) ptx::tc2_cp_32x128b_warpx4(sfa + 4, d_cp + wo + SFA_OFF + atom16);
+              if constexpr (DENSE) {
+#pragma unroll
+                for (uint32_t j = 0; j < 4; ++j)
+                  ptx::mma2_mxf4(d, d_a + wo + ((4096 * j) >> 4), d_b + so + ((256 * j) >> 4), idd[j & 1], sfa + 4 * (j >> 1),
+                                 mb + G::SFB + 8 * (j >> 1), j ? 1u : acc);
+              } else if constexpr (B32) {
+                ptx::mma2_sp_nvf4(d, d_a + wo, d_b + so, id4[0], e, sfa, mb + G::SFB, acc);
+                ptx::mma2_sp_nvf4(d, d_a + wo + (4096 >> 4), d_b + so + (512 >> 4), id4[0], e + 2, sfa + 4, mb + G::SFB + 8, 1u);
               } else {
-                ptx::tc2_cp_128x128b(mb + 0, d_e_out + so);
-                if (kk == T2) {
-                  ptx::tc2_cp_32x128b_warpx4(sfo, d_sf0 + so);
-                  ptx::tc2_cp_32x128b_warpx4(sfo + 4, d_sf1 + so);
-                  ptx::tc2_cp_32x128b_warpx4(sfo + 8, d_sf2 + so);
-                }
-                ptx::mma2_sp_mxf8(tmem, d_a + so, d_b + so, id8, mb, sfo, sfo + 4, acc);
-                ptx::mma2_sp_mxf8(tmem, d_a + so + (4096 >> 4), d_b + so + (512 >> 4), id8, mb + 2, sfo, sfo + 4, 1u);
+                ptx::mma2_sp_mxf4(d, d_a + wo, d_b + so, id4[0], e, sfa, mb + G::SFB, acc);
+                ptx::mma2_sp_mxf4(d, d_a + wo + (4096 >> 4), d_b + so + (512 >> 4), id4[1], e + 2, sfa, mb + G::SFB, 1u);
               }
-              if (ss & 1) ptx::tc2_commit_both(&empty[ss >> 1]);     // slots ss - 1 and ss may be refilled (both CTAs)
-              if (kk == S - 1) ptx::tc2_commit_both(acc_full);       // the tile's accumulator is complete (both CTAs)
-              if (++ss == NSLOT) ss = 0;
+            }
+          } else {
+            if (kk == NI) {
+              ptx::tc2_cp_32x128b_warpx4(sfo, d_cp + so + (WO_BYTES >> 4));
+              if constexpr (NU == 2) ptx::tc2_cp_32x128b_warpx4(sfo + 4, d_cp + so + wib16 + (WO_BYTES >> 4));
+              ptx::tc2_cp_32x128b_warpx4(sfo + 8, d_sf + so);
+              if (wide) ptx::tc2_cp_32x128b_warpx4(sfo + 12, d_sf + so + atom16);
+            }
+#pragma unroll
+            for (int u = 0; u < NU; ++u) {
+              const uint64_t wo = so + (u ? wib16 : 0u);
+              const uint32_t e = mb + (u ? 4u : 0u), d = u ? acc1 : acc0, sfa = sfo + (u ? 4u : 0u);
+              ptx::tc2_cp_128x128b(e, d_cp + wo + (A_OUT_BYTES >> 4));
+              ptx::mma2_sp_mxf8(d, d_a + wo, d_b + so, id8, e, sfa, sfo + 8, acc);
+              ptx::mma2_sp_mxf8(d, d_a + wo + (4096 >> 4), d_b + so + (512 >> 4), id8, e + 2, sfa, sfo + 8, 1u);
             }
           }
-          __syncwarp();
-          k += n;
-          s += (uint32_t)n;
-          if (s >= NSLOT) { s -= NSLOT; ph ^= 1; }
+          if (ss & 1) ptx::tc2_commit_both(&empty[ss >> 1], both);     // slots ss - 1 and ss may be refilled (both CTAs)
+          if (kk == S - 1) ptx::tc2_commit_both(&acc_full[ab], both);  // the task's accumulator is complete (both CTAs)
+          if (++ss == NSLOT) ss = 0;
         }
+      };
+      int k = 0;
+      while (k < S) {
+        // lane i: has slot s + i (the i-th next stage of this task) landed in both CTAs?
+        const uint32_t idx = s + lane, sl = idx >= NSLOT ? idx - NSLOT : idx;
+        const bool r = (int)lane < min(4, S - k) && ptx::mbar_test(&full[sl], idx >= NSLOT ? ph ^ 1 : ph);
+        const int n = __ffs(~__ballot_sync(0xffffffffu, r)) - 1;    // length of the run of ready slots
+        if (n == 0) {   // nothing yet: wait for the next slot, then look again (its neighbours tend to land with it)
+          ok = __all_sync(0xffffffffu, ptx::mbar_wait(&full[s], ph));
+          if (!ok) break;
+          continue;
+        }
+        if (k == 0 && use > 0) {   // the epilogues of both CTAs must have drained this accumulator's previous task
+          ok = __all_sync(0xffffffffu, ptx::mbar_wait(&acc_empty[ab], (use - 1) & 1));
+          if (!ok) break;
+        }
+        ptx::tc_fence_after();
+        if (ptx::elect_one()) {
+          if (FORM == PAIR_TWO && nu == 2) issue(std::integral_constant<int, FORM == PAIR_TWO ? 2 : 1>{}, k, n);
+          else issue(std::integral_constant<int, 1>{}, k, n);
+        }
+        __syncwarp();
+        k += n;
+        par ^= (uint32_t)n & 1u;
+        s += (uint32_t)n;
+        if (s >= NSLOT) { s -= NSLOT; ph ^= 1; }
       }
-      // (a kernel whose stage count is odd leaves its last slot unreleased: nobody waits for it)
-      if (!ok && lane == 0) atomicOr(&p.flags[FLAG_TIMEOUT], 1u);
     }
-  } else if ((warp >= 2 && warp <= 5) || warp >= 9) {
-    // ---------------- epilogue (both CTAs): warp w owns TMEM lanes 32 (w % 4) .. + 31 (own weight rows); group 0 (warps 2..5)
-    // takes tokens 0..127 of the tile, group 1 (warps 9..12) tokens 128..255
-    const uint32_t q = warp & 3;
-    const uint32_t grp = warp >= 9 ? 1u : 0u;
-    const uint32_t et = (warp - (grp ? 9u : 2u)) * 32 + lane;
+    // (a kernel whose stage count is odd leaves its last slot unreleased: nobody waits for it)
+    if (!ok && lane == 0) atomicOr(&p.flags[FLAG_TIMEOUT], 1u);
+  } else {
+    // ---------------- epilogue (both CTAs): warp w owns TMEM lanes 32 (w % 4) .. + 31 (own weight rows).  Two units: groups 0
+    // and 1 take the two halves of unit 0's tokens, groups 2 and 3 unit 1's; one unit: a quarter of the tokens each.
+    const uint32_t q = warp & 3, grp = (warp - 4) >> 2, et = tid & 127u;
     uint32_t tcount = 0;
     bool ok = true;
-    auto hand_back = [&]() {      // this warp has read its part of the accumulator
-      ptx::tc_fence_before();
-      __syncwarp();
-      if (lane == 0) { if (rank == 0) ptx::mbar_arrive(acc_empty); else ptx::mbar_arrive_remote(acc_empty, 0); }
-    };
     ptx::griddep_wait();                            // Y may still be in use by the previous kernel
-    for (int tile = pair; tile < p.total_tiles && ok; tile += n_pairs, ++tcount) {
-      const int rt = 2 * (tile % RTP) + (int)rank, mtile = tile / RTP;
-      const int64_t m0 = (int64_t)mtile * 256;
-      const int n_valid = (int)min((int64_t)256, p.M - m0);
+    for (int task = pair; task < p.pt_tasks && ok; task += n_pairs, ++tcount) {
+      const PairTask t = pair_task<FORM>(p, task);
+      const uint32_t ab = acc2 ? tcount & 1u : 0u, use = acc2 ? tcount >> 1 : tcount;
+      const int g0 = pair_group0(p, t.mt);
+      const uint32_t unit = t.nu == 2 ? grp >> 1 : 0u, nc = 2u * (uint32_t)(pair_group0(p, t.mt + 1) - g0);   // 16-token chunks
+      const uint32_t c_begin = t.nu == 2 ? (grp & 1u) * (nc / 2) : grp * nc / 4, c_end = t.nu == 2 ? (grp & 1u ? nc : nc / 2) : (grp + 1) * nc / 4;
+      const int rt = 2 * (t.u0 + (int)unit) + (int)rank;
+      const int64_t m0 = (int64_t)g0 * 32 + c_begin * 16;
+      // tokens this group stores (a multiple of 16 in tensor memory, fewer at the end of the matrix; none beyond the last row tile)
+      const int n_valid = rt < RT ? (int)max((int64_t)0, min((int64_t)(c_end - c_begin) * 16, p.M - m0)) : 0;
       // one thread per group polls the barrier and releases the other 127 through a hardware barrier: hundreds of threads
       // polling one mbarrier notice its completion late and slow the CTA's other barrier traffic down
-      if (et == 0 && !ptx::mbar_wait(acc_full, tcount & 1)) *timed_out = 1u;
-      ptx::named_bar_sync(3 + grp, 128);
+      if (et == 0 && !ptx::mbar_wait(&acc_full[ab], use & 1)) *timed_out = 1u;
+      ptx::named_bar_sync(1 + grp, 128);
       if (*timed_out) { ok = false; break; }
       ptx::tc_fence_after();
+      const uint32_t tbase = tmem + ((q * 32u) << 16) + (ab + unit) * TMAX + c_begin * 16u;   // (alternating accumulators: one unit)
       const int64_t n0 = (int64_t)rt * TILE_ROWS;
-      const int twr = p.tw ? __ldg(p.tw + n0 + q * 32 + lane) : 0;     // two-level scaling: this thread's row factor
+      const int twr = p.tw && rt < RT ? __ldg(p.tw + n0 + q * 32 + lane) : 0;     // two-level scaling: this thread's row factor
+      auto factor = [&](int64_t m) { return __int_as_float((min(max(twr + __ldg(p.tx + m), -126), 127) + 127) << 23); };
+      auto hand_back = [&]() {      // this warp has read its part of the accumulator
+        ptx::tc_fence_before();
+        __syncwarp();
+        if (lane == 0) { if (rank == 0) ptx::mbar_arrive(&acc_empty[ab]); else ptx::mbar_arrive_remote(&acc_empty[ab], lead); }
+      };
+      if (ks > 1) {
+        // K split: this CTA's fp32 partial tile [token][128 rows] goes to shared memory, where the ring is idle by now
+        float* dst = reinterpret_cast<float*>(sm) + (size_t)c_begin * 16 * TILE_ROWS + q * 32 + lane;
+#pragma unroll 1
+        for (int c0 = 0; c0 < n_valid; c0 += 16) {
+          uint32_t v[16];
+          ptx::tmem_ld_32x32b_x16(tbase + (uint32_t)c0, v);
+          ptx::tmem_ld_wait();
+#pragma unroll
+          for (int j = 0; j < 16; ++j) dst[(size_t)(c0 + j) * TILE_ROWS] = __uint_as_float(v[j]);
+        }
+        continue;
+      }
       if constexpr (F32_OUT) {
-        // fp32 output (tests): the first group stores everything, straight from TMEM
-        if (grp) { hand_back(); continue; }
+        // fp32 output (tests): straight from TMEM
         float* Y = reinterpret_cast<float*>(p.Y);
 #pragma unroll 1
-        for (int c0 = 0; c0 < 256; c0 += 16) {
+        for (int c0 = 0; c0 < n_valid; c0 += 16) {
           uint32_t v[16];
-          if (c0 < n_valid) {
-            ptx::tmem_ld_32x32b_x16(tmem + ((q * 32u) << 16) + (uint32_t)c0, v);
-            ptx::tmem_ld_wait();
-          }
-          if (c0 + 16 >= 256) hand_back();
-          if (c0 >= n_valid) continue;
+          ptx::tmem_ld_32x32b_x16(tbase + (uint32_t)c0, v);
+          ptx::tmem_ld_wait();
 #pragma unroll
           for (int j = 0; j < 16; ++j)
             if (c0 + j < n_valid) {
               float f = __uint_as_float(v[j]);
-              if (p.tw) f *= __int_as_float((min(max(twr + __ldg(p.tx + m0 + c0 + j), -126), 127) + 127) << 23);
+              if (p.tw) f *= factor(m0 + c0 + j);
               Y[(m0 + c0 + j) * p.ldy + n0 + q * 32 + lane] = f;
             }
         }
+        hand_back();
       } else {
-        // bf16 output: drain the accumulator into registers (one weight row x 128 tokens per thread as 64 packed bf16
-        // pairs), hand TMEM back, then transpose and store under the next tile's K loop
-        uint32_t pk[64];
-        {
-          uint32_t va[16], vb[16];
-          const uint32_t tbase = tmem + ((q * 32u) << 16) + 128u * grp;
-          ptx::tmem_ld_32x32b_x16(tbase, va);
+        // bf16 output: drain the accumulator into registers (one weight row x up to 112 tokens per thread as packed bf16
+        // pairs), hand TMEM back, then transpose and store under the next task's K loop
+        constexpr int CH = FORM == PAIR_TWO ? (int)FIXED_T / 32 : 4;   // 16-token chunks a group may have
+        uint32_t pk[8 * CH];
 #pragma unroll
-          for (int c = 0; c < 128; c += 32) {
+        for (int c = 0; c < CH; ++c) {
+          if (16 * c < n_valid) {                   // uniform over the group
+            uint32_t v[16];
+            ptx::tmem_ld_32x32b_x16(tbase + 16u * (uint32_t)c, v);
             ptx::tmem_ld_wait();
-            ptx::tmem_ld_32x32b_x16(tbase + (uint32_t)(c + 16), vb);
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
-              const __nv_bfloat162 h = __floats2bfloat162_rn(__uint_as_float(va[2 * j]), __uint_as_float(va[2 * j + 1]));
-              pk[c / 2 + j] = *reinterpret_cast<const uint32_t*>(&h);
-            }
-            ptx::tmem_ld_wait();
-            if (c + 32 < 128) ptx::tmem_ld_32x32b_x16(tbase + (uint32_t)(c + 32), va);
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-              const __nv_bfloat162 h = __floats2bfloat162_rn(__uint_as_float(vb[2 * j]), __uint_as_float(vb[2 * j + 1]));
-              pk[c / 2 + 8 + j] = *reinterpret_cast<const uint32_t*>(&h);
+              const __nv_bfloat162 h = __floats2bfloat162_rn(__uint_as_float(v[2 * j]), __uint_as_float(v[2 * j + 1]));
+              pk[8 * c + j] = *reinterpret_cast<const uint32_t*>(&h);
             }
           }
         }
         hand_back();
-        const int g0 = 128 * (int)grp;
         // transpose through shared memory, 4 tokens at a time per group: [4 tokens][128 features] bf16, then one 8-byte
         // store per thread (a warp writes one token's 256 B).  Two-level scaling: multiplying the rounded value by the power
         // of two is the rounding of the multiplied value, so the factors go in here, after TMEM has been handed back.
-        uint16_t* stg = reinterpret_cast<uint16_t*>(sm + G::SM_STG) + grp * 512u;
+        uint16_t* stg = reinterpret_cast<uint16_t*>(stg_base) + grp * 512u;
         __nv_bfloat16* Y = reinterpret_cast<__nv_bfloat16*>(p.Y);
 #pragma unroll
-        for (int c0 = 0; c0 < 128; c0 += 4) {
-          if (g0 + c0 < n_valid) {                  // uniform over the four warps of the group
+        for (int c0 = 0; c0 < 16 * CH; c0 += 4) {
+          if (c0 < n_valid) {                       // uniform over the group
 #pragma unroll
             for (int j = 0; j < 2; ++j) {
               uint32_t lo = pk[c0 / 2 + j] << 16, hi = pk[c0 / 2 + j] & 0xFFFF0000u;
               if (p.tw) {
-                const int t = g0 + c0 + 2 * j;
-                if (t < n_valid) lo = __float_as_uint(__uint_as_float(lo) * __int_as_float((min(max(twr + __ldg(p.tx + m0 + t), -126), 127) + 127) << 23));
-                if (t + 1 < n_valid) hi = __float_as_uint(__uint_as_float(hi) * __int_as_float((min(max(twr + __ldg(p.tx + m0 + t + 1), -126), 127) + 127) << 23));
+                const int tk = c0 + 2 * j;
+                if (tk < n_valid) lo = __float_as_uint(__uint_as_float(lo) * factor(m0 + tk));
+                if (tk + 1 < n_valid) hi = __float_as_uint(__uint_as_float(hi) * factor(m0 + tk + 1));
               }
               stg[(2 * j) * 128 + q * 32 + lane] = (uint16_t)(lo >> 16);
               stg[(2 * j + 1) * 128 + q * 32 + lane] = (uint16_t)(hi >> 16);
             }
             ptx::named_bar_sync(1 + grp, 128);
             const uint32_t tok = et >> 5, seg = et & 31;
-            if (g0 + c0 + (int)tok < n_valid) {
+            if (c0 + (int)tok < n_valid) {
               const uint2 w = *reinterpret_cast<const uint2*>(stg + tok * 128 + seg * 4);
-              *reinterpret_cast<uint2*>(Y + (m0 + g0 + c0 + tok) * p.ldy + n0 + seg * 4) = w;
+              *reinterpret_cast<uint2*>(Y + (m0 + c0 + tok) * p.ldy + n0 + seg * 4) = w;
             }
             ptx::named_bar_sync(1 + grp, 128);       // the buffer is rewritten by the next chunk
           }
@@ -391,58 +472,199 @@ sdq_linear_pair_kernel(const LinearParams p)
   }
   ptx::tc_fence_before();
   __syncthreads();
-  ptx::cluster_sync();     // neither CTA leaves (or frees TMEM) while the other may still read its shared memory
+  if (FORM == PAIR_FLEX && ks > 1) {
+    ptx::cluster_sync();   // every split's partial tile is in shared memory
+    const PairTask t = pair_task<FORM>(p, pair);
+    const int g0 = pair_group0(p, t.mt), rt = 2 * t.u0 + (int)rank;
+    const int64_t m0 = (int64_t)g0 * 32, n0 = (int64_t)rt * TILE_ROWS;
+    const int n_valid = rt < RT ? (int)min((int64_t)32 * (pair_group0(p, t.mt + 1) - g0), p.M - m0) : 0;
+    // four rows x one token per item: one 16-byte load per split, added in order.  The 32 quads of rows are dealt out over the splits
+    const uint32_t q_begin = (uint32_t)(split * 32 / ks), q_per = (uint32_t)((split + 1) * 32 / ks) - q_begin, local = ptx::smem_u32(sm);
+    uint32_t part[4];
+#pragma unroll
+    for (uint32_t sp = 0; sp < 4; ++sp) part[sp] = ptx::mapa_u32(local, sp < (uint32_t)ks ? 2 * sp + rank : crank);
+    const uint32_t n_items = q_per * (uint32_t)max(n_valid, 0);
+    for (uint32_t idx = tid; idx < n_items; idx += PAIR_THREADS) {
+      const uint32_t tok = idx / q_per, row = (q_begin + (idx - tok * q_per)) << 2, off = (tok * TILE_ROWS + row) * 4;
+      float4 v[4];
+#pragma unroll
+      for (uint32_t sp = 0; sp < 4; ++sp)
+        v[sp] = sp < (uint32_t)ks ? ptx::ld_cluster_f32x4(part[sp] + off) : make_float4(0.f, 0.f, 0.f, 0.f);
+      float4 a = v[0];
+#pragma unroll
+      for (uint32_t sp = 1; sp < 4; ++sp) { a.x += v[sp].x; a.y += v[sp].y; a.z += v[sp].z; a.w += v[sp].w; }   // absent splits add +0
+      if (p.tw) {
+        const int4 t4 = __ldg(reinterpret_cast<const int4*>(p.tw + n0 + row));
+        const int tx = __ldg(p.tx + m0 + tok);
+        auto f = [&](int e) { return __int_as_float((min(max(e + tx, -126), 127) + 127) << 23); };
+        a.x *= f(t4.x); a.y *= f(t4.y); a.z *= f(t4.z); a.w *= f(t4.w);
+      }
+      if constexpr (F32_OUT) {
+        *reinterpret_cast<float4*>(reinterpret_cast<float*>(p.Y) + (m0 + tok) * p.ldy + n0 + row) = a;
+      } else {
+        const __nv_bfloat162 lo = __floats2bfloat162_rn(a.x, a.y), hi = __floats2bfloat162_rn(a.z, a.w);
+        *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(p.Y) + (m0 + tok) * p.ldy + n0 + row) =
+            make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
+      }
+    }
+  }
+  ptx::cluster_sync();     // no CTA leaves (or frees TMEM) while another may still read its shared memory
   if (warp == 1) ptx::tmem_dealloc_pair(tmem, 512);
 }
 
-template <bool F32_OUT, bool B32, bool DENSE>
-static cudaError_t launch_one(const LinearParams& p, int pairs, cudaStream_t stream, uint32_t* attr_mask, uint32_t bit)
+template <bool F32_OUT, bool B32, bool DENSE, int FORM>
+static cudaError_t launch_form(const LinearParams& p, int pairs, cudaStream_t stream, uint32_t* attr_mask)
 {
-  using G = PairGeom<B32, DENSE>;
-  auto kern = sdq_linear_pair_kernel<F32_OUT, B32, DENSE>;
+  auto kern = sdq_linear_pair_kernel<F32_OUT, B32, DENSE, FORM>;
+  const uint32_t bit = 1u << (((F32_OUT ? 3 : 0) + (DENSE ? 2 : (B32 ? 1 : 0))) * 3 + FORM);
   if (!(*attr_mask & bit)) {     // once per device and instantiation
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::SMEM);
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
     if (e != cudaSuccess) return e;
     *attr_mask |= bit;
   }
   cudaLaunchConfig_t lc = {};
-  lc.gridDim = dim3((unsigned)(2 * pairs));
+  lc.gridDim = dim3((unsigned)(2 * p.pt_ks * pairs));
   lc.blockDim = dim3(PAIR_THREADS);
-  lc.dynamicSmemBytes = G::SMEM;
+  lc.dynamicSmemBytes = (size_t)p.nslot * (size_t)p.slot_bytes + PAIR_TAIL;
   lc.stream = stream;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = (unsigned)(2 * p.pt_ks);
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
   lc.attrs = attr;
-  lc.numAttrs = 1;
+  lc.numAttrs = 2;
   return cudaLaunchKernelEx(&lc, kern, p);
 }
-
-bool pair_kernel_applies(int64_t M, int64_t N, int64_t K, int out_n)
+template <bool F32_OUT, bool B32, bool DENSE>
+static cudaError_t launch_one(const LinearParams& p, int form, int pairs, cudaStream_t stream, uint32_t* attr_mask)
 {
-  // The accumulator is not double-buffered, so every tile pays for the epilogue's drain of TMEM (~1 us); tiles of fewer
-  // than 32 stages (no outlier part and K <= 7936, or K < 2816 with one) run faster on the single-CTA kernel's smaller
-  // tiles (measured: 4096 -> 11008 without outliers 40 against 36 us; 11008 -> 4096 without outliers 30 against 34 us).
-  const int64_t stages = K / K2 + (out_n ? K / K1 : 0);
-  return M > 128 && N % (2 * TILE_ROWS) == 0 && stages >= 32;
+  if (form == PAIR_TWO) return launch_form<F32_OUT, B32, DENSE, PAIR_TWO>(p, pairs, stream, attr_mask);
+  if (form == PAIR_FULL) return launch_form<F32_OUT, B32, DENSE, PAIR_FULL>(p, pairs, stream, attr_mask);
+  return launch_form<F32_OUT, B32, DENSE, PAIR_FLEX>(p, pairs, stream, attr_mask);
 }
 
-cudaError_t launch_linear_pair(LinearParams p, bool f32_out, int sm_count, cudaStream_t stream, uint32_t* attr_mask)
+// How a call is cut into tasks: token tiles, one or two units per task, pairs per task (K split).
+struct PairPlan { int form, T, mt, acc2, doubles, split, tasks, ks; double us; };
+
+// The plan for `mt` token tiles with one- or two-unit tasks; false if tensor memory does not hold it.  Times in us, fitted to
+// measurements (4096 x 4096 to 16384 x 4096, 130 to 8192 tokens): a stage of one unit takes 0.158 (the chain of barrier test
+// and issue) or 10.5 ns per KB that an SM stages (12.5 with every SM busy, 11.8 with compile-time geometry), one of two units 0.10 + 0.00188 T (the tensor pipe at the clock it keeps
+// under load) or 13.5 ns per KB; a call 4.2 and 0.02 per pair it uses; a task ends with a drain of its accumulator that the next one waits for unless the accumulator alternates.
+static bool pair_plan(int groups, int mt, int units, int T1, int T2, bool dbl, uint32_t wib, bool s32, int pairs, const int* max_clusters, PairPlan* out)
 {
-  const int n_mtiles = (int)((p.M + 255) / 256);
-  p.total_tiles = (int)(p.N / (2 * TILE_ROWS)) * n_mtiles;
-  int pairs = sm_count / 2;
-  if (p.total_tiles < pairs) pairs = p.total_tiles;
+  PairPlan q;
+  const int T = 32 * ((groups + mt - 1) / mt), cols = s32 ? (int)PairGeom<true, false>::COLS : (int)PairGeom<false, false>::COLS;
+  q.T = T; q.mt = mt; q.ks = 1;
+  if (T > pair_tmax(dbl ? PAIR_TWO : PAIR_FULL, s32)) return false;
+  q.acc2 = !dbl && 2 * T + cols <= 512;
+  q.form = dbl ? PAIR_TWO : (q.acc2 ? PAIR_FLEX : PAIR_FULL);
+  const double avgT = 32.0 * groups / mt;
+  const double kb1 = !dbl && units * mt < pairs ? 0.0105e-3 : (q.acc2 ? 0.0125e-3 : 0.0118e-3);
+  const double s1i = kb1 * (wib + avgT * 64.0), s1o = kb1 * (WO_BYTES + avgT * 64.0), m2 = 0.10 + 0.00188 * avgT;
+  const double c1 = T2 * (s1i > 0.158 ? s1i : 0.158) + T1 * (s1o > 0.158 ? s1o : 0.158) + (q.acc2 ? 0.3 : 1.0);
+  const double s2i = 0.0135e-3 * (2 * wib + avgT * 64.0), s2o = 0.0135e-3 * (2 * WO_BYTES + avgT * 64.0);
+  const double c2 = T2 * (s2i > m2 ? s2i : m2) + T1 * (s2o > m2 ? s2o : m2) + 1.0;
+  q.doubles = q.split = 0;
+  double us;
+  if (!dbl) {
+    q.tasks = units * mt;
+    us = c1 * ((q.tasks + pairs - 1) / pairs);
+    // few tasks: as many pairs to each as the clusters that fit the GPU allow (a reduction costs 1 us + 10 ns a token)
+    for (int k = 2; k <= 4 && q.acc2; ++k)
+      if (q.tasks <= max_clusters[k] && k <= T2 && c1 / k + 1.0 + 0.01 * avgT < us) { us = c1 / k + 1.0 + 0.01 * avgT; q.ks = k; }
+  } else {
+    const int D = (units / 2) * mt, odd = (units & 1) * mt;
+    const int full = D / pairs * pairs, left = D - full;
+    // the last, partial round either as two-unit tasks or cut into one-unit tasks
+    const double base = c2 * (D / pairs);
+    const int over = odd > pairs - left ? odd - (pairs - left) : 0;         // one-unit tasks that do not fit beside the last two-unit ones
+    const double as2 = left ? c2 + c1 * ((over + pairs - 1) / pairs) : c1 * ((odd + pairs - 1) / pairs);
+    const double as1 = c1 * ((2 * left + odd + pairs - 1) / pairs);
+    if (as1 < as2) { q.doubles = full; q.split = 2 * left; us = base + as1; }
+    else { q.doubles = D; us = base + as2; }
+    q.tasks = q.doubles + q.split + odd;
+    if (!q.doubles) return false;      // nothing but one-unit tasks: the other form has the better slots for them
+  }
+  const int used = q.tasks * q.ks < pairs ? q.tasks * q.ks : pairs;
+  q.us = us + 4.2 + 0.02 * used;
+  // the packed weights come from DRAM
+  const double stream = 4.2 + 0.02 * used + (double)units * 2 * (T2 * (double)wib + T1 * (double)WO_BYTES) / 5.5e6;
+  if (q.us < stream) q.us = stream;
+  *out = q;
+  return true;
+}
+
+static PairPlan pair_best(int64_t M, int64_t N, int64_t K, int out_n, bool b32, bool dense, int sm_count, const int* max_clusters)
+{
+  const int units = (int)((N + 2 * TILE_ROWS - 1) / (2 * TILE_ROWS)), groups = (int)((M + 31) / 32);
+  PairPlan best, q;
+  best.us = -1.0;
+  // from tiles of 256 tokens down to tiles of 128, or of 32 where the call is small (up to 1024 tokens)
+  const int mt0 = (groups + 7) / 8, mt1 = groups <= 32 ? groups : 2 * mt0;
+  for (int mt = mt0; mt <= mt1; ++mt)
+    for (int d = 0; d < 2; ++d)
+      if (pair_plan(groups, mt, units, out_n ? (int)(K / K1) : 0, (int)(K / K2), d != 0, dense ? 17408u : (b32 ? 11264u : 10752u), b32 || dense, sm_count / 2,
+                    max_clusters, &q) && (best.us < 0 || q.us < best.us))
+        best = q;
+  return best;
+}
+
+// largest grids, in clusters of 4, 6 and 8 CTAs with one CTA per SM, that run at once on the current device: [pairs per cluster]
+static const int* pair_max_clusters(DeviceInfo* d)
+{
+  if (!d->pair_clusters[1]) {
+    auto kern = sdq_linear_pair_kernel<false, false, false, PAIR_FLEX>;
+    for (int k = 2; k <= 4; ++k) {
+      cudaLaunchConfig_t lc = {};
+      lc.gridDim = dim3((unsigned)(2 * k));
+      lc.blockDim = dim3(PAIR_THREADS);
+      lc.dynamicSmemBytes = 200 * 1024;
+      cudaLaunchAttribute attr[1];
+      attr[0].id = cudaLaunchAttributeClusterDimension;
+      attr[0].val.clusterDim.x = (unsigned)(2 * k);
+      attr[0].val.clusterDim.y = 1;
+      attr[0].val.clusterDim.z = 1;
+      lc.attrs = attr;
+      lc.numAttrs = 1;
+      int n = 0;
+      if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448) != cudaSuccess ||
+          cudaOccupancyMaxActiveClusters(&n, kern, &lc) != cudaSuccess) { n = 0; (void)cudaGetLastError(); }
+      d->pair_clusters[k] = n;
+    }
+    d->pair_clusters[1] = 1;
+  }
+  return d->pair_clusters;
+}
+
+double pair_kernel_us(int64_t M, int64_t N, int64_t K, int out_n, bool b32, bool dense, DeviceInfo* d)
+{ return pair_best(M, N, K, out_n, b32, dense, d->sm_count, pair_max_clusters(d)).us; }
+
+cudaError_t launch_linear_pair(LinearParams p, bool f32_out, DeviceInfo* d, cudaStream_t stream)
+{
+  const bool s32 = p.dense || p.b32;
+  const uint32_t wib = p.dense ? 17408u : (p.b32 ? 11264u : 10752u);
+  int pairs = d->sm_count / 2;
+  const PairPlan best = pair_best(p.M, p.N, p.K, p.out_n, p.b32 != 0, p.dense != 0, d->sm_count, pair_max_clusters(d));
+  uint32_t* attr_mask = &d->pair_attr;
+  const int T = best.form == PAIR_FLEX ? best.T : pair_tmax(best.form, s32);
+  p.n_tile = T;
+  p.pt_units = (int)((p.N + 2 * TILE_ROWS - 1) / (2 * TILE_ROWS)); p.pt_mtiles = best.mt; p.pt_groups = (int)((p.M + 31) / 32);
+  p.pt_doubles = best.doubles; p.pt_split = best.split; p.pt_tasks = best.tasks; p.pt_acc2 = best.acc2; p.pt_ks = best.ks;
+  p.slot_bytes = (int)pair_slot_bytes(wib, s32, best.form == PAIR_TWO ? 2 : 1, T);
+  p.nslot = pair_slots((uint32_t)p.slot_bytes);
+  if (p.pt_tasks < pairs || best.ks > 1) pairs = p.pt_tasks;
   const int v = (f32_out ? 4 : 0) | (p.dense ? 2 : (p.b32 ? 1 : 0));
   switch (v) {
-    case 0: return launch_one<false, false, false>(p, pairs, stream, attr_mask, 1u << 0);
-    case 1: return launch_one<false, true, false>(p, pairs, stream, attr_mask, 1u << 1);
-    case 2: return launch_one<false, false, true>(p, pairs, stream, attr_mask, 1u << 2);
-    case 4: return launch_one<true, false, false>(p, pairs, stream, attr_mask, 1u << 4);
-    case 5: return launch_one<true, true, false>(p, pairs, stream, attr_mask, 1u << 5);
-    default: return launch_one<true, false, true>(p, pairs, stream, attr_mask, 1u << 6);
+    case 0: return launch_one<false, false, false>(p, best.form, pairs, stream, attr_mask);
+    case 1: return launch_one<false, true, false>(p, best.form, pairs, stream, attr_mask);
+    case 2: return launch_one<false, false, true>(p, best.form, pairs, stream, attr_mask);
+    case 4: return launch_one<true, false, false>(p, best.form, pairs, stream, attr_mask);
+    case 5: return launch_one<true, true, false>(p, best.form, pairs, stream, attr_mask);
+    default: return launch_one<true, false, true>(p, best.form, pairs, stream, attr_mask);
   }
 }
 
 }  // namespace sdq
-

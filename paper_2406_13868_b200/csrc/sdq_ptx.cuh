@@ -268,9 +268,9 @@ __device__ __forceinline__ void tc2_commit(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 // ... or one arrival on the barrier at this shared-memory offset in BOTH CTAs of the pair (a barrier signal, not a load)
-__device__ __forceinline__ void tc2_commit_both(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(smem_u32(bar)),
-               "h"((uint16_t)3)
+// (`mask`: bit per CTA of the cluster, the two of the pair)
+__device__ __forceinline__ void tc2_commit_both(uint64_t* bar, uint16_t mask) {
+  asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(smem_u32(bar)), "h"(mask)
                : "memory");
 }
 __device__ __forceinline__ void tc2_commit_remote(uint64_t* bar, uint32_t cta) {

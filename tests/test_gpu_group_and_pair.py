@@ -147,6 +147,37 @@ def test_cta_pair_many_token_kernel(M, N, K, out_n, block, gran, rule, rows):
 
 
 # ---------------------------------------------------------------------------------------------- the streamed outlier forms
+@pytest.mark.parametrize("M,N,K,cfg_args", [
+    (3371, 2560, 2048, (1, so.GRAN_PAIR, 64, 0)),     # one-unit tasks, 256-token tiles, several rounds
+    (3371, 2688, 2048, (1, so.GRAN_PAIR, 64, 0)),     # two-unit tasks, the last round cut into one-unit ones; odd units and row tiles
+    (5001, 1280, 2048, (1, so.GRAN_PAIR, 64, 0)),     # two-unit tasks and one odd unit per token tile, uneven token tiles
+    (2901, 3200, 2048, (2, so.GRAN_PAIR, 32, 1)),     # the same with one scale per 32 K, two outliers per 8
+    (4001, 2304, 2048, (1, so.GRAN_PAIR, 32, 2)),     # E4M3 scales, one-unit tasks of 256 tokens
+    (4001, 1664, 2048, (1, so.GRAN_DENSE, 32, 0)),    # one-unit tasks with alternating accumulators, dense inliers
+    (300, 384, 2048, (1, so.GRAN_PAIR, 32, 2)),       # K over four pairs, E4M3 scales, an odd number of row tiles
+    (200, 384, 1536, (1, so.GRAN_DENSE, 32, 0)),      # K over four pairs, dense inliers
+    (100, 4096, 2048, (1, so.GRAN_PAIR, 64, 0)),      # up to 128 tokens on pairs
+    (64, 2176, 4096, (2, so.GRAN_PAIR, 64, 0)),
+    (130, 128, 256, (0, so.GRAN_PAIR, 64, 0)),        # a single stage, half a unit
+])
+def test_cta_pair_task_forms(M, N, K, cfg_args):
+    """the ways the pair kernel cuts a call into tasks (on 148 SMs), sampled tokens -- the first and last of tiles among them
+    -- against the oracle; bf16 = RNE of the fp32 result, and a second call gives the same bits"""
+    m = sdq()
+    cfg = m.Config(*cfg_args)
+    W, X = sdq_synth.make_weight(N, K, 61), sdq_synth.make_act(M, K, 62)
+    p, xq = m.sdq_decompose(W.cuda(), cfg), m.sdq_quantize_act(X.cuda(), cfg)
+    y = m.sdq_linear(xq, p, f32=True)
+    y16, again = m.sdq_linear(xq, p), m.sdq_linear(xq, p, f32=True)
+    assert m.device_status() == 0
+    assert torch.equal(y16, y.to(torch.bfloat16)) and torch.equal(y, again)
+    toks = sorted({t for t in [0, 31, 32, 95, 96, 127, 128, 160, 191, 192, 223, 224, 255, 256, M // 2, M - 33, M - 2, M - 1] if 0 <= t < M})
+    oc = ocfg(cfg_args[0], cfg_args[3], cfg_args[2], cfg_args[1])
+    yref = so.linear(so.quantize_act(sdq_synth.bf16_bits(X[toks]), oc), so.decompose(sdq_synth.bf16_bits(W), oc))
+    d, tol = y_close(y[toks].cpu().numpy(), yref)
+    assert (d <= tol).all(), (d.max(), (d / tol).max())
+
+
 def _a_off(row, byte):
     j, b = byte >> 5, byte & 31
     return j * 4096 + (row >> 3) * 256 + (b >> 4) * 128 + (row & 7) * 16 + (b & 15)
