@@ -2,18 +2,21 @@
 
 Argument marshalling only -- every step of the path (weight decomposition + packing, activation
 quantization, the fused sparse GEMM) runs in the CUDA kernels of libsdq_b200.so.  PyTorch supplies
-device memory and streams.  There is no CPU fallback: importing works without a GPU (so the build can
+device memory and streams.  The calls made for every batch of activations are marshalled by a small native
+module (csrc/sdq_python.cpp), everything else by ctypes.  There is no CPU fallback: importing works without a GPU (so the build can
 be checked), but every compute call needs the CUDA library and a CUDA tensor.
 """
 from __future__ import annotations
 
 import ctypes
+import importlib.machinery
+import importlib.util
 import os
 from dataclasses import dataclass, field
 
 import torch
 
-from .build import LIB, build
+from .build import BINDING, LIB, build
 
 GRAN_PAIR, GRAN_ELEM, GRAN_DENSE = 0, 1, 2
 GRAN_3OF4 = 9      # S-Vectors of 4: 3:4 = 1:4 outliers (out_n = 2 per 8, or 0) + 2:4 inliers, stored and run like the dense pattern
@@ -107,6 +110,24 @@ def lib() -> ctypes.CDLL:
             getattr(L, n).restype = ctypes.c_int
         _lib = L
     return _lib
+
+
+_fast = None
+
+
+def _native():
+    """The binding's native module (csrc/sdq_python.cpp), loaded at first use like the CUDA library."""
+    global _fast
+    if _fast is None:
+        if not os.path.exists(LIB) or not os.path.exists(BINDING):
+            raise RuntimeError("libsdq_b200.so or _binding.so is missing: run `python -c 'import __graft_entry__ as g; g.build()'` "
+                               "(the SDQ path has no CPU or PyTorch fallback)")
+        loader = importlib.machinery.ExtensionFileLoader("_binding", BINDING)
+        mod = importlib.util.module_from_spec(importlib.util.spec_from_loader("_binding", loader))
+        loader.exec_module(mod)
+        mod.bind(_Act, _Packed, Config, QuantAct, SdqError)
+        _fast = mod
+    return _fast
 
 
 def _check(code: int, where: str):
@@ -220,6 +241,9 @@ def channel_norm(X: torch.Tensor) -> torch.Tensor:
 def sdq_quantize_act(X: torch.Tensor, cfg: Config | None = None, buf: torch.Tensor | None = None) -> QuantAct:
     """X [M, K] bf16 CUDA tensor -> 4-bit block-scaled and 8-bit per-token-scaled activations."""
     cfg = cfg or Config()
+    q = (_fast or _native()).quantize_act(X, cfg, buf)
+    if q is not None:
+        return q
     _need_cuda(X, "X")
     assert X.dtype == torch.bfloat16 and X.dim() == 2 and X.stride(1) == 1
     M, K = X.shape
@@ -251,6 +275,9 @@ def sdq_linear(xq: QuantAct, p: PackedWeight, out: torch.Tensor | None = None, f
                workspace: torch.Tensor | None = None) -> torch.Tensor:
     """Y [M, N] = A_i W_i^T + A_o W_o^T (bf16, or the fp32 accumulator itself with f32=True).
     `workspace` (from make_workspace) enables the split-K path for few tokens."""
+    y = (_fast or _native()).linear(xq, p, out, f32, workspace)
+    if y is not None:
+        return y
     dt = torch.float32 if f32 else torch.bfloat16
     if out is None:
         out = torch.empty((xq.M, p.N), dtype=dt, device=p.buf.device)
@@ -268,6 +295,9 @@ def sdq_linear(xq: QuantAct, p: PackedWeight, out: torch.Tensor | None = None, f
 def sdq_linear_group(xqs, ps, outs=None, f32: bool = False):
     """Y[i] = sdq_linear(xqs[i], ps[i]) for independent layers in one call (one persistent launch when every layer has few
     tokens and the group is large enough; see sdq_linear_group in include/sdq.h).  Returns the list of outputs."""
+    ys = (_fast or _native()).linear_group(xqs, ps, outs, f32)
+    if ys is not None:
+        return ys
     n = len(ps)
     assert n == len(xqs) and n > 0
     dt = torch.float32 if f32 else torch.bfloat16
@@ -287,6 +317,9 @@ def sdq_linear_group(xqs, ps, outs=None, f32: bool = False):
 def sdq_linear_group_x(X: torch.Tensor, ps, outs=None, f32: bool = False):
     """Y[i] = sdq_linear(sdq_quantize_act(X), ps[i]) for layers that share the bf16 activations X [M <= 16, K], the quantizer
     fused into the one persistent launch (see sdq_linear_group_x in include/sdq.h).  Returns the list of outputs."""
+    ys = (_fast or _native()).linear_group_x(X, ps, outs, f32)
+    if ys is not None:
+        return ys
     _need_cuda(X, "X")
     assert X.dtype == torch.bfloat16 and X.dim() == 2 and X.stride(1) == 1
     n, M, K = len(ps), X.shape[0], X.shape[1]

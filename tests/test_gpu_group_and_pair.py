@@ -518,3 +518,41 @@ def test_compact_buffer_serves_the_grouped_calls_and_nothing_else(cfg_args):
     with pytest.raises(RuntimeError):
         m.packed_compact(comp[0])
     assert m.device_status() == 0
+
+
+# ---------------------------------------------------------------------------------------------- the binding's two halves
+def test_native_and_ctypes_halves_of_the_binding_agree(monkeypatch):
+    """every call that has a native half gives the same bits without it (the ctypes way, taken for arguments the native
+    half leaves alone), with outputs made by the call and supplied by the caller"""
+    m = sdq()
+    cfg = m.Config()
+    ps = [m.sdq_decompose(sdq_synth.make_weight(5120, 1024, 70 + i).cuda(), cfg) for i in range(2)]
+    X = sdq_synth.make_act(9, 1024, 72).cuda()
+
+    def calls():
+        xq = m.sdq_quantize_act(X, cfg)
+        buf = torch.zeros(m.act_size(9, 1024, cfg), dtype=torch.uint8, device="cuda")
+        assert m.sdq_quantize_act(X, cfg, buf).buf is buf and (xq.M, xq.K) == (9, 1024)
+        ws = m.make_workspace(9, 5120, 1024, cfg, "cuda")
+        got = [m.act_export(xq)["xq8_code"], m.sdq_linear(xq, ps[0]), m.sdq_linear(xq, ps[0], f32=True), m.sdq_linear(xq, ps[0], workspace=ws)]
+        for f32 in (False, True):
+            got += m.sdq_linear_group([xq, xq], ps, f32=f32) + m.sdq_linear_group_x(X, ps, f32=f32)
+            outs = [torch.empty((9, 5120), dtype=torch.float32 if f32 else torch.bfloat16, device="cuda") for _ in ps]
+            assert m.sdq_linear(xq, ps[1], outs[0], f32) is outs[0]
+            assert m.sdq_linear_group_x(X, ps, outs, f32) is outs
+            got += outs
+        with pytest.raises(AssertionError):
+            m.sdq_linear(xq, ps[0], torch.empty((9, 5120), dtype=torch.float16, device="cuda"))
+        with pytest.raises(m.SdqError) as e:
+            m.sdq_quantize_act(X[:, :1000], cfg)
+        assert e.value.code == 2
+        return got
+
+    native = calls()
+
+    class Absent:
+        def __getattr__(self, name):
+            return lambda *a: None
+    monkeypatch.setattr(m, "_fast", Absent())
+    for a, b in zip(native, calls()):
+        assert torch.equal(a, b)
