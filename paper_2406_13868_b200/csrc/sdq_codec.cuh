@@ -45,6 +45,23 @@ __device__ __forceinline__ uint32_t int8_code(float x, float s) {
   return (uint32_t)(int)r & 0xFFu;
 }
 
+// The same code for a whole vector without a division per element: inv = 1 / s.  x * inv is within 2.3e-5 of the fp32
+// quotient RN(x / s) (two roundings of 2^-24 against one, at most 127), so unless it lies within 2^-14 of a half-integer both
+// round to the same integer; otherwise (one element in 8000), or where 1 / s leaves the normal range, the quotient
+// itself decides.  Adding 1.5 * 2^23 rounds to the nearest even integer and leaves its two's complement in the low bits.
+struct Int8Coder { float s, inv; bool exact; };
+__device__ __forceinline__ Int8Coder int8_coder(float s) {
+  Int8Coder c;
+  c.s = s; c.inv = __fdiv_rn(1.0f, s); c.exact = !(s > 1e-30f);
+  return c;
+}
+__device__ __forceinline__ uint32_t int8_code(float x, const Int8Coder& k) {
+  const float q = x * k.inv, t = q + 12582912.0f;
+  uint32_t c = __float_as_uint(t) & 0xFFu;
+  if (k.exact || fabsf(q - (t - 12582912.0f)) > 0.5f - 6.103515625e-5f) c = int8_code(x, k.s);
+  return c;
+}
+
 // exponent e of the power-of-two scale of an 8-bit (E4M3, max 448 = 1.75 * 2^8) operand:
 // the smallest integer with amax <= 448 * 2^e, limited to what an E8M0 byte can carry
 __device__ __forceinline__ int fp8_scale_exp(float amax) {
@@ -74,6 +91,14 @@ __device__ __forceinline__ uint32_t ue4m3_scale_code(float amax, int t) {
 __device__ __forceinline__ float ue4m3_scale_value(uint32_t c, int t) {
   const __half_raw h = __nv_cvt_fp8_to_halfraw((__nv_fp8_storage_t)c, __NV_E4M3);
   return scalbnf(__half2float(__half(h)), t);
+}
+
+// What the E2M1 converter makes of x / sv for a bf16 x and an E4M3 value sv (times a power of two), without dividing:
+// inv = 1 / sv.  The quotient either equals a rounding boundary of E2M1 (c 2^k, c = 1, 3, 5, 7) or is at least 1 / 255 of it
+// away, since x and boundary * sv are integers below 256 times powers of two; x * inv is within 2^-23 of the quotient, so
+// rounding it to 16 significant bits restores the boundaries and moves nothing across one.
+__device__ __forceinline__ float e2m1_quotient(float x, float inv) {
+  return __uint_as_float((__float_as_uint(x * inv) + 0x80u) & 0xFFFFFF00u);
 }
 
 // two floats -> two E2M1 codes in one byte (x in the low nibble)

@@ -373,7 +373,7 @@ pack_tile_kernel(const PackParams p)
       // a Q-Vector is complete: 64 K (both blocks of the half) or 32 K (this one)
       const uint32_t key = max(qmax2 & 0xFFFFu, qmax2 >> 16);
       const uint32_t c = p.ue ? ue4m3_scale_code(bf16_bits_to_float(key), tw) : e8m0_scale_code_bf16(key, p.ceil_rule != 0);
-      const float sv = p.ue ? ue4m3_scale_value(c, tw) : 0.0f, inv = pow2_inv_e8m0(c);
+      const float inv = p.ue ? __fdiv_rn(1.0f, ue4m3_scale_value(c, tw)) : pow2_inv_e8m0(c);
 #pragma unroll
       for (int hb = 0; hb < 2; ++hb) {                   // 32-K block of the half
         if (hb != (b & 1) && b32) continue;              // (one scale per 64 K: both now)
@@ -386,8 +386,8 @@ pack_tile_kernel(const PackParams p)
             const float lo = __uint_as_float(w << 16), hi = __uint_as_float(w & 0xFFFF0000u);
             if (p.ue) {
               // (an outlier's position stays +0; the quotient of a dropped one is +0 as well)
-              f[2 * j] = c ? __fdiv_rn(lo, sv) : 0.0f;
-              f[2 * j + 1] = c ? __fdiv_rn(hi, sv) : 0.0f;
+              f[2 * j] = c ? e2m1_quotient(lo, inv) : 0.0f;
+              f[2 * j + 1] = c ? e2m1_quotient(hi, inv) : 0.0f;
             } else {
               f[2 * j] = lo * inv;
               f[2 * j + 1] = hi * inv;

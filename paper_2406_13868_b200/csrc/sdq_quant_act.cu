@@ -13,7 +13,9 @@
 //
 // Bound by DRAM traffic and the conversion instructions: 2048 x 11008 at 3.74 TB/s of algorithmic bytes (21.0 us; a warp
 // per scattered 64-K Q-Vector with byte stores of scales: 24.7), 8192 x 4096 at 4.4 TB/s (26.7 us; 31.6), one token 3.6 us
-// (4.6), most of it launch and the cluster barrier.
+// (4.6), most of it launch and the cluster barrier.  E4M3 scales and int8 codes multiply by a reciprocal instead of dividing
+// every element (see sdq_codec.cuh): 4096 x 16384 with E4M3 scales 91 -> 70.7 us, int8 2048 x 4096 15.0 -> 12.6, one int8
+// token 14.1 -> 6.4 (zeros took the division's slow path).
 #include "sdq_codec.cuh"
 #include "sdq_internal.h"
 #include "sdq_layout.h"
@@ -72,7 +74,7 @@ __device__ __forceinline__ void qa_encode(const QaUnit& u, float ramax, bool liv
   const int e = fp8_scale_exp(ramax);
   const float s8 = pow2_neg(e);
   const bool i8 = cfg.out_fmt == SDQ_OUT_INT8;           // A_o in int8: fp32 token scale amax / 127
-  const float sx = int8_scale(ramax);
+  const Int8Coder k8 = int8_coder(int8_scale(ramax));
   const bool b32 = cfg.in_block == 32;                   // one scale per 32 K: a Q-Vector is a lane pair
   uint8_t* xi = buf + off.xi + (size_t)k2 * off.xi_stride + (size_t)(m >> 3) * 1024 + (uint32_t)(m & 7) * 16;
   uint8_t* xo = buf + off.xo + (size_t)(2 * k2) * off.xo_stride + (size_t)(m >> 3) * 1024 + (uint32_t)(m & 7) * 16;
@@ -108,12 +110,12 @@ __device__ __forceinline__ void qa_encode(const QaUnit& u, float ramax, bool liv
       c[i] = ue4m3_scale_code(bf16_bits_to_float(bm), e);
       if (c[i]) {
         // two-level scaling: the Q-Vector scale E4M3(c) * 2^e is not a power of two, the elements are divided by it
-        const float sv = ue4m3_scale_value(c[i], e);
+        const float inv = __fdiv_rn(1.0f, ue4m3_scale_value(c[i], e));
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
           float f[8];
 #pragma unroll
-          for (int j = 0; j < 8; ++j) f[j] = __fdiv_rn(v[8 * h + j], sv);
+          for (int j = 0; j < 8; ++j) f[j] = e2m1_quotient(v[8 * h + j], inv);
           q4[h] = e2m1x8(f);
         }
       }
@@ -123,7 +125,7 @@ __device__ __forceinline__ void qa_encode(const QaUnit& u, float ramax, bool liv
       for (int j = 0; j < 8; ++j) q8[j >> 1] |= e4m3x2(v[2 * j] * s8, v[2 * j + 1] * s8) << (16 * (j & 1));
     } else {
 #pragma unroll
-      for (int j = 0; j < 8; ++j) q8[j >> 1] |= (int8_code(v[2 * j], sx) | (int8_code(v[2 * j + 1], sx) << 8)) << (16 * (j & 1));
+      for (int j = 0; j < 8; ++j) q8[j >> 1] |= (int8_code(v[2 * j], k8) | (int8_code(v[2 * j + 1], k8) << 8)) << (16 * (j & 1));
     }
     if (live) {
       // 4-bit codes: bytes 32 i + 8 l of the token's 128; 8-bit codes: bytes 64 (i & 1) + 16 l of the 128-K record i / 2
@@ -216,9 +218,11 @@ quant_act_fused_kernel(const __nv_bfloat16* __restrict__ X, int64_t M, int64_t K
 {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int t = lane >> 2, l = lane & 3;                 // token within the group of 8, quarter of the Q-Vector
-  // launched with programmatic stream serialization: X may still be being written by the previous kernel
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  // launched with programmatic stream serialization: X may still be being written by the previous kernel.  The next launch of
+  // the stream is let in before that wait: what it does before its own wait (set-up, fetching packed weights) then overlaps
+  // the previous kernel, and its wait for this grid includes this grid's wait for the previous one
   if (tid == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   const uint32_t cx = gridDim.x, rank = blockIdx.x;      // cluster = the gridDim.x CTAs of one token group
   const int64_t m = (int64_t)blockIdx.y * 8 + t;
   const bool live = m < M;

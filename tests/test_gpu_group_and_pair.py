@@ -520,6 +520,25 @@ def test_compact_buffer_serves_the_grouped_calls_and_nothing_else(cfg_args):
     assert m.device_status() == 0
 
 
+@pytest.mark.parametrize("largest", [127.0, 126.5, 96.0, 1.0, 3e-3, 1e-34, 2e-38, 3e38])
+def test_int8_codes_next_to_half_integers(largest):
+    """activations as close to (n + 1/2) s as bf16 gets, where a product with 1 / s and the quotient by s could round to
+    different integers, on exact ties (largest = 127 * a power of two), and at both ends of the fp32 range"""
+    m = sdq()
+    cfg = m.Config(1, m.GRAN_PAIR, 64, 0, 0, m.OUT_INT8)
+    rng = np.random.default_rng(8)
+    M, K = 16, 512
+    top = (largest * (1.0 - 0.4 * rng.random(M))).astype(np.float32)
+    top[0] = largest
+    n = np.arange(K) % 254 - 127
+    X = torch.from_numpy(((n[None, :] + 0.5) * (top[:, None].astype(np.float64) / 127.0)).astype(np.float32)).to(torch.bfloat16)
+    X[:, 7] = torch.from_numpy(top).to(torch.bfloat16)
+    oq = so.quantize_act(sdq_synth.bf16_bits(X), so.Config(1, so.GRAN_PAIR, 64, 0, 0, so.OUT_INT8))
+    ae = m.act_export(m.sdq_quantize_act(X.cuda(), cfg))
+    for name in ("xq4_code", "xq4_scale", "xq8_code", "xq8_sexp"):
+        assert np.array_equal(ae[name].cpu().numpy(), getattr(oq, name)), name
+
+
 # ---------------------------------------------------------------------------------------------- the binding's two halves
 def test_native_and_ctypes_halves_of_the_binding_agree(monkeypatch):
     """every call that has a native half gives the same bits without it (the ctypes way, taken for arguments the native
