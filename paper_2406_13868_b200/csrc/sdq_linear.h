@@ -59,7 +59,7 @@ struct GroupMat {
   int item0;             // number of the matrix's first work item (= row tiles of the matrices before it)
 };
 struct GroupParams {
-  int n, n_tile, nslot, slot_bytes, total_items;
+  int n, n_tile, nslot, total_items;   // nslot: inlier ring positions
   int out_n;             // outliers per S-Vector, the same for every matrix of the call (0 or 1)
   int out_i8;            // the outlier operands are int8 with fp32 scales (else E4M3 with power-of-two scale atoms)
   // activation-resident variant (launch_linear_group with x_bf16 set): all matrices share one bf16 X [x_M][K], which every

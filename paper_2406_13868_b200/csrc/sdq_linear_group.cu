@@ -17,17 +17,23 @@
 // its bandwidth at the rate aimed for, and had room for two container pairs only, whose build -> multiply -> release
 // cycle set the pace.  Streamed bytes: 2.625 + 1.5 = 4.125 bits per weight against 4.0 algorithmic.
 //
-// The ring is organised in units of 256 K of one item: an inlier slot (the WI record with the tokens' 4-bit codes and
-// scale atom) and an outlier slot (two compact records with the tokens' 8-bit codes); tensor memory holds one container
-// set per ring position.  All of a unit is released by ONE tcgen05.commit per issuer.  An mbarrier test costs 15..50 cycles
+// The stages are organised in units of 256 K of one item, in three rings that fill and drain by themselves: inlier slots (the
+// WI record with the tokens' 4-bit codes and scale atom), compact outlier records (two of 128 K), and the tokens' 8-bit codes;
+// tensor memory holds one container set per position of the last two.  An inlier slot is free again when the inlier MMAs of
+// its unit have completed, a compact record as soon as the builders have read it, codes and container when the outlier MMAs
+// have.  What a CTA streams is bytes in flight over a position's round trip (copy 1.3 us, build 0.9, multiply, notice); with one
+// ring for everything, released as a whole, that was 2.8 us for eight units, 0.37 us a unit however few CTAs shared the
+// DRAM.  With three rings: 74 row tiles of 64 units 27.5 -> 24.4 us, of 16 units 9.6 -> 7.9; q / k / v of 16 tokens 10.2 ->
+// 9.5, gate / up 16.4 -> 15.0, 32 layers of 4096 x 4096 53.9 -> 50.5.  An mbarrier test costs 15..50 cycles
 // when the phase has completed, a tcgen05 instruction ~40 to issue, but a hand-over between roles (complete -> noticed)
 // several hundred, so every role keeps its trips few and its waits parallel: where a role waits for several barriers,
 // different lanes wait for them at the same time.
 //
-// Warps: 0 and 10 bulk-copy producers (inlier / outlier slots, six lanes each), 1 and 23 MMA issuers (inlier / outlier
+// Warps: 0, 10 and 24 bulk-copy producers (inlier slots, six lanes / compact records, two lanes / 8-bit codes and the items'
+// outlier scale atoms, four lanes), 1 and 23 MMA issuers (inlier / outlier
 // product, each into its own accumulator; warp-uniform loops, one elected lane issues; they also copy the inlier metadata
 // and the scales to TMEM), 2..5 epilogue (adds the two accumulators; accumulator pairs alternate per item, so the next
-// item's MMAs never wait for the stores), 6..9, 11..14, 15..18 and 19..22 container builders (up to four groups).
+// item's MMAs never wait for the stores), 6..9, 11..14, 15..18 and 19..22 container builders (four groups).
 // Every wait is bounded; a timeout sets the sticky flag.
 //
 // Variants.  Outlier operands in int8 (SDQ_OUT_INT8): the same containers and token codes read as integers by a sparse
@@ -36,8 +42,8 @@
 // quantizes into its own shared memory (22 warps; the codes, scales and layouts of sdq_quantize_act) while its producers
 // already stream weights; the ring slots then hold the weight records only.
 //
-// What bounds it (measured): the SM's instruction issue is half used, more than half of it by the builders' byte
-// arithmetic; a CTA runs a unit in ~0.45-0.5 us against 0.38 us at the HBM peak.
+// What bounds it (measured): with every SM at work the DRAM (0.43 us a unit against 0.385 at its peak), else the ring's round
+// trip; the SM's instruction issue is half used, more than half of it by the builders' byte arithmetic.
 #include <cuda_bf16.h>
 
 #include "sdq_codec.cuh"
@@ -48,15 +54,19 @@
 
 namespace sdq {
 
-constexpr int GRP_THREADS = 768;                 // 24 warps
-constexpr int GRP_MAX_UNITS = 8;                 // units the ring may hold (and container sets tensor memory holds)
+// 25 warps, or 24 when the tokens' codes are resident (no producer for them); 25 take at most 72 registers per thread, since
+// seven of them share a register file of 16384
+__host__ __device__ constexpr int group_threads(bool xres) { return xres ? 768 : 800; }
+constexpr int GRP_UNITS = 8;                     // outlier ring positions (container sets tensor memory holds)
+constexpr int GRP_MAX_IN = 12;                   // inlier ring positions: as many as fit, an even number
+constexpr int GRP_BUILDERS = 4;                  // builder groups (divides GRP_UNITS: a group then sees every phase of its positions' barriers)
 constexpr uint32_t GRP_TM_ACC = 0;               // per item parity 64 columns: O_i at +0, O_o at +32 (32 columns each)
 constexpr uint32_t GRP_TM_I = 128;               // 2 x 12: E_in 4 | SFA_in 4 | SFB_in 4
 constexpr uint32_t GRP_TM_SO = 152;              // 2 x 8: SFA_out 4 | SFB_out 4 (per item parity)
 constexpr uint32_t GRP_TM_C = 168;               // per ring position 40: A_out of the unit's two 128-K stages 2 x 16 | E_out 2 x 4
 constexpr uint32_t GRP_TM_C_COLS = 40;
 constexpr uint32_t GRP_TMEM_COLS = 512;
-constexpr int GRP_BAR_BYTES = (4 * GRP_MAX_UNITS + 4 + 2) * 8 + 8;
+constexpr int GRP_BAR_BYTES = (2 * GRP_MAX_IN + 5 * GRP_UNITS + 4 + 2) * 8 + 8;
 // activation-resident variant (16 tokens): per 256-K unit the tokens' 4-bit codes, their scale atom and the 8-bit codes of the
 // unit's two 128-K stages, in the operand layouts of the quantizer's buffer; then one atom of token scales for the outlier
 // product; then the quantizing warps' per-token maxima and the tokens' fp32 scales (int8 outliers)
@@ -67,8 +77,6 @@ __host__ __device__ inline int group_xres_bytes(int T2) { return T2 * (int)GRP_X
 
 // inlier slot: | WI record | 4-bit codes of the tokens | their scale atom |
 __host__ __device__ inline int group_is_bytes(int n_tile) { return WI_BYTES + n_tile * 128 + SF_ATOM_BYTES; }
-// outlier slot: | two compact records (128 K each) | 8-bit codes of the tokens, 2 x 128 K |
-__host__ __device__ inline int group_os_bytes(int n_tile) { return 2 * wc_bytes(1) + 2 * n_tile * 128; }
 // beside the ring: alternating per item, the outlier row / token scale atoms (SFA_out | SFB_out)
 constexpr int GRP_SIDE_BYTES = 2 * 2 * SF_ATOM_BYTES;
 
@@ -80,28 +88,33 @@ __device__ __forceinline__ int group_mat_of(const GroupParams& p, int item) {
 }
 
 template <bool F32_OUT, bool XRES>
-__global__ void __launch_bounds__(GRP_THREADS, 1)
+__global__ void __launch_bounds__(group_threads(XRES), 1)
 sdq_linear_group_kernel(const __grid_constant__ GroupParams p)
 {
   extern __shared__ uint8_t smem_raw[];
   const uint32_t tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   uint8_t* sm = smem_raw + ((128 - (ptx::smem_u32(smem_raw) & 127)) & 127);
-  const uint32_t NU = (uint32_t)p.nslot;                                     // units in the ring
+  constexpr uint32_t NU = GRP_UNITS;
+  const uint32_t NI = (uint32_t)p.nslot;                                     // inlier ring positions
   // (activation-resident variant: the slots hold the weight records only)
   const uint32_t xb = (uint32_t)p.n_tile * 128u, isb = XRES ? (uint32_t)WI_BYTES : (uint32_t)group_is_bytes(p.n_tile);
-  const uint32_t osb = p.out_n ? (XRES ? 2u * (uint32_t)wc_bytes(1) : (uint32_t)group_os_bytes(p.n_tile)) : 0u;
-  const uint32_t ub = isb + osb;                                             // bytes of a unit: inlier slot, then outlier slot
-  uint8_t* xres = sm + NU * ub;                                              // XRES: the quantized activations of all K
+  constexpr uint32_t wcb = 2u * (WC_CODE_BYTES + WC_POS_BYTES);              // the two compact records of a unit
+  uint8_t* wc_ring = sm + NI * isb;
+  uint8_t* x8_ring = wc_ring + (p.out_n ? NU * wcb : 0u);                    // 8-bit codes of the tokens, 2 x 128 K per position
+  uint8_t* xres = x8_ring + (p.out_n && !XRES ? NU * 2u * xb : 0u);          // XRES: the quantized activations of all K
   const uint32_t xres_main = XRES ? (uint32_t)p.m[0].T2 * GRP_XU : 0u;
   uint8_t* x_sfb = xres + xres_main;                                         // XRES: token-scale atom of the outlier product
   float* x_part = reinterpret_cast<float*>(x_sfb + SF_ATOM_BYTES);           // XRES: [quantizing warp][token of its group] maxima
   float* x_sx = x_part + GRP_XQ_WARPS * 8;                                   // XRES: the tokens' fp32 scales (int8 outliers)
   uint8_t* sfbuf = xres + (XRES ? (uint32_t)group_xres_bytes(p.m[0].T2) : 0u);   // 2 x (SFA_out | SFB_out) of the item, alternating
   uint64_t* full_is = reinterpret_cast<uint64_t*>(sfbuf + (p.out_n ? GRP_SIDE_BYTES : 0));  // inlier slot of ring position v has landed
-  uint64_t* full_os = full_is + GRP_MAX_UNITS;                               // outlier slot of ring position v has landed
-  uint64_t* done = full_os + GRP_MAX_UNITS;                                  // the MMAs of the unit at ring position v have completed
-  uint64_t* built = done + GRP_MAX_UNITS;                                    // the containers of the unit at ring position v are in tensor memory
-  uint64_t* acc_full = built + GRP_MAX_UNITS;                                // [2]
+  uint64_t* done_i = full_is + GRP_MAX_IN;                                   // the inlier MMAs of the unit at inlier position v have completed
+  uint64_t* full_wc = done_i + GRP_MAX_IN;                                   // compact records of position v have landed
+  uint64_t* free_wc = full_wc + GRP_UNITS;                                   // ... have been read by the builders
+  uint64_t* full_x8 = free_wc + GRP_UNITS;                                   // 8-bit codes of position v have landed
+  uint64_t* built = full_x8 + GRP_UNITS;                                     // the containers of position v are in tensor memory
+  uint64_t* done_o = built + GRP_UNITS;                                      // the outlier MMAs of the unit at position v have completed
+  uint64_t* acc_full = done_o + GRP_UNITS;                                   // [2]
   uint64_t* acc_empty = acc_full + 2;                                        // [2]
   uint64_t* sf_full = acc_empty + 2;                                         // [2] outlier scale atoms of the item have landed
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(sf_full + 2);
@@ -110,9 +123,10 @@ sdq_linear_group_kernel(const __grid_constant__ GroupParams p)
   if (tid == 0) ptx::griddep_launch_dependents();
   if (tid == 0) {
     *timed_out = 0u;
-    const uint32_t issuers = p.out_n ? 2u : 1u;   // MMA-issuing warps: both commit to `done` and `acc_full`
+    const uint32_t issuers = p.out_n ? 2u : 1u;   // MMA-issuing warps: both commit to `acc_full`
+    for (uint32_t v = 0; v < NI; ++v) { ptx::mbar_init(&full_is[v], 1); ptx::mbar_init(&done_i[v], 1); }
     for (uint32_t v = 0; v < NU; ++v) {
-      ptx::mbar_init(&full_is[v], 1); ptx::mbar_init(&full_os[v], 1); ptx::mbar_init(&done[v], issuers); ptx::mbar_init(&built[v], 4);
+      ptx::mbar_init(&full_wc[v], 1); ptx::mbar_init(&free_wc[v], 4); ptx::mbar_init(&full_x8[v], 1); ptx::mbar_init(&built[v], 4); ptx::mbar_init(&done_o[v], 1);
     }
     for (int a = 0; a < 2; ++a) { ptx::mbar_init(&acc_full[a], issuers); ptx::mbar_init(&acc_empty[a], 4); ptx::mbar_init(&sf_full[a], 1); }
     ptx::fence_barrier_init();
@@ -170,6 +184,7 @@ sdq_linear_group_kernel(const __grid_constant__ GroupParams p)
     for (uint32_t q2 = 0; q2 < GRP_XQ_WARPS / 2; ++q2) ramax = fmaxf(ramax, x_part[(2 * q2 + tg) * 8 + t]);
     const int e = fp8_scale_exp(ramax);
     const float s8 = pow2_neg(e), sx = int8_scale(ramax);
+    const Int8Coder k8 = int8_coder(sx);
     const bool i8 = p.out_i8 != 0;
     if (qw < 2 && l == 0) {
       x_sx[mtok] = sx;
@@ -199,7 +214,7 @@ sdq_linear_group_kernel(const __grid_constant__ GroupParams p)
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
         q4[j >> 2] |= e2m1x2(v[2 * j] * s4, v[2 * j + 1] * s4) << (8 * (j & 3));
-        q8[j >> 1] |= (i8 ? (int8_code(v[2 * j], sx) | (int8_code(v[2 * j + 1], sx) << 8)) : e4m3x2(v[2 * j] * s8, v[2 * j + 1] * s8)) << (16 * (j & 1));
+        q8[j >> 1] |= (i8 ? (int8_code(v[2 * j], k8) | (int8_code(v[2 * j + 1], k8) << 8)) : e4m3x2(v[2 * j] * s8, v[2 * j + 1] * s8)) << (16 * (j & 1));
       }
       const uint32_t k = (uint32_t)b * 64 + l * 16;          // first element of this lane
       uint8_t* xu = xres + (size_t)(k >> 8) * GRP_XU;
@@ -211,74 +226,91 @@ sdq_linear_group_kernel(const __grid_constant__ GroupParams p)
     ptx::named_bar_sync(8, GRP_XQ_WARPS * 32);
   }
 
-  if (warp == 0 || warp == 10) {
-    // ---------------- producers: warp 0 fills the inlier slots, warp 10 the outlier slots.  Six lanes each, in lockstep: lane
-    // 2 c + l issues copy c (of three) of the units u = l, l + 2, ... of this CTA's sequence (NU is even, so a lane's ring
-    // positions keep its parity) -- issuing a bulk copy costs its thread ~100 ns, so one instruction issues a copy for
-    // each of the six lanes instead of one thread issuing six in a row.
-    const bool outl = warp == 10;
+  if (warp == 0 || warp == 10 || warp == 24) {
+    // ---------------- producers: warp 0 the inlier slots (lane 2 c + l issues copy c of three), warp 10 the compact records,
+    // warp 24 the 8-bit codes (copy c of two, one per 128 K).  Lane l of a copy takes the units u = l, l + 2, ... of this CTA's
+    // sequence (the rings have an even number of positions, so a lane's positions keep its parity) -- issuing a bulk copy
+    // costs its thread ~100 ns, so one instruction issues a copy for each of the lanes instead of one thread all in a row.
+    // (Activation-resident variant: warp 0's c = 0 is the one copy of a slot, its c = 1 the row-scale atom of each item.)
     const uint32_t l = lane & 1, c = lane >> 1;
-    // (activation-resident variant: one copy per inlier slot; per outlier slot the compact records, and lane c = 1 the row-scale
-    // atom of each item)
-    if (c < (XRES ? (outl ? 2u : 1u) : 3u) && (!outl || p.out_n)) {
-      if (!XRES) ptx::griddep_wait();            // activations come from an earlier kernel
+    const bool inl = warp == 0, wc = warp == 10;
+    const uint32_t copies = inl ? (XRES ? (p.out_n && !p.out_i8 ? 2u : 1u) : 3u) : (wc ? 1u : 2u);
+    if (c < copies && (inl || p.out_n)) {
       bool ok = true;
       int item = first, k2 = (int)l;             // this lane's position: work item and 256-K unit inside the item
       int mat = -1, rt = 0, T2 = 0;
       uint32_t iseq = 0;                         // number of the item in this CTA's sequence
-      uint32_t v = l, wrapped = 0, ph = 0;       // ring position, whether the ring has wrapped, parity of `done` to wait for
-      const uint32_t wcb = 2u * (uint32_t)wc_bytes(1);
-      for (;;) {
-        for (;;) {                               // advance to the item that holds unit k2
-          if (item >= p.total_items) break;
+      const uint32_t N = inl ? NI : NU;
+      uint64_t* freed = inl ? done_i : (wc ? free_wc : done_o);
+      uint32_t v = l, wrapped = 0, ph = 0;       // ring position, whether the ring has wrapped, parity of `freed` to wait for
+      uint32_t ahead = 0;                        // units whose weights were fetched ahead of the wait below
+      // advances to the item that holds unit k2; false at the end of the sequence
+      auto seek = [&]() {
+        for (;;) {
+          if (item >= p.total_items) return false;
           if (mat < 0) { mat = group_mat_of(p, item); rt = item - p.m[mat].item0; T2 = p.m[mat].T2; }
-          if (k2 < T2) break;
+          if (k2 < T2) return true;
           k2 -= T2; item += stride; mat = -1; ++iseq;
         }
-        if (item >= p.total_items) break;
-        const GroupMat& m = p.m[mat];
-        if (wrapped && !(ok = ptx::mbar_wait(&done[v], ph ^ 1))) break;
-        uint8_t* st = sm + (size_t)v * ub + (outl ? isb : 0u);
-        if (XRES) {
-          if (!outl) {
-            ptx::mbar_expect_tx(&full_is[v], WI_BYTES);
-            ptx::bulk_g2s(st, m.w + m.wi + ((size_t)rt * m.T2 + k2) * WI_BYTES, WI_BYTES, &full_is[v]);
-          } else if (c == 0) {
-            ptx::mbar_expect_tx(&full_os[v], wcb);
-            ptx::bulk_g2s(st, m.w + m.wc + ((size_t)rt * 2 * m.T2 + 2 * k2) * (size_t)wc_bytes(1), wcb, &full_os[v]);
-          } else if (k2 == 0 && !p.out_i8) {     // the item's row-scale atom (see below); the tokens' atom is resident
-            const uint32_t sb = iseq & 1;
-            if (iseq >= 2 && !(ok = ptx::mbar_wait(&acc_full[sb], ((iseq >> 1) - 1) & 1))) break;
-            ptx::mbar_expect_tx(&sf_full[sb], SF_ATOM_BYTES);
-            ptx::bulk_g2s(sfbuf + sb * 2 * SF_ATOM_BYTES, m.w + m.sfa_out + (size_t)rt * SF_ATOM_BYTES, SF_ATOM_BYTES, &sf_full[sb]);
+      };
+      if (!XRES && !wc) {
+        // activations come from an earlier kernel; the first lap's inlier weights are fetched before the wait for it
+        if (inl && c == 0) {
+          for (uint32_t u = l; u < NI && seek(); u += 2, k2 += 2, ++ahead) {
+            const GroupMat& m = p.m[mat];
+            ptx::mbar_expect_tx(&full_is[u], WI_BYTES + xb + SF_ATOM_BYTES);
+            ptx::bulk_g2s(sm + (size_t)u * isb, m.w + m.wi + ((size_t)rt * m.T2 + k2) * WI_BYTES, WI_BYTES, &full_is[u]);
           }
-        } else if (!outl) {
-          const uint8_t* xi = m.x + m.xi + (size_t)k2 * XI_BYTES;
-          if (c == 0) ptx::mbar_expect_tx(&full_is[v], WI_BYTES + xb + SF_ATOM_BYTES);
-          const uint8_t* src = c == 0 ? m.w + m.wi + ((size_t)rt * m.T2 + k2) * WI_BYTES : (c == 1 ? xi : xi + B4_BYTES);
-          const uint32_t off = c == 0 ? 0u : (c == 1 ? (uint32_t)WI_BYTES : (uint32_t)WI_BYTES + xb);
-          ptx::bulk_g2s(st + off, src, c == 0 ? (uint32_t)WI_BYTES : (c == 1 ? xb : (uint32_t)SF_ATOM_BYTES), &full_is[v]);
+          item = first; k2 = (int)l; mat = -1; iseq = 0;
+        }
+        ptx::griddep_wait();
+      }
+      while (seek()) {
+        const GroupMat& m = p.m[mat];
+        if (wrapped && !(ok = ptx::mbar_wait(&freed[v], ph ^ 1))) break;
+        if (inl) {
+          uint8_t* st = sm + (size_t)v * isb;
+          const uint8_t* wi = m.w + m.wi + ((size_t)rt * m.T2 + k2) * WI_BYTES;
+          if (XRES) {
+            if (c == 0) {
+              ptx::mbar_expect_tx(&full_is[v], WI_BYTES);
+              ptx::bulk_g2s(st, wi, WI_BYTES, &full_is[v]);
+            } else if (k2 == 0) {                // (see warp 24; the tokens' atom is resident)
+              const uint32_t sb = iseq & 1;
+              if (iseq >= 2 && !(ok = ptx::mbar_wait(&acc_full[sb], ((iseq >> 1) - 1) & 1))) break;
+              ptx::mbar_expect_tx(&sf_full[sb], SF_ATOM_BYTES);
+              ptx::bulk_g2s(sfbuf + sb * 2 * SF_ATOM_BYTES, m.w + m.sfa_out + (size_t)rt * SF_ATOM_BYTES, SF_ATOM_BYTES, &sf_full[sb]);
+            }
+          } else if (ahead) {
+            --ahead;
+          } else {
+            const uint8_t* xi = m.x + m.xi + (size_t)k2 * XI_BYTES;
+            if (c == 0) ptx::mbar_expect_tx(&full_is[v], WI_BYTES + xb + SF_ATOM_BYTES);
+            const uint32_t off = c == 0 ? 0u : (c == 1 ? (uint32_t)WI_BYTES : (uint32_t)WI_BYTES + xb);
+            ptx::bulk_g2s(st + off, c == 0 ? wi : (c == 1 ? xi : xi + B4_BYTES), c == 0 ? (uint32_t)WI_BYTES : (c == 1 ? xb : (uint32_t)SF_ATOM_BYTES), &full_is[v]);
+          }
+        } else if (wc) {
+          ptx::mbar_expect_tx(&full_wc[v], wcb);
+          ptx::bulk_g2s(wc_ring + (size_t)v * wcb, m.w + m.wc + ((size_t)rt * m.T2 + k2) * wcb, wcb, &full_wc[v]);
         } else {
-          const uint8_t* xo = m.x + m.xo + (size_t)(2 * k2) * XO_BYTES;
-          if (c == 0) ptx::mbar_expect_tx(&full_os[v], wcb + 2 * xb);
-          const uint8_t* src = c == 0 ? m.w + m.wc + ((size_t)rt * 2 * m.T2 + 2 * k2) * (size_t)wc_bytes(1) : (c == 1 ? xo : xo + XO_BYTES);
-          ptx::bulk_g2s(st + (c == 0 ? 0u : wcb + (c - 1) * xb), src, c == 0 ? wcb : xb, &full_os[v]);
-          if (k2 == 0 && c >= 1 && !p.out_i8) {     // (int8 outliers take fp32 scales in the epilogue: no scale atoms)
-            // the item's outlier scale atoms (lane c = 1: of the weight rows, c = 2: of the tokens): a buffer and a barrier
+          const uint8_t* xo = m.x + m.xo + (size_t)(2 * k2 + (int)c) * XO_BYTES;
+          if (c == 0) ptx::mbar_expect_tx(&full_x8[v], 2 * xb);
+          ptx::bulk_g2s(x8_ring + (size_t)v * 2 * xb + c * xb, xo, xb, &full_x8[v]);
+          if (k2 == 0 && !p.out_i8) {            // (int8 outliers take fp32 scales in the epilogue: no scale atoms)
+            // the item's outlier scale atoms (lane c = 0: of the weight rows, c = 1: of the tokens): a buffer and a barrier
             // of their own per item parity.  The buffer is free once every MMA of the item two back has completed (`acc_full`
             // of that item: it cannot complete again before these atoms land, since the next item on that accumulator needs
-            // them) -- the ring alone does not say so when an item has fewer units than half the ring.
+            // them) -- the rings alone do not say so when an item has fewer units than half a ring.
             const uint32_t sb = iseq & 1;
             if (iseq >= 2 && !(ok = ptx::mbar_wait(&acc_full[sb], ((iseq >> 1) - 1) & 1))) break;
-            uint8_t* sf = sfbuf + sb * 2 * SF_ATOM_BYTES;
-            if (c == 1) ptx::mbar_expect_tx(&sf_full[sb], 2u * SF_ATOM_BYTES);
-            ptx::bulk_g2s(sf + (c - 1) * SF_ATOM_BYTES, c == 1 ? m.w + m.sfa_out + (size_t)rt * SF_ATOM_BYTES : m.x + m.sfb_out, SF_ATOM_BYTES,
-                          &sf_full[sb]);
+            if (c == 0) ptx::mbar_expect_tx(&sf_full[sb], 2u * SF_ATOM_BYTES);
+            ptx::bulk_g2s(sfbuf + sb * 2 * SF_ATOM_BYTES + c * SF_ATOM_BYTES, c == 0 ? m.w + m.sfa_out + (size_t)rt * SF_ATOM_BYTES : m.x + m.sfb_out,
+                          SF_ATOM_BYTES, &sf_full[sb]);
           }
         }
         k2 += 2;
         v += 2;
-        if (v >= NU) { v -= NU; wrapped = 1; ph ^= 1; }
+        if (v >= N) { v -= N; wrapped = 1; ph ^= 1; }
       }
       if (!ok) atomicOr(&p.flags[FLAG_TIMEOUT], 1u);
     }
@@ -289,14 +321,14 @@ sdq_linear_group_kernel(const __grid_constant__ GroupParams p)
     // lane issues (descriptors and TMEM addresses are uniform-register operands).  tcgen05.cp and tcgen05.mma of one
     // thread execute in issue order, so the inlier metadata and the scales need no barrier of their own; their TMEM buffers
     // alternate.  The outlier product takes its A operand and metadata from tensor memory, where the builders put them.
-    // The unit is released when both warps' commits have arrived.
+    // Each warp's commits release its own ring's positions.
     const bool outw = warp == 23;
     if (!outw || p.out_n) {
       bool ok = true;
       const uint32_t smb = ptx::smem_u32(sm);
       const uint32_t id4[2] = {ptx::idesc_block_scaled(128, (uint32_t)p.n_tile, 1, true, 0, 0), ptx::idesc_block_scaled(128, (uint32_t)p.n_tile, 1, true, 2, 2)};
       const uint32_t id8 = p.out_i8 ? ptx::idesc_i8(128, (uint32_t)p.n_tile, true) : ptx::idesc_block_scaled(128, (uint32_t)p.n_tile, 0, true, 0, 0);
-      const uint32_t wcb = 2u * (uint32_t)wc_bytes(1);
+      const uint32_t N = outw ? NU : NI;
       uint32_t v = 0, ph = 0, itc = 0;             // ring position and its lap parity, item count
       for (int item = first; item < p.total_items && ok; item += stride, ++itc) {
         const int T2 = p.m[group_mat_of(p, item)].T2;
@@ -306,24 +338,26 @@ sdq_linear_group_kernel(const __grid_constant__ GroupParams p)
           if (!ok) break;
         }
         for (int k2 = 0; k2 < T2 && ok;) {
-          // Up to four units of the item per trip: lane i tests unit k2 + i (for the outlier product: its containers are in
-          // tensor memory, which implies that its slot has landed -- the builders waited for that), lane 4 the item's scale
+          // Up to four units of the item per trip: lane i tests unit k2 + i (for the outlier product: lane i its containers,
+          // lane 8 + i the tokens' 8-bit codes), lane 4 the item's scale
           // atoms; the units ready in a row from k2 on are issued together.  A trip costs several hundred cycles beside the
           // instructions it issues (test, vote, fence, election, reconvergence), so taking what is ready in one trip keeps
           // the issuer ahead whenever it has fallen behind.  With nothing ready it waits for unit k2 and votes again.
           const int nb = T2 - k2 < 4 ? T2 - k2 : 4;
-          uint32_t vi = v + lane, phi = ph;
-          if (vi >= NU) { vi -= NU; phi ^= 1; }
-          const bool sf_lane = outw && k2 == 0 && lane == 4 && !p.out_i8;
-          uint64_t* bar = sf_lane ? &sf_full[ab] : (outw ? &built[vi < NU ? vi : 0] : &full_is[vi < NU ? vi : 0]);
+          const uint32_t i = lane & 3;
+          uint32_t vi = v + i, phi = ph;
+          if (vi >= N) { vi -= N; phi ^= 1; }
+          const bool sf_lane = outw && k2 == 0 && lane == 4 && !p.out_i8, x_lane = outw && !XRES && (lane >> 2) == 2;
+          uint64_t* bar = sf_lane ? &sf_full[ab] : (x_lane ? &full_x8[vi] : (outw ? &built[vi] : &full_is[vi]));
           const uint32_t par = sf_lane ? ((itc >> 1) & 1) : phi;
-          const bool mine = (int)lane < nb || sf_lane;
-          const uint32_t ready = __ballot_sync(0xffffffffu, mine ? ptx::mbar_test(bar, par) : (lane == 4));
+          const bool mine = ((lane < 4 || x_lane) && (int)i < nb) || sf_lane;
+          uint32_t ready = __ballot_sync(0xffffffffu, mine ? ptx::mbar_test(bar, par) : (lane == 4));
+          if (outw && !XRES) ready &= (ready >> 8) | ~15u;
           int n = __ffs((int)~ready) - 1;          // units ready in a row (lane 4 votes yes when it has nothing to test)
           if (n > nb) n = nb;
           if (!(ready & 16u)) n = 0;
           if (n == 0) {
-            ok = __all_sync(0xffffffffu, (lane == 0 || sf_lane) ? ptx::mbar_wait(bar, par) : true);
+            ok = __all_sync(0xffffffffu, (lane == 0 || sf_lane || (x_lane && i == 0)) ? ptx::mbar_wait(bar, par) : true);
             continue;
           }
           ptx::tc_fence_after();
@@ -331,7 +365,7 @@ sdq_linear_group_kernel(const __grid_constant__ GroupParams p)
             uint32_t vv = v;
             for (int i = 0; i < n; ++i) {
               const int kk = k2 + i;
-              const uint32_t sb = smb + vv * ub;
+              const uint32_t sb = smb + vv * isb;
               // the tokens' operands of unit kk: in the slot behind the weight records, or resident
               const uint32_t xu = ptx::smem_u32(xres) + (uint32_t)kk * GRP_XU;
               const uint32_t b4 = XRES ? xu : sb + WI_BYTES, sf4 = XRES ? xu + 16 * 128 : sb + WI_BYTES + xb;
@@ -353,7 +387,7 @@ sdq_linear_group_kernel(const __grid_constant__ GroupParams p)
 #pragma unroll
                 for (uint32_t h = 0; h < 2; ++h) {
                   const uint32_t ca = tmem + GRP_TM_C + GRP_TM_C_COLS * vv + 16u * h, eb = tmem + GRP_TM_C + GRP_TM_C_COLS * vv + 32u + 4u * h;
-                  const uint32_t xa = XRES ? xu + 16 * 128 + SF_ATOM_BYTES + h * 16 * 128 : sb + isb + wcb + h * xb;
+                  const uint32_t xa = XRES ? xu + 16 * 128 + SF_ATOM_BYTES + h * 16 * 128 : ptx::smem_u32(x8_ring) + vv * 2 * xb + h * xb;
                   if (p.out_i8) {     // the same containers and token codes as integers, int32 accumulator
                     ptx::mma_sp_i8_ta(acc_col, ca, ptx::smem_desc(xa, 128, 1024), id8, eb, (kk | (int)h) ? 1u : 0u);
                     ptx::mma_sp_i8_ta(acc_col, ca + 8, ptx::smem_desc(xa + 512, 128, 1024), id8, eb + 2, 1u);
@@ -363,15 +397,15 @@ sdq_linear_group_kernel(const __grid_constant__ GroupParams p)
                   }
                 }
               }
-              ptx::tc_commit(&done[vv]);
+              ptx::tc_commit(outw ? &done_o[vv] : &done_i[vv]);
               if (kk == T2 - 1) ptx::tc_commit(&acc_full[ab]);
-              if (++vv == NU) vv = 0;
+              if (++vv == N) vv = 0;
             }
           }
           __syncwarp();
           k2 += n;
           v += (uint32_t)n;
-          if (v >= NU) { v -= NU; ph ^= 1; }
+          if (v >= N) { v -= N; ph ^= 1; }
         }
       }
       if (!ok && lane == 0) atomicOr(&p.flags[FLAG_TIMEOUT], 1u);
@@ -436,41 +470,49 @@ sdq_linear_group_kernel(const __grid_constant__ GroupParams p)
     }
     if (!ok && lane == 0) atomicOr(&p.flags[FLAG_TIMEOUT], 1u);
   } else if (p.out_n && warp >= 6 && warp <= 22) {
-    // ---------------- outlier container builders: up to four groups of four warps (6..9, 11..14, 15..18, 19..22); group g
-    // rebuilds the containers of the units u = g, g + G, ... -- straight into tensor memory, where the outlier MMAs read their
+    // ---------------- outlier container builders: four groups of four warps (6..9, 11..14, 15..18, 19..22); group g
+    // rebuilds the containers of the units u = g, g + 4, ... -- straight into tensor memory, where the outlier MMAs read their
     // A operand and metadata: shared memory is written once (by the bulk copies) and never again.  A warp can reach the 32
     // TMEM lanes 32 (warp % 4) .., so its thread `lane` rebuilds weight row 32 (warp % 4) + lane, both 128-K stages of the
     // unit, each from 16 codes + 16 positions: per S-Vector of 8 the code goes to the 2:4 slot of its group of 4 (two
     // ascending slot indices per 4: (p, 3) with the value first, or (0, 3) with the value second when p = 3; a group without
     // outlier gets (0, 1) and zeros), the form the packer writes for the many-token kernels.  A row's 64 stored bytes per
     // stage are 16 columns of its lane, its 16 metadata bytes 4 columns.  Several groups, because a trip is mostly latency
-    // (measured ~1800 cycles, a tenth of it arithmetic): they overlap in time.  G divides the ring, so that every phase of
-    // a slot's barrier is seen by the same group.  Container set v is free when the unit's outlier slot has landed at ring
-    // position v: the producer refills a position only after the MMAs of its previous unit have completed.
+    // (measured ~1800 cycles, a tenth of it arithmetic): they overlap in time.  Container set v is free when the outlier MMAs of
+    // the unit that had it before have completed; the compact record at position v is given back once its codes and positions
+    // are in registers.
     const uint32_t bw = warp - (warp >= 11 ? 7u : 6u);       // 0..15
     const uint32_t grp = bw >> 2;
-    const uint32_t G = (NU & 3u) == 0 ? 4u : (NU % 3u == 0 ? 3u : 2u);
     const uint32_t r = (warp & 3) * 32 + lane;
     const bool poller = (bw & 3u) == 0;
     bool ok = true;
-    uint32_t v = 0, ph = 0, gu = 0;              // position of the unit in the ring, lap parity, unit count modulo G
+    uint32_t v = 0, ph = 0, lap = 0;             // position of the unit in the ring, lap parity, whether the ring has wrapped
     const uint32_t tlane = tmem + (((warp & 3) * 32u) << 16) + GRP_TM_C;
-    for (int item = first; item < p.total_items && ok && grp < G; item += stride) {
+    for (int item = first; item < p.total_items && ok; item += stride) {
       const int T2 = p.m[group_mat_of(p, item)].T2;
       for (int k2 = 0; k2 < T2; ++k2) {
-        if (gu == grp) {
+        if ((v & (GRP_BUILDERS - 1)) == grp) {
           // Only ONE thread of the group waits on the mbarrier and then releases the others through a hardware barrier: with
           // every warp waiting on the same mbarrier some of them noticed its completion more than a microsecond late.
-          if (poller && lane == 0 && !ptx::mbar_wait(&full_os[v], ph)) *timed_out = 1u;
+          // (lane 0 waits for the records, lane 1 for the container set)
+          if (poller && (lane == 0 || (lane == 1 && lap)) && !ptx::mbar_wait(lane ? &done_o[v] : &full_wc[v], lane ? ph ^ 1 : ph)) *timed_out = 1u;
           ptx::named_bar_sync(4 + grp, 128);   // (barrier 3 belongs to the epilogue)
           if (*timed_out) { ok = false; break; }
-          const uint8_t* st = sm + (size_t)v * ub + isb;
+          ptx::tc_fence_after();               // the container set is rewritten: after the MMAs that read it
+          const uint8_t* st = wc_ring + (size_t)v * wcb;
+          uint4 codes[2];
+          uint2 pos[2];
+#pragma unroll
+          for (uint32_t h = 0; h < 2; ++h) {
+            codes[h] = *reinterpret_cast<const uint4*>(st + h * (uint32_t)wc_bytes(1) + r * 16);
+            pos[h] = *reinterpret_cast<const uint2*>(st + h * (uint32_t)wc_bytes(1) + WC_CODE_BYTES + r * 8);
+          }
+          __syncwarp();
+          if (lane == 0) ptx::mbar_arrive(&free_wc[v]);
           const uint32_t tc = tlane + GRP_TM_C_COLS * v;
 #pragma unroll
           for (uint32_t h = 0; h < 2; ++h) {
-            const uint4 codes = *reinterpret_cast<const uint4*>(st + h * (uint32_t)wc_bytes(1) + r * 16);
-            const uint2 pos = *reinterpret_cast<const uint2*>(st + h * (uint32_t)wc_bytes(1) + WC_CODE_BYTES + r * 8);
-            const uint32_t cw[4] = {codes.x, codes.y, codes.z, codes.w}, pw[2] = {pos.x, pos.y};
+            const uint32_t cw[4] = {codes[h].x, codes[h].y, codes[h].z, codes[h].w}, pw[2] = {pos[h].x, pos[h].y};
             // position ps (0..7) of the outlier in its S-Vector: it sits in the group of 4 number ps >> 2 at p = ps & 3.  Stored
             // bytes of the S-Vector (two per group of 4): the code moves to byte (p == 3) + 2 (ps >> 2); metadata byte = the two
             // groups' slot-index nibbles, (p, 3) or (0, 3) for p = 3 where the outlier is, (0, 1) elsewhere.  Both come from
@@ -495,8 +537,7 @@ sdq_linear_group_kernel(const __grid_constant__ GroupParams p)
           __syncwarp();
           if (lane == 0) ptx::mbar_arrive(&built[v]);      // one arrival per warp
         }
-        if (++gu == G) gu = 0;
-        if (++v == NU) { v = 0; ph ^= 1; }
+        if (++v == NU) { v = 0; ph ^= 1; lap = 1; }
       }
     }
     if (!ok && lane == 0) atomicOr(&p.flags[FLAG_TIMEOUT], 1u);
@@ -506,27 +547,23 @@ sdq_linear_group_kernel(const __grid_constant__ GroupParams p)
   if (warp == 1) ptx::tmem_dealloc(tmem, GRP_TMEM_COLS);
 }
 
-// units the ring holds for `n_tile` tokens per tile: as many as fit (an even number)
-static int group_units(int n_tile, int out_n, int xres_bytes, int unit_bytes) {
-  const int avail = 232448 - 128 - (out_n ? GRP_SIDE_BYTES : 0) - GRP_BAR_BYTES - xres_bytes;
-  int n = avail / unit_bytes;
-  n &= ~1;
-  return n > GRP_MAX_UNITS ? GRP_MAX_UNITS : n;
+// inlier ring positions for `n_tile` tokens per tile (an even number, as many as fit beside the outlier rings)
+static int group_units(int n_tile, int out_n, int xres_bytes) {
+  const int is = xres_bytes ? WI_BYTES : group_is_bytes(n_tile), os = out_n ? 2 * wc_bytes(1) + (xres_bytes ? 0 : 2 * n_tile * 128) : 0;
+  const int n = (232448 - 128 - (out_n ? GRP_SIDE_BYTES : 0) - GRP_BAR_BYTES - xres_bytes - GRP_UNITS * os) / is & ~1;
+  return n > GRP_MAX_IN ? GRP_MAX_IN : n;
 }
 
-// shared-memory budget of the activation-resident variant: does a ring of at least six units fit beside X of K / 256 = T2 units?
-bool group_xres_fits(int T2, int out_n) {
-  const int unit = WI_BYTES + (out_n ? 2 * wc_bytes(1) : 0);
-  return group_units(16, out_n, group_xres_bytes(T2), unit) >= 6;
-}
+// shared-memory budget of the activation-resident variant: do at least six inlier slots fit beside X of K / 256 = T2 units?
+bool group_xres_fits(int T2, int out_n) { return group_units(16, out_n, group_xres_bytes(T2)) >= 6; }
 
 cudaError_t launch_linear_group(GroupParams p, bool f32_out, int sm_count, cudaStream_t stream, uint32_t* attr_done)
 {
   const bool xres = p.x_bf16 != nullptr;
   const int xbytes = xres ? group_xres_bytes(p.m[0].T2) : 0;
-  p.slot_bytes = xres ? WI_BYTES + (p.out_n ? 2 * wc_bytes(1) : 0) : group_is_bytes(p.n_tile) + (p.out_n ? group_os_bytes(p.n_tile) : 0);
-  p.nslot = group_units(p.n_tile, p.out_n, xbytes, p.slot_bytes);
-  const int smem = p.nslot * p.slot_bytes + xbytes + (p.out_n ? GRP_SIDE_BYTES : 0) + GRP_BAR_BYTES + 128;
+  const int is = xres ? WI_BYTES : group_is_bytes(p.n_tile), os = p.out_n ? 2 * wc_bytes(1) + (xres ? 0 : 2 * p.n_tile * 128) : 0;
+  p.nslot = group_units(p.n_tile, p.out_n, xbytes);
+  const int smem = p.nslot * is + GRP_UNITS * os + xbytes + (p.out_n ? GRP_SIDE_BYTES : 0) + GRP_BAR_BYTES + 128;
   if (!*attr_done) {
     const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
     if (cudaFuncSetAttribute(sdq_linear_group_kernel<false, false>, a, 232448) != cudaSuccess ||
@@ -538,7 +575,7 @@ cudaError_t launch_linear_group(GroupParams p, bool f32_out, int sm_count, cudaS
   }
   cudaLaunchConfig_t lc = {};
   lc.gridDim = dim3((unsigned)(p.total_items < sm_count ? p.total_items : sm_count));
-  lc.blockDim = dim3(GRP_THREADS);
+  lc.blockDim = dim3((unsigned)group_threads(xres));
   lc.dynamicSmemBytes = (size_t)smem;
   lc.stream = stream;
   cudaLaunchAttribute attr[1];
