@@ -496,6 +496,40 @@ extern "C" sdq_status_t sdq_workspace_size(int64_t M, int64_t N, int64_t K, cons
   return SDQ_OK;
 }
 
+// The grouped kernel carries the primary format: up to 32 tokens, pair-wise 4:8 inliers, one E8M0 scale per 64 K, at most one
+// outlier per S-Vector, and K >= 1024: an item then spans enough units that the per-item barriers never run two phases apart.
+static bool group_format(const sdq_packed_t& w) {
+  const sdq_config_t& c = w.cfg;
+  return c.in_gran == SDQ_GRAN_PAIR && c.in_block == 64 && c.scale_rule != SDQ_SCALE_UE4M3 && c.out_n <= 1 && w.K >= 4 * K2;
+}
+static bool group_kernel_takes(const sdq_act_t& x, const sdq_packed_t& w) { return x.M <= 32 && group_format(w); }
+// launch parameters of `n` layers with the format of `w`, up to `max_m` tokens; then one group_add per layer, in order
+static void group_begin(GroupParams& g, int n, int64_t max_m, const sdq_packed_t& w) {
+  g.n = n;
+  g.n_tile = max_m <= 16 ? 16 : 32;
+  g.out_n = w.cfg.out_n;
+  g.out_i8 = g.out_n > 0 && w.cfg.out_fmt == SDQ_OUT_INT8;
+  g.x_bf16 = nullptr; g.x_ld = 0; g.x_M = 0; g.scale_rule = w.cfg.scale_rule;
+  g.total_items = 0;
+  g.flags = device_flags();
+}
+// x == nullptr: the layers share g.x_bf16
+static void group_add(GroupParams& g, int i, const sdq_act_t* x, const sdq_packed_t& w, void* Y, int64_t ldy, int64_t M) {
+  const PackedOffsets po = tiled_offsets(w);
+  GroupMat& m = g.m[i];
+  m.w = (const uint8_t*)w.dev; m.Y = Y; m.ldy = ldy;
+  m.wi = po.wi; m.wc = po.wc; m.sfa_out = po.sfa_out; m.wsc = po.osexp;
+  m.x = nullptr; m.xi = m.xo = m.sfb_out = m.xsc = 0;
+  if (x) {
+    const ActOffsets ao = act_offsets(x->M, x->K, false);
+    m.x = (const uint8_t*)x->dev;
+    m.xi = ao.xi; m.xo = ao.xo; m.sfb_out = ao.sfb_out; m.xsc = ao.sexp;
+  }
+  m.M = (int)M; m.T2 = (int)(w.K / K2);
+  m.item0 = g.total_items;
+  g.total_items += (int)(w.N / TILE_ROWS);
+}
+
 static sdq_status_t launch_linear(const sdq_act_t* Xq, const sdq_packed_t* P, void* Y, int64_t ldy, void* ws, size_t ws_bytes,
                                   void* stream, bool f32)
 {
@@ -538,10 +572,27 @@ static sdq_status_t launch_linear(const sdq_act_t* Xq, const sdq_packed_t* P, vo
   p.Y = Y; p.ldy = ldy;
   p.flags = device_flags();
   if (!p.flags) return SDQ_ERR_CUDA;
-  // CTA pairs: all calls above 128 tokens; up to 128 where they are estimated faster than this file's kernel and no
-  // workspace asks for its split
+  // CTA pairs: all calls above 128 tokens.  Up to 128, unless a workspace asks for its split, the kernel with the least
+  // estimated time: this file's, the pairs, or the grouped kernel on one layer (one token: 4096 x 4096 7.7 -> 7.4 us,
+  // 4096 -> 11008 12.1 -> 8.7, 11008 -> 4096 12.7 -> 10.0; 100 tokens, 4096 -> 11008: 17.0 -> 15.1 on pairs).
   const int ws_ks = ws ? choose_ksplit(M, P->N, P->K, sm_count) : 1;
-  if (M > 128 || (ws_ks == 1 && pair_kernel_us(M, P->N, P->K, p.out_n, p.b32 != 0, p.dense != 0, dinfo) < few_token_us(M, P->N, P->K, P->cfg))) {
+  bool pairs = M > 128;
+  if (!pairs && ws_ks == 1) {
+    const double few = few_token_us(M, P->N, P->K, P->cfg), two = pair_kernel_us(M, P->N, P->K, p.out_n, p.b32 != 0, p.dense != 0, dinfo);
+    if (group_kernel_takes(*Xq, *P)) {
+      const double one = group_kernel_us(P->N / TILE_ROWS, (int)(P->K / K2), dinfo);
+      if (one < few && one < two) {
+        GroupParams g;
+        group_begin(g, 1, M, *P);
+        if (!g.flags) return SDQ_ERR_CUDA;
+        group_add(g, 0, Xq, *P, Y, ldy, M);
+        const cudaError_t ge = launch_linear_group(g, f32, dinfo, (cudaStream_t)stream);
+        return ge == cudaSuccess && cudaGetLastError() == cudaSuccess ? SDQ_OK : SDQ_ERR_CUDA;
+      }
+    }
+    pairs = two < few;
+  }
+  if (pairs) {
     const cudaError_t pe = launch_linear_pair(p, f32, dinfo, (cudaStream_t)stream);
     return pe == cudaSuccess && cudaGetLastError() == cudaSuccess ? SDQ_OK : SDQ_ERR_CUDA;
   }
@@ -674,10 +725,7 @@ static sdq_status_t launch_group(int n, const sdq_act_t* const* Xq, const sdq_pa
     if (!is_tensor_core_reading(w->cfg)) return SDQ_ERR_UNSUPPORTED;
     if (w->cfg.out_n > 0 && x->cfg.out_fmt != w->cfg.out_fmt) return SDQ_ERR_SHAPE;
     if (((uintptr_t)Y[i] & 15) || (ldy[i] % 8)) return SDQ_ERR_ALIGNMENT;
-    // the grouped kernel carries the primary format: pair-wise 4:8 inliers, one E8M0 scale per 64 K, at most one outlier per S-Vector
-    fused = fused && x->M <= 32 && w->cfg.in_gran == SDQ_GRAN_PAIR && w->cfg.in_block == 64 && w->cfg.scale_rule != SDQ_SCALE_UE4M3 &&
-            w->cfg.out_n <= 1 && w->cfg.out_n == P[0]->cfg.out_n && w->cfg.out_fmt == P[0]->cfg.out_fmt &&
-            w->K >= 4 * K2;   // an item spans at least half the ring: the kernel's per-item barriers then never run two phases apart
+    fused = fused && group_kernel_takes(*x, *w) && w->cfg.out_n == P[0]->cfg.out_n && w->cfg.out_fmt == P[0]->cfg.out_fmt;
     items += w->N / TILE_ROWS;
     if (x->M > max_m) max_m = x->M;
   }
@@ -690,28 +738,10 @@ static sdq_status_t launch_group(int n, const sdq_act_t* const* Xq, const sdq_pa
     return SDQ_OK;
   }
   GroupParams g;
-  g.n = n;
-  g.n_tile = max_m <= 16 ? 16 : 32;
-  g.out_n = P[0]->cfg.out_n;
-  g.out_i8 = g.out_n > 0 && P[0]->cfg.out_fmt == SDQ_OUT_INT8;
-  g.x_bf16 = nullptr; g.x_ld = 0; g.x_M = 0; g.scale_rule = P[0]->cfg.scale_rule;
-  g.total_items = (int)items;
-  g.flags = device_flags();
+  group_begin(g, n, max_m, *P[0]);
   if (!g.flags) return SDQ_ERR_CUDA;
-  int item0 = 0;
-  for (int i = 0; i < n; ++i) {
-    const PackedOffsets po = tiled_offsets(*P[i]);
-    const ActOffsets ao = act_offsets(Xq[i]->M, Xq[i]->K, false);
-    GroupMat& m = g.m[i];
-    m.w = (const uint8_t*)P[i]->dev; m.x = (const uint8_t*)Xq[i]->dev; m.Y = Y[i]; m.ldy = ldy[i];
-    m.wi = po.wi; m.wc = po.wc; m.sfa_out = po.sfa_out;
-    m.xi = ao.xi; m.xo = ao.xo; m.sfb_out = ao.sfb_out;
-    m.wsc = po.osexp; m.xsc = ao.sexp;
-    m.M = (int)Xq[i]->M; m.T2 = (int)(P[i]->K / K2);
-    m.item0 = item0;
-    item0 += (int)(P[i]->N / TILE_ROWS);
-  }
-  const cudaError_t e = launch_linear_group(g, f32, dinfo->sm_count, (cudaStream_t)stream, &dinfo->group_attr);
+  for (int i = 0; i < n; ++i) group_add(g, i, Xq[i], *P[i], Y[i], ldy[i], Xq[i]->M);
+  const cudaError_t e = launch_linear_group(g, f32, dinfo, (cudaStream_t)stream);
   return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? SDQ_OK : SDQ_ERR_CUDA;
 }
 
@@ -732,36 +762,18 @@ static sdq_status_t launch_group_x(int n, const void* X, int64_t M, int64_t K, i
     if (!is_tensor_core_reading(w->cfg)) return SDQ_ERR_UNSUPPORTED;
     if (((uintptr_t)Y[i] & 15) || (ldy[i] % 8)) return SDQ_ERR_ALIGNMENT;
     const sdq_config_t& c = w->cfg, &c0 = P[0]->cfg;
-    if (c.in_gran != SDQ_GRAN_PAIR || c.in_block != 64 || c.scale_rule == SDQ_SCALE_UE4M3 || c.out_n > 1 || c.out_n != c0.out_n ||
-        c.out_fmt != c0.out_fmt || c.scale_rule != c0.scale_rule)
-      return SDQ_ERR_UNSUPPORTED;
+    if (!group_format(*w) || c.out_n != c0.out_n || c.out_fmt != c0.out_fmt || c.scale_rule != c0.scale_rule) return SDQ_ERR_UNSUPPORTED;
     items += w->N / TILE_ROWS;
   }
   // (the in-kernel quantizer keeps a token's K <= 4096 elements in the registers of its 11 x 4 lanes)
   if (n > GROUP_MAX || M > 16 || K < 4 * K2 || K > 16 * K2 || !group_xres_fits((int)(K / K2), P[0]->cfg.out_n) || items * 2 < dinfo->sm_count || items >= (1 << 30))
     return SDQ_ERR_UNSUPPORTED;
   GroupParams g;
-  g.n = n;
-  g.n_tile = 16;
-  g.out_n = P[0]->cfg.out_n;
-  g.out_i8 = g.out_n > 0 && P[0]->cfg.out_fmt == SDQ_OUT_INT8;
-  g.x_bf16 = X; g.x_ld = ldx; g.x_M = (int)M; g.scale_rule = P[0]->cfg.scale_rule;
-  g.total_items = (int)items;
-  g.flags = device_flags();
+  group_begin(g, n, M, *P[0]);
   if (!g.flags) return SDQ_ERR_CUDA;
-  int item0 = 0;
-  for (int i = 0; i < n; ++i) {
-    const PackedOffsets po = tiled_offsets(*P[i]);
-    GroupMat& m = g.m[i];
-    m.w = (const uint8_t*)P[i]->dev; m.x = nullptr; m.Y = Y[i]; m.ldy = ldy[i];
-    m.wi = po.wi; m.wc = po.wc; m.sfa_out = po.sfa_out;
-    m.xi = m.xo = m.sfb_out = m.xsc = 0;
-    m.wsc = po.osexp;
-    m.M = (int)M; m.T2 = (int)(K / K2);
-    m.item0 = item0;
-    item0 += (int)(P[i]->N / TILE_ROWS);
-  }
-  const cudaError_t e = launch_linear_group(g, f32, dinfo->sm_count, (cudaStream_t)stream, &dinfo->group_attr);
+  g.x_bf16 = X; g.x_ld = ldx; g.x_M = (int)M;
+  for (int i = 0; i < n; ++i) group_add(g, i, nullptr, *P[i], Y[i], ldy[i], M);
+  const cudaError_t e = launch_linear_group(g, f32, dinfo, (cudaStream_t)stream);
   return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? SDQ_OK : SDQ_ERR_CUDA;
 }
 

@@ -60,6 +60,7 @@ struct GroupMat {
 };
 struct GroupParams {
   int n, n_tile, nslot, total_items;   // nslot: inlier ring positions
+  int cluster_log2, rounds, tail_log2; // how the items are dealt out (filled in by launch_linear_group)
   int out_n;             // outliers per S-Vector, the same for every matrix of the call (0 or 1)
   int out_i8;            // the outlier operands are int8 with fp32 scales (else E4M3 with power-of-two scale atoms)
   // activation-resident variant (launch_linear_group with x_bf16 set): all matrices share one bf16 X [x_M][K], which every
@@ -70,12 +71,15 @@ struct GroupParams {
   uint32_t* flags;
   GroupMat m[GROUP_MAX];
 };
-cudaError_t launch_linear_group(GroupParams p, bool f32_out, int sm_count, cudaStream_t stream, uint32_t* attr_done);
+cudaError_t launch_linear_group(GroupParams p, bool f32_out, DeviceInfo* d, cudaStream_t stream);
+double group_kernel_us(int64_t items, int T2, DeviceInfo* d);   // estimated time of a call of `items` row tiles of 256 T2 K, in us
 bool group_xres_fits(int T2, int out_n);   // the activation-resident variant's shared-memory budget for K = 256 T2
 
 // CTA-pair (tcgen05 cta_group::2) many-token kernel (sdq_linear_pair.cu).
 // estimated time of a call in us, to choose between the kernels
 double pair_kernel_us(int64_t M, int64_t N, int64_t K, int out_n, bool b32, bool dense, DeviceInfo* d);
+// clusters of k pairs of CTAs, one CTA per SM, that run at once on the current device: entries 2..4
+const int* pair_max_clusters(DeviceInfo* d);
 cudaError_t launch_linear_pair(LinearParams p, bool f32_out, DeviceInfo* d, cudaStream_t stream);
 
 }  // namespace sdq

@@ -5,8 +5,8 @@
 // layer costs more than the stream itself (set-up, the dependency on the previous grid, the split-K reduction).  Here
 // the work items (layer, 128-row tile) of all layers of the call are dealt out round-robin over one CTA per SM; a CTA
 // runs its items back to back through one shared-memory ring, so the weights of the next item are already landing
-// while the current one is multiplied and stored, and no K split (hence no reduction) is needed once there are about
-// as many row tiles as SMs.
+// while the current one is multiplied and stored.  Items left over after the whole rounds -- or all, when there are fewer than
+// SMs -- have their K range split over the CTAs of a cluster, which add their parts through distributed shared memory.
 //
 // The outlier part is streamed in the form the method states it -- an 8-bit code and a position per S-Vector (the WC
 // section, 1.5 bits per weight) -- not as the 2:4 FP8 container of the many-token kernels (5 bits per weight): sixteen
@@ -24,7 +24,9 @@
 // have.  What a CTA streams is bytes in flight over a position's round trip (copy 1.3 us, build 0.9, multiply, notice); with one
 // ring for everything, released as a whole, that was 2.8 us for eight units, 0.37 us a unit however few CTAs shared the
 // DRAM.  With three rings: 74 row tiles of 64 units 27.5 -> 24.4 us, of 16 units 9.6 -> 7.9; q / k / v of 16 tokens 10.2 ->
-// 9.5, gate / up 16.4 -> 15.0, 32 layers of 4096 x 4096 53.9 -> 50.5.  An mbarrier test costs 15..50 cycles
+// 9.5, gate / up 16.4 -> 15.0, 32 layers of 4096 x 4096 53.9 -> 50.5 (46.4 with the matrix of an item looked for from the last
+// one on instead of from the first).  Left-over items shared by clusters: 74 row tiles of 64 units 24.4 -> 18.0, gate / up
+// 15.0 -> 14.2; one layer 11008 -> 4096 of one token 12.7 (single-layer kernel) -> 10.0.  An mbarrier test costs 15..50 cycles
 // when the phase has completed, a tcgen05 instruction ~40 to issue, but a hand-over between roles (complete -> noticed)
 // several hundred, so every role keeps its trips few and its waits parallel: where a role waits for several barriers,
 // different lanes wait for them at the same time.
@@ -80,14 +82,26 @@ __host__ __device__ inline int group_is_bytes(int n_tile) { return WI_BYTES + n_
 // beside the ring: alternating per item, the outlier row / token scale atoms (SFA_out | SFB_out)
 constexpr int GRP_SIDE_BYTES = 2 * 2 * SF_ATOM_BYTES;
 
-// matrix of work item `item` (items are numbered matrix by matrix)
-__device__ __forceinline__ int group_mat_of(const GroupParams& p, int item) {
-  int i = 0;
-  while (i + 1 < p.n && item >= p.m[i + 1].item0) ++i;
-  return i;
+// A CTA's work is a sequence of segments: whole items dealt round-robin over the CTAs, and at the end, where the items left
+// over are fewer than the CTAs, its part of the K range of one of them.  2^p.cluster_log2 CTAs take 2^p.tail_log2 left-over
+// items (one each without clusters), 2^(cluster_log2 - tail_log2) CTAs per item.
+struct GroupSeg { int item, mat, kb, ke; };                // item, its matrix, its 256-K units [kb, ke)
+// segment i, i rising by one from 0 with s.mat = 0 before the first (items only grow, so the matrix is looked for from the last one on)
+template <bool SPLIT>
+__device__ __forceinline__ bool group_seg(const GroupParams& p, int i, GroupSeg& s) {
+  const int b = (int)blockIdx.x;
+  const bool whole = !SPLIT || i < p.rounds;
+  const int w_log2 = SPLIT ? p.cluster_log2 - p.tail_log2 : 0, r = SPLIT ? b & ((1 << p.cluster_log2) - 1) : 0;
+  s.item = whole ? b + i * (int)gridDim.x : p.rounds * (int)gridDim.x + ((b >> p.cluster_log2) << p.tail_log2) + (r >> w_log2);
+  if ((SPLIT && i > p.rounds) || s.item >= p.total_items) return false;
+  while (s.mat + 1 < p.n && s.item >= p.m[s.mat + 1].item0) ++s.mat;
+  const int T2 = p.m[s.mat].T2, part = r & ((1 << w_log2) - 1);
+  s.kb = whole ? 0 : (part * T2) >> w_log2;
+  s.ke = whole ? T2 : ((part + 1) * T2) >> w_log2;
+  return true;
 }
 
-template <bool F32_OUT, bool XRES>
+template <bool F32_OUT, bool XRES, bool SPLIT>
 __global__ void __launch_bounds__(group_threads(XRES), 1)
 sdq_linear_group_kernel(const __grid_constant__ GroupParams p)
 {
@@ -136,28 +150,30 @@ sdq_linear_group_kernel(const __grid_constant__ GroupParams p)
   __syncthreads();
   ptx::tc_fence_after();
   const uint32_t tmem = *tmem_slot;
-  const int first = (int)blockIdx.x, stride = (int)gridDim.x;
 
   if (XRES && warp != 0 && warp != 10) {
     // ---------------- activation-resident variant: every warp but the producers quantizes the shared X (up to 16 tokens x K)
     // into this CTA's shared memory, in the operand layouts and with the arithmetic of sdq_quantize_act (Section 5, Stage 3:
     // A_i as E2M1 with one scale per 64 K, A_o as E4M3 or int8 per token), while the producers already stream the first
-    // weights.  A warp takes a group of 8 tokens and every 11th Q-Vector, 4 lanes per token as in the quantizer.
+    // weights.  4 lanes per token and Q-Vector as in the quantizer; a warp takes TM tokens (the power of two that holds them
+    // all; two groups of 8 above 8 tokens, half the warps each) and 8 / TM Q-Vectors at a time.
     ptx::griddep_wait();                         // X comes from an earlier kernel
     const uint32_t qw = warp - (warp > 10 ? 2u : 1u);      // 0..21
-    const uint32_t tg = qw & 1u, t = lane >> 2, l = lane & 3;
+    const uint32_t TM = p.x_M > 4 ? 8u : (p.x_M > 2 ? 4u : (uint32_t)p.x_M), groups = p.x_M > 8 ? 2u : 1u;
+    const uint32_t tg = qw % groups, wi = qw / groups, nw = GRP_XQ_WARPS / groups, nq = 8u / TM;
+    const uint32_t t = (lane >> 2) % TM, l = lane & 3, qs = (lane >> 2) / TM;
     const uint32_t mtok = tg * 8 + t;
     const bool live = (int)mtok < p.x_M;
     const __nv_bfloat16* xrow = reinterpret_cast<const __nv_bfloat16*>(p.x_bf16) + (int64_t)mtok * p.x_ld;
     const int NB = p.m[0].T2 * 4;                // Q-Vectors of 64 per token
     // one read of X: a lane keeps its (up to six) 16-element pieces in registers across the maxima's barrier
-    constexpr int XT = 6;                        // Q-Vectors per warp: K <= 4096 -> 64 / 11
+    constexpr int XT = 6;                        // trips per warp: K <= 4096 -> 64 / 11
+    const int b0 = (int)(wi * nq + qs), bs = (int)(nw * nq);   // this lane's Q-Vectors: b0, b0 + bs, ...
     uint4 raw[XT][2];
-    uint32_t qmax[XT];
     uint32_t m2 = 0;
 #pragma unroll
     for (int i = 0; i < XT; ++i) {
-      const int b = (int)(qw >> 1) + i * (GRP_XQ_WARPS / 2);
+      const int b = b0 + i * bs;
       raw[i][0] = raw[i][1] = make_uint4(0, 0, 0, 0);
       if (live && b < NB) {
         const uint4* src = reinterpret_cast<const uint4*>(xrow + (int64_t)b * 64 + l * 16);
@@ -165,35 +181,36 @@ sdq_linear_group_kernel(const __grid_constant__ GroupParams p)
         raw[i][1] = __ldg(src + 1);
       }
     }
-#pragma unroll
-    for (int i = 0; i < XT; ++i) {
+    // largest magnitude bits of piece i; > 0x7F7F: it holds an infinity (counts as the largest finite bf16)
+    auto largest = [&](int i) {
       const uint32_t r[8] = {raw[i][0].x, raw[i][0].y, raw[i][0].z, raw[i][0].w, raw[i][1].x, raw[i][1].y, raw[i][1].z, raw[i][1].w};
       uint32_t q = 0;
 #pragma unroll
       for (int j = 0; j < 8; ++j) q = __vmaxu2(q, r[j] & 0x7FFF7FFFu);
-      q = max(q & 0xFFFFu, q >> 16);             // > 0x7F7F: the lane holds an infinity (counts as the largest finite bf16)
-      qmax[i] = q;
-      m2 = max(m2, min(q, 0x7F7Fu));
-    }
+      return max(q & 0xFFFFu, q >> 16);
+    };
+#pragma unroll
+    for (int i = 0; i < XT; ++i) m2 = max(m2, min(largest(i), 0x7F7Fu));
     float amax = __uint_as_float(m2 << 16);
     amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, 1));
     amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, 2));
-    if (l == 0) x_part[qw * 8 + t] = amax;
+    for (uint32_t d = 4 * TM; d < 32; d *= 2) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, d));
+    if (l == 0 && qs == 0) x_part[qw * 8 + t] = amax;
     ptx::named_bar_sync(8, GRP_XQ_WARPS * 32);
     float ramax = 0.0f;
-    for (uint32_t q2 = 0; q2 < GRP_XQ_WARPS / 2; ++q2) ramax = fmaxf(ramax, x_part[(2 * q2 + tg) * 8 + t]);
+    for (uint32_t q2 = 0; q2 < nw; ++q2) ramax = fmaxf(ramax, x_part[(groups * q2 + tg) * 8 + t]);
     const int e = fp8_scale_exp(ramax);
     const float s8 = pow2_neg(e), sx = int8_scale(ramax);
     const Int8Coder k8 = int8_coder(sx);
     const bool i8 = p.out_i8 != 0;
-    if (qw < 2 && l == 0) {
+    if (wi == 0 && l == 0 && qs == 0) {
       x_sx[mtok] = sx;
       *reinterpret_cast<uint32_t*>(x_sfb + sf_off(mtok, 0)) = (uint32_t)((i8 || !live) ? 127 : e + 127) * 0x01010101u;
     }
 #pragma unroll
     for (int i = 0; i < XT; ++i) {
-      const int b = (int)(qw >> 1) + i * (GRP_XQ_WARPS / 2);     // uniform over the warp
-      if (b >= NB) break;
+      const int b = b0 + i * bs;
+      if (b - (int)qs >= NB) break;               // uniform over the warp
       const uint32_t r[8] = {raw[i][0].x, raw[i][0].y, raw[i][0].z, raw[i][0].w, raw[i][1].x, raw[i][1].y, raw[i][1].z, raw[i][1].w};
       float v[16];
 #pragma unroll
@@ -201,21 +218,29 @@ sdq_linear_group_kernel(const __grid_constant__ GroupParams p)
         v[2 * j] = __uint_as_float(r[j] << 16);
         v[2 * j + 1] = __uint_as_float(r[j] & 0xFFFF0000u);
       }
-      if (qmax[i] > 0x7F7Fu) {
+      const uint32_t qmax = largest(i);
+      if (qmax > 0x7F7Fu) {
 #pragma unroll
         for (int j = 0; j < 16; ++j) v[j] = sat(v[j]);
       }
-      uint32_t bm = min(qmax[i], 0x7F7Fu);
+      uint32_t bm = min(qmax, 0x7F7Fu);
       bm = max(bm, __shfl_xor_sync(0xffffffffu, bm, 1));
       bm = max(bm, __shfl_xor_sync(0xffffffffu, bm, 2));
-      const uint32_t c = e8m0_scale_code(__uint_as_float(bm << 16), p.scale_rule);
+      const uint32_t c = e8m0_scale_code_bf16(bm, p.scale_rule == SDQ_SCALE_CEIL_NOSAT);
       const float s4 = pow2_inv_e8m0(c);
       uint32_t q4[2] = {0, 0}, q8[4] = {0, 0, 0, 0};
 #pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        float f[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) f[j] = v[8 * h + j] * s4;
+        q4[h] = e2m1x8(f);
+      }
+#pragma unroll
       for (int j = 0; j < 8; ++j) {
-        q4[j >> 2] |= e2m1x2(v[2 * j] * s4, v[2 * j + 1] * s4) << (8 * (j & 3));
         q8[j >> 1] |= (i8 ? (int8_code(v[2 * j], k8) | (int8_code(v[2 * j + 1], k8) << 8)) : e4m3x2(v[2 * j] * s8, v[2 * j + 1] * s8)) << (16 * (j & 1));
       }
+      if (!live || b >= NB) continue;             // (what the other columns of the product hold is not stored)
       const uint32_t k = (uint32_t)b * 64 + l * 16;          // first element of this lane
       uint8_t* xu = xres + (size_t)(k >> 8) * GRP_XU;
       *reinterpret_cast<uint2*>(xu + b_off(mtok, (k & 255) >> 1)) = make_uint2(q4[0], q4[1]);
@@ -237,36 +262,41 @@ sdq_linear_group_kernel(const __grid_constant__ GroupParams p)
     const uint32_t copies = inl ? (XRES ? (p.out_n && !p.out_i8 ? 2u : 1u) : 3u) : (wc ? 1u : 2u);
     if (c < copies && (inl || p.out_n)) {
       bool ok = true;
-      int item = first, k2 = (int)l;             // this lane's position: work item and 256-K unit inside the item
-      int mat = -1, rt = 0, T2 = 0;
-      uint32_t iseq = 0;                         // number of the item in this CTA's sequence
+      GroupSeg sg;                               // this lane's position: segment, unit counted from the segment's start
+      int iseq = 0, k = (int)l, k2 = 0, rt = 0;  // ... as work item: 256-K unit, row tile
+      bool have = false;
+      sg.mat = 0;
       const uint32_t N = inl ? NI : NU;
       uint64_t* freed = inl ? done_i : (wc ? free_wc : done_o);
       uint32_t v = l, wrapped = 0, ph = 0;       // ring position, whether the ring has wrapped, parity of `freed` to wait for
       uint32_t ahead = 0;                        // units whose weights were fetched ahead of the wait below
-      // advances to the item that holds unit k2; false at the end of the sequence
+      // advances to the segment that holds unit k; false at the end of the sequence
       auto seek = [&]() {
         for (;;) {
-          if (item >= p.total_items) return false;
-          if (mat < 0) { mat = group_mat_of(p, item); rt = item - p.m[mat].item0; T2 = p.m[mat].T2; }
-          if (k2 < T2) return true;
-          k2 -= T2; item += stride; mat = -1; ++iseq;
+          if (!have) {
+            if (!group_seg<SPLIT>(p, iseq, sg)) return false;
+            rt = sg.item - p.m[sg.mat].item0;
+            have = true;
+          }
+          k2 = sg.kb + k;
+          if (k2 < sg.ke) return true;
+          k = k2 - sg.ke; ++iseq; have = false;
         }
       };
       if (!XRES && !wc) {
         // activations come from an earlier kernel; the first lap's inlier weights are fetched before the wait for it
         if (inl && c == 0) {
-          for (uint32_t u = l; u < NI && seek(); u += 2, k2 += 2, ++ahead) {
-            const GroupMat& m = p.m[mat];
+          for (uint32_t u = l; u < NI && seek(); u += 2, k += 2, ++ahead) {
+            const GroupMat& m = p.m[sg.mat];
             ptx::mbar_expect_tx(&full_is[u], WI_BYTES + xb + SF_ATOM_BYTES);
             ptx::bulk_g2s(sm + (size_t)u * isb, m.w + m.wi + ((size_t)rt * m.T2 + k2) * WI_BYTES, WI_BYTES, &full_is[u]);
           }
-          item = first; k2 = (int)l; mat = -1; iseq = 0;
+          k = (int)l; iseq = 0; have = false; sg.mat = 0;
         }
         ptx::griddep_wait();
       }
       while (seek()) {
-        const GroupMat& m = p.m[mat];
+        const GroupMat& m = p.m[sg.mat];
         if (wrapped && !(ok = ptx::mbar_wait(&freed[v], ph ^ 1))) break;
         if (inl) {
           uint8_t* st = sm + (size_t)v * isb;
@@ -275,7 +305,7 @@ sdq_linear_group_kernel(const __grid_constant__ GroupParams p)
             if (c == 0) {
               ptx::mbar_expect_tx(&full_is[v], WI_BYTES);
               ptx::bulk_g2s(st, wi, WI_BYTES, &full_is[v]);
-            } else if (k2 == 0) {                // (see warp 24; the tokens' atom is resident)
+            } else if (k2 == sg.kb) {            // (see warp 24; the tokens' atom is resident)
               const uint32_t sb = iseq & 1;
               if (iseq >= 2 && !(ok = ptx::mbar_wait(&acc_full[sb], ((iseq >> 1) - 1) & 1))) break;
               ptx::mbar_expect_tx(&sf_full[sb], SF_ATOM_BYTES);
@@ -296,7 +326,7 @@ sdq_linear_group_kernel(const __grid_constant__ GroupParams p)
           const uint8_t* xo = m.x + m.xo + (size_t)(2 * k2 + (int)c) * XO_BYTES;
           if (c == 0) ptx::mbar_expect_tx(&full_x8[v], 2 * xb);
           ptx::bulk_g2s(x8_ring + (size_t)v * 2 * xb + c * xb, xo, xb, &full_x8[v]);
-          if (k2 == 0 && !p.out_i8) {            // (int8 outliers take fp32 scales in the epilogue: no scale atoms)
+          if (k2 == sg.kb && !p.out_i8) {        // (int8 outliers take fp32 scales in the epilogue: no scale atoms)
             // the item's outlier scale atoms (lane c = 0: of the weight rows, c = 1: of the tokens): a buffer and a barrier
             // of their own per item parity.  The buffer is free once every MMA of the item two back has completed (`acc_full`
             // of that item: it cannot complete again before these atoms land, since the next item on that accumulator needs
@@ -308,7 +338,7 @@ sdq_linear_group_kernel(const __grid_constant__ GroupParams p)
                           SF_ATOM_BYTES, &sf_full[sb]);
           }
         }
-        k2 += 2;
+        k += 2;
         v += 2;
         if (v >= N) { v -= N; wrapped = 1; ph ^= 1; }
       }
@@ -330,24 +360,26 @@ sdq_linear_group_kernel(const __grid_constant__ GroupParams p)
       const uint32_t id8 = p.out_i8 ? ptx::idesc_i8(128, (uint32_t)p.n_tile, true) : ptx::idesc_block_scaled(128, (uint32_t)p.n_tile, 0, true, 0, 0);
       const uint32_t N = outw ? NU : NI;
       uint32_t v = 0, ph = 0, itc = 0;             // ring position and its lap parity, item count
-      for (int item = first; item < p.total_items && ok; item += stride, ++itc) {
-        const int T2 = p.m[group_mat_of(p, item)].T2;
+      GroupSeg sg;
+      sg.mat = 0;
+      for (; ok && group_seg<SPLIT>(p, (int)itc, sg); ++itc) {
+        const int kb = sg.kb, ke = sg.ke;
         const uint32_t ab = itc & 1, acc_col = tmem + GRP_TM_ACC + 64u * ab + (outw ? 32u : 0u), so = tmem + GRP_TM_SO + 8u * ab;
         if (itc >= 2) {    // the epilogue has read this accumulator pair's previous item
           ok = __all_sync(0xffffffffu, ptx::mbar_wait(&acc_empty[ab], ((itc >> 1) - 1) & 1));
           if (!ok) break;
         }
-        for (int k2 = 0; k2 < T2 && ok;) {
+        for (int k2 = kb; k2 < ke && ok;) {
           // Up to four units of the item per trip: lane i tests unit k2 + i (for the outlier product: lane i its containers,
           // lane 8 + i the tokens' 8-bit codes), lane 4 the item's scale
           // atoms; the units ready in a row from k2 on are issued together.  A trip costs several hundred cycles beside the
           // instructions it issues (test, vote, fence, election, reconvergence), so taking what is ready in one trip keeps
           // the issuer ahead whenever it has fallen behind.  With nothing ready it waits for unit k2 and votes again.
-          const int nb = T2 - k2 < 4 ? T2 - k2 : 4;
+          const int nb = ke - k2 < 4 ? ke - k2 : 4;
           const uint32_t i = lane & 3;
           uint32_t vi = v + i, phi = ph;
           if (vi >= N) { vi -= N; phi ^= 1; }
-          const bool sf_lane = outw && k2 == 0 && lane == 4 && !p.out_i8, x_lane = outw && !XRES && (lane >> 2) == 2;
+          const bool sf_lane = outw && k2 == kb && lane == 4 && !p.out_i8, x_lane = outw && !XRES && (lane >> 2) == 2;
           uint64_t* bar = sf_lane ? &sf_full[ab] : (x_lane ? &full_x8[vi] : (outw ? &built[vi] : &full_is[vi]));
           const uint32_t par = sf_lane ? ((itc >> 1) & 1) : phi;
           const bool mine = ((lane < 4 || x_lane) && (int)i < nb) || sf_lane;
@@ -375,11 +407,11 @@ sdq_linear_group_kernel(const __grid_constant__ GroupParams p)
                 ptx::tc_cp_32x128b_warpx4(mb + 4, ptx::smem_desc(sb + A_IN_BYTES + E_IN_BYTES, 0, 128));
                 ptx::tc_cp_32x128b_warpx4(mb + 8, ptx::smem_desc(sf4, 0, 128));
                 ptx::mma_sp_mxf4(acc_col, ptx::smem_desc(sb, 128, 256), ptx::smem_desc(b4, 128, 1024), id4[0], mb, mb + 4, mb + 8,
-                                 kk ? 1u : 0u);
+                                 kk != kb ? 1u : 0u);
                 ptx::mma_sp_mxf4(acc_col, ptx::smem_desc(sb + 4096, 128, 256), ptx::smem_desc(b4 + 512, 128, 1024), id4[1], mb + 2,
                                  mb + 4, mb + 8, 1u);
               } else {
-                if (kk == 0 && !p.out_i8) {
+                if (kk == kb && !p.out_i8) {
                   const uint32_t sf = ptx::smem_u32(sfbuf) + ab * 2 * SF_ATOM_BYTES;
                   ptx::tc_cp_32x128b_warpx4(so, ptx::smem_desc(sf, 0, 128));
                   ptx::tc_cp_32x128b_warpx4(so + 4, ptx::smem_desc(XRES ? ptx::smem_u32(x_sfb) : sf + SF_ATOM_BYTES, 0, 128));
@@ -389,16 +421,16 @@ sdq_linear_group_kernel(const __grid_constant__ GroupParams p)
                   const uint32_t ca = tmem + GRP_TM_C + GRP_TM_C_COLS * vv + 16u * h, eb = tmem + GRP_TM_C + GRP_TM_C_COLS * vv + 32u + 4u * h;
                   const uint32_t xa = XRES ? xu + 16 * 128 + SF_ATOM_BYTES + h * 16 * 128 : ptx::smem_u32(x8_ring) + vv * 2 * xb + h * xb;
                   if (p.out_i8) {     // the same containers and token codes as integers, int32 accumulator
-                    ptx::mma_sp_i8_ta(acc_col, ca, ptx::smem_desc(xa, 128, 1024), id8, eb, (kk | (int)h) ? 1u : 0u);
+                    ptx::mma_sp_i8_ta(acc_col, ca, ptx::smem_desc(xa, 128, 1024), id8, eb, (kk != kb || h) ? 1u : 0u);
                     ptx::mma_sp_i8_ta(acc_col, ca + 8, ptx::smem_desc(xa + 512, 128, 1024), id8, eb + 2, 1u);
                   } else {
-                    ptx::mma_sp_mxf8_ta(acc_col, ca, ptx::smem_desc(xa, 128, 1024), id8, eb, so, so + 4, (kk | (int)h) ? 1u : 0u);
+                    ptx::mma_sp_mxf8_ta(acc_col, ca, ptx::smem_desc(xa, 128, 1024), id8, eb, so, so + 4, (kk != kb || h) ? 1u : 0u);
                     ptx::mma_sp_mxf8_ta(acc_col, ca + 8, ptx::smem_desc(xa + 512, 128, 1024), id8, eb + 2, so, so + 4, 1u);
                   }
                 }
               }
               ptx::tc_commit(outw ? &done_o[vv] : &done_i[vv]);
-              if (kk == T2 - 1) ptx::tc_commit(&acc_full[ab]);
+              if (kk == ke - 1) ptx::tc_commit(&acc_full[ab]);
               if (++vv == N) vv = 0;
             }
           }
@@ -416,10 +448,12 @@ sdq_linear_group_kernel(const __grid_constant__ GroupParams p)
     bool ok = true;
     uint32_t itc = 0;
     ptx::griddep_wait();                   // Y may still be in use by the previous kernel
-    for (int item = first; item < p.total_items && ok; item += stride, ++itc) {
-      const int mat = group_mat_of(p, item);
-      const GroupMat& m = p.m[mat];
-      const int64_t n0 = (int64_t)(item - m.item0) * TILE_ROWS;
+    GroupSeg sg;
+    sg.mat = 0;
+    for (; ok && group_seg<SPLIT>(p, (int)itc, sg); ++itc) {
+      const GroupMat& m = p.m[sg.mat];
+      const int64_t n0 = (int64_t)(sg.item - m.item0) * TILE_ROWS;
+      const bool split = SPLIT && sg.ke - sg.kb < m.T2;      // a part of a left-over item: the last segment
       const uint32_t ab = itc & 1;
       // one thread polls the barrier and releases the other 127 through a hardware barrier: many threads polling an mbarrier
       // slow every other barrier operation of the CTA down
@@ -443,7 +477,11 @@ sdq_linear_group_kernel(const __grid_constant__ GroupParams p)
             ptx::tmem_ld_wait();
 #pragma unroll
             for (int i = 0; i < 16; ++i) val[c + i] = p.out_n ? __float_as_uint(__uint_as_float(a[i]) + __uint_as_float(b[i])) : a[i];
-            if (p.out_i8) {      // b holds exact int32 sums: scale them, tokens that exist only
+            if (split && p.out_i8) {     // the parts' sums are added as integers, then scaled
+              int* pb = reinterpret_cast<int*>(sm + 32 * TILE_ROWS * 4);
+#pragma unroll
+              for (int i = 0; i < 16; ++i) { val[c + i] = a[i]; pb[(c + i) * TILE_ROWS + qd * 32 + lane] = (int)b[i]; }
+            } else if (p.out_i8) {      // b holds exact int32 sums: scale them, tokens that exist only
 #pragma unroll
               for (int i = 0; i < 16; ++i) {
                 const float o = (int)(c + i) < m.M ? (float)(int)b[i] * (sw * (XRES ? x_sx[c + i] : __ldg(sxp + c + i))) : 0.0f;
@@ -459,6 +497,13 @@ sdq_linear_group_kernel(const __grid_constant__ GroupParams p)
       ptx::tc_fence_before();
       __syncwarp();
       if (lane == 0) ptx::mbar_arrive(&acc_empty[ab]);
+      if (split) {       // to shared memory, where the rings are idle by now
+        float* pa = reinterpret_cast<float*>(sm);
+#pragma unroll
+        for (int t = 0; t < 32; ++t)
+          if (t < m.M) pa[t * TILE_ROWS + qd * 32 + lane] = __uint_as_float(val[t]);
+        continue;
+      }
 #pragma unroll
       for (int t = 0; t < 32; ++t) {
         if (t < m.M) {
@@ -488,9 +533,10 @@ sdq_linear_group_kernel(const __grid_constant__ GroupParams p)
     bool ok = true;
     uint32_t v = 0, ph = 0, lap = 0;             // position of the unit in the ring, lap parity, whether the ring has wrapped
     const uint32_t tlane = tmem + (((warp & 3) * 32u) << 16) + GRP_TM_C;
-    for (int item = first; item < p.total_items && ok; item += stride) {
-      const int T2 = p.m[group_mat_of(p, item)].T2;
-      for (int k2 = 0; k2 < T2; ++k2) {
+    GroupSeg sg;
+    sg.mat = 0;
+    for (int iseq = 0; ok && group_seg<SPLIT>(p, iseq, sg); ++iseq) {
+      for (int k2 = sg.kb; k2 < sg.ke; ++k2) {
         if ((v & (GRP_BUILDERS - 1)) == grp) {
           // Only ONE thread of the group waits on the mbarrier and then releases the others through a hardware barrier: with
           // every warp waiting on the same mbarrier some of them noticed its completion more than a microsecond late.
@@ -545,6 +591,48 @@ sdq_linear_group_kernel(const __grid_constant__ GroupParams p)
   ptx::tc_fence_before();
   __syncthreads();
   if (warp == 1) ptx::tmem_dealloc(tmem, GRP_TMEM_COLS);
+  if constexpr (SPLIT) {
+    // ---------------- left-over items: every CTA adds its share of the item's rows over the parts, in order
+    ptx::cluster_sync();                           // the parts are in shared memory
+    GroupSeg sg;
+    sg.mat = 0;
+    const uint32_t w_log2 = (uint32_t)(p.cluster_log2 - p.tail_log2), tail_w = 1u << w_log2;   // CTAs per left-over item
+    if (group_seg<SPLIT>(p, p.rounds, sg)) {
+      const GroupMat& m = p.m[sg.mat];
+      const uint32_t rank = ptx::cluster_ctarank(), part = rank & (tail_w - 1u), r0 = rank - part;
+      const uint32_t q_per = 32u >> w_log2, q_begin = part * q_per;      // quads of rows
+      const uint32_t local = ptx::smem_u32(sm);
+      const int64_t n0 = (int64_t)(sg.item - m.item0) * TILE_ROWS;
+      for (uint32_t idx = tid; idx < q_per * (uint32_t)m.M; idx += blockDim.x) {
+        const uint32_t t = idx >> (5 - w_log2), row = (q_begin + (idx & (q_per - 1u))) << 2, off = (t * TILE_ROWS + row) * 4;
+        float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+        int4 b = make_int4(0, 0, 0, 0);
+        for (uint32_t i = 0; i < tail_w; ++i) {
+          const uint32_t peer = ptx::mapa_u32(local, r0 + i) + off;
+          const float4 v = ptx::ld_cluster_f32x4(peer);
+          a.x += v.x; a.y += v.y; a.z += v.z; a.w += v.w;
+          if (p.out_i8) {
+            const float4 w = ptx::ld_cluster_f32x4(peer + 32 * TILE_ROWS * 4);
+            b.x += __float_as_int(w.x); b.y += __float_as_int(w.y); b.z += __float_as_int(w.z); b.w += __float_as_int(w.w);
+          }
+        }
+        if (p.out_i8) {
+          const float4 sw = __ldg(reinterpret_cast<const float4*>(m.w + m.wsc) + (n0 + row) / 4);
+          const float sx = XRES ? x_sx[t] : __ldg(reinterpret_cast<const float*>(m.x + m.xsc) + t);
+          a.x += (float)b.x * (sw.x * sx); a.y += (float)b.y * (sw.y * sx); a.z += (float)b.z * (sw.z * sx); a.w += (float)b.w * (sw.w * sx);
+        }
+        const int64_t at = (int64_t)t * m.ldy + n0 + row;
+        if (F32_OUT) {
+          *reinterpret_cast<float4*>(reinterpret_cast<float*>(m.Y) + at) = a;
+        } else {
+          const __nv_bfloat162 lo = __floats2bfloat162_rn(a.x, a.y), hi = __floats2bfloat162_rn(a.z, a.w);
+          *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(m.Y) + at) =
+              make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
+        }
+      }
+    }
+    ptx::cluster_sync();                           // nobody leaves while its parts may still be read
+  }
 }
 
 // inlier ring positions for `n_tile` tokens per tile (an even number, as many as fit beside the outlier rings)
@@ -557,8 +645,48 @@ static int group_units(int n_tile, int out_n, int xres_bytes) {
 // shared-memory budget of the activation-resident variant: do at least six inlier slots fit beside X of K / 256 = T2 units?
 bool group_xres_fits(int T2, int out_n) { return group_units(16, out_n, group_xres_bytes(T2)) >= 6; }
 
-cudaError_t launch_linear_group(GroupParams p, bool f32_out, int sm_count, cudaStream_t stream, uint32_t* attr_done)
+// How the items are dealt out: clusters of 1, 2 or 4 CTAs, whole rounds of items, left-over items per cluster.  Times in us,
+// fitted to measurements (74 to 1024 items of 4 to 64 units): 3.5 for the launch, 0.28 a unit or 0.42 with every SM
+// pulling from DRAM, 2.3 for the clusters and adding the parts.
+struct GroupPlan { int cluster, ctas, rounds, tail_items; double us; };
+static GroupPlan group_plan(int64_t items, int T2, int T2_min, int sm_count, const int* max_clusters)
 {
+  GroupPlan best;
+  best.us = -1.0;
+  for (int c = 1; c <= 4; c *= 2) {
+    const int64_t C = c == 1 ? sm_count : (c == 2 ? sm_count / 2 : max_clusters[2]);   // clusters that run at once
+    if (C <= 0) continue;
+    GroupPlan q;
+    q.cluster = c;
+    q.rounds = (int)(items / (C * c));
+    const int64_t left = items - q.rounds * C * c;
+    q.tail_items = c;
+    while (q.tail_items > 1 && left <= C * (q.tail_items / 2) && c / (q.tail_items / 2) <= T2_min) q.tail_items /= 2;
+    const int w = c / q.tail_items;
+    if (c > 1 && w == 1) continue;                      // nothing is split: clusters only cost
+    q.ctas = (int)(q.rounds ? C * c : (left + q.tail_items - 1) / q.tail_items * c);
+    const double unit = 0.42 * q.ctas / sm_count > 0.28 ? 0.42 * q.ctas / sm_count : 0.28;
+    const int64_t tail_ctas = left * w;
+    const double tail_unit = 0.42 * tail_ctas / sm_count > 0.28 ? 0.42 * tail_ctas / sm_count : 0.28;
+    q.us = 3.5 + q.rounds * T2 * unit + (left ? (double)((T2 + w - 1) / w) * tail_unit : 0.0) + (w > 1 ? 2.3 : 0.0);
+    if (best.us < 0 || q.us < best.us) best = q;
+  }
+  return best;
+}
+double group_kernel_us(int64_t items, int T2, DeviceInfo* d) { return group_plan(items, T2, T2, d->sm_count, pair_max_clusters(d)).us; }
+
+cudaError_t launch_linear_group(GroupParams p, bool f32_out, DeviceInfo* d, cudaStream_t stream)
+{
+  uint32_t* attr_done = &d->group_attr;
+  int T2_min = p.m[0].T2;
+  int64_t units = 0;
+  for (int i = 0; i < p.n; ++i) {
+    T2_min = p.m[i].T2 < T2_min ? p.m[i].T2 : T2_min;
+    units += (int64_t)((i + 1 < p.n ? p.m[i + 1].item0 : p.total_items) - p.m[i].item0) * p.m[i].T2;
+  }
+  const GroupPlan plan = group_plan(p.total_items, (int)((units + p.total_items - 1) / p.total_items), T2_min, d->sm_count, pair_max_clusters(d));
+  auto log2 = [](int v) { return v == 4 ? 2 : v - 1; };
+  p.cluster_log2 = log2(plan.cluster); p.tail_log2 = log2(plan.tail_items); p.rounds = plan.rounds;
   const bool xres = p.x_bf16 != nullptr;
   const int xbytes = xres ? group_xres_bytes(p.m[0].T2) : 0;
   const int is = xres ? WI_BYTES : group_is_bytes(p.n_tile), os = p.out_n ? 2 * wc_bytes(1) + (xres ? 0 : 2 * p.n_tile * 128) : 0;
@@ -566,25 +694,37 @@ cudaError_t launch_linear_group(GroupParams p, bool f32_out, int sm_count, cudaS
   const int smem = p.nslot * is + GRP_UNITS * os + xbytes + (p.out_n ? GRP_SIDE_BYTES : 0) + GRP_BAR_BYTES + 128;
   if (!*attr_done) {
     const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    if (cudaFuncSetAttribute(sdq_linear_group_kernel<false, false>, a, 232448) != cudaSuccess ||
-        cudaFuncSetAttribute(sdq_linear_group_kernel<true, false>, a, 232448) != cudaSuccess ||
-        cudaFuncSetAttribute(sdq_linear_group_kernel<false, true>, a, 232448) != cudaSuccess ||
-        cudaFuncSetAttribute(sdq_linear_group_kernel<true, true>, a, 232448) != cudaSuccess)
+    bool ok = true;
+    auto set = [&](auto kern) { ok = ok && cudaFuncSetAttribute(kern, a, 232448) == cudaSuccess; };
+    set(sdq_linear_group_kernel<false, false, false>); set(sdq_linear_group_kernel<true, false, false>);
+    set(sdq_linear_group_kernel<false, true, false>); set(sdq_linear_group_kernel<true, true, false>);
+    set(sdq_linear_group_kernel<false, false, true>); set(sdq_linear_group_kernel<true, false, true>);
+    set(sdq_linear_group_kernel<false, true, true>); set(sdq_linear_group_kernel<true, true, true>);
+    if (!ok)
       return cudaErrorUnknown;
     *attr_done = 1;
   }
   cudaLaunchConfig_t lc = {};
-  lc.gridDim = dim3((unsigned)(p.total_items < sm_count ? p.total_items : sm_count));
+  lc.gridDim = dim3((unsigned)plan.ctas);
   lc.blockDim = dim3((unsigned)group_threads(xres));
   lc.dynamicSmemBytes = (size_t)smem;
   lc.stream = stream;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = (unsigned)plan.cluster;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
   lc.attrs = attr;
-  lc.numAttrs = 1;
-  if (xres) return f32_out ? cudaLaunchKernelEx(&lc, sdq_linear_group_kernel<true, true>, p) : cudaLaunchKernelEx(&lc, sdq_linear_group_kernel<false, true>, p);
-  return f32_out ? cudaLaunchKernelEx(&lc, sdq_linear_group_kernel<true, false>, p) : cudaLaunchKernelEx(&lc, sdq_linear_group_kernel<false, false>, p);
+  lc.numAttrs = plan.cluster > 1 ? 2 : 1;
+  auto go = [&](auto kern) { return cudaLaunchKernelEx(&lc, kern, p); };
+  if (plan.cluster > 1) {      // (without left-over items to share the kernel carries no cluster code: 0.6 us a launch)
+    if (xres) return f32_out ? go(sdq_linear_group_kernel<true, true, true>) : go(sdq_linear_group_kernel<false, true, true>);
+    return f32_out ? go(sdq_linear_group_kernel<true, false, true>) : go(sdq_linear_group_kernel<false, false, true>);
+  }
+  if (xres) return f32_out ? go(sdq_linear_group_kernel<true, true, false>) : go(sdq_linear_group_kernel<false, true, false>);
+  return f32_out ? go(sdq_linear_group_kernel<true, false, false>) : go(sdq_linear_group_kernel<false, false, false>);
 }
 
 }  // namespace sdq

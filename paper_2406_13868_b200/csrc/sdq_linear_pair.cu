@@ -613,7 +613,7 @@ static PairPlan pair_best(int64_t M, int64_t N, int64_t K, int out_n, bool b32, 
 }
 
 // largest grids, in clusters of 4, 6 and 8 CTAs with one CTA per SM, that run at once on the current device: [pairs per cluster]
-static const int* pair_max_clusters(DeviceInfo* d)
+const int* pair_max_clusters(DeviceInfo* d)
 {
   if (!d->pair_clusters[1]) {
     auto kern = sdq_linear_pair_kernel<false, false, false, PAIR_FLEX>;

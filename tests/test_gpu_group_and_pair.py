@@ -72,6 +72,38 @@ def test_group_call_matches_oracle(shapes, Ms, out_n, share_x):
             assert (d <= tol).all()
 
 
+@pytest.mark.parametrize("shapes,M,cfg_args", [
+    ([(9600, 1024)], 3, (1, so.GRAN_PAIR, 64, 0)),                       # one item each for 75 CTAs: nothing to split
+    ([(11008, 1024), (8192, 1536)], 16, (1, so.GRAN_PAIR, 64, 0)),       # 150 items: a round and two left over, K differs
+    ([(4352, 1280)] * 5, 20, (1, so.GRAN_PAIR, 64, 0)),                  # 170 items of five units: uneven parts, 32-token tile
+    ([(11008, 1024), (8192, 1024)], 5, (1, so.GRAN_PAIR, 64, 0, 0, 1)),  # int8: the parts are added as integers
+    ([(11008, 1024), (8448, 1024)], 7, (0, so.GRAN_PAIR, 64, 0)),        # no outlier part
+])
+def test_group_items_left_over_after_whole_rounds(shapes, M, cfg_args):
+    """left-over items share a cluster's CTAs along K: every layer's last row tiles and a few others against the oracle, the
+    fused-quantizer call bit for bit"""
+    m, cfg, Ws, Xs, ps, xqs = _layers(shapes, [M] * len(shapes), cfg_args, 4300)
+    y32, y16 = m.sdq_linear_group(xqs, ps, f32=True), m.sdq_linear_group(xqs, ps)
+    assert m.device_status() == 0
+    oc = so.Config(*cfg_args)
+    for W, X, a, b in zip(Ws, Xs, y32, y16):
+        rows = sorted({r for r in [0, 1, 127, 128, W.shape[0] // 2 + 5, W.shape[0] - 129, W.shape[0] - 128, W.shape[0] - 97, W.shape[0] - 1]})
+        yref = so.linear(so.quantize_act(sdq_synth.bf16_bits(X), oc), so.decompose(sdq_synth.bf16_bits(W[rows]), oc))
+        d, tol = y_close(a[:, rows].cpu().numpy(), yref)
+        assert (d <= tol).all(), (d.max(), (d / tol).max())
+        assert torch.equal(b, a.to(torch.bfloat16))
+    if len({k for _, k in shapes}) == 1 and M <= 16:
+        xq = m.sdq_quantize_act(Xs[0].cuda(), cfg)
+        for a, b in zip(m.sdq_linear_group_x(Xs[0].cuda(), ps), m.sdq_linear_group([xq] * len(ps), ps)):
+            assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("M,N,K,out_n", [(1, 4096, 4096, 1), (17, 4224, 1024, 1), (32, 8448, 2048, 1), (3, 128, 1280, 1), (9, 16640, 1024, 0)])
+def test_single_layers_on_the_grouped_kernel(M, N, K, out_n):
+    """few-token calls that the grouped kernel takes: one, two and four CTAs per row tile, a tile count just above the clusters"""
+    run_case(M, N, K, 4400 + M, out_n=out_n, check_rows=None if N <= 4224 else (N - 256, N))
+
+
 def test_group_call_runs_twice_in_a_row_and_inside_a_graph():
     cfg_args = (1, so.GRAN_PAIR, 64, 0)
     m, cfg, Ws, Xs, ps, xqs = _layers([(4096, 1024)] * 4, [9] * 4, cfg_args, 4300)
