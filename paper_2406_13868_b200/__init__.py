@@ -125,7 +125,7 @@ def _native():
         loader = importlib.machinery.ExtensionFileLoader("_binding", BINDING)
         mod = importlib.util.module_from_spec(importlib.util.spec_from_loader("_binding", loader))
         loader.exec_module(mod)
-        mod.bind(_Act, _Packed, Config, QuantAct, SdqError)
+        mod.bind(_Act, _Packed, Config, QuantAct, PackedWeight, SdqError)
         _fast = mod
     return _fast
 
@@ -181,6 +181,9 @@ def sdq_decompose(W: torch.Tensor, cfg: Config | None = None, buf: torch.Tensor 
     """W [N, K] bf16 CUDA tensor -> packed inlier/outlier parts (sdq_decompose of the C-ABI; with col_weight [K] fp32,
     sdq_decompose_metric: selections rank by the weight-activation product |w| * col_weight[k])."""
     cfg = cfg or Config()
+    p = (_fast or _native()).decompose(W, cfg, buf, col_weight)
+    if p is not None:
+        return p
     _need_cuda(W, "W")
     assert W.dtype == torch.bfloat16 and W.dim() == 2 and W.stride(1) == 1
     N, K = W.shape
@@ -213,6 +216,9 @@ def packed_attach(buf: torch.Tensor) -> PackedWeight:
 def packed_compact(p: PackedWeight) -> PackedWeight:
     """The packed matrix without its 2:4 outlier containers (4.2 instead of 9.1 bits per weight): the form the grouped
     few-token calls stream.  Returns a new PackedWeight in its own buffer (see sdq_packed_compact in include/sdq.h)."""
+    q = (_fast or _native()).compact(p)
+    if q is not None:
+        return q
     n = ctypes.c_size_t(0)
     _check(lib().sdq_packed_compact_size(ctypes.c_int64(p.N), ctypes.c_int64(p.K), ctypes.byref(p.cfg), ctypes.byref(n)), "sdq_packed_compact_size")
     buf = torch.empty(int(n.value), dtype=torch.uint8, device=p.buf.device)
@@ -230,6 +236,9 @@ def diag_wait_timeout(polls: int = 64) -> None:
 def channel_norm(X: torch.Tensor) -> torch.Tensor:
     """X [M, K] bf16 CUDA tensor -> fp32 [K]: Euclidean norm of every input channel over the tokens
     (the per-channel weight of the product metric)."""
+    c = (_fast or _native()).channel_norm(X)
+    if c is not None:
+        return c
     _need_cuda(X, "X")
     assert X.dtype == torch.bfloat16 and X.dim() == 2 and X.stride(1) == 1
     M, K = X.shape

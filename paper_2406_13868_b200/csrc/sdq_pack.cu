@@ -1,17 +1,19 @@
 // Offline weight decomposition + packing (Section 5, Stage 2 -> Stage 1 -> Stage 3) and its exporter.
 //
-// Two launches.  `row_scale_kernel` reads W once and leaves, per row, what needs the whole row: the exponent (or fp32 scale)
-// of the outliers, for two-level scaling the inlier factor, the scale atom, and the non-finite flag.  `pack_tile_kernel`
-// reads W again (a matrix up to ~100 MB is then still in L2) and writes the stage-tiled layout of sdq_layout.h: a CTA takes
-// 128 rows x 256 K, one record of the layout, and a thread 128 K of one row -- 16 S-Vectors, whole Q-Vectors, so that scales
-// need no exchange between threads and everything a thread produces is 4 to 16 contiguous bytes of the layout; the 32
-// lanes of a warp are 32 consecutive rows, whose pieces make whole 128-byte lines.  W comes in through shared memory, rows
-// 528 B apart (the 16-byte reads of 8 lanes then touch all banks once).
+// One launch for rows up to 16384 long (`pack_kernel<FUSED>`): a CTA takes 16 rows x 2048 K, the CTAs of a thread-block cluster
+// share the rows' K range, and a thread takes 128 K of one row -- 16 S-Vectors, whole Q-Vectors, so that scales need no
+// exchange between threads and everything a thread produces is 4 to 16 contiguous bytes of the layout; the lanes of a warp
+// are 16 consecutive rows, whose pieces make whole 128-byte lines.  W is read once, through shared memory (rows 4112 B
+// apart: the 16-byte reads of 8 lanes then touch all banks once).  What needs the whole row -- the exponent (or fp32 scale) of
+// the outliers, for two-level scaling the inlier factor -- is found in a first pass over the staged rows and exchanged
+// through distributed shared memory.  Longer rows: `row_scale_kernel` finds it and the same kernel follows without clusters.
 //
 // What bounds it: the integer pipe (77 % busy at ~140 instructions per S-Vector; selections on packed keys instead of index
 // loops took it from ~350 over two passes), DRAM is at 30 %.  11008 x 4096, 1:8 + pair-wise 4:8: 189 us as one kernel with a
-// CTA per row and a thread per S-Vector scattering bytes -> 20 + 42 us.
+// CTA per row and a thread per S-Vector scattering bytes -> 20 + 42 us with the row scales in a launch of their own ->
+// 51 us.
 #include <cstring>
+#include <type_traits>
 #include <mutex>
 #include <condition_variable>
 
@@ -164,7 +166,50 @@ struct PackParams {
   int sv4, elem, ue, i8, b32, ceil_rule;
 };
 
-// ---- launch 1: per row the outlier scale, the inlier factor of two-level scaling, non-finite check.  One warp per row.
+// outlier scale of a row from its largest outlier: exponent, or the bit pattern of the fp32 scale amax / 127 (int8)
+__device__ __forceinline__ int row_scale(const PackParams& p, uint32_t omax) {
+  const float a = bf16_bits_to_float(omax);
+  return p.i8 ? __float_as_int(int8_scale(a)) : fp8_scale_exp(a);
+}
+// exponent of the row's inlier factor 2^t (two-level scaling)
+__device__ __forceinline__ int row_factor(const PackParams& p, uint32_t imax) { return p.ue ? fp8_scale_exp(bf16_bits_to_float(imax)) : 0; }
+__device__ __forceinline__ void store_row_scale(const PackParams& p, int64_t n, uint32_t omax, uint32_t imax) {
+  const int e = row_scale(p, omax), tw = row_factor(p, imax);
+  reinterpret_cast<int32_t*>(p.blob + p.off.osexp)[n] = e;
+  reinterpret_cast<int32_t*>(p.blob + p.off.wtexp)[n] = tw;
+  // the accumulator of a row is kept in units of 2^tw (the inlier scale codes leave that factor out), so the outlier
+  // row scale is 2^(e - tw); the GEMM's epilogue multiplies the factor back in
+  const uint32_t c = p.i8 ? 127u : (uint32_t)min(max(e - tw + 127, 0), 254);    // (int8: the epilogue applies the scales)
+  *reinterpret_cast<uint32_t*>(p.blob + p.off.sfa_out + (size_t)(n / TILE_ROWS) * SF_ATOM_BYTES + sf_off((uint32_t)(n % TILE_ROWS), 0)) = c * 0x01010101u;
+}
+// the self-describing header, zero-filled to its reservation, by one block of at least 64 threads
+__device__ __forceinline__ void store_header(const PackParams& p, const BlobHeader& hdr) {
+  if (threadIdx.x < HEADER_BYTES / 4)
+    reinterpret_cast<uint32_t*>(p.blob)[threadIdx.x] = threadIdx.x < sizeof(BlobHeader) / 4 ? reinterpret_cast<const uint32_t*>(&hdr)[threadIdx.x] : 0u;
+}
+// the largest outlier (and, two-level scaling, the largest inlier that stays) of one S-Vector, into running maxima
+template <bool WGT, int OUTN>
+__device__ __forceinline__ void group_maxima(const PackParams& p, uint32_t (&r)[4], const float* c, uint32_t& omax, uint32_t& imax) {
+  int k[8], o0, o1;
+  rank_keys<WGT>(r, c, k);
+  pick_outliers<WGT, OUTN>(k, p.order_mask, p.sv4 != 0, o0, o1);
+  if constexpr (OUTN > 0) omax = max(omax, __float_as_uint(pick_value(r, o0)) << 1 >> 17);
+  if constexpr (OUTN > 1) omax = max(omax, __float_as_uint(pick_value(r, o1)) << 1 >> 17);
+  if (p.ue) {                                                     // pair-wise pattern
+    if constexpr (OUTN > 0) zero_at(r, o0);
+    if constexpr (OUTN > 1) zero_at(r, o1);
+    uint32_t w0, w1, nibble;
+    pick_pairs<WGT>(r, k, o0, o1, w0, w1, nibble);
+    const uint32_t m = __vmaxu2(w0 & 0x7FFF7FFFu, w1 & 0x7FFF7FFFu);
+    imax = max(imax, max(m & 0xFFFFu, m >> 16));
+  }
+}
+__device__ __forceinline__ uint32_t max_magnitudes(const uint32_t (&r)[4]) {      // two packed maxima
+  return __vmaxu2(__vmaxu2(r[0] & 0x7FFF7FFFu, r[1] & 0x7FFF7FFFu), __vmaxu2(r[2] & 0x7FFF7FFFu, r[3] & 0x7FFF7FFFu));
+}
+__device__ __forceinline__ bool bad_weight(float c) { return !(c >= 0.0f && c <= 3.4028234663852886e38f); }
+
+// ---- what a row needs as a whole (K > 16384): per row the outlier scale, the inlier factor of two-level scaling, non-finite check.  One warp per row.
 // SELECT = false: the outliers hold the row's largest magnitude, so nothing has to be selected (magnitude metric, most
 // significant values first, no two-level scaling).
 template <bool SELECT, bool WGT, int OUTN>
@@ -173,9 +218,7 @@ row_scale_kernel(const PackParams p, const BlobHeader hdr)
 {
   const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t n = (int64_t)blockIdx.x * 8 + warp;               // N is a multiple of 128
-  if (blockIdx.x == 0 && threadIdx.x < HEADER_BYTES / 4)          // the self-describing header, zero-filled to its reservation
-    reinterpret_cast<uint32_t*>(p.blob)[threadIdx.x] =
-        threadIdx.x < sizeof(BlobHeader) / 4 ? reinterpret_cast<const uint32_t*>(&hdr)[threadIdx.x] : 0u;
+  if (blockIdx.x == 0) store_header(p, hdr);
   const uint4* row = reinterpret_cast<const uint4*>(p.W + n * p.ldw);
   const int G = (int)(p.K / 8);
   uint32_t all2 = 0, omax = 0, imax = 0, bad = 0;                 // all2: two packed running maxima of the magnitudes
@@ -200,25 +243,12 @@ row_scale_kernel(const PackParams p, const BlobHeader hdr)
     for (int g = (int)lane; g < G; g += 32) {
       const uint4 v = __ldg(row + g);
       uint32_t r[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-      for (int j = 0; j < 4; ++j) all2 = __vmaxu2(all2, r[j] & 0x7FFF7FFFu);
+      all2 = __vmaxu2(all2, max_magnitudes(r));
       if constexpr (WGT) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) { const float c = __ldg(p.colw + 8 * (int64_t)g + i); bad |= !(c >= 0.0f && c <= 3.4028234663852886e38f); }
+        for (int i = 0; i < 8; ++i) bad |= bad_weight(__ldg(p.colw + 8 * (int64_t)g + i));
       }
-      int k[8], o0, o1;
-      rank_keys<WGT>(r, WGT ? p.colw + 8 * (int64_t)g : nullptr, k);
-      pick_outliers<WGT, OUTN>(k, p.order_mask, p.sv4 != 0, o0, o1);
-      if constexpr (OUTN > 0) omax = max(omax, __float_as_uint(pick_value(r, o0)) << 1 >> 17);
-      if constexpr (OUTN > 1) omax = max(omax, __float_as_uint(pick_value(r, o1)) << 1 >> 17);
-      if (p.ue) {                                                 // pair-wise pattern: the largest inlier that stays
-        if constexpr (OUTN > 0) zero_at(r, o0);
-        if constexpr (OUTN > 1) zero_at(r, o1);
-        uint32_t w0, w1, nibble;
-        pick_pairs<WGT>(r, k, o0, o1, w0, w1, nibble);
-        const uint32_t m = __vmaxu2(w0 & 0x7FFF7FFFu, w1 & 0x7FFF7FFFu);
-        imax = max(imax, max(m & 0xFFFFu, m >> 16));
-      }
+      group_maxima<WGT, OUTN>(p, r, WGT ? p.colw + 8 * (int64_t)g : nullptr, omax, imax);
     }
     bad |= max(all2 & 0xFFFFu, all2 >> 16) >= 0x7F80u;
   }
@@ -227,59 +257,110 @@ row_scale_kernel(const PackParams p, const BlobHeader hdr)
   bad = __any_sync(0xffffffffu, bad != 0);
   if (lane == 0) {
     if (bad) *reinterpret_cast<volatile uint32_t*>(p.nonfinite) = 1u;
-    const float a = bf16_bits_to_float(OUTN ? omax : 0u);
-    // int8 outliers: the row's fp32 scale amax / 127 travels as its bit pattern in the place of the exponent
-    const int e = p.i8 ? __float_as_int(int8_scale(a)) : fp8_scale_exp(a);
-    const int tw = p.ue ? fp8_scale_exp(bf16_bits_to_float(imax)) : 0;       // exponent of the row's inlier factor 2^t
-    reinterpret_cast<int32_t*>(p.blob + p.off.osexp)[n] = e;
-    reinterpret_cast<int32_t*>(p.blob + p.off.wtexp)[n] = tw;
-    // the accumulator of a row is kept in units of 2^tw (the inlier scale codes leave that factor out), so the outlier
-    // row scale is 2^(e - tw); the GEMM's epilogue multiplies the factor back in
-    const uint32_t c = p.i8 ? 127u : (uint32_t)min(max(e - tw + 127, 0), 254);    // (int8: the epilogue applies the scales)
-    *reinterpret_cast<uint32_t*>(p.blob + p.off.sfa_out + (size_t)(n / TILE_ROWS) * SF_ATOM_BYTES + sf_off((uint32_t)(n % TILE_ROWS), 0)) = c * 0x01010101u;
+    store_row_scale(p, n, OUTN ? omax : 0u, imax);
   }
 }
 
-// ---- launch 2
-constexpr int PK_THREADS = 256;
-constexpr int PK_PITCH = 512 + 16;                       // bytes between rows of the staged tile
-constexpr int PK_SMEM = TILE_ROWS * PK_PITCH;            // 67584: three CTAs per SM
+// ---- the packer
+constexpr int PK_THREADS = 256, PK_ROWS = 16, PK_K = 2048;
+constexpr int PK_PITCH = PK_K * 2 + 16;                  // bytes between rows of the staged tile
+constexpr int PK_SMEM = PK_ROWS * PK_PITCH;              // 65792: three CTAs per SM
 
-template <bool DENSE, bool WGT, int OUTN>
+template <bool DENSE, bool WGT, int OUTN, bool FUSED>
 __global__ void __launch_bounds__(PK_THREADS, 3)
-pack_tile_kernel(const PackParams p)
+pack_kernel(const PackParams p, const BlobHeader hdr)
 {
   extern __shared__ __align__(16) uint8_t tile[];
+  __shared__ uint32_t s_part[2][PK_ROWS][PK_ROWS + 1];   // [outliers / inliers][row][128-K chunk]: largest magnitudes
+  __shared__ uint32_t s_all[2][8][PK_ROWS];              // [outliers / inliers][cluster rank][row], pushed by their owners
   const uint32_t tid = threadIdx.x;
-  const int T2 = (int)(p.K / K2), T1 = 2 * T2;
-  const int rt = (int)(blockIdx.x / (uint32_t)T2), k2 = (int)(blockIdx.x % (uint32_t)T2);
+  const int T1 = (int)(p.K / K1), T2 = T1 / 2;
+  const int cx = (int)((p.K + PK_K - 1) / PK_K), rank = (int)(blockIdx.x % (uint32_t)cx);   // FUSED: a cluster is the cx CTAs of these rows
+  const bool first_rows = blockIdx.x < (uint32_t)cx;
+  const int64_t n_first = (int64_t)(blockIdx.x / (uint32_t)cx) * PK_ROWS;
   {
-    // 256 threads: 8 rows per round, 32 lanes x 16 B = the 512 B of one row
-    const uint32_t row = tid >> 5, lane = tid & 31;
-    const uint8_t* src = reinterpret_cast<const uint8_t*>(p.W + ((int64_t)rt * TILE_ROWS + row) * p.ldw + (int64_t)k2 * K2) + lane * 16;
-    const uint32_t dst = (uint32_t)__cvta_generic_to_shared(tile) + row * PK_PITCH + lane * 16;
+    // 256 threads x 16 B = the 4096 B of one row per round
+    const int64_t k = (int64_t)rank * PK_K + tid * 8;
+    const uint8_t* src = reinterpret_cast<const uint8_t*>(p.W + n_first * p.ldw + k);
+    const uint32_t dst = (uint32_t)__cvta_generic_to_shared(tile) + tid * 16;
+    if (k < p.K) {
 #pragma unroll
-    for (int i = 0; i < TILE_ROWS / 8; ++i)
-      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + i * 8 * PK_PITCH), "l"(src + (int64_t)i * 16 * p.ldw) : "memory");
+      for (int i = 0; i < PK_ROWS; ++i)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + i * PK_PITCH), "l"(src + (int64_t)i * 2 * p.ldw) : "memory");
+    }
     asm volatile("cp.async.wait_all;" ::: "memory");
   }
-  const uint32_t r = tid & 127u, h = tid >> 7;           // this thread's row and 128-K half
-  const int64_t n = (int64_t)rt * TILE_ROWS + r;
-  const int e = reinterpret_cast<const int32_t*>(p.blob + p.off.osexp)[n];
-  const int tw = p.ue ? reinterpret_cast<const int32_t*>(p.blob + p.off.wtexp)[n] : 0;
+  const uint32_t row = tid & 15u, ch = tid >> 4;         // this thread's row and 128-K chunk of the tile
+  const int kc = rank * 16 + (int)ch;                    // ... and of the matrix
+  const bool on = kc < T1;
+  const int64_t n = n_first + row;
+  const uint8_t* mine = tile + row * PK_PITCH + ch * 256;
+  const float* colw = WGT ? p.colw + (int64_t)kc * K1 : nullptr;
   __syncthreads();
 
+  int e, tw;
+  if constexpr (FUSED) {
+    // ---- first pass: the row's largest outlier (and inlier), non-finite check.  By magnitude, most significant first, the
+    // outliers hold the row's largest magnitude, so nothing has to be selected.
+    uint32_t all2 = 0, omax = 0, imax = 0, bad = 0;
+    if (on) {
+      const bool select = WGT || p.order_mask || p.ue;
+#pragma unroll 4
+      for (int i = 0; i < 16; ++i) {
+        const uint4 v = *reinterpret_cast<const uint4*>(mine + i * 16);
+        uint32_t r[4] = {v.x, v.y, v.z, v.w};
+        all2 = __vmaxu2(all2, max_magnitudes(r));
+        if (select) group_maxima<WGT, OUTN>(p, r, WGT ? colw + 8 * i : nullptr, omax, imax);
+      }
+      const uint32_t all = max(all2 & 0xFFFFu, all2 >> 16);
+      if (!select) omax = all;
+      bad = all >= 0x7F80u;
+      if (WGT && first_rows)                             // the channel weights are the same for every row
+        for (int i = (int)row; i < K1; i += PK_ROWS) bad |= bad_weight(__ldg(colw + i));
+    }
+    if (bad) *reinterpret_cast<volatile uint32_t*>(p.nonfinite) = 1u;
+    s_part[0][row][ch] = OUTN ? omax : 0u;
+    s_part[1][row][ch] = imax;
+    __syncthreads();
+    if (tid < 2 * PK_ROWS) {
+      const uint32_t which = tid >> 4, r = tid & 15u;
+      uint32_t m = 0;
+#pragma unroll
+      for (int c = 0; c < 16; ++c) m = max(m, s_part[which][r][c]);
+      const uint32_t mine_at = (uint32_t)__cvta_generic_to_shared(&s_all[which][rank][r]);
+      for (uint32_t peer = 0; peer < (uint32_t)cx; ++peer) {
+        uint32_t ra;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(mine_at), "r"(peer));
+        asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(ra), "r"(m) : "memory");
+      }
+    }
+    // one barrier: every push is visible after it, and nobody touches another CTA's memory afterwards
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    omax = imax = 0;
+    for (int c = 0; c < cx; ++c) { omax = max(omax, s_all[0][c][row]); imax = max(imax, s_all[1][c][row]); }
+    if (rank == 0 && ch == 0) store_row_scale(p, n, omax, imax);
+    if (rank == 0 && first_rows) store_header(p, hdr);
+    e = row_scale(p, omax);
+    tw = row_factor(p, imax);
+  } else {
+    e = reinterpret_cast<const int32_t*>(p.blob + p.off.osexp)[n];
+    tw = p.ue ? reinterpret_cast<const int32_t*>(p.blob + p.off.wtexp)[n] : 0;
+  }
+  if (!on) return;
+
+  // ---- second pass
+  const int rt = (int)(n / TILE_ROWS), k2 = kc >> 1;
+  const uint32_t r = (uint32_t)(n % TILE_ROWS), h = (uint32_t)kc & 1u;   // row of the row tile, 128-K half of the record
   const bool b32 = DENSE || p.b32 != 0;
   uint8_t* wi = p.blob + p.off.wi + ((size_t)rt * T2 + k2) * (size_t)wi_bytes(b32, DENSE);
-  uint8_t* wo = p.blob + p.off.wo + ((size_t)rt * T1 + 2 * k2 + h) * (size_t)WO_BYTES;
-  uint8_t* wc = p.blob + p.off.wc + ((size_t)rt * T1 + 2 * k2 + h) * (size_t)wc_bytes(OUTN);
-  const uint8_t* mine = tile + r * PK_PITCH + h * 256;
-  const float* colw = WGT ? p.colw + (int64_t)k2 * K2 + h * K1 : nullptr;
+  uint8_t* wo = p.blob + p.off.wo + ((size_t)rt * T1 + kc) * (size_t)WO_BYTES;
+  uint8_t* wc = p.blob + p.off.wc + ((size_t)rt * T1 + kc) * (size_t)wc_bytes(OUTN);
   const float s8 = pow2_neg(e);
   const uint32_t core = (r >> 3) * 256 + (r & 7) * 16;   // this row inside a K-block of an A operand
 
   uint32_t in_word[2][2];                                // pair-wise inliers: the 64-K half's codes, two S-Vectors per word
   uint32_t nib = 0, sc = 0;                              // its pattern nibbles; scale bytes of the 128 K
+  uint32_t nibs[2], codes[4], sels[4], metas[4];         // pattern nibbles and outlier bytes of the 128 K
   uint32_t kept[16];                                     // pair-wise inliers of a Q-Vector of 64 K, outlier positions zeroed
   uint32_t qmax2 = 0;                                    // packed running maximum of the Q-Vector
 #pragma unroll
@@ -404,7 +485,7 @@ pack_tile_kernel(const PackParams p)
       if (b & 1) {
         // 16 code bytes per 64 K (K-block h, chunk b / 2) and 4 bytes of pattern nibbles
         *reinterpret_cast<uint4*>(wi + h * 4096 + core + (b >> 1) * 128) = make_uint4(in_word[0][0], in_word[0][1], in_word[1][0], in_word[1][1]);
-        *reinterpret_cast<uint32_t*>(wi + A_IN_BYTES + r * 16 + h * 8 + (b >> 1) * 4) = nib;
+        nibs[b >> 1] = nib;
         nib = 0;
       }
     }
@@ -415,14 +496,13 @@ pack_tile_kernel(const PackParams p)
       // per S-Vector: position ps (0..7) sits in group of 4 number ps >> 2 at p = ps & 3, whose slots are (p, 3), the value
       // first, or (0, 3), the value second, when p = 3; the other group has slots (0, 1).  Metadata bytes and byte shifts
       // come from 8-entry tables looked up by byte-permutes, the four position nibbles being the selector.
-      const uint32_t codes = ocode[0] | (ocode[1] << 8) | (ocode[2] << 16) | (ocode[3] << 24);
+      codes[b] = ocode[0] | (ocode[1] << 8) | (ocode[2] << 16) | (ocode[3] << 24);
       const uint32_t sel = opos[0] | (opos[1] << 4) | (opos[2] << 8) | (opos[3] << 12);
-      const uint32_t meta = __byte_perm(0x4C4E4D4Cu, 0xC4E4D4C4u, sel), sh = __byte_perm(0x08000000u, 0x18101010u, sel);
+      const uint32_t sh = __byte_perm(0x08000000u, 0x18101010u, sel);
+      metas[b] = __byte_perm(0x4C4E4D4Cu, 0xC4E4D4C4u, sel);
+      sels[b] = sel;
       *reinterpret_cast<uint4*>(wo + (b >> 1) * 4096 + core + (b & 1) * 128) =
           make_uint4(ocode[0] << (sh & 31u), ocode[1] << ((sh >> 8) & 31u), ocode[2] << ((sh >> 16) & 31u), ocode[3] << (sh >> 24));
-      *reinterpret_cast<uint32_t*>(wo + A_OUT_BYTES + r * 16 + 4 * b) = meta;
-      *reinterpret_cast<uint32_t*>(wc + r * 16 + 4 * b) = codes;
-      *reinterpret_cast<uint16_t*>(wc + WC_CODE_BYTES + r * 8 + 2 * b) = (uint16_t)sel;
     } else if constexpr (OUTN == 2) {
       uint32_t st[4], meta = 0;
 #pragma unroll
@@ -444,12 +524,18 @@ pack_tile_kernel(const PackParams p)
         }
       }
       *reinterpret_cast<uint4*>(wo + (b >> 1) * 4096 + core + (b & 1) * 128) = make_uint4(st[0], st[1], st[2], st[3]);
-      *reinterpret_cast<uint32_t*>(wo + A_OUT_BYTES + r * 16 + 4 * b) = meta;
+      metas[b] = meta;
       *reinterpret_cast<uint2*>(wc + r * 32 + 8 * b) =
           make_uint2(ocode[0] | (ocode1[0] << 8) | (ocode[1] << 16) | (ocode1[1] << 24), ocode[2] | (ocode1[2] << 8) | (ocode[3] << 16) | (ocode1[3] << 24));
       *reinterpret_cast<uint32_t*>(wc + 2 * WC_CODE_BYTES + r * 16 + 4 * b) =
           opos[0] | (opos1[0] << 4) | (opos[1] << 8) | (opos1[1] << 12) | (opos[2] << 16) | (opos1[2] << 20) | (opos[3] << 24) | (opos1[3] << 28);
     }
+  }
+  if constexpr (!DENSE) *reinterpret_cast<uint2*>(wi + A_IN_BYTES + r * 16 + h * 8) = make_uint2(nibs[0], nibs[1]);
+  if constexpr (OUTN > 0) *reinterpret_cast<uint4*>(wo + A_OUT_BYTES + r * 16) = make_uint4(metas[0], metas[1], metas[2], metas[3]);
+  if constexpr (OUTN == 1) {
+    *reinterpret_cast<uint4*>(wc + r * 16) = make_uint4(codes[0], codes[1], codes[2], codes[3]);
+    *reinterpret_cast<uint2*>(wc + WC_CODE_BYTES + r * 8) = make_uint2(sels[0] | (sels[1] << 16), sels[2] | (sels[3] << 16));
   }
   // ---- inlier scales: one atom per 128-K half with four scales of 32 K, or two scales of 64 K of the one atom
   uint8_t* sf = wi + a_in_bytes(DENSE) + e_in_bytes(DENSE) + (r & 31) * 16 + (r >> 5) * 4;
@@ -457,19 +543,31 @@ pack_tile_kernel(const PackParams p)
   else *reinterpret_cast<uint16_t*>(sf + 2 * h) = (uint16_t)sc;
 }
 
-template <bool WGT, int OUTN>
-static void launch_pack(const PackParams& p, const BlobHeader& hdr, bool dense, cudaStream_t st)
+template <bool DENSE, bool WGT, int OUTN>
+static void launch_pack(const PackParams& p, const BlobHeader& hdr, cudaStream_t st)
 {
-  const unsigned rows = (unsigned)(p.N / 8), tiles = (unsigned)((p.N / TILE_ROWS) * (p.K / K2));
+  const unsigned cx = (unsigned)((p.K + PK_K - 1) / PK_K);
+  cudaLaunchConfig_t lc = {};
+  lc.gridDim = dim3(cx * (unsigned)(p.N / PK_ROWS));
+  lc.blockDim = dim3(PK_THREADS);
+  lc.dynamicSmemBytes = PK_SMEM;
+  lc.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = cx;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  lc.attrs = attr;
+  auto go = [&](auto kern, int n_attrs) {
+    lc.numAttrs = n_attrs;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, PK_SMEM) == cudaSuccess) (void)cudaLaunchKernelEx(&lc, kern, p, hdr);
+  };
+  if (cx <= 8) { go(pack_kernel<DENSE, WGT, OUTN, true>, 1); return; }
+  // rows longer than a cluster of eight CTAs holds
+  const unsigned rows = (unsigned)(p.N / 8);
   if (WGT || p.order_mask || p.ue) row_scale_kernel<true, WGT, OUTN><<<rows, 256, 0, st>>>(p, hdr);
   else row_scale_kernel<false, WGT, OUTN><<<rows, 256, 0, st>>>(p, hdr);
-  if (dense) {
-    cudaFuncSetAttribute(pack_tile_kernel<true, WGT, OUTN>, cudaFuncAttributeMaxDynamicSharedMemorySize, PK_SMEM);
-    pack_tile_kernel<true, WGT, OUTN><<<tiles, PK_THREADS, PK_SMEM, st>>>(p);
-  } else {
-    cudaFuncSetAttribute(pack_tile_kernel<false, WGT, OUTN>, cudaFuncAttributeMaxDynamicSharedMemorySize, PK_SMEM);
-    pack_tile_kernel<false, WGT, OUTN><<<tiles, PK_THREADS, PK_SMEM, st>>>(p);
-  }
+  go(pack_kernel<DENSE, WGT, OUTN, false>, 0);
 }
 
 // One host-visible word per call in flight, where the kernels report a non-finite weight: a page of pinned memory, taken
@@ -570,6 +668,27 @@ export_packed_kernel(const uint8_t* __restrict__ blob, int64_t N, int64_t K, sdq
     out.out_sexp[n] = reinterpret_cast<const int32_t*>(blob + off.osexp)[n];
     if (out.in_texp) out.in_texp[n] = reinterpret_cast<const int32_t*>(blob + off.wtexp)[n];
   }
+}
+
+// two ranges of a packed buffer (16-byte units) to their places in another, and its header: one pass at DRAM speed
+struct CopyRange { const uint4* src; uint4* dst; size_t n; };
+__global__ void __launch_bounds__(256)
+compact_kernel(const CopyRange a, const CopyRange b, uint32_t* __restrict__ header, const BlobHeader hdr)
+{
+  if (blockIdx.x == 0 && threadIdx.x < HEADER_BYTES / 4)
+    header[threadIdx.x] = threadIdx.x < sizeof(BlobHeader) / 4 ? reinterpret_cast<const uint32_t*>(&hdr)[threadIdx.x] : 0u;
+  const size_t step = (size_t)gridDim.x * 256, n = a.n + b.n;
+  auto from = [&](size_t i) { return i < a.n ? a.src + i : b.src + (i - a.n); };
+  auto to = [&](size_t i) { return i < a.n ? a.dst + i : b.dst + (i - a.n); };
+  size_t i = (size_t)blockIdx.x * 256 + threadIdx.x;
+  for (; i + 3 * step < n; i += 4 * step) {
+    uint4 v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) v[u] = __ldcs(from(i + u * step));
+#pragma unroll
+    for (int u = 0; u < 4; ++u) *to(i + u * step) = v[u];
+  }
+  for (; i < n; i += step) *to(i) = __ldcs(from(i));
 }
 
 }  // namespace sdq
@@ -673,15 +792,19 @@ extern "C" sdq_status_t sdq_decompose_metric(const void* W, int64_t N, int64_t K
     p.i8 = cfg->out_fmt == SDQ_OUT_INT8;
     p.b32 = cfg->in_block == 32;
     p.ceil_rule = cfg->scale_rule == SDQ_SCALE_CEIL_NOSAT;
-    const bool dense = is_dense_layout(*cfg);
-    switch ((col_weight ? 3 : 0) + cfg->out_n) {
-      case 0: launch_pack<false, 0>(p, *hdr, dense, st); break;
-      case 1: launch_pack<false, 1>(p, *hdr, dense, st); break;
-      case 2: launch_pack<false, 2>(p, *hdr, dense, st); break;
-      case 3: launch_pack<true, 0>(p, *hdr, dense, st); break;
-      case 4: launch_pack<true, 1>(p, *hdr, dense, st); break;
-      default: launch_pack<true, 2>(p, *hdr, dense, st); break;
-    }
+    const int v = (col_weight ? 3 : 0) + cfg->out_n;
+    auto pick = [&](auto dense) {
+      constexpr bool D = decltype(dense)::value;
+      switch (v) {
+        case 0: launch_pack<D, false, 0>(p, *hdr, st); break;
+        case 1: launch_pack<D, false, 1>(p, *hdr, st); break;
+        case 2: launch_pack<D, false, 2>(p, *hdr, st); break;
+        case 3: launch_pack<D, true, 0>(p, *hdr, st); break;
+        case 4: launch_pack<D, true, 1>(p, *hdr, st); break;
+        default: launch_pack<D, true, 2>(p, *hdr, st); break;
+      }
+    };
+    if (is_dense_layout(*cfg)) pick(std::true_type{}); else pick(std::false_type{});
   } else if (ok) {
     launch_pack_plain(W, N, K, ldw, *cfg, col_weight, packed_buf, report_dev, st);
     ok = cudaMemcpyAsync(packed_buf, raw, HEADER_BYTES, cudaMemcpyHostToDevice, st) == cudaSuccess;
@@ -755,20 +878,20 @@ extern "C" sdq_status_t sdq_packed_compact(const sdq_packed_t* P, void* dst, siz
   cudaStream_t st = (cudaStream_t)stream;
   const uint8_t* s = (const uint8_t*)P->dev;
   uint8_t* d = (uint8_t*)dst;
-  // every section but the 2:4 containers, each to its place in the shorter buffer
-  bool ok = cudaMemcpyAsync(d + off.wi, s + src.wi, src.wo - src.wi, cudaMemcpyDeviceToDevice, st) == cudaSuccess;
-  ok = ok && cudaMemcpyAsync(d + off.sfa_out, s + src.sfa_out, src.total - src.sfa_out, cudaMemcpyDeviceToDevice, st) == cudaSuccess;
-  if (!ok) return SDQ_ERR_CUDA;
   sdq_packed_t q;
   q.dev = dst; q.bytes = off.total; q.N = P->N; q.K = P->K; q.cfg = P->cfg;
   for (int i = 0; i < 8; ++i) q.off[i] = 0;
   q.off[0] = off.wi; q.off[1] = 0; q.off[2] = off.sfa_out; q.off[3] = off.wc; q.off[5] = off.osexp; q.off[6] = off.wtexp;
-  alignas(16) static thread_local unsigned char raw[HEADER_BYTES];
-  memset(raw, 0, HEADER_BYTES);
-  fill_header(reinterpret_cast<BlobHeader*>(raw), q, true);
-  reinterpret_cast<BlobHeader*>(raw)->tiled = 2u;
-  if (cudaMemcpyAsync(dst, raw, HEADER_BYTES, cudaMemcpyHostToDevice, st) != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess)
-    return SDQ_ERR_CUDA;
+  BlobHeader hdr;
+  fill_header(&hdr, q, true);
+  hdr.tiled = 2u;
+  // every section but the 2:4 containers, each to its place in the shorter buffer
+  const CopyRange a = {(const uint4*)(s + src.wi), (uint4*)(d + off.wi), (src.wo - src.wi) / 16};
+  const CopyRange b = {(const uint4*)(s + src.sfa_out), (uint4*)(d + off.sfa_out), (src.total - src.sfa_out) / 16};
+  const DeviceInfo* dinfo = device_info();
+  if (!dinfo) return SDQ_ERR_CUDA;
+  compact_kernel<<<(unsigned)(dinfo->sm_count * 8), 256, 0, st>>>(a, b, (uint32_t*)d, hdr);
+  if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess) return SDQ_ERR_CUDA;
   *out = q;
   return SDQ_OK;
 }

@@ -1,5 +1,5 @@
 // Native half of the Python binding: the calls a program makes for every batch of activations (quantize, linear, grouped
-// linear), marshalled without ctypes.  Each function takes the arguments of its namesake in __init__.py, does what that
+// linear) or for every weight matrix (decompose, compact, channel norm), marshalled without ctypes.  Each function takes the arguments of its namesake in __init__.py, does what that
 // does -- allocate what was not supplied, look up the current stream, call the C-ABI, raise SdqError -- and returns None
 // where an argument is not what such a call has in the ordinary case (a CPU tensor, another type, another shape); the Python
 // function then goes its own way, which checks and reports.
@@ -24,8 +24,9 @@ PyTypeObject* act_type = nullptr;        // the ctypes structures of sdq_act_t, 
 PyTypeObject* packed_type = nullptr;
 PyTypeObject* config_type = nullptr;
 PyObject* quant_act = nullptr;           // class QuantAct
+PyObject* packed_weight = nullptr;       // class PackedWeight
 PyObject* sdq_error = nullptr;           // class SdqError
-PyObject *s_desc, *s_buf;
+PyObject *s_desc, *s_buf, *s_N, *s_K, *s_cfg, *s_algo;
 
 // memory of a ctypes structure, held for the lifetime of this object
 class View {
@@ -82,10 +83,13 @@ at::Tensor new_output(int64_t M, int64_t N, at::ScalarType type, const at::Devic
 #define NOT_HERE Py_RETURN_NONE
 
 PyObject* bind(PyObject*, PyObject* const* a, Py_ssize_t n) {
-  if (n != 5 || !PyType_Check(a[0]) || !PyType_Check(a[1]) || !PyType_Check(a[2])) { PyErr_SetString(PyExc_TypeError, "bind(Act, Packed, Config, QuantAct, SdqError)"); return nullptr; }
-  for (int i = 0; i < 5; ++i) Py_INCREF(a[i]);
+  if (n != 6 || !PyType_Check(a[0]) || !PyType_Check(a[1]) || !PyType_Check(a[2])) {
+    PyErr_SetString(PyExc_TypeError, "bind(Act, Packed, Config, QuantAct, PackedWeight, SdqError)");
+    return nullptr;
+  }
+  for (int i = 0; i < 6; ++i) Py_INCREF(a[i]);
   act_type = (PyTypeObject*)a[0]; packed_type = (PyTypeObject*)a[1]; config_type = (PyTypeObject*)a[2];
-  quant_act = a[3]; sdq_error = a[4];
+  quant_act = a[3]; packed_weight = a[4]; sdq_error = a[5];
   Py_RETURN_NONE;
 }
 
@@ -265,7 +269,106 @@ PyObject* linear_group_x(PyObject*, PyObject* const* a, Py_ssize_t n) {
   END_HANDLE_TH_ERRORS
 }
 
-PyMethodDef methods[] = {{"bind", (PyCFunction)(void (*)(void))bind, METH_FASTCALL, nullptr},
+// decompose(W, cfg, buf or None, col_weight or None) -> PackedWeight
+PyObject* decompose(PyObject*, PyObject* const* a, Py_ssize_t n) {
+  HANDLE_TH_ERRORS
+  if (n != 4 || !is_cuda_matrix(a[0], at::kBFloat16)) NOT_HERE;
+  View vc;
+  const sdq_config_t* cfg = (const sdq_config_t*)vc.open(a[1], config_type);
+  if (!cfg) NOT_HERE;
+  const at::Tensor& W = THPVariable_Unpack(a[0]);
+  const int64_t N = W.size(0), K = W.size(1);
+  const float* colw = nullptr;
+  if (a[3] != Py_None) {
+    if (!THPVariable_Check(a[3])) NOT_HERE;
+    const at::Tensor& c = THPVariable_Unpack(a[3]);
+    if (!c.is_cuda() || c.scalar_type() != at::kFloat || c.dim() != 1 || c.size(0) != K || !c.is_contiguous()) NOT_HERE;
+    colw = (const float*)c.data_ptr();
+  }
+  size_t bytes = 0, algo = 0;
+  sdq_status_t st = sdq_packed_size(N, K, cfg, &bytes, &algo);
+  if (st != SDQ_OK) return raise(st, "sdq_packed_size");
+  at::Tensor buf;
+  if (a[2] == Py_None) {
+    buf = at::empty({(int64_t)bytes}, at::TensorOptions().dtype(at::kByte).device(W.device()));
+  } else {
+    if (!THPVariable_Check(a[2])) NOT_HERE;
+    buf = THPVariable_Unpack(a[2]);
+    if (!buf.is_cuda() || buf.scalar_type() != at::kByte) NOT_HERE;
+  }
+  Ref desc(PyObject_CallNoArgs((PyObject*)packed_type));
+  if (!desc.get()) return nullptr;
+  {
+    View vd;
+    sdq_packed_t* d = (sdq_packed_t*)vd.open(desc.get(), packed_type);
+    if (!d) NOT_HERE;
+    void *stream = current_stream(), *w = W.data_ptr(), *b = buf.data_ptr();
+    const int64_t ldw = W.stride(0);
+    const size_t room = (size_t)buf.numel();
+    Py_BEGIN_ALLOW_THREADS
+    st = sdq_decompose_metric(w, N, K, ldw, cfg, colw, b, room, d, stream);
+    Py_END_ALLOW_THREADS
+    if (st != SDQ_OK) return raise(st, colw ? "sdq_decompose_metric" : "sdq_decompose");
+  }
+  Ref b(a[2] == Py_None ? THPVariable_Wrap(std::move(buf)) : Py_NewRef(a[2])), pn(PyLong_FromLongLong(N)), pk(PyLong_FromLongLong(K)), pa(PyLong_FromSize_t(algo));
+  if (!b.get() || !pn.get() || !pk.get() || !pa.get()) return nullptr;
+  PyObject* args[6] = {b.get(), desc.get(), pn.get(), pk.get(), a[1], pa.get()};
+  return PyObject_Vectorcall(packed_weight, args, 6, nullptr);
+  END_HANDLE_TH_ERRORS
+}
+
+// compact(p) -> PackedWeight
+PyObject* compact(PyObject*, PyObject* const* a, Py_ssize_t n) {
+  HANDLE_TH_ERRORS
+  if (n != 1) NOT_HERE;
+  Ref dp(attr(a[0], s_desc)), pb(attr(a[0], s_buf)), pn(attr(a[0], s_N)), pk(attr(a[0], s_K)), pc(attr(a[0], s_cfg)), pa(attr(a[0], s_algo));
+  View vp;
+  const sdq_packed_t* p = (const sdq_packed_t*)vp.open(dp.get(), packed_type);
+  if (!p || !pb.get() || !THPVariable_Check(pb.get()) || !pn.get() || !pk.get() || !pc.get() || !pa.get()) NOT_HERE;
+  size_t bytes = 0;
+  sdq_status_t st = sdq_packed_compact_size(p->N, p->K, &p->cfg, &bytes);
+  if (st != SDQ_OK) return raise(st, "sdq_packed_compact_size");
+  at::Tensor buf = at::empty({(int64_t)bytes}, at::TensorOptions().dtype(at::kByte).device(THPVariable_Unpack(pb.get()).device()));
+  Ref desc(PyObject_CallNoArgs((PyObject*)packed_type));
+  if (!desc.get()) return nullptr;
+  {
+    View vd;
+    sdq_packed_t* d = (sdq_packed_t*)vd.open(desc.get(), packed_type);
+    if (!d) NOT_HERE;
+    void *stream = current_stream(), *b = buf.data_ptr();
+    Py_BEGIN_ALLOW_THREADS
+    st = sdq_packed_compact(p, b, bytes, d, stream);
+    Py_END_ALLOW_THREADS
+    if (st != SDQ_OK) return raise(st, "sdq_packed_compact");
+  }
+  Ref b(THPVariable_Wrap(std::move(buf)));
+  if (!b.get()) return nullptr;
+  PyObject* args[6] = {b.get(), desc.get(), pn.get(), pk.get(), pc.get(), pa.get()};
+  return PyObject_Vectorcall(packed_weight, args, 6, nullptr);
+  END_HANDLE_TH_ERRORS
+}
+
+// channel_norm(X) -> fp32 [K]
+PyObject* channel_norm(PyObject*, PyObject* const* a, Py_ssize_t n) {
+  HANDLE_TH_ERRORS
+  if (n != 1 || !is_cuda_matrix(a[0], at::kBFloat16)) NOT_HERE;
+  const at::Tensor& X = THPVariable_Unpack(a[0]);
+  at::Tensor c = at::empty({X.size(1)}, at::TensorOptions().dtype(at::kFloat).device(X.device()));
+  void *stream = current_stream(), *x = X.data_ptr(), *y = c.data_ptr();
+  const int64_t M = X.size(0), K = X.size(1), ldx = X.stride(0);
+  sdq_status_t st;
+  Py_BEGIN_ALLOW_THREADS
+  st = sdq_channel_norm(x, M, K, ldx, (float*)y, stream);
+  Py_END_ALLOW_THREADS
+  if (st != SDQ_OK) return raise(st, "sdq_channel_norm");
+  return THPVariable_Wrap(std::move(c));
+  END_HANDLE_TH_ERRORS
+}
+
+PyMethodDef methods[] = {{"decompose", (PyCFunction)(void (*)(void))decompose, METH_FASTCALL, nullptr},
+                         {"compact", (PyCFunction)(void (*)(void))compact, METH_FASTCALL, nullptr},
+                         {"channel_norm", (PyCFunction)(void (*)(void))channel_norm, METH_FASTCALL, nullptr},
+                         {"bind", (PyCFunction)(void (*)(void))bind, METH_FASTCALL, nullptr},
                          {"quantize_act", (PyCFunction)(void (*)(void))quantize_act, METH_FASTCALL, nullptr},
                          {"linear", (PyCFunction)(void (*)(void))linear, METH_FASTCALL, nullptr},
                          {"linear_group", (PyCFunction)(void (*)(void))linear_group, METH_FASTCALL, nullptr},
@@ -278,5 +381,9 @@ PyModuleDef module = {PyModuleDef_HEAD_INIT, "_binding", nullptr, -1, methods, n
 PyMODINIT_FUNC PyInit__binding() {
   s_desc = PyUnicode_InternFromString("desc");
   s_buf = PyUnicode_InternFromString("buf");
+  s_N = PyUnicode_InternFromString("N");
+  s_K = PyUnicode_InternFromString("K");
+  s_cfg = PyUnicode_InternFromString("cfg");
+  s_algo = PyUnicode_InternFromString("algorithmic_bytes");
   return PyModule_Create(&module);
 }

@@ -585,7 +585,12 @@ def test_native_and_ctypes_halves_of_the_binding_agree(monkeypatch):
         buf = torch.zeros(m.act_size(9, 1024, cfg), dtype=torch.uint8, device="cuda")
         assert m.sdq_quantize_act(X, cfg, buf).buf is buf and (xq.M, xq.K) == (9, 1024)
         ws = m.make_workspace(9, 5120, 1024, cfg, "cuda")
-        got = [m.act_export(xq)["xq8_code"], m.sdq_linear(xq, ps[0]), m.sdq_linear(xq, ps[0], f32=True), m.sdq_linear(xq, ps[0], workspace=ws)]
+        W = sdq_synth.make_weight(128, 1024, 73).cuda()
+        norms = m.channel_norm(X)
+        packed = [m.sdq_decompose(W, cfg), m.sdq_decompose(W, cfg, col_weight=norms), m.sdq_decompose(W, cfg, torch.zeros_like(ps[0].buf))]
+        packed.append(m.packed_compact(packed[1]))
+        assert all((q.N, q.K, q.algorithmic_bytes) == (128, 1024, m.packed_size(128, 1024, cfg)[1]) for q in packed)
+        got = [norms] + [t for q in packed for t in m.packed_export(q).values()] + [m.act_export(xq)["xq8_code"], m.sdq_linear(xq, ps[0]), m.sdq_linear(xq, ps[0], f32=True), m.sdq_linear(xq, ps[0], workspace=ws)]
         for f32 in (False, True):
             got += m.sdq_linear_group([xq, xq], ps, f32=f32) + m.sdq_linear_group_x(X, ps, f32=f32)
             outs = [torch.empty((9, 5120), dtype=torch.float32 if f32 else torch.bfloat16, device="cuda") for _ in ps]
