@@ -117,7 +117,7 @@ sdq_linear_pair_kernel(const __grid_constant__ LinearParams p)
   const uint32_t NSLOT = FORM == PAIR_FLEX ? (uint32_t)p.nslot : (uint32_t)pair_slots(FIXED_SLOT), SL_SF = SL_B + TMAX * 64u;
   const bool acc2 = FORM == PAIR_FLEX && p.pt_acc2;
   uint8_t* stg_base = sm + NSLOT * SLOT;
-  uint64_t* full = reinterpret_cast<uint64_t*>(stg_base + PAIR_STG);   // the three producers' parts of slot s have landed (leader: + the peer's)
+  uint64_t* full = reinterpret_cast<uint64_t*>(stg_base + PAIR_STG);   // the producers' parts of slot s have landed (leader: + the peer's)
   uint64_t* empty = full + PAIR_MAX_SLOTS;                         // [s / 2]: the MMAs that read slots s and s ^ 1 have completed
   uint64_t* acc_full = empty + PAIR_MAX_SLOTS;                     // [2]
   uint64_t* acc_empty = acc_full + 2;                              // [2] leader: all epilogue warps of the pair have drained the accumulator
@@ -139,7 +139,7 @@ sdq_linear_pair_kernel(const __grid_constant__ LinearParams p)
   if (tid == 0) {
     *timed_out = 0u;
     for (uint32_t s = 0; s < NSLOT; ++s) {
-      ptx::mbar_init(&full[s], rank == 0 ? 4 : 3);
+      ptx::mbar_init(&full[s], rank == 0 ? 3 : 2);
       if (!(s & 1)) ptx::mbar_init(&empty[s >> 1], 1);
     }
     for (int a = 0; a < 2; ++a) { ptx::mbar_init(&acc_full[a], 1); ptx::mbar_init(&acc_empty[a], 32); }
@@ -157,71 +157,90 @@ sdq_linear_pair_kernel(const __grid_constant__ LinearParams p)
     if (lane < 2) {
       // ---------------- producers (both CTAs): role 0 = own weight records, 1 = own activation codes, 2 = scale atoms.
       // Ring slots are released in pairs, so lanes 0 and 1 of the warp run the loop in lockstep, lane l filling the slots of
-      // parity l: two stages per trip.
-      const int role = warp == 0 ? 0 : (int)warp - 1;
-      if (role != 0) ptx::griddep_wait();    // activations come from an earlier kernel; weights do not
+      // parity l: two stages per trip.  A trip has to stay short -- with the addresses worked out from scratch and the release
+      // tested at its head it took 0.3 us, and no stage could take less than half of that: what belongs to a task is worked out
+      // once, and the next release is tested while this trip's copies go out.
+      // The expected bytes of codes and atoms are announced by role 1, so role 2 has nothing to do for an outlier stage but
+      // the first.
       bool ok = true;
-      uint32_t s = lane, wrapped = 0, ph = 0;
-      int tseq = 0, k = (int)lane;                                           // this lane's stage: task number in the CTA's sequence, stage in the task
-      while (k >= S) { k -= S; ++tseq; }
-      int cur = -1, rt0 = 0, rt1 = 0, nu = 1, have = 0;
-      int64_t t0 = 0;
-      size_t a0 = 0;
-      uint32_t own = 0;
-      for (int i = (int)lane; i < total && ok; i += 2) {
-        if (tseq != cur) {
-          cur = tseq;
-          const PairTask t = pair_task<FORM>(p, pair + tseq * n_pairs);
-          nu = t.nu;
-          rt0 = min(2 * t.u0 + (int)rank, RT - 1);                           // (an odd number of row tiles: the last unit's second half
-          rt1 = min(2 * t.u0 + 2 + (int)rank, RT - 1);                       //  repeats the last tile and is not stored)
-          a0 = (size_t)pair_group0(p, t.mt);                                 // the tile's first scale atom
-          const int T = 32 * (pair_group0(p, t.mt + 1) - (int)a0);
-          t0 = (int64_t)a0 * 32 + rank * (T / 2);
-          own = (uint32_t)max((int64_t)0, min((int64_t)(T / 2), p.aoff.Mpad - t0)) * 128u;   // this CTA's code bytes that exist
-          have = T > 128 && (int)a0 + 4 < p.aoff.atoms ? 2 : 1;
-        }
-        if (wrapped && !(ok = ptx::mbar_wait(&empty[s >> 1], ph ^ 1))) break;
-        uint8_t* st = sm + (size_t)s * SLOT;
-        const bool inl = k < NI, first_o = (k == NI);
-        const int ki = i0 + k, ko = o0 + k - NI;                             // inlier / outlier stage number
-        if (role == 0) {
-          const uint32_t nb = inl ? G::WIB : (uint32_t)WO_BYTES;
-          const uint8_t* base = inl ? p.w + p.poff.wi + (size_t)ki * G::WIB : p.w + p.poff.wo + (size_t)ko * WO_BYTES;
-          const size_t step = inl ? (size_t)T2 * G::WIB : (size_t)T1 * WO_BYTES;   // bytes between row tiles
-          ptx::mbar_expect_tx(&full[s], (uint32_t)nu * (nb + (first_o ? SF_ATOM_BYTES : 0u)));
-          ptx::bulk_g2s(st, base + (size_t)rt0 * step, nb, &full[s]);
-          if (FORM == PAIR_TWO && nu == 2) ptx::bulk_g2s(st + G::WIB, base + (size_t)rt1 * step, nb, &full[s]);
-          if (first_o) {
-            ptx::bulk_g2s(st + WO_BYTES, p.w + p.poff.sfa_out + (size_t)rt0 * SF_ATOM_BYTES, SF_ATOM_BYTES, &full[s]);
-            if (FORM == PAIR_TWO && nu == 2) ptx::bulk_g2s(st + G::WIB + WO_BYTES, p.w + p.poff.sfa_out + (size_t)rt1 * SF_ATOM_BYTES, SF_ATOM_BYTES, &full[s]);
-          }
-        } else if (role == 1) {
-          if (!own) {
-            ptx::mbar_arrive(&full[s]);
-          } else {
-            ptx::mbar_expect_tx(&full[s], own);
-            ptx::bulk_g2s(st + SL_B, (inl ? p.x + p.aoff.xi + (size_t)ki * p.aoff.xi_stride : p.x + p.aoff.xo + (size_t)ko * p.aoff.xo_stride) + (size_t)t0 * 128u,
-                          own, &full[s]);
-          }
-        } else {
-          if (inl) {
-            const uint8_t* xs = p.x + p.aoff.xi + (size_t)ki * p.aoff.xi_stride + (size_t)p.aoff.Mpad * 128u + a0 * (NA * SF_ATOM_BYTES);
-            ptx::mbar_expect_tx(&full[s], (uint32_t)have * NA * SF_ATOM_BYTES);
-            for (int a = 0; a < have; ++a)
-              ptx::bulk_g2s(st + SL_SF + a * NA * SF_ATOM_BYTES, xs + a * (4 * NA * SF_ATOM_BYTES), NA * SF_ATOM_BYTES, &full[s]);
-          } else if (first_o) {
-            ptx::mbar_expect_tx(&full[s], (uint32_t)have * SF_ATOM_BYTES);
-            for (int a = 0; a < have; ++a)
-              ptx::bulk_g2s(st + SL_SF + a * SF_ATOM_BYTES, p.x + p.aoff.sfb_out + (a0 + 4 * (size_t)a) * SF_ATOM_BYTES, SF_ATOM_BYTES, &full[s]);
-          } else {
-            ptx::mbar_arrive(&full[s]);
-          }
-        }
-        s += 2;
-        if (s >= NSLOT) { s -= NSLOT; wrapped = 1; ph ^= 1; }
-        k += 2;
+      auto produce = [&](auto on_task, auto on_stage) {
+        uint32_t s = lane, wrapped = 0, ph = 0;
+        int tseq = 0, k = (int)lane, cur = -1;                               // this lane's stage: task number in the CTA's sequence, stage in the task
         while (k >= S) { k -= S; ++tseq; }
+        bool ready = false;
+        for (int i = (int)lane; i < total; i += 2) {
+          if (tseq != cur) { cur = tseq; on_task(pair_task<FORM>(p, pair + tseq * n_pairs)); }
+          if (wrapped && !ready && !(ok = ptx::mbar_wait(&empty[s >> 1], ph ^ 1))) break;
+          on_stage(k, sm + (size_t)s * SLOT, &full[s]);
+          s += 2;
+          if (s >= NSLOT) { s -= NSLOT; wrapped = 1; ph ^= 1; }
+          ready = wrapped && ptx::mbar_test(&empty[s >> 1], ph ^ 1);
+          k += 2;
+          while (k >= S) { k -= S; ++tseq; }
+        }
+      };
+      if (warp == 0) {
+        // weight records of the one or two units
+        const uint8_t *wi0 = nullptr, *wi1 = nullptr, *wo0 = nullptr, *wo1 = nullptr, *sf0 = nullptr, *sf1 = nullptr;
+        uint32_t nu = 1;
+        produce([&](const PairTask& t) {
+          nu = (uint32_t)t.nu;
+          // (an odd number of row tiles: the last unit's second half repeats the last tile and is not stored)
+          const int rt0 = min(2 * t.u0 + (int)rank, RT - 1), rt1 = min(2 * t.u0 + 2 + (int)rank, RT - 1);
+          wi0 = p.w + p.poff.wi + ((size_t)rt0 * T2 + i0) * G::WIB;
+          wo0 = p.w + p.poff.wo + ((size_t)rt0 * T1 + o0) * WO_BYTES;
+          sf0 = p.w + p.poff.sfa_out + (size_t)rt0 * SF_ATOM_BYTES;
+          if (FORM == PAIR_TWO) {
+            wi1 = p.w + p.poff.wi + ((size_t)rt1 * T2 + i0) * G::WIB;
+            wo1 = p.w + p.poff.wo + ((size_t)rt1 * T1 + o0) * WO_BYTES;
+            sf1 = p.w + p.poff.sfa_out + (size_t)rt1 * SF_ATOM_BYTES;
+          }
+        }, [&](int k, uint8_t* st, uint64_t* bar) {
+          const bool two = FORM == PAIR_TWO && nu == 2;
+          if (k < NI) {
+            const uint32_t off = (uint32_t)k * G::WIB;
+            ptx::mbar_expect_tx(bar, (two ? 2u : 1u) * G::WIB);
+            ptx::bulk_g2s(st, wi0 + off, G::WIB, bar);
+            if (two) ptx::bulk_g2s(st + G::WIB, wi1 + off, G::WIB, bar);
+          } else {
+            const uint32_t off = (uint32_t)(k - NI) * WO_BYTES;
+            const bool first_o = k == NI;
+            ptx::mbar_expect_tx(bar, (two ? 2u : 1u) * (WO_BYTES + (first_o ? SF_ATOM_BYTES : 0u)));
+            ptx::bulk_g2s(st, wo0 + off, WO_BYTES, bar);
+            if (two) ptx::bulk_g2s(st + G::WIB, wo1 + off, WO_BYTES, bar);
+            if (first_o) {
+              ptx::bulk_g2s(st + WO_BYTES, sf0, SF_ATOM_BYTES, bar);
+              if (two) ptx::bulk_g2s(st + G::WIB + WO_BYTES, sf1, SF_ATOM_BYTES, bar);
+            }
+          }
+        });
+      } else {
+        // own activation codes (role 1) and the scale atoms of both token halves (role 2)
+        const bool codes = warp == 2;
+        const uint8_t *xi = nullptr, *xo = nullptr, *sf = nullptr;
+        uint32_t own = 0, have = 1;
+        ptx::griddep_wait();                   // activations come from an earlier kernel; weights do not
+        produce([&](const PairTask& t) {
+          const int g0 = pair_group0(p, t.mt), T = 32 * (pair_group0(p, t.mt + 1) - g0);   // the tile's first scale atom, its tokens
+          const int64_t t0 = (int64_t)g0 * 32 + rank * (T / 2);
+          own = (uint32_t)max((int64_t)0, min((int64_t)(T / 2), p.aoff.Mpad - t0)) * 128u; // this CTA's code bytes that exist
+          have = T > 128 && g0 + 4 < p.aoff.atoms ? 2u : 1u;
+          xi = p.x + p.aoff.xi + (size_t)i0 * p.aoff.xi_stride + (codes ? (size_t)t0 * 128u : (size_t)p.aoff.Mpad * 128u + (size_t)g0 * (NA * SF_ATOM_BYTES));
+          xo = p.x + p.aoff.xo + (size_t)o0 * p.aoff.xo_stride + (size_t)t0 * 128u;
+          sf = p.x + p.aoff.sfb_out + (size_t)g0 * SF_ATOM_BYTES;
+        }, [&](int k, uint8_t* st, uint64_t* bar) {
+          const bool inl = k < NI, first_o = k == NI;
+          if (codes) {
+            const uint32_t bytes = own + (inl ? have * NA * SF_ATOM_BYTES : (first_o ? have * SF_ATOM_BYTES : 0u));
+            if (bytes) ptx::mbar_expect_tx(bar, bytes); else ptx::mbar_arrive(bar);
+            if (own) ptx::bulk_g2s(st + SL_B, inl ? xi + (size_t)k * p.aoff.xi_stride : xo + (size_t)(k - NI) * p.aoff.xo_stride, own, bar);
+          } else if (inl || first_o) {
+            const uint8_t* src = inl ? xi + (size_t)k * p.aoff.xi_stride : sf;
+            const uint32_t nb = inl ? NA * SF_ATOM_BYTES : SF_ATOM_BYTES;
+            ptx::bulk_g2s(st + SL_SF, src, nb, bar);
+            if (have == 2) ptx::bulk_g2s(st + SL_SF + nb, src + 4 * nb, nb, bar);
+          }
+        });
       }
       if (!ok) atomicOr(&p.flags[FLAG_TIMEOUT], 1u);
     }
