@@ -79,26 +79,25 @@ __device__ __forceinline__ int fp8_scale_exp(float amax) {
 __device__ __forceinline__ float pow2_inv_e8m0(uint32_t c) { return __uint_as_float((254u - c) << 23); }
 __device__ __forceinline__ float pow2_neg(int e) { return __uint_as_float((uint32_t)(127 - e) << 23); }
 
-// Two-level scaling (SDQ_SCALE_UE4M3): unsigned E4M3 code of the Q-Vector scale nearest to amax / (6 * 2^t), at least
-// the smallest positive code unless amax == 0, and the value scale * 2^t the elements are divided by (0 for code 0).
-// amax * 2^-t is exact (amax <= 448 * 2^t); the one rounding of the division is far from every E4M3 midpoint or
-// lands on it exactly, so the converter's round-to-nearest-even is that of the exact quotient.
-__device__ __forceinline__ uint32_t ue4m3_scale_code(float amax, int t) {
-  if (amax == 0.0f) return 0u;
-  const uint32_t c = (uint32_t)__nv_cvt_float_to_fp8(__fdiv_rn(scalbnf(amax, -t), 6.0f), __NV_SATFINITE, __NV_E4M3);
-  return c == 0u ? 1u : c;
-}
-__device__ __forceinline__ float ue4m3_scale_value(uint32_t c, int t) {
-  const __half_raw h = __nv_cvt_fp8_to_halfraw((__nv_fp8_storage_t)c, __NV_E4M3);
-  return scalbnf(__half2float(__half(h)), t);
-}
-
-// What the E2M1 converter makes of x / sv for a bf16 x and an E4M3 value sv (times a power of two), without dividing:
-// inv = 1 / sv.  The quotient either equals a rounding boundary of E2M1 (c 2^k, c = 1, 3, 5, 7) or is at least 1 / 255 of it
-// away, since x and boundary * sv are integers below 256 times powers of two; x * inv is within 2^-23 of the quotient, so
-// rounding it to 16 significant bits restores the boundaries and moves nothing across one.
-__device__ __forceinline__ float e2m1_quotient(float x, float inv) {
+// Quotients x / y that are about to be rounded to a small format, without dividing: inv is 1 / y to within 2^-22 of it.  If
+// x and (every rounding boundary) * y are integers below 256 times powers of two, the quotient either equals a boundary or is at
+// least 1 / 255 of it away; x * inv is within 2^-21 of the quotient, so rounding it to 16 significant bits restores the
+// boundaries and moves nothing across one.
+__device__ __forceinline__ float small_quotient(float x, float inv) {
   return __uint_as_float((__float_as_uint(x * inv) + 0x80u) & 0xFFFFFF00u);
+}
+// Two-level scaling (SDQ_SCALE_UE4M3), on magnitudes already multiplied by 2^-t (pow2_neg): unsigned E4M3 code of the Q-Vector
+// scale nearest to a / 6 (ties to even; 6 times an E4M3 midpoint has 8 significant bits), at least the smallest positive code
+// unless a == 0
+__device__ __forceinline__ uint32_t ue4m3_scale_code(float a, bool nonzero) {
+  const uint32_t c = (uint32_t)__nv_cvt_float_to_fp8(small_quotient(a, 1.0f / 6.0f), __NV_SATFINITE, __NV_E4M3);
+  return nonzero ? max(c, 1u) : 0u;
+}
+// 1 / scale of code c > 0 for small_quotient (an E4M3 value times an E2M1 boundary, 1, 3, 5 or 7 times a power of two, has 7
+// significant bits)
+__device__ __forceinline__ float ue4m3_scale_inverse(uint32_t c) {
+  const __half_raw h = __nv_cvt_fp8_to_halfraw((__nv_fp8_storage_t)c, __NV_E4M3);
+  return __fdividef(1.0f, __half2float(__half(h)));
 }
 
 // two floats -> two E2M1 codes in one byte (x in the low nibble)
@@ -116,6 +115,21 @@ __device__ __forceinline__ uint32_t e2m1x8(const float (&v)[8]) {
       "mov.b32 %0, {a, b, c, d};\n}"
       : "=r"(d) : "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]));
   return d;
+}
+// four floats -> four E4M3 codes in one word (the first in the lowest byte)
+__device__ __forceinline__ uint32_t e4m3x4(float a, float b, float c, float d) {
+  uint32_t w;
+  asm("{\n.reg .b16 l, h;\n"
+      "cvt.rn.satfinite.e4m3x2.f32 l, %2, %1;\n"
+      "cvt.rn.satfinite.e4m3x2.f32 h, %4, %3;\n"
+      "mov.b32 %0, {l, h};\n}"
+      : "=r"(w) : "f"(a), "f"(b), "f"(c), "f"(d));
+  return w;
+}
+// running maxima of two packed bf16 magnitudes; a NaN stays, as one above infinity
+__device__ __forceinline__ uint32_t max_abs2(uint32_t m, uint32_t x) {
+  const __nv_bfloat162 r = __hmax2_nan(*reinterpret_cast<const __nv_bfloat162*>(&m), __habs2(*reinterpret_cast<const __nv_bfloat162*>(&x)));
+  return *reinterpret_cast<const uint32_t*>(&r);
 }
 // two floats -> two E4M3 codes in 16 bits (x in the low byte)
 __device__ __forceinline__ uint32_t e4m3x2(float x, float y) {

@@ -186,7 +186,7 @@ sdq_linear_group_kernel(const __grid_constant__ GroupParams p)
       const uint32_t r[8] = {raw[i][0].x, raw[i][0].y, raw[i][0].z, raw[i][0].w, raw[i][1].x, raw[i][1].y, raw[i][1].z, raw[i][1].w};
       uint32_t q = 0;
 #pragma unroll
-      for (int j = 0; j < 8; ++j) q = __vmaxu2(q, r[j] & 0x7FFF7FFFu);
+      for (int j = 0; j < 8; ++j) q = max_abs2(q, r[j]);
       return max(q & 0xFFFFu, q >> 16);
     };
 #pragma unroll

@@ -453,8 +453,8 @@ pack_kernel(const PackParams p, const BlobHeader hdr)
     } else if ((b & 1) || b32) {
       // a Q-Vector is complete: 64 K (both blocks of the half) or 32 K (this one)
       const uint32_t key = max(qmax2 & 0xFFFFu, qmax2 >> 16);
-      const uint32_t c = p.ue ? ue4m3_scale_code(bf16_bits_to_float(key), tw) : e8m0_scale_code_bf16(key, p.ceil_rule != 0);
-      const float inv = p.ue ? __fdiv_rn(1.0f, ue4m3_scale_value(c, tw)) : pow2_inv_e8m0(c);
+      const uint32_t c = p.ue ? ue4m3_scale_code(bf16_bits_to_float(key) * pow2_neg(tw), key != 0) : e8m0_scale_code_bf16(key, p.ceil_rule != 0);
+      const float inv = p.ue ? ue4m3_scale_inverse(max(c, 1u)) : pow2_inv_e8m0(c);
 #pragma unroll
       for (int hb = 0; hb < 2; ++hb) {                   // 32-K block of the half
         if (hb != (b & 1) && b32) continue;              // (one scale per 64 K: both now)
@@ -467,14 +467,14 @@ pack_kernel(const PackParams p, const BlobHeader hdr)
             const float lo = __uint_as_float(w << 16), hi = __uint_as_float(w & 0xFFFF0000u);
             if (p.ue) {
               // (an outlier's position stays +0; the quotient of a dropped one is +0 as well)
-              f[2 * j] = c ? e2m1_quotient(lo, inv) : 0.0f;
-              f[2 * j + 1] = c ? e2m1_quotient(hi, inv) : 0.0f;
+              f[2 * j] = small_quotient(lo * pow2_neg(tw), inv);
+              f[2 * j + 1] = small_quotient(hi * pow2_neg(tw), inv);
             } else {
               f[2 * j] = lo * inv;
               f[2 * j + 1] = hi * inv;
             }
           }
-          in_word[hb][i] = e2m1x8(f);
+          in_word[hb][i] = p.ue && c == 0 ? 0u : e2m1x8(f);
         }
       }
       if (b32) { sc |= c << (8 * b); }

@@ -326,6 +326,10 @@ __device__ __forceinline__ uint32_t mapa_u32(uint32_t saddr, uint32_t cta) {
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(saddr), "r"(cta));
   return ra;
 }
+// asynchronous 4-byte store to a shared::cluster address whose arrival is counted on the mbarrier at `rbar` in the same CTA
+__device__ __forceinline__ void st_async_u32(uint32_t raddr, uint32_t v, uint32_t rbar) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(raddr), "r"(v), "r"(rbar) : "memory");
+}
 // 16-byte load from a shared::cluster address (see mapa_u32)
 __device__ __forceinline__ float4 ld_cluster_f32x4(uint32_t raddr) {
   float4 v;

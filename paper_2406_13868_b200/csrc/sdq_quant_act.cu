@@ -20,6 +20,7 @@
 #include "sdq_internal.h"
 #include "sdq_layout.h"
 #include "sdq_plain.h"
+#include "sdq_ptx.cuh"
 
 namespace sdq {
 
@@ -44,8 +45,8 @@ __device__ __forceinline__ void qa_load(QaUnit& u, const __nv_bfloat16* p, bool 
     }
   }
 }
-// fills qmax and returns the largest magnitude bits of all the lane's elements.  Magnitudes are compared as 15-bit integers,
-// two per word; +-Inf counts as the largest finite bf16: maxima are clamped, the elements only where a lane holds one
+// fills qmax and returns the largest magnitude bits of all the lane's elements.  +-Inf counts as the largest
+// finite bf16: maxima are clamped, the elements only where a lane holds one
 __device__ __forceinline__ uint32_t qa_maxima(QaUnit& u) {
   uint32_t m = 0;
 #pragma unroll
@@ -53,7 +54,7 @@ __device__ __forceinline__ uint32_t qa_maxima(QaUnit& u) {
     const uint32_t r[8] = {u.raw[i][0].x, u.raw[i][0].y, u.raw[i][0].z, u.raw[i][0].w, u.raw[i][1].x, u.raw[i][1].y, u.raw[i][1].z, u.raw[i][1].w};
     uint32_t q = 0;
 #pragma unroll
-    for (int j = 0; j < 8; ++j) q = __vmaxu2(q, r[j] & 0x7FFF7FFFu);
+    for (int j = 0; j < 8; ++j) q = max_abs2(q, r[j]);
     q = max(q & 0xFFFFu, q >> 16);
     u.qmax[i] = q;
     m = max(m, min(q, 0x7F7Fu));
@@ -107,22 +108,22 @@ __device__ __forceinline__ void qa_encode(const QaUnit& u, float ramax, bool liv
         q4[h] = e2m1x8(f);
       }
     } else {
-      c[i] = ue4m3_scale_code(bf16_bits_to_float(bm), e);
+      c[i] = ue4m3_scale_code(bf16_bits_to_float(bm) * s8, bm != 0);
       if (c[i]) {
         // two-level scaling: the Q-Vector scale E4M3(c) * 2^e is not a power of two, the elements are divided by it
-        const float inv = __fdiv_rn(1.0f, ue4m3_scale_value(c[i], e));
+        const float inv = ue4m3_scale_inverse(c[i]);
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
           float f[8];
 #pragma unroll
-          for (int j = 0; j < 8; ++j) f[j] = e2m1_quotient(v[8 * h + j], inv);
+          for (int j = 0; j < 8; ++j) f[j] = small_quotient(v[8 * h + j] * s8, inv);
           q4[h] = e2m1x8(f);
         }
       }
     }
     if (!i8) {
 #pragma unroll
-      for (int j = 0; j < 8; ++j) q8[j >> 1] |= e4m3x2(v[2 * j] * s8, v[2 * j + 1] * s8) << (16 * (j & 1));
+      for (int j = 0; j < 4; ++j) q8[j] = e4m3x4(v[4 * j] * s8, v[4 * j + 1] * s8, v[4 * j + 2] * s8, v[4 * j + 3] * s8);
     } else {
 #pragma unroll
       for (int j = 0; j < 8; ++j) q8[j >> 1] |= (int8_code(v[2 * j], k8) | (int8_code(v[2 * j + 1], k8) << 8)) << (16 * (j & 1));
@@ -214,43 +215,51 @@ quant_act_kernel(const __nv_bfloat16* __restrict__ X, int64_t M, int64_t K, int6
 template <bool UE>
 __global__ void __launch_bounds__(QA_THREADS, UE ? 3 : 4)
 quant_act_fused_kernel(const __nv_bfloat16* __restrict__ X, int64_t M, int64_t K, int64_t ldx, sdq_config_t cfg, uint8_t* __restrict__ buf,
-                       ActOffsets off)
+                       ActOffsets off, uint32_t* __restrict__ flags)
 {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int t = lane >> 2, l = lane & 3;                 // token within the group of 8, quarter of the Q-Vector
+  const uint32_t cx = gridDim.x, rank = blockIdx.x;      // cluster = the gridDim.x CTAs of one token group
+  __shared__ float s_warp[QA_WARPS][8];
+  __shared__ float s_all[8][8];                          // [cluster rank][token]: every CTA's maxima, pushed by their owners
+  __shared__ uint64_t s_bar;                             // ... all of which have arrived
+  if (tid == 0) {
+    ptx::mbar_init(&s_bar, 1);
+    ptx::fence_barrier_init();
+    ptx::mbar_expect_tx(&s_bar, cx * 8u * 4u);
+  }
+  // (waited for before the first push: by then, behind the loads, every CTA's barrier has long been set up)
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
   // launched with programmatic stream serialization: X may still be being written by the previous kernel.  The next launch of
   // the stream is let in before that wait: what it does before its own wait (set-up, fetching packed weights) then overlaps
   // the previous kernel, and its wait for this grid includes this grid's wait for the previous one
   if (tid == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  const uint32_t cx = gridDim.x, rank = blockIdx.x;      // cluster = the gridDim.x CTAs of one token group
   const int64_t m = (int64_t)blockIdx.y * 8 + t;
   const bool live = m < M;
   const int k2 = (int)rank * QA_WARPS + warp;            // this warp's unit
   const bool on = k2 < (int)(K / K2);
-  __shared__ float s_warp[QA_WARPS][8];
-  __shared__ float s_all[8][8];                          // [cluster rank][token]: every CTA's maxima, pushed by their owners
-
   QaUnit u;
   qa_load(u, X + m * ldx + (int64_t)k2 * K2 + l * 16, live && on);
   float amax = bf16_bits_to_float(qa_maxima(u));
   amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, 1));
   amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, 2));
   if (l == 0) s_warp[warp][t] = amax;
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
   __syncthreads();
   if (tid < 8 * (int)cx) {
-    // thread (peer, token): this CTA's maximum of the token goes into row `rank` of the peer's table
+    // thread (peer, token): this CTA's maximum of the token goes into row `rank` of the peer's table; the store counts its bytes
+    // on the peer's barrier, so that nothing but its own copies' arrival keeps a CTA waiting (a cluster barrier behind
+    // plain stores cost a quarter of the stalls)
     const int tok = tid & 7;
     const uint32_t peer = (uint32_t)tid >> 3;
     float a = 0.0f;
 #pragma unroll
     for (int w = 0; w < QA_WARPS; ++w) a = fmaxf(a, s_warp[w][tok]);
-    uint32_t ra;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"((uint32_t)__cvta_generic_to_shared(&s_all[rank][tok])), "r"(peer));
-    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(ra), "f"(a) : "memory");
+    ptx::st_async_u32(ptx::mapa_u32(ptx::smem_u32(&s_all[rank][tok]), peer), __float_as_uint(a), ptx::mapa_u32(ptx::smem_u32(&s_bar), peer));
   }
-  // one barrier: every push is visible after it, and nobody touches another CTA's memory afterwards
-  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  // no CTA leaves before all pushes to it have arrived, and its own go to CTAs that wait for them
+  if (!ptx::mbar_wait_cluster(&s_bar, 0) && lane == 0) atomicOr(&flags[FLAG_TIMEOUT], 1u);
   float ramax = 0.0f;
   for (uint32_t c = 0; c < cx; ++c) ramax = fmaxf(ramax, s_all[c][t]);
   if (live && rank == 0 && warp == 0) qa_token_scale<UE>(ramax, m, (uint32_t)l, cfg, buf, off);
@@ -311,6 +320,8 @@ extern "C" sdq_status_t sdq_quantize_act(const void* X, int64_t M, int64_t K, in
   const bool ue = cfg->scale_rule == SDQ_SCALE_UE4M3;
   const int n_chunks = (int)((K + QA_CHUNK - 1) / QA_CHUNK);      // = CTAs per token group: one 256-K unit per warp
   if (n_chunks <= 8) {
+    uint32_t* flags = device_flags();
+    if (!flags) return SDQ_ERR_CUDA;
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3((unsigned)n_chunks, (unsigned)((M + 7) / 8));
     lc.blockDim = dim3(QA_THREADS);
@@ -324,8 +335,8 @@ extern "C" sdq_status_t sdq_quantize_act(const void* X, int64_t M, int64_t K, in
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     lc.attrs = attr;
     lc.numAttrs = 2;
-    const cudaError_t le = ue ? cudaLaunchKernelEx(&lc, quant_act_fused_kernel<true>, Xb, M, K, ldx, *cfg, bufp, off)
-                              : cudaLaunchKernelEx(&lc, quant_act_fused_kernel<false>, Xb, M, K, ldx, *cfg, bufp, off);
+    const cudaError_t le = ue ? cudaLaunchKernelEx(&lc, quant_act_fused_kernel<true>, Xb, M, K, ldx, *cfg, bufp, off, flags)
+                              : cudaLaunchKernelEx(&lc, quant_act_fused_kernel<false>, Xb, M, K, ldx, *cfg, bufp, off, flags);
     if (le != cudaSuccess || cudaGetLastError() != cudaSuccess) return SDQ_ERR_CUDA;
   } else {
     float* partial = reinterpret_cast<float*>(bufp + off.amax);
