@@ -126,6 +126,12 @@ __device__ __forceinline__ uint32_t e4m3x4(float a, float b, float c, float d) {
       : "=r"(w) : "f"(a), "f"(b), "f"(c), "f"(d));
   return w;
 }
+// bytes of {b, a} picked by the four nibbles of sel (bit 3 of a nibble: the byte's sign bit, spread over it)
+__device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
+  uint32_t d;
+  asm("prmt.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(sel));
+  return d;
+}
 // running maxima of two packed bf16 magnitudes; a NaN stays, as one above infinity
 __device__ __forceinline__ uint32_t max_abs2(uint32_t m, uint32_t x) {
   const __nv_bfloat162 r = __hmax2_nan(*reinterpret_cast<const __nv_bfloat162*>(&m), __habs2(*reinterpret_cast<const __nv_bfloat162*>(&x)));

@@ -11,7 +11,7 @@
 // What bounds it: the integer pipe (77 % busy at ~140 instructions per S-Vector; selections on packed keys instead of index
 // loops took it from ~350 over two passes), DRAM is at 30 %.  11008 x 4096, 1:8 + pair-wise 4:8: 189 us as one kernel with a
 // CTA per row and a thread per S-Vector scattering bytes -> 20 + 42 us with the row scales in a launch of their own ->
-// 51 us.
+// 49 us.  4096 x 11008, 1:8 + 6:8 with channel weights: 98 us choosing in both passes -> 67.
 #include <cstring>
 #include <type_traits>
 #include <mutex>
@@ -33,8 +33,9 @@ __device__ __forceinline__ void rank_keys(const uint32_t (&r)[4], const float* _
   if constexpr (!WGT) {
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      k[2 * j] = (int)(((r[j] & 0x7FFFu) << 16) | (uint32_t)(7 - 2 * j));
-      k[2 * j + 1] = (int)((r[j] & 0x7FFF0000u) | (uint32_t)(6 - 2 * j));
+      const uint32_t a = r[j] & 0x7FFF7FFFu;
+      k[2 * j] = (int)prmt(a, (uint32_t)(7 - 2 * j), 0x1054u);
+      k[2 * j + 1] = (int)((a & 0xFFFF0000u) | (uint32_t)(6 - 2 * j));
     }
   } else {
     const float4 c0 = __ldg(reinterpret_cast<const float4*>(c)), c1 = __ldg(reinterpret_cast<const float4*>(c) + 1);
@@ -46,27 +47,33 @@ __device__ __forceinline__ void rank_keys(const uint32_t (&r)[4], const float* _
     }
   }
 }
-// position of the largest key of k[B .. B + n), ties to the lower index
+// position of the largest key of k[B .. E), ties to the lower index
 template <bool WGT, int B, int E>
 __device__ __forceinline__ int arg_max(const int (&k)[8]) {
-  int best = k[B], at = B;
+  if constexpr (!WGT) {
+    int best = __vimax3_s32(k[B], k[B + 1], k[B + 2]);
+    if constexpr (E - B == 8) best = __vimax3_s32(__vimax3_s32(k[B + 4], k[B + 5], k[B + 6]), k[B + 7], best);
+    return 7 - (max(best, k[B + 3]) & 7);
+  } else {
+    int best = k[B], at = B;
 #pragma unroll
-  for (int i = B + 1; i < E; ++i) {
-    if constexpr (WGT) { if (k[i] > best) { best = k[i]; at = i; } }
-    else best = max(best, k[i]);
+    for (int i = B + 1; i < E; ++i)
+      if (k[i] > best) { best = k[i]; at = i; }
+    return at;
   }
-  return WGT ? at : 7 - (best & 7);
 }
 // position of the smallest key, ties to the higher index (the last in rank order)
 template <bool WGT>
 __device__ __forceinline__ int arg_min(const int (&k)[8]) {
-  int best = k[0], at = 0;
+  if constexpr (!WGT) {
+    return 7 - (min(__vimin3_s32(__vimin3_s32(k[0], k[1], k[2]), k[3], k[4]), __vimin3_s32(k[5], k[6], k[7])) & 7);
+  } else {
+    int best = k[0], at = 0;
 #pragma unroll
-  for (int i = 1; i < 8; ++i) {
-    if constexpr (WGT) { if (k[i] <= best) { best = k[i]; at = i; } }
-    else best = min(best, k[i]);
+    for (int i = 1; i < 8; ++i)
+      if (k[i] <= best) { best = k[i]; at = i; }
+    return at;
   }
-  return WGT ? at : 7 - (best & 7);
 }
 // Stage 2: positions of the outliers, ascending (-1: none).  order_mask turns the ranking round when the least significant
 // values are taken (SDQ_ORDER_SMALL); sv4: S-Vectors of 4, one outlier in each half.
@@ -76,7 +83,10 @@ __device__ __forceinline__ void pick_outliers(const int (&key)[8], int order_mas
   if constexpr (OUTN > 0) {
     int k[8];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) k[i] = key[i] ^ order_mask;
+    for (int i = 0; i < 8; ++i) k[i] = key[i];
+    if (order_mask)
+#pragma unroll
+      for (int i = 0; i < 8; ++i) k[i] ^= order_mask;
     if (OUTN == 2 && sv4) {
       o0 = arg_max<WGT, 0, 4>(k);
       o1 = arg_max<WGT, 4, 8>(k);
@@ -95,14 +105,26 @@ __device__ __forceinline__ void pick_outliers(const int (&key)[8], int order_mas
 }
 // element `at` of the S-Vector as a float
 __device__ __forceinline__ float pick_value(const uint32_t (&r)[4], int at) {
-  const uint32_t w = (at & 4) ? ((at & 2) ? r[3] : r[2]) : ((at & 2) ? r[1] : r[0]);
-  return __uint_as_float((at & 1) ? (w & 0xFFFF0000u) : (w << 16));
+  const uint32_t sel = (uint32_t)(at & 3) * 0x2200u + 0x1000u;      // its two bytes, to the upper half
+  return __uint_as_float(((at & 4) ? prmt(r[2], r[3], sel) : prmt(r[0], r[1], sel)) & 0xFFFF0000u);
 }
+// bf16 bits of |x|
+__device__ __forceinline__ uint32_t magnitude(float x) { return __float_as_uint(x) << 1 >> 17; }
+__device__ __forceinline__ uint32_t larger_half(uint32_t x) { return max(x & 0xFFFFu, x >> 16); }
 // r with position `at` zeroed (at = -1: nothing)
 __device__ __forceinline__ void zero_at(uint32_t (&r)[4], int at) {
   const uint32_t keep = (at & 1) ? 0x0000FFFFu : 0xFFFF0000u;
 #pragma unroll
   for (int j = 0; j < 4; ++j) r[j] &= (at >> 1) == j ? keep : 0xFFFFFFFFu;
+}
+// r with the positions of the set `gone` (bit i: position i) zeroed: bit i of four goes to the top of byte i, whose sign is
+// then spread over a half word
+__device__ __forceinline__ void zero_set(uint32_t (&r)[4], uint32_t gone) {
+  const uint32_t lo = (gone & 15u) * 0x10204080u, hi = ((gone >> 4) & 15u) * 0x10204080u;
+  r[0] &= ~prmt(lo, 0u, 0x9988u);
+  r[1] &= ~prmt(lo, 0u, 0xBBAAu);
+  r[2] &= ~prmt(hi, 0u, 0x9988u);
+  r[3] &= ~prmt(hi, 0u, 0xBBAAu);
 }
 // Stage 1, pair-wise 4:8: the 2 pairs (of 4) with the largest summed significance among the non-outliers (x: outliers
 // zeroed), largest first, ties to the lower index.  A pair stays if it comes before at least two of the other three.
@@ -129,20 +151,25 @@ __device__ __forceinline__ void pick_pairs(const uint32_t (&x)[4], const int (&k
   w1 = k3 ? x[3] : (k2 ? x[2] : x[1]);
   nibble = (k0 ? 0u : (k1 ? 1u : 2u)) | (k3 ? 12u : (k2 ? 8u : 4u));
 }
-// Stage 1 for the patterns stored dense: nibble i of the result is 15 if position i holds +0 -- the outliers and, among the
-// others, all but the keep_in most significant (of every 8, or of every 4 with grp4).  k: ranking keys, -1 at the outliers.
+// Stage 1 for the patterns stored dense: the set of positions that hold +0 -- the outliers and, among the others, all but the
+// keep_in most significant (of every 8, or of every 4 with grp4).  k: ranking keys.
 template <bool WGT, int OUTN>
-__device__ __forceinline__ uint32_t dropped_nibbles(int (&k)[8], int o0, int o1, int keep_in, bool grp4) {
-  uint32_t m = 0;                                   // bit 4 i: position i holds +0
+__device__ __forceinline__ uint32_t dropped_set(int (&k)[8], int o0, int o1, int keep_in, bool grp4, int order_mask) {
+  uint32_t m = 0;
+  if (OUTN > 0) m |= 1u << o0;
+  if (OUTN > 1) m |= 1u << o1;
   if (!grp4 && keep_in + OUTN >= 7) {
-    if (OUTN > 0) m |= 1u << (4 * o0);
-    if (OUTN > 1) m |= 1u << (4 * o1);
-    if (keep_in + OUTN == 7) {                      // exactly one value more: the last in rank order
+    if (keep_in + OUTN == 7) {
+      // exactly one value more: the last in rank order, which is no outlier unless these are the least significant
+      if (OUTN > 0 && order_mask)
 #pragma unroll
-      for (int i = 0; i < 8; ++i) k[i] = k[i] < 0 ? 0x7FFFFFFF : k[i];
-      m |= 1u << (4 * arg_min<WGT>(k));
+        for (int i = 0; i < 8; ++i) k[i] = (m >> i) & 1u ? 0x7FFFFFFF : k[i];
+      m |= 1u << arg_min<WGT>(k);
     }
   } else {
+    if (OUTN > 0)
+#pragma unroll
+      for (int i = 0; i < 8; ++i) k[i] = (m >> i) & 1u ? -1 : k[i];
     uint32_t rank = 0;                              // nibble i: how many come before position i
 #pragma unroll
     for (int i = 0; i < 8; ++i)
@@ -151,8 +178,11 @@ __device__ __forceinline__ uint32_t dropped_nibbles(int (&k)[8], int o0, int o1,
         if ((i >> 2) == (j >> 2) || !grp4) rank += k[i] >= k[j] ? (1u << (4 * j)) : (1u << (4 * i));
       }
     m = ((rank + (uint32_t)(8 - keep_in) * 0x11111111u) >> 3) & 0x11111111u;
+    m = (m | m >> 3) & 0x03030303u;                 // every fourth bit -> 8 bits
+    m = (m | m >> 6) & 0x000F000Fu;
+    m = (m | m >> 12) & 0xFFu;
   }
-  return m * 15u;
+  return m;
 }
 
 struct PackParams {
@@ -187,25 +217,38 @@ __device__ __forceinline__ void store_header(const PackParams& p, const BlobHead
   if (threadIdx.x < HEADER_BYTES / 4)
     reinterpret_cast<uint32_t*>(p.blob)[threadIdx.x] = threadIdx.x < sizeof(BlobHeader) / 4 ? reinterpret_cast<const uint32_t*>(&hdr)[threadIdx.x] : 0u;
 }
-// the largest outlier (and, two-level scaling, the largest inlier that stays) of one S-Vector, into running maxima
+// the choices of one S-Vector: outlier positions and values, pattern nibble and the two pairs that stay, outlier positions at +0
+template <bool WGT, int OUTN>
+__device__ __forceinline__ void choose_pairs(const PackParams& p, uint32_t (&r)[4], const float* c, int& o0, int& o1, float& f0, float& f1,
+                                             uint32_t& w0, uint32_t& w1, uint32_t& nibble) {
+  int k[8];
+  rank_keys<WGT>(r, c, k);
+  pick_outliers<WGT, OUTN>(k, p.order_mask, p.sv4 != 0, o0, o1);
+  f0 = OUTN > 0 ? pick_value(r, o0) : 0.0f;
+  f1 = OUTN > 1 ? pick_value(r, o1) : 0.0f;
+  if constexpr (OUTN > 0) zero_at(r, o0);
+  if constexpr (OUTN > 1) zero_at(r, o1);
+  pick_pairs<WGT>(r, k, o0, o1, w0, w1, nibble);
+}
+// its largest outlier (and, two-level scaling, the largest inlier that stays), into running maxima
 template <bool WGT, int OUTN>
 __device__ __forceinline__ void group_maxima(const PackParams& p, uint32_t (&r)[4], const float* c, uint32_t& omax, uint32_t& imax) {
   int k[8], o0, o1;
   rank_keys<WGT>(r, c, k);
   pick_outliers<WGT, OUTN>(k, p.order_mask, p.sv4 != 0, o0, o1);
-  if constexpr (OUTN > 0) omax = max(omax, __float_as_uint(pick_value(r, o0)) << 1 >> 17);
-  if constexpr (OUTN > 1) omax = max(omax, __float_as_uint(pick_value(r, o1)) << 1 >> 17);
-  if (p.ue) {                                                     // pair-wise pattern
+  if constexpr (OUTN > 0) omax = max(omax, magnitude(pick_value(r, o0)));
+  if constexpr (OUTN > 1) omax = max(omax, magnitude(pick_value(r, o1)));
+  if (p.ue) {                                            // pair-wise pattern
     if constexpr (OUTN > 0) zero_at(r, o0);
     if constexpr (OUTN > 1) zero_at(r, o1);
     uint32_t w0, w1, nibble;
     pick_pairs<WGT>(r, k, o0, o1, w0, w1, nibble);
-    const uint32_t m = __vmaxu2(w0 & 0x7FFF7FFFu, w1 & 0x7FFF7FFFu);
-    imax = max(imax, max(m & 0xFFFFu, m >> 16));
+    imax = max_abs2(max_abs2(imax, w0), w1);
   }
 }
-__device__ __forceinline__ uint32_t max_magnitudes(const uint32_t (&r)[4]) {      // two packed maxima
-  return __vmaxu2(__vmaxu2(r[0] & 0x7FFF7FFFu, r[1] & 0x7FFF7FFFu), __vmaxu2(r[2] & 0x7FFF7FFFu, r[3] & 0x7FFF7FFFu));
+// two packed running maxima of the magnitudes
+__device__ __forceinline__ uint32_t max_magnitudes(uint32_t m, const uint32_t (&r)[4]) {
+  return max_abs2(max_abs2(max_abs2(max_abs2(m, r[0]), r[1]), r[2]), r[3]);
 }
 __device__ __forceinline__ bool bad_weight(float c) { return !(c >= 0.0f && c <= 3.4028234663852886e38f); }
 
@@ -229,28 +272,32 @@ row_scale_kernel(const PackParams p, const BlobHeader hdr)
 #pragma unroll
       for (int u = 0; u < 4; ++u) v[u] = __ldg(row + g + 32 * u);
 #pragma unroll
-      for (int u = 0; u < 4; ++u)
-        all2 = __vmaxu2(all2, __vmaxu2(__vmaxu2(v[u].x & 0x7FFF7FFFu, v[u].y & 0x7FFF7FFFu), __vmaxu2(v[u].z & 0x7FFF7FFFu, v[u].w & 0x7FFF7FFFu)));
+      for (int u = 0; u < 4; ++u) {
+        const uint32_t r[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
+        all2 = max_magnitudes(all2, r);
+      }
     }
     for (; g < G; g += 32) {
       const uint4 v = __ldg(row + g);
-      all2 = __vmaxu2(all2, __vmaxu2(__vmaxu2(v.x & 0x7FFF7FFFu, v.y & 0x7FFF7FFFu), __vmaxu2(v.z & 0x7FFF7FFFu, v.w & 0x7FFF7FFFu)));
+      const uint32_t r[4] = {v.x, v.y, v.z, v.w};
+      all2 = max_magnitudes(all2, r);
     }
-    omax = max(all2 & 0xFFFFu, all2 >> 16);
+    omax = larger_half(all2);
     bad = omax >= 0x7F80u;
   } else {
 #pragma unroll 2
     for (int g = (int)lane; g < G; g += 32) {
       const uint4 v = __ldg(row + g);
       uint32_t r[4] = {v.x, v.y, v.z, v.w};
-      all2 = __vmaxu2(all2, max_magnitudes(r));
+      all2 = max_magnitudes(all2, r);
       if constexpr (WGT) {
 #pragma unroll
         for (int i = 0; i < 8; ++i) bad |= bad_weight(__ldg(p.colw + 8 * (int64_t)g + i));
       }
       group_maxima<WGT, OUTN>(p, r, WGT ? p.colw + 8 * (int64_t)g : nullptr, omax, imax);
     }
-    bad |= max(all2 & 0xFFFFu, all2 >> 16) >= 0x7F80u;
+    bad |= larger_half(all2) >= 0x7F80u;
+    imax = larger_half(imax);
   }
   omax = __reduce_max_sync(0xffffffffu, omax);
   imax = __reduce_max_sync(0xffffffffu, imax);
@@ -266,7 +313,8 @@ constexpr int PK_THREADS = 256, PK_ROWS = 16, PK_K = 2048;
 constexpr int PK_PITCH = PK_K * 2 + 16;                  // bytes between rows of the staged tile
 constexpr int PK_SMEM = PK_ROWS * PK_PITCH;              // 65792: three CTAs per SM
 
-template <bool DENSE, bool WGT, int OUTN, bool FUSED>
+// CHOSEN: the first pass chooses for good (see there)
+template <bool DENSE, bool WGT, bool CHOSEN, int OUTN, bool FUSED>
 __global__ void __launch_bounds__(PK_THREADS, 3)
 pack_kernel(const PackParams p, const BlobHeader hdr)
 {
@@ -294,27 +342,64 @@ pack_kernel(const PackParams p, const BlobHeader hdr)
   const int kc = rank * 16 + (int)ch;                    // ... and of the matrix
   const bool on = kc < T1;
   const int64_t n = n_first + row;
-  const uint8_t* mine = tile + row * PK_PITCH + ch * 256;
+  uint8_t* mine = tile + row * PK_PITCH + ch * 256;
   const float* colw = WGT ? p.colw + (int64_t)kc * K1 : nullptr;
   __syncthreads();
 
+  // ---- first pass: the choices, the row's largest outlier (and inlier), non-finite check.
+  // CHOSEN, pair-wise: everything is chosen here and the S-Vector's 16 bytes in the tile become what is left to encode, the two
+  // pairs that stay and the outliers' values; positions and pattern nibbles are collected in registers, as the layout wants
+  // them.  CHOSEN, stored dense: the same, but the values stay where they are and the sets of dropped positions are collected.
+  // Otherwise the second pass chooses: the outliers, if the most significant by magnitude, hold the row's largest magnitude,
+  // and then this pass has to choose nothing.
+  [[maybe_unused]] uint32_t c_o0[2] = {0, 0}, c_o1[2] = {0, 0}, c_nib[2] = {0, 0}, c_gone[4] = {0, 0, 0, 0};
+  uint32_t all2 = 0, omax = 0, imax = 0, bad = 0;        // all2, imax: packed running maxima
+  if constexpr (CHOSEN) {
+    const bool look_at_all = WGT || OUTN == 0 || p.order_mask;    // for non-finite values: otherwise they are outliers
+    if (on) {
+#pragma unroll
+      for (int i = 0; i < 16; ++i) {
+        uint4* at = reinterpret_cast<uint4*>(mine) + i;
+        const uint4 v = *at;
+        uint32_t r[4] = {v.x, v.y, v.z, v.w};
+        const float* c = WGT ? colw + 8 * i : nullptr;
+        int o0, o1;
+        float f0, f1;
+        if (look_at_all) all2 = max_magnitudes(all2, r);
+        if constexpr (!DENSE) {
+          uint32_t w0, w1, nibble;
+          choose_pairs<WGT, OUTN>(p, r, c, o0, o1, f0, f1, w0, w1, nibble);
+          if (p.ue) imax = max_abs2(max_abs2(imax, w0), w1);
+          *at = make_uint4(w0, w1, __float_as_uint(f0), __float_as_uint(f1));
+          c_nib[i >> 3] |= nibble << (4 * (i & 7));
+        } else {
+          int k[8];
+          rank_keys<WGT>(r, c, k);
+          pick_outliers<WGT, OUTN>(k, p.order_mask, p.sv4 != 0, o0, o1);
+          f0 = OUTN > 0 ? pick_value(r, o0) : 0.0f;
+          f1 = OUTN > 1 ? pick_value(r, o1) : 0.0f;
+          c_gone[i >> 2] |= dropped_set<WGT, OUTN>(k, o0, o1, p.keep_in, p.sv4 || p.elem, p.order_mask) << (8 * (i & 3));
+        }
+        if constexpr (OUTN > 0) { omax = max(omax, magnitude(f0)); c_o0[i >> 3] |= (uint32_t)o0 << (4 * (i & 7)); }
+        if constexpr (OUTN > 1) { omax = max(omax, magnitude(f1)); c_o1[i >> 3] |= (uint32_t)o1 << (4 * (i & 7)); }
+      }
+    }
+  }
   int e, tw;
   if constexpr (FUSED) {
-    // ---- first pass: the row's largest outlier (and inlier), non-finite check.  By magnitude, most significant first, the
-    // outliers hold the row's largest magnitude, so nothing has to be selected.
-    uint32_t all2 = 0, omax = 0, imax = 0, bad = 0;
     if (on) {
-      const bool select = WGT || p.order_mask || p.ue;
+      if constexpr (!CHOSEN) {
 #pragma unroll 4
-      for (int i = 0; i < 16; ++i) {
-        const uint4 v = *reinterpret_cast<const uint4*>(mine + i * 16);
-        uint32_t r[4] = {v.x, v.y, v.z, v.w};
-        all2 = __vmaxu2(all2, max_magnitudes(r));
-        if (select) group_maxima<WGT, OUTN>(p, r, WGT ? colw + 8 * i : nullptr, omax, imax);
+        for (int i = 0; i < 16; ++i) {
+          const uint4 v = *reinterpret_cast<const uint4*>(mine + i * 16);
+          uint32_t r[4] = {v.x, v.y, v.z, v.w};
+          all2 = max_magnitudes(all2, r);
+          if (DENSE && p.order_mask) group_maxima<false, OUTN>(p, r, nullptr, omax, imax);
+        }
+        if (!DENSE || !p.order_mask) omax = OUTN ? larger_half(all2) : 0u;
       }
-      const uint32_t all = max(all2 & 0xFFFFu, all2 >> 16);
-      if (!select) omax = all;
-      bad = all >= 0x7F80u;
+      imax = larger_half(imax);
+      bad = max(omax, larger_half(all2)) >= 0x7F80u;
       if (WGT && first_rows)                             // the channel weights are the same for every row
         for (int i = (int)row; i < K1; i += PK_ROWS) bad |= bad_weight(__ldg(colw + i));
     }
@@ -359,8 +444,8 @@ pack_kernel(const PackParams p, const BlobHeader hdr)
   const uint32_t core = (r >> 3) * 256 + (r & 7) * 16;   // this row inside a K-block of an A operand
 
   uint32_t in_word[2][2];                                // pair-wise inliers: the 64-K half's codes, two S-Vectors per word
-  uint32_t nib = 0, sc = 0;                              // its pattern nibbles; scale bytes of the 128 K
-  uint32_t nibs[2], codes[4], sels[4], metas[4];         // pattern nibbles and outlier bytes of the 128 K
+  uint32_t sc = 0;                                       // scale bytes of the 128 K
+  uint32_t codes[4], sels[4], metas[4];                  // outlier bytes of the 128 K
   uint32_t kept[16];                                     // pair-wise inliers of a Q-Vector of 64 K, outlier positions zeroed
   uint32_t qmax2 = 0;                                    // packed running maximum of the Q-Vector
 #pragma unroll
@@ -371,51 +456,44 @@ pack_kernel(const PackParams p, const BlobHeader hdr)
     for (int i = 0; i < 4; ++i) {
       const uint4 v = *reinterpret_cast<const uint4*>(mine + (4 * b + i) * 16);
       uint32_t x[4] = {v.x, v.y, v.z, v.w};
-      int k[8], o0, o1;
-      rank_keys<WGT>(x, WGT ? colw + 8 * (4 * b + i) : nullptr, k);
-      pick_outliers<WGT, OUTN>(k, p.order_mask, p.sv4 != 0, o0, o1);
+      const int sv = 4 * b + i;
+      [[maybe_unused]] int k[8];
+      int o0, o1;
+      [[maybe_unused]] float f0, f1;
+      if constexpr (!DENSE && !CHOSEN) {
+        uint32_t w0, w1, nibble;
+        choose_pairs<WGT, OUTN>(p, x, WGT ? colw + 8 * sv : nullptr, o0, o1, f0, f1, w0, w1, nibble);
+        x[0] = w0;
+        x[1] = w1;
+        c_nib[sv >> 3] |= nibble << (4 * (sv & 7));
+      } else if constexpr (CHOSEN) {
+        o0 = (int)((c_o0[sv >> 3] >> (4 * (sv & 7))) & 7u);
+        o1 = (int)((c_o1[sv >> 3] >> (4 * (sv & 7))) & 7u);
+      } else {
+        rank_keys<false>(x, nullptr, k);
+        pick_outliers<false, OUTN>(k, p.order_mask, p.sv4 != 0, o0, o1);
+      }
       // Stage 3, outliers: E4M3 codes of w / 2^e, or int8 codes of w / s
       if constexpr (OUTN > 0) {
-        const float f = pick_value(x, o0);
-        ocode[i] = p.i8 ? int8_code(f, __int_as_float(e)) : e4m3x1(f * s8);
+        const float f = DENSE ? pick_value(x, o0) : (CHOSEN ? __uint_as_float(x[2]) : f0);
+        ocode[i] = !DENSE && p.i8 ? int8_code(f, __int_as_float(e)) : e4m3x1(f * s8);
         opos[i] = (uint32_t)o0;
       }
       if constexpr (OUTN > 1) {
-        const float f = pick_value(x, o1);
-        ocode1[i] = p.i8 ? int8_code(f, __int_as_float(e)) : e4m3x1(f * s8);
+        const float f = DENSE ? pick_value(x, o1) : (CHOSEN ? __uint_as_float(x[3]) : f1);
+        ocode1[i] = !DENSE && p.i8 ? int8_code(f, __int_as_float(e)) : e4m3x1(f * s8);
         opos1[i] = (uint32_t)o1;
       }
       if constexpr (!DENSE) {
-        // Stage 1: the two pairs that stay, outlier positions at +0
-        if constexpr (OUTN > 0) zero_at(x, o0);
-        if constexpr (OUTN > 1) zero_at(x, o1);
-        uint32_t w0, w1, nibble;
-        pick_pairs<WGT>(x, k, o0, o1, w0, w1, nibble);
-        kept[2 * (4 * (b & 1) + i)] = w0;
-        kept[2 * (4 * (b & 1) + i) + 1] = w1;
-        qmax2 = __vmaxu2(qmax2, __vmaxu2(w0 & 0x7FFF7FFFu, w1 & 0x7FFF7FFFu));
-        nib |= nibble << (4 * (4 * (b & 1) + i));
+        kept[2 * (4 * (b & 1) + i)] = x[0];
+        kept[2 * (4 * (b & 1) + i) + 1] = x[1];
+        qmax2 = max_abs2(max_abs2(qmax2, x[0]), x[1]);
       } else {
-        if constexpr (OUTN > 0) {
-#pragma unroll
-          for (int j = 0; j < 8; ++j) k[j] = (j == o0 || (OUTN > 1 && j == o1)) ? -1 : k[j];
-        }
-        uint32_t mag = 0;                                // largest magnitude of the inliers
-        if constexpr (!WGT) {
-#pragma unroll
-          for (int j = 0; j < 8; ++j) mag = (uint32_t)max((int)mag, k[j]);   // the most significant non-outlier always stays
-          mag >>= 16;
-        }
-        const uint32_t gone = dropped_nibbles<WGT, OUTN>(k, o0, o1, p.keep_in, p.sv4 || p.elem);
-        if constexpr (WGT) {
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            mag = max(mag, (gone >> (8 * j)) & 1u ? 0u : (x[j] & 0x7FFFu));
-            mag = max(mag, (gone >> (8 * j + 4)) & 1u ? 0u : ((x[j] >> 16) & 0x7FFFu));
-          }
-        }
-        qmax2 = max(qmax2, mag);
-        dense_codes[i] = ~gone;
+        uint32_t gone;
+        if constexpr (CHOSEN) gone = (c_gone[b] >> (8 * i)) & 255u;
+        else gone = dropped_set<false, OUTN>(k, o0, o1, p.keep_in, p.sv4 || p.elem, p.order_mask);
+        zero_set(x, gone);
+        qmax2 = max_magnitudes(qmax2, x);
 #pragma unroll
         for (int j = 0; j < 4; ++j) dval[4 * i + j] = x[j];
         if (p.elem) {
@@ -423,8 +501,7 @@ pack_kernel(const PackParams p, const BlobHeader hdr)
           uint32_t mb = 0;
 #pragma unroll
           for (int q = 0; q < 2; ++q) {
-            const uint32_t g4 = ~gone >> (16 * q);       // nibbles of the group's four positions, exactly two of them set
-            const uint32_t bits = (g4 & 1u) | ((g4 >> 3) & 2u) | ((g4 >> 6) & 4u) | ((g4 >> 9) & 8u);
+            const uint32_t bits = (~gone >> (4 * q)) & 15u;          // the group's four positions, exactly two of them set
             mb |= (uint32_t)((__ffs((int)bits) - 1) | ((31 - __clz((int)bits)) << 2)) << (8 * q);
           }
           reinterpret_cast<uint16_t*>(p.blob + p.off.emeta + (size_t)n * (size_t)(p.K / 4))[(k2 * 2 + (int)h) * 16 + 4 * b + i] = (uint16_t)mb;
@@ -434,7 +511,7 @@ pack_kernel(const PackParams p, const BlobHeader hdr)
 
     // ---- Stage 3, inliers
     if constexpr (DENSE) {
-      const uint32_t c = e8m0_scale_code_bf16(qmax2, p.ceil_rule != 0);
+      const uint32_t c = e8m0_scale_code_bf16(larger_half(qmax2), p.ceil_rule != 0);
       const float inv = pow2_inv_e8m0(c);
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
@@ -444,7 +521,7 @@ pack_kernel(const PackParams p, const BlobHeader hdr)
           f[2 * j] = __uint_as_float(dval[4 * i + j] << 16) * inv;
           f[2 * j + 1] = __uint_as_float(dval[4 * i + j] & 0xFFFF0000u) * inv;
         }
-        dense_codes[i] &= e2m1x8(f);
+        dense_codes[i] = e2m1x8(f);
       }
       // 16 code bytes per 32 K: K-block (64 K) 2 h + b / 2 of the record, chunk b & 1
       *reinterpret_cast<uint4*>(wi + (2 * h + (b >> 1)) * 4096 + core + (b & 1) * 128) = make_uint4(dense_codes[0], dense_codes[1], dense_codes[2], dense_codes[3]);
@@ -452,7 +529,7 @@ pack_kernel(const PackParams p, const BlobHeader hdr)
       qmax2 = 0;
     } else if ((b & 1) || b32) {
       // a Q-Vector is complete: 64 K (both blocks of the half) or 32 K (this one)
-      const uint32_t key = max(qmax2 & 0xFFFFu, qmax2 >> 16);
+      const uint32_t key = larger_half(qmax2);
       const uint32_t c = p.ue ? ue4m3_scale_code(bf16_bits_to_float(key) * pow2_neg(tw), key != 0) : e8m0_scale_code_bf16(key, p.ceil_rule != 0);
       const float inv = p.ue ? ue4m3_scale_inverse(max(c, 1u)) : pow2_inv_e8m0(c);
 #pragma unroll
@@ -483,10 +560,8 @@ pack_kernel(const PackParams p, const BlobHeader hdr)
     }
     if constexpr (!DENSE) {
       if (b & 1) {
-        // 16 code bytes per 64 K (K-block h, chunk b / 2) and 4 bytes of pattern nibbles
+        // 16 code bytes per 64 K (K-block h, chunk b / 2)
         *reinterpret_cast<uint4*>(wi + h * 4096 + core + (b >> 1) * 128) = make_uint4(in_word[0][0], in_word[0][1], in_word[1][0], in_word[1][1]);
-        nibs[b >> 1] = nib;
-        nib = 0;
       }
     }
 
@@ -497,7 +572,7 @@ pack_kernel(const PackParams p, const BlobHeader hdr)
       // first, or (0, 3), the value second, when p = 3; the other group has slots (0, 1).  Metadata bytes and byte shifts
       // come from 8-entry tables looked up by byte-permutes, the four position nibbles being the selector.
       codes[b] = ocode[0] | (ocode[1] << 8) | (ocode[2] << 16) | (ocode[3] << 24);
-      const uint32_t sel = opos[0] | (opos[1] << 4) | (opos[2] << 8) | (opos[3] << 12);
+      const uint32_t sel = CHOSEN ? (c_o0[b >> 1] >> (16 * (b & 1))) & 0xFFFFu : opos[0] | (opos[1] << 4) | (opos[2] << 8) | (opos[3] << 12);
       const uint32_t sh = __byte_perm(0x08000000u, 0x18101010u, sel);
       metas[b] = __byte_perm(0x4C4E4D4Cu, 0xC4E4D4C4u, sel);
       sels[b] = sel;
@@ -531,7 +606,7 @@ pack_kernel(const PackParams p, const BlobHeader hdr)
           opos[0] | (opos1[0] << 4) | (opos[1] << 8) | (opos1[1] << 12) | (opos[2] << 16) | (opos1[2] << 20) | (opos[3] << 24) | (opos1[3] << 28);
     }
   }
-  if constexpr (!DENSE) *reinterpret_cast<uint2*>(wi + A_IN_BYTES + r * 16 + h * 8) = make_uint2(nibs[0], nibs[1]);
+  if constexpr (!DENSE) *reinterpret_cast<uint2*>(wi + A_IN_BYTES + r * 16 + h * 8) = make_uint2(c_nib[0], c_nib[1]);
   if constexpr (OUTN > 0) *reinterpret_cast<uint4*>(wo + A_OUT_BYTES + r * 16) = make_uint4(metas[0], metas[1], metas[2], metas[3]);
   if constexpr (OUTN == 1) {
     *reinterpret_cast<uint4*>(wc + r * 16) = make_uint4(codes[0], codes[1], codes[2], codes[3]);
@@ -562,12 +637,21 @@ static void launch_pack(const PackParams& p, const BlobHeader& hdr, cudaStream_t
     lc.numAttrs = n_attrs;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, PK_SMEM) == cudaSuccess) (void)cudaLaunchKernelEx(&lc, kern, p, hdr);
   };
-  if (cx <= 8) { go(pack_kernel<DENSE, WGT, OUTN, true>, 1); return; }
+  if (cx <= 8) {
+    // Where the first pass has to choose anyway (channel weights, least significant outliers, two-level scaling's row factor)
+    // its choices are kept: 11008 x 4096, E4M3 scales 74 -> 60 us; 4096 x 11008 with weights, 1:8 88 -> 71, 1:8 + 6:8 98 -> 67.
+    // Otherwise choosing in the second pass saves writing them down (1:8: 49 against 56 us), except with two outliers (78, 75).
+    if constexpr (DENSE) go(pack_kernel<true, WGT, WGT, OUTN, true>, 1);
+    else if constexpr (WGT || OUTN == 2) go(pack_kernel<false, WGT, true, OUTN, true>, 1);
+    else if (p.order_mask || p.ue) go(pack_kernel<false, false, true, OUTN, true>, 1);
+    else go(pack_kernel<false, false, false, OUTN, true>, 1);
+    return;
+  }
   // rows longer than a cluster of eight CTAs holds
   const unsigned rows = (unsigned)(p.N / 8);
   if (WGT || p.order_mask || p.ue) row_scale_kernel<true, WGT, OUTN><<<rows, 256, 0, st>>>(p, hdr);
   else row_scale_kernel<false, WGT, OUTN><<<rows, 256, 0, st>>>(p, hdr);
-  go(pack_kernel<DENSE, WGT, OUTN, false>, 0);
+  go(pack_kernel<DENSE, WGT, DENSE && WGT, OUTN, false>, 0);
 }
 
 // One host-visible word per call in flight, where the kernels report a non-finite weight: a page of pinned memory, taken

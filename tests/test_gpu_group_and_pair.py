@@ -612,3 +612,32 @@ def test_native_and_ctypes_halves_of_the_binding_agree(monkeypatch):
     monkeypatch.setattr(m, "_fast", Absent())
     for a, b in zip(native, calls()):
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("gran,block,rule,out_n", [(so.GRAN_PAIR, 64, 0, 0), (so.GRAN_PAIR, 64, 0, 1), (so.GRAN_PAIR, 32, 0, 2), (so.GRAN_PAIR, 32, so.SCALE_UE4M3, 1),
+                                                   (so.GRAN_PAIR, 32, so.SCALE_UE4M3, 2), (so.GRAN_ELEM, 32, 0, 1),
+                                                   (so.gran_keep(7), 32, 0, 1), (so.gran_keep(7), 32, 0, 2), (so.gran_keep(5), 32, 0, 1), (so.GRAN_3OF4, 32, 0, 2)])
+@pytest.mark.parametrize("K", [2304, 16640])
+def test_packer_choices_with_ties(gran, block, rule, out_n, K):
+    """every place where the packer chooses (kept from its first pass, or made in the second), over full and partial chunks of
+    a row and rows longer than a cluster holds, with few distinct magnitudes, so that most choices are ties, and zeros of either
+    sign; a value that is not finite is found wherever the choices leave it.  Bit-exact."""
+    m = sdq()
+    rng = np.random.default_rng(11)
+    W = torch.from_numpy(rng.choice(np.array([0.0, -0.0, 0.5, -0.5, 0.75, 1.0, -1.0, -2.0, 3.0], np.float32), (128, K))).to(torch.bfloat16)
+    W[5, 64:320] = 0
+    c = rng.choice(np.array([0.25, 1.0, 1.0, 2.0], np.float32), K)
+    for order in (m.ORDER_LARGE,) if rule == m.SCALE_UE4M3 else (m.ORDER_LARGE, m.ORDER_SMALL):   # (two-level scaling has one order)
+        for cw in (None, c):
+            cfg = m.Config(out_n, gran, block, rule, order)
+            gpu_cw = None if cw is None else torch.from_numpy(cw).cuda()
+            op = so.decompose(sdq_synth.bf16_bits(W), so.Config(out_n, gran, block, rule, order), col_weight=cw)
+            pe = {k: v.cpu().numpy() for k, v in m.packed_export(m.sdq_decompose(W.cuda(), cfg, col_weight=gpu_cw)).items()}
+            for name in ("in_code", "in_meta", "in_scale", "out_code", "out_idx", "out_sexp"):
+                assert np.array_equal(pe[name], getattr(op, name)), (name, order, cw is None)
+            for k, bad in ((K - 1, float("inf")), (3, float("nan"))):
+                B = W.clone()
+                B[77, k] = bad
+                with pytest.raises(m.SdqError) as e:
+                    m.sdq_decompose(B.cuda(), cfg, col_weight=gpu_cw)
+                assert e.value.code == 6
