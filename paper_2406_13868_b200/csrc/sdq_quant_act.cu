@@ -6,16 +6,16 @@
 // keep their elements in registers, exchange the per-token maxima through distributed shared memory and encode.
 // Longer rows take two launches: `act_amax_kernel` reduces, per token, the largest magnitude of each 2048-K chunk,
 // `quant_act_kernel` then encodes, one CTA per (group of 8 tokens = one row group of the operand layout, 2048-K chunk).
-// In all of them a warp works on one unit: 8 tokens x 256 K, i.e. what 8 tokens have in one record of the layout; 4 lanes
+// In all of them (but the spread form of few tokens, see its dispatch) a warp works on one unit: 8 tokens x 256 K, i.e. what 8 tokens have in one record of the layout; 4 lanes
 // per token, for each of the unit's four 64-K Q-Vectors 16 elements (two 16-byte loads) per lane.  A Q-Vector maximum is
 // then a 4-lane shuffle, a token's four scales are one word, and every store instruction of codes writes whole 128-byte
 // lines (8 tokens x 16 B per core matrix).  Codes come from the hardware E2M1 / E4M3 converters.
 //
-// Bound by DRAM traffic and the conversion instructions: 2048 x 11008 at 3.74 TB/s of algorithmic bytes (21.0 us; a warp
-// per scattered 64-K Q-Vector with byte stores of scales: 24.7), 8192 x 4096 at 4.4 TB/s (26.7 us; 31.6), one token 3.6 us
-// (4.6), most of it launch and the cluster barrier.  E4M3 scales and int8 codes multiply by a reciprocal instead of dividing
-// every element (see sdq_codec.cuh): 4096 x 16384 with E4M3 scales 91 -> 70.7 us, int8 2048 x 4096 15.0 -> 12.6, one int8
-// token 14.1 -> 6.4 (zeros took the division's slow path).
+// Bound by DRAM traffic and the conversion instructions: 2048 x 11008 at 3.8 TB/s of algorithmic bytes (20.8 us; a warp
+// per scattered 64-K Q-Vector with byte stores of scales: 24.7), 8192 x 4096 at 4.8 TB/s (24.6 us; 31.6), one token 2.3 us
+// (4.6), most of it the launch.  E4M3 scales and int8 codes multiply by a reciprocal instead of dividing
+// every element (see sdq_codec.cuh): 4096 x 16384 with E4M3 scales 91 -> 61.3 us, int8 2048 x 4096 15.0 -> 12.6, one int8
+// token 14.1 -> 3.0 (zeros took the division's slow path).
 #include "sdq_codec.cuh"
 #include "sdq_internal.h"
 #include "sdq_layout.h"
@@ -28,15 +28,17 @@ constexpr int QA_THREADS = 256;
 constexpr int QA_WARPS = QA_THREADS / 32;
 constexpr int QA_CHUNK = QA_WARPS * K2;                  // K per CTA: one 256-K unit per warp
 
-// a lane's part of a unit: its token's elements 64 i + 16 l .. + 15 for the four Q-Vectors i
+// a lane's part of a unit: its token's elements 64 i + 16 l .. + 15 for NQ of the four Q-Vectors i
+template <int NQ>
 struct QaUnit {
-  uint4 raw[4][2];
-  uint32_t qmax[4];                                      // largest magnitude bits of the 16 elements; > 0x7F7F: an infinity
+  uint4 raw[NQ][2];
+  uint32_t qmax[NQ];                                     // largest magnitude bits of the 16 elements; > 0x7F7F: an infinity
 };
 // `on`: the token exists and the unit lies inside the row (zeros otherwise)
-__device__ __forceinline__ void qa_load(QaUnit& u, const __nv_bfloat16* p, bool on) {
+template <int NQ>
+__device__ __forceinline__ void qa_load(QaUnit<NQ>& u, const __nv_bfloat16* p, bool on) {
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
+  for (int i = 0; i < NQ; ++i) {
     u.raw[i][0] = u.raw[i][1] = make_uint4(0, 0, 0, 0);
     if (on) {
       const uint4* q = reinterpret_cast<const uint4*>(p + i * 64);
@@ -47,10 +49,11 @@ __device__ __forceinline__ void qa_load(QaUnit& u, const __nv_bfloat16* p, bool 
 }
 // fills qmax and returns the largest magnitude bits of all the lane's elements.  +-Inf counts as the largest
 // finite bf16: maxima are clamped, the elements only where a lane holds one
-__device__ __forceinline__ uint32_t qa_maxima(QaUnit& u) {
+template <int NQ>
+__device__ __forceinline__ uint32_t qa_maxima(QaUnit<NQ>& u) {
   uint32_t m = 0;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
+  for (int i = 0; i < NQ; ++i) {
     const uint32_t r[8] = {u.raw[i][0].x, u.raw[i][0].y, u.raw[i][0].z, u.raw[i][0].w, u.raw[i][1].x, u.raw[i][1].y, u.raw[i][1].z, u.raw[i][1].w};
     uint32_t q = 0;
 #pragma unroll
@@ -68,9 +71,10 @@ __device__ __forceinline__ void qa_store_scales(uint8_t* atoms, uint32_t step, i
   if (a >= 0) *reinterpret_cast<uint32_t*>(atoms + (size_t)a * step + (uint32_t)(m & 31) * 16 + l * 4) = w;
 }
 
-// encodes a unit: token m (existing: `live`), 256-K record k2 of the buffer, the token's largest magnitude `ramax`
-template <bool UE>                                       // UE: two-level scaling with E4M3 Q-Vector scales
-__device__ __forceinline__ void qa_encode(const QaUnit& u, float ramax, bool live, int64_t m, int k2, uint32_t l, const sdq_config_t& cfg,
+// encodes a unit: token m (existing: `live`), 256-K record k2 of the buffer, the token's largest magnitude `ramax`; with NQ < 4
+// only its Q-Vectors from `first` on
+template <bool UE, int NQ>                               // UE: two-level scaling with E4M3 Q-Vector scales
+__device__ __forceinline__ void qa_encode(const QaUnit<NQ>& u, int first, float ramax, bool live, int64_t m, int k2, uint32_t l, const sdq_config_t& cfg,
                                           uint8_t* __restrict__ buf, const ActOffsets& off) {
   const int e = fp8_scale_exp(ramax);
   const float s8 = pow2_neg(e);
@@ -79,9 +83,10 @@ __device__ __forceinline__ void qa_encode(const QaUnit& u, float ramax, bool liv
   const bool b32 = cfg.in_block == 32;                   // one scale per 32 K: a Q-Vector is a lane pair
   uint8_t* xi = buf + off.xi + (size_t)k2 * off.xi_stride + (size_t)(m >> 3) * 1024 + (uint32_t)(m & 7) * 16;
   uint8_t* xo = buf + off.xo + (size_t)(2 * k2) * off.xo_stride + (size_t)(m >> 3) * 1024 + (uint32_t)(m & 7) * 16;
-  uint32_t c[4];
+  uint32_t c[NQ];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
+  for (int i = 0; i < NQ; ++i) {
+    const int iq = first + i;
     const uint32_t r[8] = {u.raw[i][0].x, u.raw[i][0].y, u.raw[i][0].z, u.raw[i][0].w, u.raw[i][1].x, u.raw[i][1].y, u.raw[i][1].z, u.raw[i][1].w};
     float v[16];
 #pragma unroll
@@ -130,12 +135,29 @@ __device__ __forceinline__ void qa_encode(const QaUnit& u, float ramax, bool liv
     }
     if (live) {
       // 4-bit codes: bytes 32 i + 8 l of the token's 128; 8-bit codes: bytes 64 (i & 1) + 16 l of the 128-K record i / 2
-      *reinterpret_cast<uint2*>(xi + (uint32_t)(2 * i + (l >> 1)) * 128 + (l & 1) * 8) = make_uint2(q4[0], q4[1]);
-      *reinterpret_cast<uint4*>(xo + (size_t)(i >> 1) * off.xo_stride + (uint32_t)(4 * (i & 1) + l) * 128) = make_uint4(q8[0], q8[1], q8[2], q8[3]);
+      *reinterpret_cast<uint2*>(xi + (uint32_t)(2 * iq + (l >> 1)) * 128 + (l & 1) * 8) = make_uint2(q4[0], q4[1]);
+      *reinterpret_cast<uint4*>(xo + (size_t)(iq >> 1) * off.xo_stride + (uint32_t)(4 * (iq & 1) + l) * 128) = make_uint4(q8[0], q8[1], q8[2], q8[3]);
     }
   }
   uint8_t* sf = buf + off.xi + (size_t)k2 * off.xi_stride + (size_t)off.Mpad * 128;
-  if (!b32) {
+  if constexpr (NQ < 4) {
+    // its bytes of the words that qa_store_scales writes whole
+    const int64_t a = m / 32 - (int64_t)l;
+    const uint32_t at = (uint32_t)(m & 31) * 16 + l * 4 + (b32 ? 2u * ((uint32_t)first & 1u) : (uint32_t)first);
+    uint8_t* dst = sf + ((size_t)a * (b32 ? 2 : 1) + (b32 ? first >> 1 : 0)) * SF_ATOM_BYTES + at;
+    uint32_t w = c[0];
+    if constexpr (NQ == 2) w |= c[1] << (b32 ? 16 : 8);
+    if (b32) {                                           // two scales per Q-Vector, one of each lane pair
+      w <<= 8 * (l >> 1);
+      w |= __shfl_xor_sync(0xffffffffu, w, 2);
+    }
+    if (live && a >= 0) {
+      const int bytes = NQ * (b32 ? 2 : 1);
+      if (bytes == 1) *dst = (uint8_t)w;
+      else if (bytes == 2) *reinterpret_cast<uint16_t*>(dst) = (uint16_t)w;
+      else *reinterpret_cast<uint32_t*>(dst) = w;
+    }
+  } else if (!b32) {
     if (live) qa_store_scales(sf, SF_ATOM_BYTES, m, l, c[0] | (c[1] << 8) | (c[2] << 16) | (c[3] << 24));
   } else {
 #pragma unroll
@@ -166,7 +188,7 @@ act_amax_kernel(const __nv_bfloat16* __restrict__ X, int64_t M, int64_t K, int64
   const int64_t m = (int64_t)blockIdx.x * 8 + t;
   const int64_t k = (int64_t)blockIdx.y * QA_CHUNK + warp * K2;
   __shared__ float s_amax[QA_WARPS][8];
-  QaUnit u;
+  QaUnit<4> u;
   qa_load(u, X + m * ldx + k + l * 16, m < M && k < K);
   float amax = bf16_bits_to_float(qa_maxima(u));
   amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, 1));
@@ -202,25 +224,26 @@ quant_act_kernel(const __nv_bfloat16* __restrict__ X, int64_t M, int64_t K, int6
   ramax = fmaxf(ramax, __shfl_xor_sync(0xffffffffu, ramax, 2));
   if (live && blockIdx.y == 0 && warp == 0) qa_token_scale<UE>(ramax, m, (uint32_t)l, cfg, buf, off);
   if (k >= K) return;
-  QaUnit u;
+  QaUnit<4> u;
   qa_load(u, X + m * ldx + k + l * 16, live);
   qa_maxima(u);
-  qa_encode<UE>(u, ramax, live, m, (int)(k / K2), (uint32_t)l, cfg, buf, off);
+  qa_encode<UE>(u, 0, ramax, live, m, (int)(k / K2), (uint32_t)l, cfg, buf, off);
 }
 
-// Single pass: the CTAs of a cluster share one group of 8 tokens and split its 256-K units, one per warp; every thread keeps
+// Single pass: the CTAs of a cluster share one group of 8 tokens and split its Q-Vectors, NQ per warp; every thread keeps
 // its elements in registers (packed bf16) from the one read of X, the per-token maxima meet through distributed shared
 // memory, and the codes are produced from the registers.  The two-launch path stays for rows longer than a cluster of
 // eight CTAs holds (K > 16384).
-template <bool UE>
-__global__ void __launch_bounds__(QA_THREADS, UE ? 3 : 4)
+template <bool UE, int NQ>
+__global__ void __launch_bounds__(NQ == 4 ? QA_THREADS : 512, NQ == 4 ? (UE ? 3 : 4) : 1)
 quant_act_fused_kernel(const __nv_bfloat16* __restrict__ X, int64_t M, int64_t K, int64_t ldx, sdq_config_t cfg, uint8_t* __restrict__ buf,
                        ActOffsets off, uint32_t* __restrict__ flags)
 {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int t = lane >> 2, l = lane & 3;                 // token within the group of 8, quarter of the Q-Vector
   const uint32_t cx = gridDim.x, rank = blockIdx.x;      // cluster = the gridDim.x CTAs of one token group
-  __shared__ float s_warp[QA_WARPS][8];
+  const int warps = NQ == 4 ? QA_WARPS : (int)(blockDim.x >> 5);
+  __shared__ float s_warp[NQ == 4 ? QA_WARPS : 16][8];
   __shared__ float s_all[8][8];                          // [cluster rank][token]: every CTA's maxima, pushed by their owners
   __shared__ uint64_t s_bar;                             // ... all of which have arrived
   if (tid == 0) {
@@ -237,10 +260,10 @@ quant_act_fused_kernel(const __nv_bfloat16* __restrict__ X, int64_t M, int64_t K
   asm volatile("griddepcontrol.wait;" ::: "memory");
   const int64_t m = (int64_t)blockIdx.y * 8 + t;
   const bool live = m < M;
-  const int k2 = (int)rank * QA_WARPS + warp;            // this warp's unit
-  const bool on = k2 < (int)(K / K2);
-  QaUnit u;
-  qa_load(u, X + m * ldx + (int64_t)k2 * K2 + l * 16, live && on);
+  const int q = ((int)rank * warps + warp) * NQ;         // this warp's first Q-Vector
+  const bool on = q < (int)(K / 64);
+  QaUnit<NQ> u;
+  qa_load(u, X + m * ldx + (int64_t)q * 64 + l * 16, live && on);
   float amax = bf16_bits_to_float(qa_maxima(u));
   amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, 1));
   amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, 2));
@@ -254,8 +277,8 @@ quant_act_fused_kernel(const __nv_bfloat16* __restrict__ X, int64_t M, int64_t K
     const int tok = tid & 7;
     const uint32_t peer = (uint32_t)tid >> 3;
     float a = 0.0f;
-#pragma unroll
-    for (int w = 0; w < QA_WARPS; ++w) a = fmaxf(a, s_warp[w][tok]);
+#pragma unroll 8
+    for (int w = 0; w < warps; ++w) a = fmaxf(a, s_warp[w][tok]);
     ptx::st_async_u32(ptx::mapa_u32(ptx::smem_u32(&s_all[rank][tok]), peer), __float_as_uint(a), ptx::mapa_u32(ptx::smem_u32(&s_bar), peer));
   }
   // no CTA leaves before all pushes to it have arrived, and its own go to CTAs that wait for them
@@ -263,7 +286,7 @@ quant_act_fused_kernel(const __nv_bfloat16* __restrict__ X, int64_t M, int64_t K
   float ramax = 0.0f;
   for (uint32_t c = 0; c < cx; ++c) ramax = fmaxf(ramax, s_all[c][t]);
   if (live && rank == 0 && warp == 0) qa_token_scale<UE>(ramax, m, (uint32_t)l, cfg, buf, off);
-  if (on) qa_encode<UE>(u, ramax, live, m, k2, (uint32_t)l, cfg, buf, off);
+  if (on) qa_encode<UE>(u, q & 3, ramax, live, m, q >> 2, (uint32_t)l, cfg, buf, off);
 }
 
 __global__ void __launch_bounds__(QA_THREADS)
@@ -323,20 +346,33 @@ extern "C" sdq_status_t sdq_quantize_act(const void* X, int64_t M, int64_t K, in
     uint32_t* flags = device_flags();
     if (!flags) return SDQ_ERR_CUDA;
     cudaLaunchConfig_t lc = {};
-    lc.gridDim = dim3((unsigned)n_chunks, (unsigned)((M + 7) / 8));
-    lc.blockDim = dim3(QA_THREADS);
+    const DeviceInfo* dinfo = device_info();
+    if (!dinfo) return SDQ_ERR_CUDA;
+    // Q-Vectors (64 K) per warp.  A whole unit of four costs the fewest instructions, but a warp then encodes one after the other
+    // for about a microsecond, so where there are too few to fill the chip they are spread: one each for up to 7 warps per SM
+    // (16 x 4096: 2.3 us, two 2.5, four 3.2; int8 3.0, 4.1, 6.2), in CTAs of up to 16 warps (8 x 16384, 32 warps: 3.4, 3.2, 3.2),
+    // two while all these warps run at once, 28 per SM (256 x 4096: 3.1, 2.9, 3.5; 1000 x 4096: 6.2, 4.4, 5.1; 500 x 11008: 14.8,
+    // 7.3, 6.5).
+    const int64_t groups = (M + 7) / 8, vecs = groups * (K / 64);
+    const int nq = vecs <= 7 * (int64_t)dinfo->sm_count && K <= 8192 ? 1 : (vecs <= 56 * (int64_t)dinfo->sm_count ? 2 : 4);
+    const int warps = (int)(K / 64 + nq - 1) / nq;       // per token group
+    const unsigned cx = (unsigned)((warps + QA_WARPS - 1) / QA_WARPS < 8 ? (warps + QA_WARPS - 1) / QA_WARPS : 8);
+    lc.gridDim = dim3(cx, (unsigned)groups);
+    lc.blockDim = dim3(nq < 4 ? 32 * (((unsigned)warps + cx - 1) / cx) : QA_THREADS);
     lc.stream = (cudaStream_t)stream;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)n_chunks;
+    attr[0].val.clusterDim.x = cx;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     lc.attrs = attr;
     lc.numAttrs = 2;
-    const cudaError_t le = ue ? cudaLaunchKernelEx(&lc, quant_act_fused_kernel<true>, Xb, M, K, ldx, *cfg, bufp, off, flags)
-                              : cudaLaunchKernelEx(&lc, quant_act_fused_kernel<false>, Xb, M, K, ldx, *cfg, bufp, off, flags);
+    auto go = [&](auto kern) { return cudaLaunchKernelEx(&lc, kern, Xb, M, K, ldx, *cfg, bufp, off, flags); };
+    const cudaError_t le = nq == 4   ? (ue ? go(quant_act_fused_kernel<true, 4>) : go(quant_act_fused_kernel<false, 4>))
+                           : nq == 2 ? (ue ? go(quant_act_fused_kernel<true, 2>) : go(quant_act_fused_kernel<false, 2>))
+                                     : (ue ? go(quant_act_fused_kernel<true, 1>) : go(quant_act_fused_kernel<false, 1>));
     if (le != cudaSuccess || cudaGetLastError() != cudaSuccess) return SDQ_ERR_CUDA;
   } else {
     float* partial = reinterpret_cast<float*>(bufp + off.amax);

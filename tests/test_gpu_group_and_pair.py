@@ -641,3 +641,20 @@ def test_packer_choices_with_ties(gran, block, rule, out_n, K):
                 with pytest.raises(m.SdqError) as e:
                     m.sdq_decompose(B.cuda(), cfg, col_weight=gpu_cw)
                 assert e.value.code == 6
+
+
+@pytest.mark.parametrize("M,K", [(1, 256), (9, 1280), (130, 4096), (9, 8192), (9, 8448), (600, 1024), (1040, 4096), (270, 16384)])
+@pytest.mark.parametrize("rule,block,fmt", [(0, 64, 0), (1, 32, 0), (so.SCALE_UE4M3, 32, 0), (0, 64, 1)])
+def test_quantizer_one_two_and_four_q_vectors_per_warp(M, K, rule, block, fmt):
+    """few tokens are spread over more warps: the three forms and the token counts and row lengths around their limits, bit for
+    bit"""
+    m = sdq()
+    X = sdq_synth.make_act(M, K, 300 + M)
+    X[M // 2, K // 3] = float("-inf")
+    X[M - 1, K - 64:] = 0.0
+    xq = m.sdq_quantize_act(X.cuda(), m.Config(1, m.GRAN_PAIR, block, rule, 0, fmt))
+    oq = so.quantize_act(sdq_synth.bf16_bits(X), so.Config(1, so.GRAN_PAIR, block, rule, 0, fmt))
+    ae = {k: v.cpu().numpy() for k, v in m.act_export(xq).items()}
+    assert m.device_status() == 0
+    for name in ("xq4_code", "xq4_scale", "xq8_code", "xq8_sexp"):
+        assert np.array_equal(ae[name], getattr(oq, name)), name
