@@ -705,7 +705,7 @@ def measure_model(sdq, dev, peaks, token_counts=(1, 16, 128, 1024, 8192)):
 
         def model(grouped=False, fused=False):
             for ps in layers:
-                if fused:                                      # quantizer inside the grouped kernel: no quantized buffer, no launch
+                if fused:                                      # one call that quantizes and multiplies
                     sdq.sdq_linear_group_x(X, ps[0:3], Ya)
                     xq = sdq.sdq_quantize_act(X, cfg, bx)      # input of o
                     sdq.sdq_linear(xq, ps[3], Ya[0])

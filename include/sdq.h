@@ -293,6 +293,14 @@ sdq_status_t sdq_linear_group_x(int n, const void* X_bf16, int64_t M, int64_t K,
                                 void* const* Y_bf16, const int64_t* ldy, void* stream);
 sdq_status_t sdq_linear_group_x_f32(int n, const void* X_bf16, int64_t M, int64_t K, int64_t ldx, const sdq_packed_t* const* P,
                                     float* const* Y_f32, const int64_t* ldy, void* stream);
+/* The same with scratch, sdq_act_size(M, K, &P[0]->cfg) bytes of device memory, 16-byte aligned, in use until the call's work on
+ * `stream` is done: the activations are quantized into it by a launch of their own in front of the grouped kernel, whose first
+ * weights stream in meanwhile.  Same bits, less time: X is quantized once instead of once per CTA.  ws == NULL: as above.
+ * Further errors: BUFFER_TOO_SMALL, ALIGNMENT. */
+sdq_status_t sdq_linear_group_x_ws(int n, const void* X_bf16, int64_t M, int64_t K, int64_t ldx, const sdq_packed_t* const* P,
+                                   void* const* Y_bf16, const int64_t* ldy, void* ws, size_t ws_bytes, void* stream);
+sdq_status_t sdq_linear_group_x_f32_ws(int n, const void* X_bf16, int64_t M, int64_t K, int64_t ldx, const sdq_packed_t* const* P,
+                                       float* const* Y_f32, const int64_t* ldy, void* ws, size_t ws_bytes, void* stream);
 
 /* Built-in scratch variant of sdq_linear_ws (the paper has no counterpart: this is a packaging choice of the
  * library, not part of the method).

@@ -69,7 +69,7 @@ class _ActCanon(ctypes.Structure):
 
 EXPORTS = ["sdq_packed_size", "sdq_decompose", "sdq_decompose_metric", "sdq_channel_norm", "sdq_packed_export", "sdq_packed_attach", "sdq_packed_compact_size", "sdq_packed_compact", "sdq_act_size", "sdq_quantize_act", "sdq_act_export",
            "sdq_linear", "sdq_linear_f32", "sdq_workspace_size", "sdq_workspace_init", "sdq_linear_ws", "sdq_linear_f32_ws", "sdq_linear_noalloc",
-           "sdq_linear_group", "sdq_linear_group_f32", "sdq_linear_group_x", "sdq_linear_group_x_f32", "sdq_diag_l2_copy", "sdq_diag_wait_timeout", "sdq_device_status", "sdq_status_string"]
+           "sdq_linear_group", "sdq_linear_group_f32", "sdq_linear_group_x", "sdq_linear_group_x_f32", "sdq_linear_group_x_ws", "sdq_linear_group_x_f32_ws", "sdq_diag_l2_copy", "sdq_diag_wait_timeout", "sdq_device_status", "sdq_status_string"]
 
 _lib = None
 
@@ -324,8 +324,9 @@ def sdq_linear_group(xqs, ps, outs=None, f32: bool = False):
 
 
 def sdq_linear_group_x(X: torch.Tensor, ps, outs=None, f32: bool = False):
-    """Y[i] = sdq_linear(sdq_quantize_act(X), ps[i]) for layers that share the bf16 activations X [M <= 16, K], the quantizer
-    fused into the one persistent launch (see sdq_linear_group_x in include/sdq.h).  Returns the list of outputs."""
+    """Y[i] = sdq_linear(sdq_quantize_act(X), ps[i]) for layers that share the bf16 activations X [M <= 16, K], in one call (see
+    sdq_linear_group_x_ws in include/sdq.h; the ctypes way takes sdq_linear_group_x, which needs no scratch).  Returns the list
+    of outputs."""
     ys = (_fast or _native()).linear_group_x(X, ps, outs, f32)
     if ys is not None:
         return ys

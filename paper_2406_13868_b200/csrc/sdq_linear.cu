@@ -745,9 +745,12 @@ static sdq_status_t launch_group(int n, const sdq_act_t* const* Xq, const sdq_pa
   return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? SDQ_OK : SDQ_ERR_CUDA;
 }
 
-// The same with the activation quantizer inside the kernel: all layers read one bf16 X (see include/sdq.h).
+// The same from one bf16 X that all layers read (see include/sdq.h): with scratch, the quantizer's launch and then the grouped
+// kernel's, whose first weights are on their way while the quantizer runs; without, the quantizer inside the kernel, once per
+// CTA.  gate and up of 11008 x 4096, 1 / 5 / 16 tokens: 15.3 / 15.5 / 15.7 us against 15.5 / 17.2 / 20.5, int8 outliers 16.0 / 16.2 /
+// 16.6 against 16.3 / 19.8 / 25.8; three of 8192 x 1024: 8.0 / 8.1 / 8.9 against 8.9 / 9.1 / 9.8.
 static sdq_status_t launch_group_x(int n, const void* X, int64_t M, int64_t K, int64_t ldx, const sdq_packed_t* const* P, void* const* Y,
-                                   const int64_t* ldy, void* stream, bool f32)
+                                   const int64_t* ldy, void* ws, size_t ws_bytes, void* stream, bool f32)
 {
   if (n <= 0 || !X || !P || !Y || !ldy) return SDQ_ERR_INVALID_ARG;
   if (M <= 0 || K <= 0 || K % K2 || ldx < K) return SDQ_ERR_SHAPE;
@@ -765,25 +768,39 @@ static sdq_status_t launch_group_x(int n, const void* X, int64_t M, int64_t K, i
     if (!group_format(*w) || c.out_n != c0.out_n || c.out_fmt != c0.out_fmt || c.scale_rule != c0.scale_rule) return SDQ_ERR_UNSUPPORTED;
     items += w->N / TILE_ROWS;
   }
-  // (the in-kernel quantizer keeps a token's K <= 4096 elements in the registers of its 11 x 4 lanes)
+  // (the same range with and without scratch: the in-kernel quantizer keeps a token's K <= 4096 elements in the registers of its 11 x 4 lanes)
   if (n > GROUP_MAX || M > 16 || K < 4 * K2 || K > 16 * K2 || !group_xres_fits((int)(K / K2), P[0]->cfg.out_n) || items * 2 < dinfo->sm_count || items >= (1 << 30))
     return SDQ_ERR_UNSUPPORTED;
   GroupParams g;
   group_begin(g, n, M, *P[0]);
   if (!g.flags) return SDQ_ERR_CUDA;
-  g.x_bf16 = X; g.x_ld = ldx; g.x_M = (int)M;
-  for (int i = 0; i < n; ++i) group_add(g, i, nullptr, *P[i], Y[i], ldy[i], M);
+  sdq_act_t xq;
+  if (ws) {
+    const sdq_status_t st = sdq_quantize_act(X, M, K, ldx, &P[0]->cfg, ws, ws_bytes, &xq, stream);
+    if (st != SDQ_OK) return st;
+  } else {
+    g.x_bf16 = X; g.x_ld = ldx; g.x_M = (int)M;
+  }
+  for (int i = 0; i < n; ++i) group_add(g, i, ws ? &xq : nullptr, *P[i], Y[i], ldy[i], M);
   const cudaError_t e = launch_linear_group(g, f32, dinfo, (cudaStream_t)stream);
   return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? SDQ_OK : SDQ_ERR_CUDA;
 }
 
 extern "C" sdq_status_t sdq_linear_group_x(int n, const void* X_bf16, int64_t M, int64_t K, int64_t ldx, const sdq_packed_t* const* P,
                                            void* const* Y, const int64_t* ldy, void* stream)
-{ return launch_group_x(n, X_bf16, M, K, ldx, P, Y, ldy, stream, false); }
+{ return launch_group_x(n, X_bf16, M, K, ldx, P, Y, ldy, nullptr, 0, stream, false); }
 
 extern "C" sdq_status_t sdq_linear_group_x_f32(int n, const void* X_bf16, int64_t M, int64_t K, int64_t ldx, const sdq_packed_t* const* P,
                                                float* const* Y, const int64_t* ldy, void* stream)
-{ return launch_group_x(n, X_bf16, M, K, ldx, P, (void* const*)Y, ldy, stream, true); }
+{ return launch_group_x(n, X_bf16, M, K, ldx, P, (void* const*)Y, ldy, nullptr, 0, stream, true); }
+
+extern "C" sdq_status_t sdq_linear_group_x_ws(int n, const void* X_bf16, int64_t M, int64_t K, int64_t ldx, const sdq_packed_t* const* P,
+                                              void* const* Y, const int64_t* ldy, void* ws, size_t ws_bytes, void* stream)
+{ return launch_group_x(n, X_bf16, M, K, ldx, P, Y, ldy, ws, ws_bytes, stream, false); }
+
+extern "C" sdq_status_t sdq_linear_group_x_f32_ws(int n, const void* X_bf16, int64_t M, int64_t K, int64_t ldx, const sdq_packed_t* const* P,
+                                                  float* const* Y, const int64_t* ldy, void* ws, size_t ws_bytes, void* stream)
+{ return launch_group_x(n, X_bf16, M, K, ldx, P, (void* const*)Y, ldy, ws, ws_bytes, stream, true); }
 
 extern "C" sdq_status_t sdq_linear_group(int n, const sdq_act_t* const* Xq, const sdq_packed_t* const* P, void* const* Y,
                                          const int64_t* ldy, void* stream)

@@ -240,11 +240,19 @@ PyObject* group(PyObject* xqs, PyObject* X, PyObject* ps, PyObject* outs, PyObje
   void* stream = current_stream();
   const void* xp = nullptr;
   int64_t M = 0, K = 0, ldx = 0;
-  if (X) { const at::Tensor& t = THPVariable_Unpack(X); xp = t.data_ptr(); M = t.size(0); K = t.size(1); ldx = t.stride(0); }
+  at::Tensor ws;                         // the quantized activations, for the caching allocator to hand on in stream order
+  if (X) {
+    const at::Tensor& t = THPVariable_Unpack(X);
+    xp = t.data_ptr(); M = t.size(0); K = t.size(1); ldx = t.stride(0);
+    size_t bytes = 0;
+    if (sdq_act_size(M, K, &g.p[0]->cfg, &bytes) == SDQ_OK) ws = at::empty({(int64_t)bytes}, at::TensorOptions().dtype(at::kByte).device(t.device()));
+  }
+  void* wp = ws.defined() ? ws.data_ptr() : nullptr;
+  const size_t ws_bytes = ws.defined() ? (size_t)ws.numel() : 0;
   sdq_status_t st;
   Py_BEGIN_ALLOW_THREADS
-  if (X) st = f32 ? sdq_linear_group_x_f32((int)n, xp, M, K, ldx, g.p.data(), (float* const*)g.y.data(), g.ldy.data(), stream)
-                  : sdq_linear_group_x((int)n, xp, M, K, ldx, g.p.data(), g.y.data(), g.ldy.data(), stream);
+  if (X) st = f32 ? sdq_linear_group_x_f32_ws((int)n, xp, M, K, ldx, g.p.data(), (float* const*)g.y.data(), g.ldy.data(), wp, ws_bytes, stream)
+                  : sdq_linear_group_x_ws((int)n, xp, M, K, ldx, g.p.data(), g.y.data(), g.ldy.data(), wp, ws_bytes, stream);
   else st = f32 ? sdq_linear_group_f32((int)n, g.x.data(), g.p.data(), (float* const*)g.y.data(), g.ldy.data(), stream)
                 : sdq_linear_group((int)n, g.x.data(), g.p.data(), g.y.data(), g.ldy.data(), stream);
   Py_END_ALLOW_THREADS

@@ -1,5 +1,7 @@
 """GPU parity of the grouped few-token call, the CTA-pair many-token kernel and the streamed outlier forms,
 against the CPU oracle, through the C-ABI."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -658,3 +660,31 @@ def test_quantizer_one_two_and_four_q_vectors_per_warp(M, K, rule, block, fmt):
     assert m.device_status() == 0
     for name in ("xq4_code", "xq4_scale", "xq8_code", "xq8_sexp"):
         assert np.array_equal(ae[name], getattr(oq, name)), name
+
+
+@pytest.mark.parametrize("M,K,out_fmt", [(1, 1024, 0), (16, 4096, 0), (5, 2304, 1)])
+def test_group_x_with_and_without_scratch(M, K, out_fmt):
+    """the quantizer in a launch of its own, into the caller's scratch, and inside the grouped kernel: the same bits; scratch of
+    any contents, one byte short of it refused"""
+    m = sdq()
+    cfg = m.Config(1, m.GRAN_PAIR, 64, 0, 0, out_fmt)
+    ps = [m.sdq_decompose(sdq_synth.make_weight(5120, K, 90 + i).cuda(), cfg) for i in range(2)]
+    X = sdq_synth.make_act(M, K, 92).cuda()
+    need = m.act_size(M, K, cfg)
+    ws = torch.randint(0, 256, (need,), dtype=torch.uint8, device="cuda")
+    PA = (ctypes.POINTER(m._Packed) * 2)(*[ctypes.pointer(p.desc) for p in ps])
+    LD = (ctypes.c_int64 * 2)(5120, 5120)
+    st = torch.cuda.current_stream().cuda_stream
+
+    def call(fn, *scratch):
+        Y = torch.zeros((2, M, 5120), dtype=torch.float32, device="cuda")
+        YA = (ctypes.c_void_p * 2)(Y[0].data_ptr(), Y[1].data_ptr())
+        i64 = ctypes.c_int64
+        return fn(2, ctypes.c_void_p(X.data_ptr()), i64(M), i64(K), i64(K), PA, YA, LD, *scratch, ctypes.c_void_p(st)), Y
+    rc0, inside = call(m.lib().sdq_linear_group_x_f32)
+    rc1, apart = call(m.lib().sdq_linear_group_x_f32_ws, ctypes.c_void_p(ws.data_ptr()), ctypes.c_size_t(need))
+    rc2, none = call(m.lib().sdq_linear_group_x_f32_ws, None, ctypes.c_size_t(0))
+    short, _ = call(m.lib().sdq_linear_group_x_f32_ws, ctypes.c_void_p(ws.data_ptr()), ctypes.c_size_t(need - 1))
+    assert (rc0, rc1, rc2, short) == (0, 0, 0, 5) and m.device_status() == 0
+    assert torch.equal(inside, apart) and torch.equal(inside, none)
+    assert all(torch.equal(a, b) for a, b in zip(m.sdq_linear_group_x(X, ps, f32=True), apart))
