@@ -180,7 +180,7 @@ sdq_status_t sdq_decompose_metric(const void* W_bf16, int64_t N, int64_t K, int6
 
 /* Calibration helper for sdq_decompose_metric (Section 5, Stage 1: metrics that use calibration data):
  * col_norm[k] = sqrt(sum over the M tokens of X[m][k]^2), the Euclidean norm of input channel k, accumulated
- * in token order in fp64 and rounded to fp32 (reproducible).
+ * in fp64 in a fixed order and rounded to fp32 (reproducible).
  *   X (device) [M][ldx] bf16, 4-byte aligned, ldx >= K, K and ldx even; col_norm (device) [K] fp32.
  *   Asynchronous on `stream`.  Errors: INVALID_ARG, SHAPE, ALIGNMENT, CUDA. */
 sdq_status_t sdq_channel_norm(const void* X_bf16, int64_t M, int64_t K, int64_t ldx, float* col_norm, void* stream);
@@ -268,7 +268,8 @@ sdq_status_t sdq_linear_f32_ws(const sdq_act_t* Xq, const sdq_packed_t* P, float
  *   When every layer has at most 32 tokens, K >= 1024, the primary format (SDQ_GRAN_PAIR, in_block 64, out_n <= 1,
  *   power-of-two scales), n <= 32 and the layers together have at least half as many 128-row tiles as the GPU has SMs, the
  *   call is ONE persistent kernel launch that streams all weights once, the outlier part in its compact form (8-bit code +
- *   position per S-Vector, rebuilt into the tensor core's 2:4 form in tensor memory); the summation order over K of an output differs
+ *   position per S-Vector, rebuilt into the tensor core's 2:4 form in tensor memory); row tiles left over after whole rounds of the
+ *   SMs have their K range split over clusters of two or four thread blocks; the summation order over K of an output differs
  *   from sdq_linear's split-K paths, so results agree to fp32 rounding, not bit for bit.  Otherwise the layers are
  *   enqueued one after the other exactly as sdq_linear would.
  *   Asynchronous on `stream`; allocates nothing.  Errors as sdq_linear (the first failing layer's). */
