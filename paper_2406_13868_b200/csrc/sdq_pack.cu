@@ -8,10 +8,11 @@
 // the outliers, for two-level scaling the inlier factor -- is found in a first pass over the staged rows and exchanged
 // through distributed shared memory.  Longer rows: `row_scale_kernel` finds it and the same kernel follows without clusters.
 //
-// What bounds it: the integer pipe (77 % busy at ~140 instructions per S-Vector; selections on packed keys instead of index
-// loops took it from ~350 over two passes), DRAM is at 30 %.  11008 x 4096, 1:8 + pair-wise 4:8: 189 us as one kernel with a
-// CTA per row and a thread per S-Vector scattering bytes -> 20 + 42 us with the row scales in a launch of their own ->
-// 49 us.  4096 x 11008, 1:8 + 6:8 with channel weights: 98 us choosing in both passes -> 67.
+// What bounds it: the integer pipe (selections on packed keys instead of index loops took it from ~350 instructions per S-Vector
+// over two passes to ~120), DRAM is at 35 %.  11008 x 4096, 1:8 + pair-wise 4:8: 189 us as one kernel with a CTA per row and a
+// thread per S-Vector scattering bytes -> 20 + 42 us with the row scales in a launch of their own -> 49 us -> 42 us with the
+// pairs picked by two minima and two maxima instead of six comparisons and the choices kept from the first pass.  4096 x 11008,
+// 1:8 + 6:8 with channel weights: 98 us choosing in both passes -> 67.
 #include <cstring>
 #include <type_traits>
 #include <mutex>
@@ -127,7 +128,7 @@ __device__ __forceinline__ void zero_set(uint32_t (&r)[4], uint32_t gone) {
   r[3] &= ~prmt(hi, 0u, 0xBBAAu);
 }
 // Stage 1, pair-wise 4:8: the 2 pairs (of 4) with the largest summed significance among the non-outliers (x: outliers
-// zeroed), largest first, ties to the lower index.  A pair stays if it comes before at least two of the other three.
+// zeroed), largest first, ties to the lower index.
 // Returns the two pairs in ascending order and the pattern nibble j0 | j1 << 2.
 template <bool WGT>
 __device__ __forceinline__ void pick_pairs(const uint32_t (&x)[4], const int (&key)[8], int o0, int o1, uint32_t& w0, uint32_t& w1, uint32_t& nibble) {
@@ -142,14 +143,12 @@ __device__ __forceinline__ void pick_pairs(const uint32_t (&x)[4], const int (&k
       s[j] = __fadd_rn(fabsf(__uint_as_float(x[j] << 16)), fabsf(__uint_as_float(x[j] & 0xFFFF0000u)));
     }
   }
-  const bool b01 = s[0] >= s[1], b02 = s[0] >= s[2], b03 = s[0] >= s[3], b12 = s[1] >= s[2], b13 = s[1] >= s[3], b23 = s[2] >= s[3];
-  const bool k0 = (b01 && b02) || (b03 && (b01 || b02));
-  const bool k1 = (!b01 && b12) || (b13 && (!b01 || b12));
-  const bool k3 = (!b03 && !b13) || (!b23 && (!b03 || !b13));
-  const bool k2 = !((k0 && k1) || (k3 && (k0 || k1)));
-  w0 = k0 ? x[0] : (k1 ? x[1] : x[2]);
-  w1 = k3 ? x[3] : (k2 ? x[2] : x[1]);
-  nibble = (k0 ? 0u : (k1 ? 1u : 2u)) | (k3 ? 12u : (k2 ? 8u : 4u));
+  // the weaker of the first two beats the stronger of the last two; or the other way round; else one of each
+  const bool first = fminf(s[0], s[1]) >= fmaxf(s[2], s[3]), last = fminf(s[2], s[3]) > fmaxf(s[0], s[1]);
+  const bool k0 = first || s[0] >= s[1], k2 = !last && s[2] >= s[3];
+  w0 = last ? x[2] : (k0 ? x[0] : x[1]);
+  w1 = first ? x[1] : (k2 ? x[2] : x[3]);
+  nibble = (last ? 2u : (k0 ? 0u : 1u)) | (first ? 4u : (k2 ? 8u : 12u));
 }
 // Stage 1 for the patterns stored dense: the set of positions that hold +0 -- the outliers and, among the others, all but the
 // keep_in most significant (of every 8, or of every 4 with grp4).  k: ranking keys.
@@ -313,8 +312,7 @@ constexpr int PK_THREADS = 256, PK_ROWS = 16, PK_K = 2048;
 constexpr int PK_PITCH = PK_K * 2 + 16;                  // bytes between rows of the staged tile
 constexpr int PK_SMEM = PK_ROWS * PK_PITCH;              // 65792: three CTAs per SM
 
-// CHOSEN: the first pass chooses for good (see there)
-template <bool DENSE, bool WGT, bool CHOSEN, int OUTN, bool FUSED>
+template <bool DENSE, bool WGT, int OUTN, bool FUSED>
 __global__ void __launch_bounds__(PK_THREADS, 3)
 pack_kernel(const PackParams p, const BlobHeader hdr)
 {
@@ -347,11 +345,13 @@ pack_kernel(const PackParams p, const BlobHeader hdr)
   __syncthreads();
 
   // ---- first pass: the choices, the row's largest outlier (and inlier), non-finite check.
-  // CHOSEN, pair-wise: everything is chosen here and the S-Vector's 16 bytes in the tile become what is left to encode, the two
-  // pairs that stay and the outliers' values; positions and pattern nibbles are collected in registers, as the layout wants
-  // them.  CHOSEN, stored dense: the same, but the values stay where they are and the sets of dropped positions are collected.
-  // Otherwise the second pass chooses: the outliers, if the most significant by magnitude, hold the row's largest magnitude,
-  // and then this pass has to choose nothing.
+  // Pair-wise: everything is chosen here and the S-Vector's 16 bytes in the tile become what is left to encode, the two pairs that
+  // stay and the outliers' values; positions and pattern nibbles are collected in registers, as the layout wants them (11008 x 4096
+  // against choosing in the second pass: 1:8 42.3 and 45.7 us, with E4M3 scales, where both passes have to choose, 49 and 74).
+  // Stored dense, with channel weights: the same, but the values stay where they are and the sets of dropped positions are
+  // collected (4096 x 11008, 1:8 + 6:8: 67 and 98).  Dense by magnitude: the outliers, if the most significant, hold the row's
+  // largest magnitude, this pass has nothing to choose and leaves it to the second.
+  constexpr bool CHOSEN = !DENSE || WGT;
   [[maybe_unused]] uint32_t c_o0[2] = {0, 0}, c_o1[2] = {0, 0}, c_nib[2] = {0, 0}, c_gone[4] = {0, 0, 0, 0};
   uint32_t all2 = 0, omax = 0, imax = 0, bad = 0;        // all2, imax: packed running maxima
   if constexpr (CHOSEN) {
@@ -394,9 +394,9 @@ pack_kernel(const PackParams p, const BlobHeader hdr)
           const uint4 v = *reinterpret_cast<const uint4*>(mine + i * 16);
           uint32_t r[4] = {v.x, v.y, v.z, v.w};
           all2 = max_magnitudes(all2, r);
-          if (DENSE && p.order_mask) group_maxima<false, OUTN>(p, r, nullptr, omax, imax);
+          if (p.order_mask) group_maxima<false, OUTN>(p, r, nullptr, omax, imax);
         }
-        if (!DENSE || !p.order_mask) omax = OUTN ? larger_half(all2) : 0u;
+        if (!p.order_mask) omax = larger_half(all2);
       }
       imax = larger_half(imax);
       bad = max(omax, larger_half(all2)) >= 0x7F80u;
@@ -459,14 +459,7 @@ pack_kernel(const PackParams p, const BlobHeader hdr)
       const int sv = 4 * b + i;
       [[maybe_unused]] int k[8];
       int o0, o1;
-      [[maybe_unused]] float f0, f1;
-      if constexpr (!DENSE && !CHOSEN) {
-        uint32_t w0, w1, nibble;
-        choose_pairs<WGT, OUTN>(p, x, WGT ? colw + 8 * sv : nullptr, o0, o1, f0, f1, w0, w1, nibble);
-        x[0] = w0;
-        x[1] = w1;
-        c_nib[sv >> 3] |= nibble << (4 * (sv & 7));
-      } else if constexpr (CHOSEN) {
+      if constexpr (CHOSEN) {
         o0 = (int)((c_o0[sv >> 3] >> (4 * (sv & 7))) & 7u);
         o1 = (int)((c_o1[sv >> 3] >> (4 * (sv & 7))) & 7u);
       } else {
@@ -475,12 +468,12 @@ pack_kernel(const PackParams p, const BlobHeader hdr)
       }
       // Stage 3, outliers: E4M3 codes of w / 2^e, or int8 codes of w / s
       if constexpr (OUTN > 0) {
-        const float f = DENSE ? pick_value(x, o0) : (CHOSEN ? __uint_as_float(x[2]) : f0);
+        const float f = DENSE ? pick_value(x, o0) : __uint_as_float(x[2]);
         ocode[i] = !DENSE && p.i8 ? int8_code(f, __int_as_float(e)) : e4m3x1(f * s8);
         opos[i] = (uint32_t)o0;
       }
       if constexpr (OUTN > 1) {
-        const float f = DENSE ? pick_value(x, o1) : (CHOSEN ? __uint_as_float(x[3]) : f1);
+        const float f = DENSE ? pick_value(x, o1) : __uint_as_float(x[3]);
         ocode1[i] = !DENSE && p.i8 ? int8_code(f, __int_as_float(e)) : e4m3x1(f * s8);
         opos1[i] = (uint32_t)o1;
       }
@@ -638,20 +631,14 @@ static void launch_pack(const PackParams& p, const BlobHeader& hdr, cudaStream_t
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, PK_SMEM) == cudaSuccess) (void)cudaLaunchKernelEx(&lc, kern, p, hdr);
   };
   if (cx <= 8) {
-    // Where the first pass has to choose anyway (channel weights, least significant outliers, two-level scaling's row factor)
-    // its choices are kept: 11008 x 4096, E4M3 scales 74 -> 60 us; 4096 x 11008 with weights, 1:8 88 -> 71, 1:8 + 6:8 98 -> 67.
-    // Otherwise choosing in the second pass saves writing them down (1:8: 49 against 56 us), except with two outliers (78, 75).
-    if constexpr (DENSE) go(pack_kernel<true, WGT, WGT, OUTN, true>, 1);
-    else if constexpr (WGT || OUTN == 2) go(pack_kernel<false, WGT, true, OUTN, true>, 1);
-    else if (p.order_mask || p.ue) go(pack_kernel<false, false, true, OUTN, true>, 1);
-    else go(pack_kernel<false, false, false, OUTN, true>, 1);
+    go(pack_kernel<DENSE, WGT, OUTN, true>, 1);
     return;
   }
   // rows longer than a cluster of eight CTAs holds
   const unsigned rows = (unsigned)(p.N / 8);
   if (WGT || p.order_mask || p.ue) row_scale_kernel<true, WGT, OUTN><<<rows, 256, 0, st>>>(p, hdr);
   else row_scale_kernel<false, WGT, OUTN><<<rows, 256, 0, st>>>(p, hdr);
-  go(pack_kernel<DENSE, WGT, DENSE && WGT, OUTN, false>, 0);
+  go(pack_kernel<DENSE, WGT, OUTN, false>, 0);
 }
 
 // One host-visible word per call in flight, where the kernels report a non-finite weight: a page of pinned memory, taken
