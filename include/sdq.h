@@ -114,8 +114,8 @@ typedef struct {
 } sdq_packed_t;
 
 /* Host-side descriptor of a quantized activation matrix (filled by sdq_quantize_act).
- *   off: 0 activation stages (4-bit codes | 8-bit codes | 4-bit scales per 128-token x 256-K tile)
- *        1 per-token 8-bit scale atoms   2 per-token 8-bit scale exponents   3.. reserved */
+ *   off: 0 records of 256 K: 4-bit codes | 4-bit scale atoms of all tokens   1 records of 128 K: 8-bit codes of all tokens
+ *        2 per-token 8-bit scale atoms   3 per-token 8-bit scale exponents   4.. reserved */
 typedef struct {
   void* dev;
   size_t bytes;
