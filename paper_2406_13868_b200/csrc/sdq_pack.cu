@@ -169,6 +169,16 @@ __device__ __forceinline__ uint32_t dropped_set(int (&k)[8], int o0, int o1, int
     if (OUTN > 0)
 #pragma unroll
       for (int i = 0; i < 8; ++i) k[i] = (m >> i) & 1u ? -1 : k[i];
+    if (grp4 && keep_in == 2) {                     // two of four, as in pick_pairs (11008 x 4096, 2:4: 71.5 us ranking all four -> 65.3)
+      m = 0xFFu;
+#pragma unroll
+      for (int g = 0; g < 8; g += 4) {
+        const bool first = min(k[g], k[g + 1]) >= max(k[g + 2], k[g + 3]), last = min(k[g + 2], k[g + 3]) > max(k[g], k[g + 1]);
+        const uint32_t one = k[g] >= k[g + 1] ? 1u : 2u, two = k[g + 2] >= k[g + 3] ? 4u : 8u;
+        m ^= (first ? 3u : (last ? 12u : one | two)) << g;
+      }
+      return m;
+    }
     uint32_t rank = 0;                              // nibble i: how many come before position i
 #pragma unroll
     for (int i = 0; i < 8; ++i)
@@ -452,6 +462,7 @@ pack_kernel(const PackParams p, const BlobHeader hdr)
   for (int b = 0; b < 4; ++b) {                          // blocks of 4 S-Vectors (32 K)
     uint32_t ocode[4], ocode1[4], opos[4], opos1[4];
     uint32_t dense_codes[4], dval[16];
+    [[maybe_unused]] uint32_t emeta[2] = {0, 0};
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const uint4 v = *reinterpret_cast<const uint4*>(mine + (4 * b + i) * 16);
@@ -490,14 +501,11 @@ pack_kernel(const PackParams p, const BlobHeader hdr)
 #pragma unroll
         for (int j = 0; j < 4; ++j) dval[4 * i + j] = x[j];
         if (p.elem) {
-          // the kept indices (two ascending 2-bit values per group of 4) are only needed by the exporter
-          uint32_t mb = 0;
-#pragma unroll
-          for (int q = 0; q < 2; ++q) {
-            const uint32_t bits = (~gone >> (4 * q)) & 15u;          // the group's four positions, exactly two of them set
-            mb |= (uint32_t)((__ffs((int)bits) - 1) | ((31 - __clz((int)bits)) << 2)) << (8 * q);
-          }
-          reinterpret_cast<uint16_t*>(p.blob + p.off.emeta + (size_t)n * (size_t)(p.K / 4))[(k2 * 2 + (int)h) * 16 + 4 * b + i] = (uint16_t)mb;
+          // the kept indices (two ascending 2-bit values per group of 4) are only needed by the exporter.  Exactly two of a
+          // group's four bits are set: the nibble that such a set stands for, looked up
+          const uint32_t lo = (~gone) & 15u, hi = (~gone >> 4) & 15u;
+          const uint32_t ml = ((lo & 8u) ? 0x000E0DC0u : 0x09804000u) >> (4 * (lo & 7u)), mh = ((hi & 8u) ? 0x000E0DC0u : 0x09804000u) >> (4 * (hi & 7u));
+          emeta[i >> 1] |= ((ml & 15u) | ((mh & 15u) << 8)) << (16 * (i & 1));
         }
       }
     }
@@ -516,6 +524,7 @@ pack_kernel(const PackParams p, const BlobHeader hdr)
         }
         dense_codes[i] = e2m1x8(f);
       }
+      if (p.elem) *reinterpret_cast<uint2*>(p.blob + p.off.emeta + (size_t)n * (size_t)(p.K / 4) + (kc * 16 + 4 * b) * 2) = make_uint2(emeta[0], emeta[1]);
       // 16 code bytes per 32 K: K-block (64 K) 2 h + b / 2 of the record, chunk b & 1
       *reinterpret_cast<uint4*>(wi + (2 * h + (b >> 1)) * 4096 + core + (b & 1) * 128) = make_uint4(dense_codes[0], dense_codes[1], dense_codes[2], dense_codes[3]);
       sc |= c << (8 * b);
