@@ -9,7 +9,7 @@
 // through distributed shared memory.  Longer rows: `row_scale_kernel` finds it and the same kernel follows without clusters.
 //
 // What bounds it: the integer pipe (selections on packed keys instead of index loops took it from ~350 instructions per S-Vector
-// over two passes to ~120), DRAM is at 35 %.  11008 x 4096, 1:8 + pair-wise 4:8: 189 us as one kernel with a CTA per row and a
+// over two passes to 138), DRAM is at 30 %.  11008 x 4096, 1:8 + pair-wise 4:8: 189 us as one kernel with a CTA per row and a
 // thread per S-Vector scattering bytes -> 20 + 42 us with the row scales in a launch of their own -> 49 us -> 42 us with the
 // pairs picked by two minima and two maxima instead of six comparisons and the choices kept from the first pass.  4096 x 11008,
 // 1:8 + 6:8 with channel weights: 98 us choosing in both passes -> 67.
