@@ -132,6 +132,13 @@ __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
   asm("prmt.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(sel));
   return d;
 }
+// two packed bf16, infinities as the largest finite number of their sign
+__device__ __forceinline__ uint32_t finite2(uint32_t x) {
+  const uint32_t top = 0x7F7F7F7Fu, bottom = 0xFF7FFF7Fu;
+  const __nv_bfloat162 r = __hmin2(__hmax2(*reinterpret_cast<const __nv_bfloat162*>(&x), *reinterpret_cast<const __nv_bfloat162*>(&bottom)),
+                                   *reinterpret_cast<const __nv_bfloat162*>(&top));
+  return *reinterpret_cast<const uint32_t*>(&r);
+}
 // running maxima of two packed bf16 magnitudes; a NaN stays, as one above infinity
 __device__ __forceinline__ uint32_t max_abs2(uint32_t m, uint32_t x) {
   const __nv_bfloat162 r = __hmax2_nan(*reinterpret_cast<const __nv_bfloat162*>(&m), __habs2(*reinterpret_cast<const __nv_bfloat162*>(&x)));

@@ -11,10 +11,10 @@
 // then a 4-lane shuffle, a token's four scales are one word, and every store instruction of codes writes whole 128-byte
 // lines (8 tokens x 16 B per core matrix).  Codes come from the hardware E2M1 / E4M3 converters.
 //
-// Bound by DRAM traffic and the conversion instructions: 2048 x 11008 at 3.8 TB/s of algorithmic bytes (20.8 us; a warp
-// per scattered 64-K Q-Vector with byte stores of scales: 24.7), 8192 x 4096 at 4.8 TB/s (24.6 us; 31.6), one token 2.3 us
+// Bound by DRAM traffic and the conversion instructions: 2048 x 11008 at 3.9 TB/s of algorithmic bytes (20.2 us; a warp
+// per scattered 64-K Q-Vector with byte stores of scales: 24.7), 8192 x 4096 at 5.0 TB/s (23.5 us; 31.6), one token 2.3 us
 // (4.6), most of it the launch.  E4M3 scales and int8 codes multiply by a reciprocal instead of dividing
-// every element (see sdq_codec.cuh): 4096 x 16384 with E4M3 scales 91 -> 61.3 us, int8 2048 x 4096 15.0 -> 12.6, one int8
+// every element (see sdq_codec.cuh): 4096 x 16384 with E4M3 scales 91 -> 60.0 us, int8 2048 x 4096 15.0 -> 12.3, one int8
 // token 14.1 -> 3.0 (zeros took the division's slow path).
 #include "sdq_codec.cuh"
 #include "sdq_internal.h"
@@ -32,7 +32,7 @@ constexpr int QA_CHUNK = QA_WARPS * K2;                  // K per CTA: one 256-K
 template <int NQ>
 struct QaUnit {
   uint4 raw[NQ][2];
-  uint32_t qmax[NQ];                                     // largest magnitude bits of the 16 elements; > 0x7F7F: an infinity
+  uint32_t qmax[NQ];                                     // largest magnitude bits of the 16 elements
 };
 // `on`: the token exists and the unit lies inside the row (zeros otherwise)
 template <int NQ>
@@ -48,7 +48,7 @@ __device__ __forceinline__ void qa_load(QaUnit<NQ>& u, const __nv_bfloat16* p, b
   }
 }
 // fills qmax and returns the largest magnitude bits of all the lane's elements.  +-Inf counts as the largest
-// finite bf16: maxima are clamped, the elements only where a lane holds one
+// finite bf16: maxima are clamped, the elements only where a lane of the warp holds one
 template <int NQ>
 __device__ __forceinline__ uint32_t qa_maxima(QaUnit<NQ>& u) {
   uint32_t m = 0;
@@ -59,10 +59,20 @@ __device__ __forceinline__ uint32_t qa_maxima(QaUnit<NQ>& u) {
 #pragma unroll
     for (int j = 0; j < 8; ++j) q = max_abs2(q, r[j]);
     q = max(q & 0xFFFFu, q >> 16);
-    u.qmax[i] = q;
-    m = max(m, min(q, 0x7F7Fu));
+    u.qmax[i] = min(q, 0x7F7Fu);
+    m = max(m, q);
   }
-  return m;
+  // (a branch of the warp: as predicated instructions in the encoding, the clamping cost 2 to 5 %)
+  if (__any_sync(0xffffffffu, m > 0x7F7Fu)) {
+#pragma unroll
+    for (int i = 0; i < NQ; ++i)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        uint4& w = u.raw[i][h];
+        w = make_uint4(finite2(w.x), finite2(w.y), finite2(w.z), finite2(w.w));
+      }
+  }
+  return min(m, 0x7F7Fu);
 }
 // writes `w` (a token's four scales of one 128- or 256-K block) to the overlapping atoms that hold the token: lane l (0..3)
 // of the token writes word l of atom m / 32 - l; `step` = bytes between atom numbers
@@ -94,11 +104,7 @@ __device__ __forceinline__ void qa_encode(const QaUnit<NQ>& u, int first, float 
       v[2 * j] = __uint_as_float(r[j] << 16);
       v[2 * j + 1] = __uint_as_float(r[j] & 0xFFFF0000u);
     }
-    if (u.qmax[i] > 0x7F7Fu) {
-#pragma unroll
-      for (int j = 0; j < 16; ++j) v[j] = sat(v[j]);
-    }
-    uint32_t bm = min(u.qmax[i], 0x7F7Fu);
+    uint32_t bm = u.qmax[i];
     bm = max(bm, __shfl_xor_sync(0xffffffffu, bm, 1));
     if (!b32) bm = max(bm, __shfl_xor_sync(0xffffffffu, bm, 2));
     uint32_t q4[2] = {0, 0}, q8[4] = {0, 0, 0, 0};
