@@ -333,6 +333,8 @@ pack_kernel(const PackParams p, const BlobHeader hdr)
   const int T1 = (int)(p.K / K1), T2 = T1 / 2;
   const int cx = (int)((p.K + PK_K - 1) / PK_K), rank = (int)(blockIdx.x % (uint32_t)cx);   // FUSED: a cluster is the cx CTAs of these rows
   const bool first_rows = blockIdx.x < (uint32_t)cx;
+  // (waited for before the first store into another CTA's shared memory: every CTA of the cluster has started by then)
+  if constexpr (FUSED) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
   const int64_t n_first = (int64_t)(blockIdx.x / (uint32_t)cx) * PK_ROWS;
   {
     // 256 threads x 16 B = the 4096 B of one row per round
@@ -416,6 +418,7 @@ pack_kernel(const PackParams p, const BlobHeader hdr)
     if (bad) *reinterpret_cast<volatile uint32_t*>(p.nonfinite) = 1u;
     s_part[0][row][ch] = OUTN ? omax : 0u;
     s_part[1][row][ch] = imax;
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
     __syncthreads();
     if (tid < 2 * PK_ROWS) {
       const uint32_t which = tid >> 4, r = tid & 15u;
@@ -429,7 +432,7 @@ pack_kernel(const PackParams p, const BlobHeader hdr)
         asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(ra), "r"(m) : "memory");
       }
     }
-    // one barrier: every push is visible after it, and nobody touches another CTA's memory afterwards
+    // every push is visible after this barrier, and nobody touches another CTA's memory afterwards
     asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
     omax = imax = 0;
     for (int c = 0; c < cx; ++c) { omax = max(omax, s_all[0][c][row]); imax = max(imax, s_all[1][c][row]); }

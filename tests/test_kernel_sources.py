@@ -1,0 +1,45 @@
+"""Orders that a kernel has to keep and that no run shows reliably, read from the sources."""
+import os
+import re
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2406_13868_b200", "csrc")
+
+
+def kernels():
+    """(file, name, body without comments) of every __global__ function"""
+    out = []
+    for f in sorted(os.listdir(CSRC)):
+        if not f.endswith(".cu"):
+            continue
+        src = re.sub(r"//[^\n]*|/\*.*?\*/", "", open(os.path.join(CSRC, f)).read(), flags=re.S)
+        for m in re.finditer(r"__global__", src):
+            open_brace = src.index("{", m.end())
+            name = re.findall(r"(\w+)\s*\((?=[^()]*\)\s*$)", src[m.end():open_brace])[-1]
+            depth, at = 1, open_brace + 1
+            while depth:
+                depth += {"{": 1, "}": -1}.get(src[at], 0)
+                at += 1
+            out.append((f, name, src[open_brace:at]))
+    return out
+
+
+# what reaches another CTA's shared memory, and what says that every CTA of the cluster has started
+REMOTE = re.compile(r"(?:st|ld)\.shared::cluster|ptx::(?:st_async|ld_cluster|mbar_arrive_remote|tc2_commit_both|tc2_commit_remote)\w*")
+STARTED = re.compile(r"ptx::cluster_sync\(\)|barrier\.cluster\.wait")
+
+
+def test_the_sources_are_read():
+    names = [n for _, n, _ in kernels()]
+    assert {"pack_kernel", "quant_act_fused_kernel", "channel_norm_kernel", "sdq_linear_kernel", "sdq_linear_pair_kernel", "sdq_linear_group_kernel"} <= set(names)
+    assert sum(bool(REMOTE.search(b)) for _, _, b in kernels()) == 6
+
+
+@pytest.mark.parametrize("name", [n for _, n, b in kernels() if REMOTE.search(b)])
+def test_no_remote_shared_memory_before_the_cluster_has_started(name):
+    """distributed shared memory may be touched only when all CTAs of the cluster are known to have started"""
+    for _, n, body in kernels():
+        if n == name:
+            first, started = REMOTE.search(body).start(), STARTED.search(body)
+            assert started and started.start() < first
