@@ -220,7 +220,7 @@ sdq_status_t sdq_act_size(int64_t M, int64_t K, const sdq_config_t* cfg, size_t*
  * E4M3 codes (A_o).  X (device) [M][ldx] bf16; xq_buf (device) >= sdq_act_size bytes; out (host).
  * +-Inf saturates, NaN input is undefined.  Asynchronous on `stream`; for K <= 16384 the one kernel it
  * enqueues carries programmatic stream serialization and waits for the previous kernel of the stream
- * before it reads X. */
+ * before it reads X and before it lets the next one begin. */
 sdq_status_t sdq_quantize_act(const void* X_bf16, int64_t M, int64_t K, int64_t ldx, const sdq_config_t* cfg,
                               void* xq_buf, size_t xq_bytes, sdq_act_t* out, void* stream);
 
@@ -272,6 +272,8 @@ sdq_status_t sdq_linear_f32_ws(const sdq_act_t* Xq, const sdq_packed_t* P, float
  *   SMs have their K range split over clusters of two or four thread blocks; the summation order over K of an output differs
  *   from sdq_linear's split-K paths, so results agree to fp32 rounding, not bit for bit.  Otherwise the layers are
  *   enqueued one after the other exactly as sdq_linear would.
+ *   The one launch waits for the previous kernel of the stream before it reads activations or packed weights or writes Y
+ *   (layers enqueued one after the other: as sdq_linear says).
  *   Asynchronous on `stream`; allocates nothing.  Errors as sdq_linear (the first failing layer's). */
 sdq_status_t sdq_linear_group(int n, const sdq_act_t* const* Xq, const sdq_packed_t* const* P, void* const* Y_bf16,
                               const int64_t* ldy, void* stream);
@@ -289,6 +291,8 @@ sdq_status_t sdq_linear_group_f32(int n, const sdq_act_t* const* Xq, const sdq_p
  *   Range: the fused kernel's (primary format, out_n <= 1, power-of-two scales, n <= 32, at least half as many 128-row
  *   tiles as SMs) with 1024 <= K <= 4096 (X has to fit beside the weight ring); outside it the call returns
  *   SDQ_ERR_UNSUPPORTED and launches nothing: quantize with sdq_quantize_act and use sdq_linear_group then.
+ *   The packed weights must be complete before the call is enqueued, as for sdq_linear: they are read before the previous kernel
+ *   of the stream has ended (so too with scratch, below).
  *   Asynchronous on `stream`; allocates nothing. */
 sdq_status_t sdq_linear_group_x(int n, const void* X_bf16, int64_t M, int64_t K, int64_t ldx, const sdq_packed_t* const* P,
                                 void* const* Y_bf16, const int64_t* ldy, void* stream);

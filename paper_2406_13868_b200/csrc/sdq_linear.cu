@@ -510,6 +510,7 @@ static void group_begin(GroupParams& g, int n, int64_t max_m, const sdq_packed_t
   g.out_n = w.cfg.out_n;
   g.out_i8 = g.out_n > 0 && w.cfg.out_fmt == SDQ_OUT_INT8;
   g.x_bf16 = nullptr; g.x_ld = 0; g.x_M = 0; g.scale_rule = w.cfg.scale_rule;
+  g.w_early = 0;
   g.total_items = 0;
   g.flags = device_flags();
 }
@@ -776,8 +777,9 @@ static sdq_status_t launch_group_x(int n, const void* X, int64_t M, int64_t K, i
   if (!g.flags) return SDQ_ERR_CUDA;
   sdq_act_t xq;
   if (ws) {
-    const sdq_status_t st = sdq_quantize_act(X, M, K, ldx, &P[0]->cfg, ws, ws_bytes, &xq, stream);
+    const sdq_status_t st = quantize_act(X, M, K, ldx, &P[0]->cfg, ws, ws_bytes, &xq, stream, true);
     if (st != SDQ_OK) return st;
+    g.w_early = 1;
   } else {
     g.x_bf16 = X; g.x_ld = ldx; g.x_M = (int)M;
   }

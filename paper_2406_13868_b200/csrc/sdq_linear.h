@@ -61,6 +61,7 @@ struct GroupMat {
 struct GroupParams {
   int n, n_tile, nslot, total_items;   // nslot: inlier ring positions
   int cluster_log2, rounds, tail_log2; // how the items are dealt out (filled in by launch_linear_group)
+  int w_early;           // 1: the packed weights are complete and may be read before the previous launch of the stream has ended
   int out_n;             // outliers per S-Vector, the same for every matrix of the call (0 or 1)
   int out_i8;            // the outlier operands are int8 with fp32 scales (else E4M3 with power-of-two scale atoms)
   // activation-resident variant (launch_linear_group with x_bf16 set): all matrices share one bf16 X [x_M][K], which every

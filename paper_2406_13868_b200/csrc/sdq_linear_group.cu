@@ -283,9 +283,11 @@ sdq_linear_group_kernel(const __grid_constant__ GroupParams p)
           k = k2 - sg.ke; ++iseq; have = false;
         }
       };
-      if (!XRES && !wc) {
-        // activations come from an earlier kernel; the first lap's inlier weights are fetched before the wait for it
-        if (inl && c == 0) {
+      if (!XRES) {
+        // activations come from an earlier kernel.  Packed weights are waited for too, but in calls that start from bf16 activations
+        // and are documented to want them complete: there the first lap's inlier records and all compact ones are fetched before the
+        // wait (gate / up int8, 5 tokens: 18.0 us per pass waiting for them, 17.3)
+        if (p.w_early && inl && c == 0) {
           for (uint32_t u = l; u < NI && seek(); u += 2, k += 2, ++ahead) {
             const GroupMat& m = p.m[sg.mat];
             ptx::mbar_expect_tx(&full_is[u], WI_BYTES + xb + SF_ATOM_BYTES);
@@ -293,7 +295,7 @@ sdq_linear_group_kernel(const __grid_constant__ GroupParams p)
           }
           k = (int)l; iseq = 0; have = false; sg.mat = 0;
         }
-        ptx::griddep_wait();
+        if (!(p.w_early && wc)) ptx::griddep_wait();
       }
       while (seek()) {
         const GroupMat& m = p.m[sg.mat];

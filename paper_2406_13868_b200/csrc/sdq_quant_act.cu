@@ -243,7 +243,7 @@ quant_act_kernel(const __nv_bfloat16* __restrict__ X, int64_t M, int64_t K, int6
 template <bool UE, int NQ>
 __global__ void __launch_bounds__(NQ == 4 ? QA_THREADS : 512, NQ == 4 ? (UE ? 3 : 4) : 1)
 quant_act_fused_kernel(const __nv_bfloat16* __restrict__ X, int64_t M, int64_t K, int64_t ldx, sdq_config_t cfg, uint8_t* __restrict__ buf,
-                       ActOffsets off, uint32_t* __restrict__ flags)
+                       ActOffsets off, uint32_t* __restrict__ flags, int early_next)
 {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int t = lane >> 2, l = lane & 3;                 // token within the group of 8, quarter of the Q-Vector
@@ -260,10 +260,11 @@ quant_act_fused_kernel(const __nv_bfloat16* __restrict__ X, int64_t M, int64_t K
   // (waited for before the first push: by then, behind the loads, every CTA's barrier has long been set up)
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
   // launched with programmatic stream serialization: X may still be being written by the previous kernel.  The next launch of
-  // the stream is let in before that wait: what it does before its own wait (set-up, fetching packed weights) then overlaps
-  // the previous kernel, and its wait for this grid includes this grid's wait for the previous one
-  if (tid == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // the stream is let in behind that wait: a linear kernel reads packed weights before its own, and those may be what the
+  // kernel in front of this one writes.  Before it only in calls that want the packed weights complete
+  if (early_next && tid == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (!early_next && tid == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int64_t m = (int64_t)blockIdx.y * 8 + t;
   const bool live = m < M;
   const int q = ((int)rank * warps + warp) * NQ;         // this warp's first Q-Vector
@@ -336,6 +337,10 @@ extern "C" sdq_status_t sdq_act_size(int64_t M, int64_t K, const sdq_config_t* c
 
 extern "C" sdq_status_t sdq_quantize_act(const void* X, int64_t M, int64_t K, int64_t ldx, const sdq_config_t* cfg, void* xq_buf,
                                          size_t xq_bytes, sdq_act_t* out, void* stream)
+{ return quantize_act(X, M, K, ldx, cfg, xq_buf, xq_bytes, out, stream, false); }
+
+sdq_status_t sdq::quantize_act(const void* X, int64_t M, int64_t K, int64_t ldx, const sdq_config_t* cfg, void* xq_buf, size_t xq_bytes, sdq_act_t* out,
+                               void* stream, bool early_next)
 {
   if (!X || !xq_buf || !out || !act_cfg_ok(cfg)) return SDQ_ERR_INVALID_ARG;
   if (cfg->scale_rule == SDQ_SCALE_UE4M3 && cfg->in_block != 32) return SDQ_ERR_UNSUPPORTED;
@@ -375,7 +380,7 @@ extern "C" sdq_status_t sdq_quantize_act(const void* X, int64_t M, int64_t K, in
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     lc.attrs = attr;
     lc.numAttrs = 2;
-    auto go = [&](auto kern) { return cudaLaunchKernelEx(&lc, kern, Xb, M, K, ldx, *cfg, bufp, off, flags); };
+    auto go = [&](auto kern) { return cudaLaunchKernelEx(&lc, kern, Xb, M, K, ldx, *cfg, bufp, off, flags, (int)early_next); };
     const cudaError_t le = nq == 4   ? (ue ? go(quant_act_fused_kernel<true, 4>) : go(quant_act_fused_kernel<false, 4>))
                            : nq == 2 ? (ue ? go(quant_act_fused_kernel<true, 2>) : go(quant_act_fused_kernel<false, 2>))
                                      : (ue ? go(quant_act_fused_kernel<true, 1>) : go(quant_act_fused_kernel<false, 1>));

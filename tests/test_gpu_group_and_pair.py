@@ -688,3 +688,34 @@ def test_group_x_with_and_without_scratch(M, K, out_fmt):
     assert (rc0, rc1, rc2, short) == (0, 0, 0, 5) and m.device_status() == 0
     assert torch.equal(inside, apart) and torch.equal(inside, none)
     assert all(torch.equal(a, b) for a, b in zip(m.sdq_linear_group_x(X, ps, f32=True), apart))
+
+
+@pytest.mark.parametrize("call", ["quantize_linear", "quantize_linear_many", "group"])
+def test_weights_written_by_the_kernel_in_front(call):
+    """packed weights written on the stream by a kernel that ends just before the call (or before its quantizer): never the bytes
+    that were there before"""
+    m = sdq()
+    cfg = m.Config()
+    M, N, K = (200 if call == "quantize_linear_many" else 5), 5120, 1024
+    sets = [[m.sdq_decompose(sdq_synth.make_weight(N, K, 400 + 2 * s + i).cuda(), cfg) for i in range(2)] for s in range(2)]
+    live = [m.packed_attach(p.buf.clone()) for p in sets[0]]
+    X = sdq_synth.make_act(M, K, 410).cuda()
+
+    def run(ps, xq):
+        if call == "group":
+            return m.sdq_linear_group([xq, xq], ps)
+        xq = m.sdq_quantize_act(X, cfg)
+        return [m.sdq_linear(xq, ps[0])]
+    xq = m.sdq_quantize_act(X, cfg)
+    want = [run(ps, xq) for ps in sets]
+    zero = torch.zeros_like(sets[0][0].buf)
+    got = []
+    for i in range(60):
+        src = sets[i % 2]
+        for d, p in zip(live[::-1], src[::-1]):          # (the matrix that is multiplied first is written last)
+            torch.bitwise_or(p.buf, zero, out=d.buf)
+        got.append(run(live, xq))
+    assert m.device_status() == 0
+    for i, ys in enumerate(got):
+        for a, b in zip(ys, want[i % 2]):
+            assert torch.equal(a, b), i

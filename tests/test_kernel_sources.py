@@ -43,3 +43,20 @@ def test_no_remote_shared_memory_before_the_cluster_has_started(name):
         if n == name:
             first, started = REMOTE.search(body).start(), STARTED.search(body)
             assert started and started.start() < first
+
+
+def test_packed_weights_are_ordered_behind_the_kernels_in_front():
+    """a quantizer lets the next launch in (which may read packed weights at once) only behind its own wait for the previous
+    one, and the grouped kernel copies nothing before its wait -- but in the calls that want the weights complete"""
+    body = {n: b for _, n, b in kernels()}
+    q = body["quant_act_fused_kernel"]
+    wait = q.index("griddepcontrol.wait")
+    lets_in = [(m.start() < wait, m.group(1)) for m in re.finditer(r"if \(([^()]*)\) asm volatile\(\"griddepcontrol\.launch_dependents", q)]
+    assert lets_in == [(True, "early_next && tid == 0"), (False, "!early_next && tid == 0")]
+    g = body["sdq_linear_group_kernel"]
+    assert re.search(r"if \(p\.w_early && inl && c == 0\) \{\s*for [^{}]*seek\(\)", g)
+    assert "if (!(p.w_early && wc)) ptx::griddep_wait();" in g
+    src = open(os.path.join(CSRC, "sdq_linear.cu")).read()
+    assert src.count("stream, true)") - src.count("stream, true); }") == src.count("w_early = 1") == 1
+    assert 0 < src.index("w_early = 1") - src.index("&xq, stream, true)") < 100
+    assert "out, stream, false); }" in open(os.path.join(CSRC, "sdq_quant_act.cu")).read()
