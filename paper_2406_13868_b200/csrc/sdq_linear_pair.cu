@@ -106,7 +106,7 @@ __global__ void __maxnreg__(96)
 sdq_linear_pair_kernel(const __grid_constant__ LinearParams p)
 {
   using G = PairGeom<B32, DENSE>;
-  constexpr bool S32 = G::S32;
+  constexpr bool S32 = G::S32, TWO_LEVEL = B32 && !DENSE && !F32_OUT;   // (bf16 outputs of two-level scaling)
   constexpr uint32_t NA = G::NA;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -393,15 +393,29 @@ sdq_linear_pair_kernel(const __grid_constant__ LinearParams p)
       const int64_t m0 = (int64_t)g0 * 32 + c_begin * 16;
       // tokens this group stores (a multiple of 16 in tensor memory, fewer at the end of the matrix; none beyond the last row tile)
       const int n_valid = rt < RT ? (int)max((int64_t)0, min((int64_t)(c_end - c_begin) * 16, p.M - m0)) : 0;
+      const int64_t n0 = (int64_t)rt * TILE_ROWS;
+      const int twr = p.tw && rt < RT ? __ldg(p.tw + n0 + q * 32 + lane) : 0;     // two-level scaling: this thread's row factor
+      // The bf16 output is rounded first and multiplied by its power of two when it is stored, which is the rounding of the
+      // multiplied value unless that falls below the normal range.  `tiny`: in this group of warps it may.  Accumulators are
+      // multiples of 2^-20 (products of two codes and two subnormal E4M3 scales) and of 2^-18 times the outliers' row scale
+      [[maybe_unused]] bool tiny = false;
+      if constexpr (TWO_LEVEL) {
+        if (p.tw && ks == 1 && n_valid) {
+          int tx = 127;
+          for (int i = (int)lane; i < n_valid; i += 32) tx = min(tx, __ldg(p.tx + m0 + i));
+          tx = __reduce_min_sync(0xffffffffu, tx);
+          const int e = T1 ? __ldg(reinterpret_cast<const int32_t*>(p.w + p.poff.osexp) + n0 + q * 32 + lane) : 0;
+          tiny = max(twr + tx, -126) + min(-20, T1 ? e - twr - 18 : -20) < -126;
+        }
+      }
       // one thread per group polls the barrier and releases the other 127 through a hardware barrier: hundreds of threads
       // polling one mbarrier notice its completion late and slow the CTA's other barrier traffic down
       if (et == 0 && !ptx::mbar_wait(&acc_full[ab], use & 1)) *timed_out = 1u;
-      ptx::named_bar_sync(1 + grp, 128);
+      if constexpr (TWO_LEVEL) tiny = ptx::named_bar_any(1 + grp, 128, tiny);
+      else ptx::named_bar_sync(1 + grp, 128);
       if (*timed_out) { ok = false; break; }
       ptx::tc_fence_after();
       const uint32_t tbase = tmem + ((q * 32u) << 16) + (ab + unit) * TMAX + c_begin * 16u;   // (alternating accumulators: one unit)
-      const int64_t n0 = (int64_t)rt * TILE_ROWS;
-      const int twr = p.tw && rt < RT ? __ldg(p.tw + n0 + q * 32 + lane) : 0;     // two-level scaling: this thread's row factor
       auto factor = [&](int64_t m) { return __int_as_float((min(max(twr + __ldg(p.tx + m), -126), 127) + 127) << 23); };
       auto hand_back = [&]() {      // this warp has read its part of the accumulator
         ptx::tc_fence_before();
@@ -421,9 +435,8 @@ sdq_linear_pair_kernel(const __grid_constant__ LinearParams p)
         }
         continue;
       }
-      if constexpr (F32_OUT) {
-        // fp32 output (tests): straight from TMEM
-        float* Y = reinterpret_cast<float*>(p.Y);
+      if (F32_OUT || tiny) {
+        // fp32 output (tests), or a scaled one that is rounded after the scaling: straight from TMEM
 #pragma unroll 1
         for (int c0 = 0; c0 < n_valid; c0 += 16) {
           uint32_t v[16];
@@ -434,7 +447,9 @@ sdq_linear_pair_kernel(const __grid_constant__ LinearParams p)
             if (c0 + j < n_valid) {
               float f = __uint_as_float(v[j]);
               if (p.tw) f *= factor(m0 + c0 + j);
-              Y[(m0 + c0 + j) * p.ldy + n0 + q * 32 + lane] = f;
+              const int64_t at = (m0 + c0 + j) * p.ldy + n0 + q * 32 + lane;
+              if constexpr (F32_OUT) reinterpret_cast<float*>(p.Y)[at] = f;
+              else reinterpret_cast<__nv_bfloat16*>(p.Y)[at] = __float2bfloat16_rn(f);
             }
         }
         hand_back();
@@ -459,7 +474,7 @@ sdq_linear_pair_kernel(const __grid_constant__ LinearParams p)
         hand_back();
         // transpose through shared memory, 4 tokens at a time per group: [4 tokens][128 features] bf16, then one 8-byte
         // store per thread (a warp writes one token's 256 B).  Two-level scaling: multiplying the rounded value by the power
-        // of two is the rounding of the multiplied value, so the factors go in here, after TMEM has been handed back.
+        // of two is the rounding of the multiplied value (not `tiny`), so the factors go in here, after TMEM has been handed back.
         uint16_t* stg = reinterpret_cast<uint16_t*>(stg_base) + grp * 512u;
         __nv_bfloat16* Y = reinterpret_cast<__nv_bfloat16*>(p.Y);
 #pragma unroll

@@ -339,6 +339,13 @@ __device__ __forceinline__ float4 ld_cluster_f32x4(uint32_t raddr) {
 __device__ __forceinline__ void named_bar_sync(uint32_t id, uint32_t threads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
+// the same barrier; true on all of its threads if `v` is true on any
+__device__ __forceinline__ bool named_bar_any(uint32_t id, uint32_t nthreads, bool v) {
+  uint32_t r;
+  asm volatile("{\n.reg .pred p, q;\nsetp.ne.u32 p, %3, 0;\nbarrier.cta.red.or.pred q, %1, %2, p;\nselp.u32 %0, 1, 0, q;\n}"
+               : "=r"(r) : "r"(id), "r"(nthreads), "r"((uint32_t)v) : "memory");
+  return r != 0;
+}
 
 }  // namespace ptx
 }  // namespace sdq

@@ -212,6 +212,26 @@ def test_cta_pair_task_forms(M, N, K, cfg_args):
     assert (d <= tol).all(), (d.max(), (d / tol).max())
 
 
+@pytest.mark.parametrize("M,N,K", [(100, 4096, 2048), (300, 384, 2048), (4001, 2304, 2048), (3371, 2688, 2048), (20, 1024, 512)])
+@pytest.mark.parametrize("order", [0, 1])
+def test_two_level_scaling_rounds_once_below_the_normal_range(M, N, K, order):
+    """two-level scaling, outputs on both sides of the smallest normal bf16 number: the bf16 output is the fp32 one rounded once, to
+    the nearest even"""
+    m = sdq()
+    cfg = m.Config(1, so.GRAN_PAIR, 32, so.SCALE_UE4M3, order)
+    W, X = sdq_synth.make_weight(N, K, 63).float(), sdq_synth.make_act(M, K, 64).float()
+    W[:, 0] = 0.0                      # a channel that sets the tokens' scale and adds nothing to the product
+    X *= 2.0 ** -11
+    X[:, 0] = 100.0
+    W, X = (W * 2.0 ** -60).to(torch.bfloat16), (X * 2.0 ** -53).to(torch.bfloat16)
+    p, xq = m.sdq_decompose(W.cuda(), cfg), m.sdq_quantize_act(X.cuda(), cfg)
+    y, y16 = m.sdq_linear(xq, p, f32=True), m.sdq_linear(xq, p)
+    assert m.device_status() == 0
+    below = (y.abs() < 2.0 ** -126) & (y != 0)
+    assert 0.02 < float(below.float().mean()) < 0.98
+    assert torch.equal(y16.view(torch.int16), y.to(torch.bfloat16).view(torch.int16))
+
+
 def _a_off(row, byte):
     j, b = byte >> 5, byte & 31
     return j * 4096 + (row >> 3) * 256 + (b >> 4) * 128 + (row & 7) * 16 + (b & 15)
