@@ -220,7 +220,8 @@ sdq_status_t sdq_act_size(int64_t M, int64_t K, const sdq_config_t* cfg, size_t*
  * E4M3 codes (A_o).  X (device) [M][ldx] bf16; xq_buf (device) >= sdq_act_size bytes; out (host).
  * +-Inf saturates, NaN input is undefined.  Asynchronous on `stream`; for K <= 16384 the one kernel it
  * enqueues carries programmatic stream serialization and waits for the previous kernel of the stream
- * before it reads X and before it lets the next one begin. */
+ * before it reads X and before it lets the next one begin.
+ * Errors: INVALID_ARG, UNSUPPORTED, SHAPE (for K <= 16384 also more than 524280 tokens), ALIGNMENT, BUFFER_TOO_SMALL, CUDA. */
 sdq_status_t sdq_quantize_act(const void* X_bf16, int64_t M, int64_t K, int64_t ldx, const sdq_config_t* cfg,
                               void* xq_buf, size_t xq_bytes, sdq_act_t* out, void* stream);
 

@@ -29,6 +29,12 @@ DeviceInfo* device_info_slot(int dev);
 // entry of the current device with sm_count filled in (nullptr on failure).  First use per device takes a lock.
 DeviceInfo* device_info();
 
+// status of a launch that returned `e`; takes the thread's last error with it, or the next call would report it as its own
+inline sdq_status_t launch_status(cudaError_t e) {
+  const cudaError_t last = cudaGetLastError();
+  return e == cudaSuccess && last == cudaSuccess ? SDQ_OK : SDQ_ERR_CUDA;
+}
+
 // sdq_quantize_act; early_next: the next launch of the stream, the caller's own, may begin and read packed weights before this
 // one has waited for its predecessor
 sdq_status_t quantize_act(const void* X, int64_t M, int64_t K, int64_t ldx, const sdq_config_t* cfg, void* xq_buf, size_t xq_bytes, sdq_act_t* out,

@@ -588,14 +588,14 @@ static sdq_status_t launch_linear(const sdq_act_t* Xq, const sdq_packed_t* P, vo
         if (!g.flags) return SDQ_ERR_CUDA;
         group_add(g, 0, Xq, *P, Y, ldy, M);
         const cudaError_t ge = launch_linear_group(g, f32, dinfo, (cudaStream_t)stream);
-        return ge == cudaSuccess && cudaGetLastError() == cudaSuccess ? SDQ_OK : SDQ_ERR_CUDA;
+        return launch_status(ge);
       }
     }
     pairs = two < few;
   }
   if (pairs) {
     const cudaError_t pe = launch_linear_pair(p, f32, dinfo, (cudaStream_t)stream);
-    return pe == cudaSuccess && cudaGetLastError() == cudaSuccess ? SDQ_OK : SDQ_ERR_CUDA;
+    return launch_status(pe);
   }
   p.n_tile = n_tile_for(M);
   p.slot_bytes = slot_bytes_for(p.n_tile, p.b32 != 0, p.dense != 0);
@@ -682,7 +682,7 @@ static sdq_status_t launch_linear(const sdq_act_t* Xq, const sdq_packed_t* P, vo
   lc.attrs = attr;
   lc.numAttrs = na;
   const cudaError_t le = f32 ? cudaLaunchKernelEx(&lc, sdq_linear_kernel<true>, p) : cudaLaunchKernelEx(&lc, sdq_linear_kernel<false>, p);
-  return le == cudaSuccess && cudaGetLastError() == cudaSuccess ? SDQ_OK : SDQ_ERR_CUDA;
+  return launch_status(le);
 }
 
 extern "C" sdq_status_t sdq_linear(const sdq_act_t* Xq, const sdq_packed_t* P, void* Y, int64_t ldy, void* stream)
@@ -743,7 +743,7 @@ static sdq_status_t launch_group(int n, const sdq_act_t* const* Xq, const sdq_pa
   if (!g.flags) return SDQ_ERR_CUDA;
   for (int i = 0; i < n; ++i) group_add(g, i, Xq[i], *P[i], Y[i], ldy[i], Xq[i]->M);
   const cudaError_t e = launch_linear_group(g, f32, dinfo, (cudaStream_t)stream);
-  return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? SDQ_OK : SDQ_ERR_CUDA;
+  return launch_status(e);
 }
 
 // The same from one bf16 X that all layers read (see include/sdq.h): with scratch, the quantizer's launch and then the grouped
@@ -785,7 +785,7 @@ static sdq_status_t launch_group_x(int n, const void* X, int64_t M, int64_t K, i
   }
   for (int i = 0; i < n; ++i) group_add(g, i, ws ? &xq : nullptr, *P[i], Y[i], ldy[i], M);
   const cudaError_t e = launch_linear_group(g, f32, dinfo, (cudaStream_t)stream);
-  return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? SDQ_OK : SDQ_ERR_CUDA;
+  return launch_status(e);
 }
 
 extern "C" sdq_status_t sdq_linear_group_x(int n, const void* X_bf16, int64_t M, int64_t K, int64_t ldx, const sdq_packed_t* const* P,

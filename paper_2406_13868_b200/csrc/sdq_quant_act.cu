@@ -354,6 +354,7 @@ sdq_status_t sdq::quantize_act(const void* X, int64_t M, int64_t K, int64_t ldx,
   const bool ue = cfg->scale_rule == SDQ_SCALE_UE4M3;
   const int n_chunks = (int)((K + QA_CHUNK - 1) / QA_CHUNK);      // = CTAs per token group: one 256-K unit per warp
   if (n_chunks <= 8) {
+    if ((M + 7) / 8 > 65535) return SDQ_ERR_SHAPE;                // token groups are the grid's second dimension
     uint32_t* flags = device_flags();
     if (!flags) return SDQ_ERR_CUDA;
     cudaLaunchConfig_t lc = {};
@@ -384,7 +385,7 @@ sdq_status_t sdq::quantize_act(const void* X, int64_t M, int64_t K, int64_t ldx,
     const cudaError_t le = nq == 4   ? (ue ? go(quant_act_fused_kernel<true, 4>) : go(quant_act_fused_kernel<false, 4>))
                            : nq == 2 ? (ue ? go(quant_act_fused_kernel<true, 2>) : go(quant_act_fused_kernel<false, 2>))
                                      : (ue ? go(quant_act_fused_kernel<true, 1>) : go(quant_act_fused_kernel<false, 1>));
-    if (le != cudaSuccess || cudaGetLastError() != cudaSuccess) return SDQ_ERR_CUDA;
+    if (launch_status(le) != SDQ_OK) return SDQ_ERR_CUDA;
   } else {
     float* partial = reinterpret_cast<float*>(bufp + off.amax);
     const dim3 grid((unsigned)((M + 7) / 8), (unsigned)n_chunks);

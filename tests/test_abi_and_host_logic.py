@@ -148,3 +148,11 @@ def test_bench_starts_its_own_ranks_when_run_without_a_launcher():
     # rank 1 "took" 20 ms for its 400 units, rank 0 10 ms: the job took the max, and processed both batches
     assert abs(d["ms_per_step"] - 20.0 / 4) < 1e-9
     assert abs(d["value"] - 2 * 400.0 / 20e-3) < 1e-6
+
+
+def test_quantizer_refuses_more_tokens_than_its_grid_holds(m):
+    """before anything is launched: the pointers are not looked at"""
+    L, cfg, b = m.lib(), m.Config(), ctypes.c_size_t()
+    i64, x, M = ctypes.c_int64, ctypes.c_void_p(0x1000), 65535 * 8 + 1
+    assert L.sdq_act_size(M, 256, ctypes.byref(cfg), ctypes.byref(b)) == 0
+    assert L.sdq_quantize_act(x, i64(M), i64(256), i64(256), ctypes.byref(cfg), x, b, ctypes.byref(m._Act()), None) == 2

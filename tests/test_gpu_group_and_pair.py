@@ -739,3 +739,16 @@ def test_weights_written_by_the_kernel_in_front(call):
     for i, ys in enumerate(got):
         for a, b in zip(ys, want[i % 2]):
             assert torch.equal(a, b), i
+
+
+def test_a_refused_call_leaves_nothing_behind_for_the_next_one():
+    """more tokens than one quantizer launch takes: refused as a shape, and the next call is not told of it"""
+    m = sdq()
+    cfg = m.Config()
+    X = torch.zeros((65535 * 8 + 1, 256), dtype=torch.bfloat16, device="cuda")
+    with pytest.raises(m.SdqError) as e:
+        m.sdq_quantize_act(X, cfg)
+    assert e.value.code == 2
+    assert m.sdq_quantize_act(X[:9], cfg).M == 9
+    torch.zeros(8, device="cuda").sum().item()
+    assert m.device_status() == 0
