@@ -600,7 +600,7 @@ static sdq_status_t launch_linear(const sdq_act_t* Xq, const sdq_packed_t* P, vo
   p.n_tile = n_tile_for(M);
   p.slot_bytes = slot_bytes_for(p.n_tile, p.b32 != 0, p.dense != 0);
   const int tiles = (int)(P->N / TILE_ROWS), T2c = (int)(P->K / K2);
-  if (!ws) {
+  if (ws_ks == 1) {              // (also with a workspace that this shape does not use: few_token_us is the time of this split)
     // cluster split-K: a cluster of up to 8 CTAs per row tile, one tile per CTA
     // as many members (1..8) as the budget and the inlier stages allow.  Clusters are placed inside one GPC, whose SM count
     // varies: sizes 3, 5, 6, 7 pack worse than powers of two, and a grid that needs every slot then runs a second wave
@@ -621,7 +621,7 @@ static sdq_status_t launch_linear(const sdq_act_t* Xq, const sdq_packed_t* P, vo
     // split in two and let the grid run in waves of two CTAs per SM (K >= 2048: below that the halves are too short)
     if (ks == 1 && tiles > sm_count && T2c >= 8) ks = 2;
     if (ks > 1) { p.ksplit = ks; p.cluster_ks = ks; }
-  } else if (ws_ks > 1) {
+  } else {
     size_t need = 0;
     sdq_workspace_size(M, P->N, P->K, &P->cfg, &need);
     if (ws_bytes < need) return SDQ_ERR_BUFFER_TOO_SMALL;

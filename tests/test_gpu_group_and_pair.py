@@ -752,3 +752,22 @@ def test_a_refused_call_leaves_nothing_behind_for_the_next_one():
     assert m.sdq_quantize_act(X[:9], cfg).M == 9
     torch.zeros(8, device="cuda").sum().item()
     assert m.device_status() == 0
+
+
+@pytest.mark.parametrize("M,N,K,block", [(5, 19072, 2048, 32), (64, 18944, 4096, 64), (5, 1024, 1024, 64)])
+def test_a_workspace_that_is_not_needed_changes_nothing(M, N, K, block):
+    """more row tiles than a split over a workspace is made for: the call runs as without one (the last shape does use it)"""
+    m = sdq()
+    cfg = m.Config(1, m.GRAN_PAIR, block)
+    p = m.sdq_decompose(sdq_synth.make_weight(N, K, 95).cuda(), cfg)
+    xq = m.sdq_quantize_act(sdq_synth.make_act(M, K, 96).cuda(), cfg)
+    need = m.workspace_size(M, N, K, cfg)
+    assert (need == 0) == (N > 1024)
+    ws = torch.zeros(max(need, 1 << 16), dtype=torch.uint8, device="cuda")
+    y = m.sdq_linear(xq, p, f32=True)
+    with_ws = m.sdq_linear(xq, p, f32=True, workspace=ws)
+    assert m.device_status() == 0
+    if need == 0:
+        assert torch.equal(y, with_ws) and not ws.any()
+    else:
+        assert torch.allclose(y, with_ws, rtol=1e-4, atol=1e-5)
