@@ -3,12 +3,17 @@ from __future__ import annotations
 
 import os
 import subprocess
+import sys
 import sysconfig
+import warnings
+
+import torch
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(_HERE, "csrc")
 LIB = os.path.join(_HERE, "libsdq_b200.so")
-BINDING = os.path.join(_HERE, "_binding.so")
+# C++ against torch's headers: the versions it was built for are part of the name, so a module of another torch is never loaded
+BINDING = os.path.join(_HERE, "_binding-%s-torch%s.so" % (sys.implementation.cache_tag, torch.__version__))
 BINDING_SOURCE = "sdq_python.cpp"
 SOURCES = ["sdq_api.cu", "sdq_pack.cu", "sdq_quant_act.cu", "sdq_linear.cu", "sdq_linear_pair.cu", "sdq_linear_group.cu", "sdq_plain.cu", "sdq_calib.cu", "sdq_diag.cu"]
 HEADERS = ["sdq_internal.h", "sdq_layout.h", "sdq_linear.h", "sdq_plain.h", "sdq_ptx.cuh", "sdq_codec.cuh", os.path.join("..", "..", "include", "sdq.h"), os.path.join("..", "..", "include", "sdq_diag.h")]
@@ -31,7 +36,6 @@ def _binding_stale() -> bool:
 
 
 def _build_binding() -> None:
-    import torch
     root = os.path.dirname(torch.__file__)
     inc = [os.path.join(root, "include"), os.path.join(root, "include", "torch", "csrc", "api", "include"), sysconfig.get_paths()["include"],
            os.path.join(os.environ.get("CUDA_HOME", "/usr/local/cuda"), "include")]
@@ -51,7 +55,10 @@ def build(force: bool = False, verbose: bool = False) -> str:
         subprocess.check_call(cmd, cwd=CSRC)
         os.replace(LIB + ".tmp", LIB)
     if force or _binding_stale():
-        _build_binding()
+        try:
+            _build_binding()
+        except (OSError, subprocess.CalledProcessError) as e:
+            warnings.warn("the binding's native half was not built (%s): calls go through ctypes, 6 to 12 us slower each" % e)
     return LIB
 
 

@@ -156,3 +156,19 @@ def test_quantizer_refuses_more_tokens_than_its_grid_holds(m):
     i64, x, M = ctypes.c_int64, ctypes.c_void_p(0x1000), 65535 * 8 + 1
     assert L.sdq_act_size(M, 256, ctypes.byref(cfg), ctypes.byref(b)) == 0
     assert L.sdq_quantize_act(x, i64(M), i64(256), i64(256), ctypes.byref(cfg), x, b, ctypes.byref(m._Act()), None) == 2
+
+
+def test_binding_without_its_native_half(m, monkeypatch, tmp_path):
+    """the native half is built for one torch, which its name says; where it is missing or does not load, calls go through ctypes,
+    and say so once"""
+    name = os.path.basename(m.BINDING)
+    assert torch.__version__ in name and sys.implementation.cache_tag in name
+    broken = tmp_path / "broken.so"
+    broken.write_bytes(b"not a module")
+    for path in (str(broken), str(tmp_path / "absent.so")):
+        monkeypatch.setattr(m, "BINDING", path)
+        monkeypatch.setattr(m, "_fast", None)
+        with pytest.warns(UserWarning, match="ctypes"):
+            assert m._native().quantize_act(None, None, None) is None
+        with pytest.raises(ValueError):                  # the ctypes form's own check
+            m.sdq_quantize_act(torch.zeros((8, 256), dtype=torch.bfloat16))
