@@ -245,7 +245,14 @@ PyObject* group(PyObject* xqs, PyObject* X, PyObject* ps, PyObject* outs, PyObje
     const at::Tensor& t = THPVariable_Unpack(X);
     xp = t.data_ptr(); M = t.size(0); K = t.size(1); ldx = t.stride(0);
     size_t bytes = 0;
-    if (sdq_act_size(M, K, &g.p[0]->cfg, &bytes) == SDQ_OK) ws = at::empty({(int64_t)bytes}, at::TensorOptions().dtype(at::kByte).device(t.device()));
+    // (16 tokens of 4096: the call's range, anything else is refused; X on another device, whose streams the allocator would hand
+    // the scratch on by, or no memory left: the form that needs none)
+    if (M <= 16 && K <= 4096 && t.device().index() == c10::cuda::current_device() && sdq_act_size(M, K, &g.p[0]->cfg, &bytes) == SDQ_OK) {
+      try {
+        ws = at::empty({(int64_t)bytes}, at::TensorOptions().dtype(at::kByte).device(t.device()));
+      } catch (const c10::OutOfMemoryError&) {
+      }
+    }
   }
   void* wp = ws.defined() ? ws.data_ptr() : nullptr;
   const size_t ws_bytes = ws.defined() ? (size_t)ws.numel() : 0;

@@ -771,3 +771,32 @@ def test_a_workspace_that_is_not_needed_changes_nothing(M, N, K, block):
         assert torch.equal(y, with_ws) and not ws.any()
     else:
         assert torch.allclose(y, with_ws, rtol=1e-4, atol=1e-5)
+
+
+def test_group_x_needs_no_memory():
+    """with no memory left for scratch the call runs in the form that needs none: the same bits"""
+    m = sdq()
+    cfg = m.Config()
+    ps = [m.sdq_decompose(sdq_synth.make_weight(5120, 4096, 97 + i).cuda(), cfg) for i in range(2)]
+    X = sdq_synth.make_act(16, 4096, 99).cuda()
+    want = m.sdq_linear_group_x(X, ps)
+    outs = [torch.zeros_like(y) for y in want]
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    total = torch.cuda.get_device_properties(0).total_memory
+    torch.cuda.set_per_process_memory_fraction(torch.cuda.memory_reserved() / total)
+    held = []
+    try:
+        with pytest.raises(torch.cuda.OutOfMemoryError):
+            while True:
+                held.append(torch.empty(1 << 18, dtype=torch.uint8, device="cuda"))
+        m.sdq_linear_group_x(X, ps, outs)
+    finally:
+        torch.cuda.set_per_process_memory_fraction(1.0)
+    assert m.device_status() == 0
+    for a, b in zip(outs, want):
+        assert torch.equal(a, b)
+    big = torch.zeros((17, 4096), dtype=torch.bfloat16, device="cuda")
+    with pytest.raises(m.SdqError) as e:
+        m.sdq_linear_group_x(big, ps)
+    assert e.value.code == 4
