@@ -3,6 +3,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "../../include/sdq.h"
 
 namespace sdq {
@@ -15,13 +17,15 @@ uint32_t* device_flags();
 
 // Host-side facts about one device, looked up by the CURRENT device of the calling thread: they differ between the
 // GPUs of one process (SM count; function attributes are per context), so nothing of this kind is a process-wide static.
+// Threads share the table: sm_count is filled in under a lock, and so are pair_clusters, before clusters_known says so.
 struct DeviceInfo {
   int sm_count;            // 0 until queried
-  uint32_t linear_attr;    // 1: the single-CTA GEMM instantiations carry their shared-memory attribute
-  uint32_t pair_attr;      // bit per CTA-pair GEMM instantiation
-  uint32_t diag_attr;      // the copy-rate diagnostic
-  uint32_t group_attr;     // the grouped few-token GEMM
-  int pair_clusters[5];    // CTA-pair GEMM: clusters of k pairs that run at once (entry 1 set: filled in)
+  std::atomic<uint32_t> linear_attr;    // 1: the single-CTA GEMM instantiations carry their shared-memory attribute
+  std::atomic<uint32_t> pair_attr;      // bit per CTA-pair GEMM instantiation
+  std::atomic<uint32_t> diag_attr;      // the copy-rate diagnostic
+  std::atomic<uint32_t> group_attr;     // the grouped few-token GEMM
+  std::atomic<uint32_t> clusters_known; // 1: pair_clusters is filled in
+  int pair_clusters[5];    // CTA-pair GEMM: clusters of k pairs that run at once
 };
 constexpr int MAX_DEVICES = 64;
 // entry of device `dev` (0 <= dev < MAX_DEVICES) in the table; nullptr outside that range

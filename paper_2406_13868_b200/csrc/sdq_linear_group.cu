@@ -679,7 +679,6 @@ double group_kernel_us(int64_t items, int T2, DeviceInfo* d) { return group_plan
 
 cudaError_t launch_linear_group(GroupParams p, bool f32_out, DeviceInfo* d, cudaStream_t stream)
 {
-  uint32_t* attr_done = &d->group_attr;
   int T2_min = p.m[0].T2;
   int64_t units = 0;
   for (int i = 0; i < p.n; ++i) {
@@ -694,7 +693,7 @@ cudaError_t launch_linear_group(GroupParams p, bool f32_out, DeviceInfo* d, cuda
   const int is = xres ? WI_BYTES : group_is_bytes(p.n_tile), os = p.out_n ? 2 * wc_bytes(1) + (xres ? 0 : 2 * p.n_tile * 128) : 0;
   p.nslot = group_units(p.n_tile, p.out_n, xbytes);
   const int smem = p.nslot * is + GRP_UNITS * os + xbytes + (p.out_n ? GRP_SIDE_BYTES : 0) + GRP_BAR_BYTES + 128;
-  if (!*attr_done) {
+  if (!d->group_attr) {
     const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
     bool ok = true;
     auto set = [&](auto kern) { ok = ok && cudaFuncSetAttribute(kern, a, 232448) == cudaSuccess; };
@@ -704,7 +703,7 @@ cudaError_t launch_linear_group(GroupParams p, bool f32_out, DeviceInfo* d, cuda
     set(sdq_linear_group_kernel<false, true, true>); set(sdq_linear_group_kernel<true, true, true>);
     if (!ok)
       return cudaErrorUnknown;
-    *attr_done = 1;
+    d->group_attr = 1;
   }
   cudaLaunchConfig_t lc = {};
   lc.gridDim = dim3((unsigned)plan.ctas);

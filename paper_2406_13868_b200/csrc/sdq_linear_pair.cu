@@ -37,6 +37,7 @@
 // uniform-register operands, so the issue loop is warp-uniform with one elected lane; a trip of a single-thread loop costs
 // 0.3 us, hence two lanes per producer and runs of landed slots in the issuer; a pair-wide commit costs the pipe ~80 ns.
 #include <cuda_bf16.h>
+#include <mutex>
 #include <type_traits>
 
 #include "sdq_internal.h"
@@ -547,7 +548,7 @@ sdq_linear_pair_kernel(const __grid_constant__ LinearParams p)
 }
 
 template <bool F32_OUT, bool B32, bool DENSE, int FORM>
-static cudaError_t launch_form(const LinearParams& p, int pairs, cudaStream_t stream, uint32_t* attr_mask)
+static cudaError_t launch_form(const LinearParams& p, int pairs, cudaStream_t stream, std::atomic<uint32_t>* attr_mask)
 {
   auto kern = sdq_linear_pair_kernel<F32_OUT, B32, DENSE, FORM>;
   const uint32_t bit = 1u << (((F32_OUT ? 3 : 0) + (DENSE ? 2 : (B32 ? 1 : 0))) * 3 + FORM);
@@ -573,7 +574,7 @@ static cudaError_t launch_form(const LinearParams& p, int pairs, cudaStream_t st
   return cudaLaunchKernelEx(&lc, kern, p);
 }
 template <bool F32_OUT, bool B32, bool DENSE>
-static cudaError_t launch_one(const LinearParams& p, int form, int pairs, cudaStream_t stream, uint32_t* attr_mask)
+static cudaError_t launch_one(const LinearParams& p, int form, int pairs, cudaStream_t stream, std::atomic<uint32_t>* attr_mask)
 {
   if (form == PAIR_TWO) return launch_form<F32_OUT, B32, DENSE, PAIR_TWO>(p, pairs, stream, attr_mask);
   if (form == PAIR_FULL) return launch_form<F32_OUT, B32, DENSE, PAIR_FULL>(p, pairs, stream, attr_mask);
@@ -649,9 +650,12 @@ static PairPlan pair_best(int64_t M, int64_t N, int64_t K, int out_n, bool b32, 
 // largest grids, in clusters of 4, 6 and 8 CTAs with one CTA per SM, that run at once on the current device: [pairs per cluster]
 const int* pair_max_clusters(DeviceInfo* d)
 {
-  if (!d->pair_clusters[1]) {
+  static const int none[5] = {0, 0, 0, 0, 0};
+  static std::mutex filling;
+  if (!d->clusters_known) {
+    std::lock_guard<std::mutex> lock(filling);
     auto kern = sdq_linear_pair_kernel<false, false, false, PAIR_FLEX>;
-    for (int k = 2; k <= 4; ++k) {
+    for (int k = 2; k <= 4 && !d->clusters_known; ++k) {
       cudaLaunchConfig_t lc = {};
       lc.gridDim = dim3((unsigned)(2 * k));
       lc.blockDim = dim3(PAIR_THREADS);
@@ -663,12 +667,11 @@ const int* pair_max_clusters(DeviceInfo* d)
       attr[0].val.clusterDim.z = 1;
       lc.attrs = attr;
       lc.numAttrs = 1;
-      int n = 0;
+      // (not answered: plans without larger clusters, and the next call asks again)
       if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448) != cudaSuccess ||
-          cudaOccupancyMaxActiveClusters(&n, kern, &lc) != cudaSuccess) { n = 0; (void)cudaGetLastError(); }
-      d->pair_clusters[k] = n;
+          cudaOccupancyMaxActiveClusters(&d->pair_clusters[k], kern, &lc) != cudaSuccess) { (void)cudaGetLastError(); return none; }
     }
-    d->pair_clusters[1] = 1;
+    d->clusters_known = 1;
   }
   return d->pair_clusters;
 }
@@ -682,7 +685,7 @@ cudaError_t launch_linear_pair(LinearParams p, bool f32_out, DeviceInfo* d, cuda
   const uint32_t wib = p.dense ? 17408u : (p.b32 ? 11264u : 10752u);
   int pairs = d->sm_count / 2;
   const PairPlan best = pair_best(p.M, p.N, p.K, p.out_n, p.b32 != 0, p.dense != 0, d->sm_count, pair_max_clusters(d));
-  uint32_t* attr_mask = &d->pair_attr;
+  std::atomic<uint32_t>* attr_mask = &d->pair_attr;
   const int T = best.form == PAIR_FLEX ? best.T : pair_tmax(best.form, s32);
   p.n_tile = T;
   p.pt_units = (int)((p.N + 2 * TILE_ROWS - 1) / (2 * TILE_ROWS)); p.pt_mtiles = best.mt; p.pt_groups = (int)((p.M + 31) / 32);

@@ -60,3 +60,13 @@ def test_packed_weights_are_ordered_behind_the_kernels_in_front():
     assert src.count("stream, true)") - src.count("stream, true); }") == src.count("w_early = 1") == 1
     assert 0 < src.index("w_early = 1") - src.index("&xq, stream, true)") < 100
     assert "out, stream, false); }" in open(os.path.join(CSRC, "sdq_quant_act.cu")).read()
+
+
+def test_the_device_table_is_safe_to_share():
+    """what host threads share per device is atomic, or filled in under a lock before an atomic word says so"""
+    src = open(os.path.join(CSRC, "sdq_internal.h")).read()
+    members = re.findall(r"^  ([\w:<>]+) (\w+)(?:\[\d\])?;", src[src.index("struct DeviceInfo {"):src.index("constexpr int MAX_DEVICES")], flags=re.M)
+    assert {n for t, n in members if not t.startswith("std::atomic")} == {"sm_count", "pair_clusters"}
+    pair = open(os.path.join(CSRC, "sdq_linear_pair.cu")).read()
+    body = pair[pair.index("const int* pair_max_clusters(DeviceInfo* d)\n{"):]
+    assert body.index("lock_guard") < body.index("&d->pair_clusters[k]") < body.index("d->clusters_known = 1")
