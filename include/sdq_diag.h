@@ -31,6 +31,33 @@ sdq_status_t sdq_diag_l2_copy(const void* src, size_t src_bytes, int slot_bytes,
  * the context stays usable.  Asynchronous on `stream`.  Errors: SHAPE (polls out of range), CUDA. */
 sdq_status_t sdq_diag_wait_timeout(int polls, void* stream);
 
+/* What a call would run, decided by the functions that decide it in the call itself; nothing is launched.
+ *   sm_count > 0: for a GPU of that many SMs, of which max_clusters[k] (k = 2, 3, 4; NULL: none) clusters of 2 k thread blocks, one
+ *   per SM, run at once -- host code only; sm_count == 0: for the current device (max_clusters is then ignored).
+ *   sdq_diag_linear_plan: sdq_linear (workspace != 0: sdq_linear_ws with one that is large enough) of M tokens and an N x K matrix.
+ *   sdq_diag_group_plan: the one launch of sdq_linear_group on n layers N[i] x K[i] in its range.
+ *   tasks (may be NULL): the first `cap` of out->tasks pieces of work, in the order that thread blocks take them.  CTA pairs: row units
+ *   (256 rows) row .. row + rows - 1 of 32-token groups begin .. end - 1 of the call, all of K.  Grouped kernel: row tile (128 rows)
+ *   `row` of layer `layer`, its 256-K units begin .. end - 1.  The few-token kernel has none to tell.
+ *   Errors: INVALID_ARG, SHAPE, UNSUPPORTED, CUDA. */
+enum { SDQ_DIAG_FEW = 0, SDQ_DIAG_PAIRS = 1, SDQ_DIAG_GROUP = 2 };
+typedef struct {
+  int32_t kernel;      /* SDQ_DIAG_* */
+  int32_t token_tile;  /* tokens of the widest tile there is room for */
+  int32_t ksplit;      /* parts of the K range: of a row tile (few-token), of a task (pairs), of a left-over item (grouped) */
+  int32_t cluster;     /* thread blocks per cluster (few-token with a workspace: 1) */
+  int32_t ctas, tasks; /* (pairs, grouped) */
+  int32_t form;        /* pairs: 0 two row units per task, 1 one, 2 one with geometry from the launch */
+  int32_t alternate;   /* pairs: the accumulator alternates between two sets of columns */
+  int32_t doubles, halves;   /* pairs, form 0: tasks of two units, and the tasks behind them that are halves of such */
+  int32_t rounds, tail_items;   /* grouped: whole items per thread block, left-over items per cluster */
+} sdq_diag_plan_t;
+typedef struct { int32_t layer, row, rows, begin, end; } sdq_diag_task_t;
+sdq_status_t sdq_diag_linear_plan(int64_t M, int64_t N, int64_t K, const sdq_config_t* cfg, int workspace, int sm_count,
+                                  const int* max_clusters, sdq_diag_plan_t* out, sdq_diag_task_t* tasks, int64_t cap);
+sdq_status_t sdq_diag_group_plan(int n, int64_t M, const int64_t* N, const int64_t* K, int sm_count, const int* max_clusters,
+                                 sdq_diag_plan_t* out, sdq_diag_task_t* segs, int64_t cap);
+
 #ifdef __cplusplus
 }
 #endif

@@ -498,11 +498,10 @@ extern "C" sdq_status_t sdq_workspace_size(int64_t M, int64_t N, int64_t K, cons
 
 // The grouped kernel carries the primary format: up to 32 tokens, pair-wise 4:8 inliers, one E8M0 scale per 64 K, at most one
 // outlier per S-Vector, and K >= 1024: an item then spans enough units that the per-item barriers never run two phases apart.
-static bool group_format(const sdq_packed_t& w) {
-  const sdq_config_t& c = w.cfg;
-  return c.in_gran == SDQ_GRAN_PAIR && c.in_block == 64 && c.scale_rule != SDQ_SCALE_UE4M3 && c.out_n <= 1 && w.K >= 4 * K2;
+static bool group_format(const sdq_config_t& c, int64_t K) {
+  return c.in_gran == SDQ_GRAN_PAIR && c.in_block == 64 && c.scale_rule != SDQ_SCALE_UE4M3 && c.out_n <= 1 && K >= 4 * K2;
 }
-static bool group_kernel_takes(const sdq_act_t& x, const sdq_packed_t& w) { return x.M <= 32 && group_format(w); }
+static bool group_kernel_takes(int64_t M, const sdq_packed_t& w) { return M <= 32 && group_format(w.cfg, w.K); }
 // launch parameters of `n` layers with the format of `w`, up to `max_m` tokens; then one group_add per layer, in order
 static void group_begin(GroupParams& g, int n, int64_t max_m, const sdq_packed_t& w) {
   g.n = n;
@@ -529,6 +528,49 @@ static void group_add(GroupParams& g, int i, const sdq_act_t* x, const sdq_packe
   m.M = (int)M; m.T2 = (int)(w.K / K2);
   m.item0 = g.total_items;
   g.total_items += (int)(w.N / TILE_ROWS);
+}
+
+// How a single call is run: CTA pairs above 128 tokens.  Up to 128, unless a workspace asks for its split, the kernel with the least
+// estimated time: this file's, the pairs, or the grouped kernel on one layer (one token: 4096 x 4096 7.7 -> 7.4 us,
+// 4096 -> 11008 12.1 -> 8.7, 11008 -> 4096 12.7 -> 10.0; 100 tokens, 4096 -> 11008: 17.0 -> 15.1 on pairs).
+struct LinearRoute { int kernel, ksplit, cluster_ks; };            // SDQ_DIAG_*; the split of K of this file's kernel (cluster_ks = 1: over the workspace)
+static LinearRoute linear_route(int64_t M, int64_t N, int64_t K, const sdq_config_t& cfg, bool ws, int sm_count, const int* max_clusters) {
+  LinearRoute r = {SDQ_DIAG_PAIRS, 1, 1};
+  if (M > 128) return r;
+  if (ws) {
+    r.ksplit = choose_ksplit(M, N, K, sm_count);
+    if (r.ksplit > 1) { r.kernel = SDQ_DIAG_FEW; return r; }
+  }
+  const bool dense = is_dense_layout(cfg);
+  const int tiles = (int)(N / TILE_ROWS), T2 = (int)(K / K2);
+  const double few = few_token_us(M, N, K, cfg), two = pair_kernel_us(M, N, K, cfg.out_n, cfg.in_block == 32, dense, sm_count, max_clusters);
+  if (M <= 32 && group_format(cfg, K)) {
+    const double one = group_kernel_us(tiles, T2, sm_count, max_clusters);
+    if (one < few && one < two) { r.kernel = SDQ_DIAG_GROUP; return r; }
+  }
+  if (two < few) return r;
+  r.kernel = SDQ_DIAG_FEW;
+  // cluster split-K: a cluster of up to 8 CTAs per row tile, one tile per CTA
+  // as many members (1..8) as the budget and the inlier stages allow.  Clusters are placed inside one GPC, whose SM count
+  // varies: sizes 3, 5, 6, 7 pack worse than powers of two, and a grid that needs every slot then runs a second wave
+  // (96 clusters of 3 took 21 us, 96 of 2 take 14), so odd sizes only get 88 % of the budget
+  auto split_for = [&](int cta_budget) {
+    for (int k = 8; k > 1; --k) {
+      const bool pow2 = (k & (k - 1)) == 0;
+      if (k <= T2 && (int64_t)k * tiles <= (pow2 ? cta_budget : cta_budget * 22 / 25)) return k;
+    }
+    return 1;
+  };
+  // CTAs the grid may have: up to 64 tokens the CTAs are small enough for two per SM; from 65 to 128 tokens two
+  // per SM leave only three ring slots, which pays only when one per SM would leave many SMs idle
+  int ks = split_for(M <= 64 ? 2 * sm_count : sm_count);
+  if (M > 64 && ks * tiles * 5 <= sm_count * 3) ks = split_for(2 * sm_count);
+  // more row tiles than SMs: one CTA per SM walking whole-K tiles streams a tile in ~19 us however few tiles its
+  // last round holds (149 tiles took 38 us, 148 took 16), while two half-K CTAs per SM keep more bytes in flight;
+  // split in two and let the grid run in waves of two CTAs per SM (K >= 2048: below that the halves are too short)
+  if (ks == 1 && tiles > sm_count && T2 >= 8) ks = 2;
+  r.ksplit = r.cluster_ks = ks;
+  return r;
 }
 
 static sdq_status_t launch_linear(const sdq_act_t* Xq, const sdq_packed_t* P, void* Y, int64_t ldy, void* ws, size_t ws_bytes,
@@ -566,66 +608,29 @@ static sdq_status_t launch_linear(const sdq_act_t* Xq, const sdq_packed_t* P, vo
   p.M = Xq->M; p.N = P->N; p.K = P->K;
   p.out_n = P->cfg.out_n;
   const int64_t M = Xq->M;
-  p.ksplit = 1;
-  p.cluster_ks = 1;
   p.ws_counter = nullptr;
   p.ws_partial = nullptr;
   p.Y = Y; p.ldy = ldy;
   p.flags = device_flags();
   if (!p.flags) return SDQ_ERR_CUDA;
-  // CTA pairs: all calls above 128 tokens.  Up to 128, unless a workspace asks for its split, the kernel with the least
-  // estimated time: this file's, the pairs, or the grouped kernel on one layer (one token: 4096 x 4096 7.7 -> 7.4 us,
-  // 4096 -> 11008 12.1 -> 8.7, 11008 -> 4096 12.7 -> 10.0; 100 tokens, 4096 -> 11008: 17.0 -> 15.1 on pairs).
-  const int ws_ks = ws ? choose_ksplit(M, P->N, P->K, sm_count) : 1;
-  bool pairs = M > 128;
-  if (!pairs && ws_ks == 1) {
-    const double few = few_token_us(M, P->N, P->K, P->cfg), two = pair_kernel_us(M, P->N, P->K, p.out_n, p.b32 != 0, p.dense != 0, dinfo);
-    if (group_kernel_takes(*Xq, *P)) {
-      const double one = group_kernel_us(P->N / TILE_ROWS, (int)(P->K / K2), dinfo);
-      if (one < few && one < two) {
-        GroupParams g;
-        group_begin(g, 1, M, *P);
-        if (!g.flags) return SDQ_ERR_CUDA;
-        group_add(g, 0, Xq, *P, Y, ldy, M);
-        const cudaError_t ge = launch_linear_group(g, f32, dinfo, (cudaStream_t)stream);
-        return launch_status(ge);
-      }
-    }
-    pairs = two < few;
+  const LinearRoute route = linear_route(M, P->N, P->K, P->cfg, ws != nullptr, sm_count, pair_max_clusters(dinfo));
+  if (route.kernel == SDQ_DIAG_GROUP) {
+    GroupParams g;
+    group_begin(g, 1, M, *P);
+    if (!g.flags) return SDQ_ERR_CUDA;
+    group_add(g, 0, Xq, *P, Y, ldy, M);
+    return launch_status(launch_linear_group(g, f32, dinfo, (cudaStream_t)stream));
   }
-  if (pairs) {
-    const cudaError_t pe = launch_linear_pair(p, f32, dinfo, (cudaStream_t)stream);
-    return launch_status(pe);
-  }
+  if (route.kernel == SDQ_DIAG_PAIRS) return launch_status(launch_linear_pair(p, f32, dinfo, (cudaStream_t)stream));
   p.n_tile = n_tile_for(M);
   p.slot_bytes = slot_bytes_for(p.n_tile, p.b32 != 0, p.dense != 0);
-  const int tiles = (int)(P->N / TILE_ROWS), T2c = (int)(P->K / K2);
-  if (ws_ks == 1) {              // (also with a workspace that this shape does not use: few_token_us is the time of this split)
-    // cluster split-K: a cluster of up to 8 CTAs per row tile, one tile per CTA
-    // as many members (1..8) as the budget and the inlier stages allow.  Clusters are placed inside one GPC, whose SM count
-    // varies: sizes 3, 5, 6, 7 pack worse than powers of two, and a grid that needs every slot then runs a second wave
-    // (96 clusters of 3 took 21 us, 96 of 2 take 14), so odd sizes only get 88 % of the budget
-    auto split_for = [&](int cta_budget) {
-      for (int k = 8; k > 1; --k) {
-        const bool pow2 = (k & (k - 1)) == 0;
-        if (k <= T2c && (int64_t)k * tiles <= (pow2 ? cta_budget : cta_budget * 22 / 25)) return k;
-      }
-      return 1;
-    };
-    // CTAs the grid may have: up to 64 tokens the CTAs are small enough for two per SM; from 65 to 128 tokens two
-    // per SM leave only three ring slots, which pays only when one per SM would leave many SMs idle
-    int ks = split_for(M <= 64 ? 2 * sm_count : sm_count);
-    if (M > 64 && ks * tiles * 5 <= sm_count * 3) ks = split_for(2 * sm_count);
-    // more row tiles than SMs: one CTA per SM walking whole-K tiles streams a tile in ~19 us however few tiles its
-    // last round holds (149 tiles took 38 us, 148 took 16), while two half-K CTAs per SM keep more bytes in flight;
-    // split in two and let the grid run in waves of two CTAs per SM (K >= 2048: below that the halves are too short)
-    if (ks == 1 && tiles > sm_count && T2c >= 8) ks = 2;
-    if (ks > 1) { p.ksplit = ks; p.cluster_ks = ks; }
-  } else {
+  const int tiles = (int)(P->N / TILE_ROWS);
+  p.ksplit = route.ksplit;
+  p.cluster_ks = route.cluster_ks;
+  if (p.ksplit > 1 && p.cluster_ks == 1) {
     size_t need = 0;
     sdq_workspace_size(M, P->N, P->K, &P->cfg, &need);
     if (ws_bytes < need) return SDQ_ERR_BUFFER_TOO_SMALL;
-    p.ksplit = ws_ks;
     p.ws_counter = (uint32_t*)ws;
     p.ws_partial = (float*)((uint8_t*)ws + (((size_t)tiles * 4 + 255) & ~(size_t)255));
   }
@@ -726,7 +731,7 @@ static sdq_status_t launch_group(int n, const sdq_act_t* const* Xq, const sdq_pa
     if (!is_tensor_core_reading(w->cfg)) return SDQ_ERR_UNSUPPORTED;
     if (w->cfg.out_n > 0 && x->cfg.out_fmt != w->cfg.out_fmt) return SDQ_ERR_SHAPE;
     if (((uintptr_t)Y[i] & 15) || (ldy[i] % 8)) return SDQ_ERR_ALIGNMENT;
-    fused = fused && group_kernel_takes(*x, *w) && w->cfg.out_n == P[0]->cfg.out_n && w->cfg.out_fmt == P[0]->cfg.out_fmt;
+    fused = fused && group_kernel_takes(x->M, *w) && w->cfg.out_n == P[0]->cfg.out_n && w->cfg.out_fmt == P[0]->cfg.out_fmt;
     items += w->N / TILE_ROWS;
     if (x->M > max_m) max_m = x->M;
   }
@@ -766,7 +771,7 @@ static sdq_status_t launch_group_x(int n, const void* X, int64_t M, int64_t K, i
     if (!is_tensor_core_reading(w->cfg)) return SDQ_ERR_UNSUPPORTED;
     if (((uintptr_t)Y[i] & 15) || (ldy[i] % 8)) return SDQ_ERR_ALIGNMENT;
     const sdq_config_t& c = w->cfg, &c0 = P[0]->cfg;
-    if (!group_format(*w) || c.out_n != c0.out_n || c.out_fmt != c0.out_fmt || c.scale_rule != c0.scale_rule) return SDQ_ERR_UNSUPPORTED;
+    if (!group_format(c, w->K) || c.out_n != c0.out_n || c.out_fmt != c0.out_fmt || c.scale_rule != c0.scale_rule) return SDQ_ERR_UNSUPPORTED;
     items += w->N / TILE_ROWS;
   }
   // (the same range with and without scratch: the in-kernel quantizer keeps a token's K <= 4096 elements in the registers of its 11 x 4 lanes)
@@ -811,6 +816,57 @@ extern "C" sdq_status_t sdq_linear_group(int n, const sdq_act_t* const* Xq, cons
 extern "C" sdq_status_t sdq_linear_group_f32(int n, const sdq_act_t* const* Xq, const sdq_packed_t* const* P, float* const* Y,
                                              const int64_t* ldy, void* stream)
 { return launch_group(n, Xq, P, (void* const*)Y, ldy, stream, true); }
+
+// ---------------------------------------------------------------------------------------------------------
+// What a call would run, for tests (see include/sdq_diag.h): the functions above decide, nothing is launched.
+static bool diag_machine(int& sm_count, const int*& max_clusters) {
+  static const int none[5] = {0, 0, 0, 0, 0};
+  if (sm_count > 0) { if (!max_clusters) max_clusters = none; return true; }
+  DeviceInfo* d = device_info();
+  if (!d) return false;
+  sm_count = d->sm_count; max_clusters = pair_max_clusters(d);
+  return true;
+}
+
+extern "C" sdq_status_t sdq_diag_linear_plan(int64_t M, int64_t N, int64_t K, const sdq_config_t* cfg, int workspace, int sm_count,
+                                             const int* max_clusters, sdq_diag_plan_t* out, sdq_diag_task_t* tasks, int64_t cap)
+{
+  if (!cfg || !out) return SDQ_ERR_INVALID_ARG;
+  if (M <= 0 || N <= 0 || K <= 0 || N % TILE_ROWS || K % K2) return SDQ_ERR_SHAPE;
+  if (!is_tensor_core_reading(*cfg)) return SDQ_ERR_UNSUPPORTED;
+  if (!diag_machine(sm_count, max_clusters)) return SDQ_ERR_CUDA;
+  *out = sdq_diag_plan_t{};
+  const LinearRoute r = linear_route(M, N, K, *cfg, workspace != 0, sm_count, max_clusters);
+  out->kernel = r.kernel;
+  if (r.kernel == SDQ_DIAG_FEW) { out->ksplit = r.ksplit; out->cluster = r.cluster_ks; out->token_tile = n_tile_for(M); }
+  if (r.kernel == SDQ_DIAG_PAIRS) {
+    LinearParams p = {};
+    p.M = M; p.N = N; p.K = K; p.out_n = cfg->out_n; p.b32 = cfg->in_block == 32; p.dense = is_dense_layout(*cfg);
+    pair_describe(p, sm_count, max_clusters, out, tasks, cap);
+  }
+  if (r.kernel == SDQ_DIAG_GROUP) return sdq_diag_group_plan(1, M, &N, &K, sm_count, max_clusters, out, tasks, cap);
+  return SDQ_OK;
+}
+
+extern "C" sdq_status_t sdq_diag_group_plan(int n, int64_t M, const int64_t* N, const int64_t* K, int sm_count, const int* max_clusters,
+                                            sdq_diag_plan_t* out, sdq_diag_task_t* segs, int64_t cap)
+{
+  if (n <= 0 || n > GROUP_MAX || !N || !K || !out) return SDQ_ERR_INVALID_ARG;
+  if (!diag_machine(sm_count, max_clusters)) return SDQ_ERR_CUDA;
+  GroupParams g = {};
+  g.n = n;
+  for (int i = 0; i < n; ++i) {
+    if (N[i] <= 0 || N[i] % TILE_ROWS || K[i] < 4 * K2 || K[i] % K2) return SDQ_ERR_SHAPE;
+    g.m[i].T2 = (int)(K[i] / K2);
+    g.m[i].item0 = g.total_items;
+    g.total_items += (int)(N[i] / TILE_ROWS);
+  }
+  *out = sdq_diag_plan_t{};
+  out->kernel = SDQ_DIAG_GROUP;
+  out->token_tile = M <= 16 ? 16 : 32;
+  group_describe(g, sm_count, max_clusters, out, segs, cap);
+  return SDQ_OK;
+}
 
 // ---------------------------------------------------------------------------------------------------------
 // Allocation-free variant of sdq_linear_ws (see include/sdq.h).  The split-K scratch lives in this library's

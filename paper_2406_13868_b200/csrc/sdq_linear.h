@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "../../include/sdq_diag.h"
 #include "sdq_internal.h"
 #include "sdq_layout.h"
 
@@ -73,14 +74,17 @@ struct GroupParams {
   GroupMat m[GROUP_MAX];
 };
 cudaError_t launch_linear_group(GroupParams p, bool f32_out, DeviceInfo* d, cudaStream_t stream);
-double group_kernel_us(int64_t items, int T2, DeviceInfo* d);   // estimated time of a call of `items` row tiles of 256 T2 K, in us
+double group_kernel_us(int64_t items, int T2, int sm_count, const int* max_clusters);   // estimated time of a call of `items` row tiles of 256 T2 K, in us
 bool group_xres_fits(int T2, int out_n);   // the activation-resident variant's shared-memory budget for K = 256 T2
 
 // CTA-pair (tcgen05 cta_group::2) many-token kernel (sdq_linear_pair.cu).
 // estimated time of a call in us, to choose between the kernels
-double pair_kernel_us(int64_t M, int64_t N, int64_t K, int out_n, bool b32, bool dense, DeviceInfo* d);
+double pair_kernel_us(int64_t M, int64_t N, int64_t K, int out_n, bool b32, bool dense, int sm_count, const int* max_clusters);
 // clusters of k pairs of CTAs, one CTA per SM, that run at once on the current device: entries 2..4
 const int* pair_max_clusters(DeviceInfo* d);
+// what sdq_diag_linear_plan and sdq_diag_group_plan report (the parameters as for a launch, pointers unset)
+void pair_describe(LinearParams p, int sm_count, const int* max_clusters, sdq_diag_plan_t* out, sdq_diag_task_t* tasks, int64_t cap);
+void group_describe(GroupParams p, int sm_count, const int* max_clusters, sdq_diag_plan_t* out, sdq_diag_task_t* segs, int64_t cap);
 cudaError_t launch_linear_pair(LinearParams p, bool f32_out, DeviceInfo* d, cudaStream_t stream);
 
 }  // namespace sdq

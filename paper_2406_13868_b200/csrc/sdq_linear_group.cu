@@ -88,11 +88,10 @@ constexpr int GRP_SIDE_BYTES = 2 * 2 * SF_ATOM_BYTES;
 struct GroupSeg { int item, mat, kb, ke; };                // item, its matrix, its 256-K units [kb, ke)
 // segment i, i rising by one from 0 with s.mat = 0 before the first (items only grow, so the matrix is looked for from the last one on)
 template <bool SPLIT>
-__device__ __forceinline__ bool group_seg(const GroupParams& p, int i, GroupSeg& s) {
-  const int b = (int)blockIdx.x;
+__host__ __device__ __forceinline__ bool group_seg_of(const GroupParams& p, int b, int ctas, int i, GroupSeg& s) {   // CTA b of `ctas`
   const bool whole = !SPLIT || i < p.rounds;
   const int w_log2 = SPLIT ? p.cluster_log2 - p.tail_log2 : 0, r = SPLIT ? b & ((1 << p.cluster_log2) - 1) : 0;
-  s.item = whole ? b + i * (int)gridDim.x : p.rounds * (int)gridDim.x + ((b >> p.cluster_log2) << p.tail_log2) + (r >> w_log2);
+  s.item = whole ? b + i * ctas : p.rounds * ctas + ((b >> p.cluster_log2) << p.tail_log2) + (r >> w_log2);
   if ((SPLIT && i > p.rounds) || s.item >= p.total_items) return false;
   while (s.mat + 1 < p.n && s.item >= p.m[s.mat + 1].item0) ++s.mat;
   const int T2 = p.m[s.mat].T2, part = r & ((1 << w_log2) - 1);
@@ -100,6 +99,8 @@ __device__ __forceinline__ bool group_seg(const GroupParams& p, int i, GroupSeg&
   s.ke = whole ? T2 : ((part + 1) * T2) >> w_log2;
   return true;
 }
+template <bool SPLIT>
+__device__ __forceinline__ bool group_seg(const GroupParams& p, int i, GroupSeg& s) { return group_seg_of<SPLIT>(p, (int)blockIdx.x, (int)gridDim.x, i, s); }
 
 template <bool F32_OUT, bool XRES, bool SPLIT>
 __global__ void __launch_bounds__(group_threads(XRES), 1)
@@ -675,9 +676,10 @@ static GroupPlan group_plan(int64_t items, int T2, int T2_min, int sm_count, con
   }
   return best;
 }
-double group_kernel_us(int64_t items, int T2, DeviceInfo* d) { return group_plan(items, T2, T2, d->sm_count, pair_max_clusters(d)).us; }
+double group_kernel_us(int64_t items, int T2, int sm_count, const int* max_clusters) { return group_plan(items, T2, T2, sm_count, max_clusters).us; }
 
-cudaError_t launch_linear_group(GroupParams p, bool f32_out, DeviceInfo* d, cudaStream_t stream)
+// how p's items are dealt out, into p
+static GroupPlan group_deal(GroupParams& p, int sm_count, const int* max_clusters)
 {
   int T2_min = p.m[0].T2;
   int64_t units = 0;
@@ -685,9 +687,30 @@ cudaError_t launch_linear_group(GroupParams p, bool f32_out, DeviceInfo* d, cuda
     T2_min = p.m[i].T2 < T2_min ? p.m[i].T2 : T2_min;
     units += (int64_t)((i + 1 < p.n ? p.m[i + 1].item0 : p.total_items) - p.m[i].item0) * p.m[i].T2;
   }
-  const GroupPlan plan = group_plan(p.total_items, (int)((units + p.total_items - 1) / p.total_items), T2_min, d->sm_count, pair_max_clusters(d));
+  const GroupPlan plan = group_plan(p.total_items, (int)((units + p.total_items - 1) / p.total_items), T2_min, sm_count, max_clusters);
   auto log2 = [](int v) { return v == 4 ? 2 : v - 1; };
   p.cluster_log2 = log2(plan.cluster); p.tail_log2 = log2(plan.tail_items); p.rounds = plan.rounds;
+  return plan;
+}
+
+void group_describe(GroupParams p, int sm_count, const int* max_clusters, sdq_diag_plan_t* out, sdq_diag_task_t* segs, int64_t cap)
+{
+  const GroupPlan plan = group_deal(p, sm_count, max_clusters);
+  out->cluster = plan.cluster; out->ctas = plan.ctas; out->rounds = plan.rounds; out->tail_items = plan.tail_items;
+  out->ksplit = plan.cluster / plan.tail_items;
+  int64_t n = 0;
+  for (int b = 0; b < plan.ctas; ++b) {
+    GroupSeg s;
+    s.mat = 0;
+    for (int i = 0; plan.cluster > 1 ? group_seg_of<true>(p, b, plan.ctas, i, s) : group_seg_of<false>(p, b, plan.ctas, i, s); ++i, ++n)
+      if (segs && n < cap) segs[n] = {s.mat, s.item - p.m[s.mat].item0, 1, s.kb, s.ke};
+  }
+  out->tasks = (int32_t)n;
+}
+
+cudaError_t launch_linear_group(GroupParams p, bool f32_out, DeviceInfo* d, cudaStream_t stream)
+{
+  const GroupPlan plan = group_deal(p, d->sm_count, pair_max_clusters(d));
   const bool xres = p.x_bf16 != nullptr;
   const int xbytes = xres ? group_xres_bytes(p.m[0].T2) : 0;
   const int is = xres ? WI_BYTES : group_is_bytes(p.n_tile), os = p.out_n ? 2 * wc_bytes(1) + (xres ? 0 : 2 * p.n_tile * 128) : 0;

@@ -78,7 +78,7 @@ __host__ __device__ constexpr int pair_slots(uint32_t slot) {      // released t
 
 struct PairTask { int u0, nu, mt; };
 template <int FORM>
-__device__ __forceinline__ PairTask pair_task(const LinearParams& p, int task) {
+__host__ __device__ __forceinline__ PairTask pair_task(const LinearParams& p, int task) {
   PairTask t;
   if (FORM != PAIR_TWO) {
     t.mt = task / p.pt_units; t.u0 = task - t.mt * p.pt_units; t.nu = 1;
@@ -100,7 +100,7 @@ __device__ __forceinline__ PairTask pair_task(const LinearParams& p, int task) {
   return t;
 }
 // first 32-token group of token tile `mt`
-__device__ __forceinline__ int pair_group0(const LinearParams& p, int mt) { return (int)((int64_t)mt * p.pt_groups / p.pt_mtiles); }
+__host__ __device__ __forceinline__ int pair_group0(const LinearParams& p, int mt) { return (int)((int64_t)mt * p.pt_groups / p.pt_mtiles); }
 
 template <bool F32_OUT, bool B32, bool DENSE, int FORM>
 __global__ void __maxnreg__(96)
@@ -676,23 +676,39 @@ const int* pair_max_clusters(DeviceInfo* d)
   return d->pair_clusters;
 }
 
-double pair_kernel_us(int64_t M, int64_t N, int64_t K, int out_n, bool b32, bool dense, DeviceInfo* d)
-{ return pair_best(M, N, K, out_n, b32, dense, d->sm_count, pair_max_clusters(d)).us; }
+double pair_kernel_us(int64_t M, int64_t N, int64_t K, int out_n, bool b32, bool dense, int sm_count, const int* max_clusters)
+{ return pair_best(M, N, K, out_n, b32, dense, sm_count, max_clusters).us; }
 
-cudaError_t launch_linear_pair(LinearParams p, bool f32_out, DeviceInfo* d, cudaStream_t stream)
+// the plan's numbers into the launch parameters (p.M, N, K and the format are there); returns the pairs to launch
+static int pair_apply(LinearParams& p, const PairPlan& best, int sm_count)
 {
   const bool s32 = p.dense || p.b32;
-  const uint32_t wib = p.dense ? 17408u : (p.b32 ? 11264u : 10752u);
-  int pairs = d->sm_count / 2;
-  const PairPlan best = pair_best(p.M, p.N, p.K, p.out_n, p.b32 != 0, p.dense != 0, d->sm_count, pair_max_clusters(d));
-  std::atomic<uint32_t>* attr_mask = &d->pair_attr;
   const int T = best.form == PAIR_FLEX ? best.T : pair_tmax(best.form, s32);
   p.n_tile = T;
   p.pt_units = (int)((p.N + 2 * TILE_ROWS - 1) / (2 * TILE_ROWS)); p.pt_mtiles = best.mt; p.pt_groups = (int)((p.M + 31) / 32);
   p.pt_doubles = best.doubles; p.pt_split = best.split; p.pt_tasks = best.tasks; p.pt_acc2 = best.acc2; p.pt_ks = best.ks;
-  p.slot_bytes = (int)pair_slot_bytes(wib, s32, best.form == PAIR_TWO ? 2 : 1, T);
+  p.slot_bytes = (int)pair_slot_bytes(p.dense ? 17408u : (p.b32 ? 11264u : 10752u), s32, best.form == PAIR_TWO ? 2 : 1, T);
   p.nslot = pair_slots((uint32_t)p.slot_bytes);
-  if (p.pt_tasks < pairs || best.ks > 1) pairs = p.pt_tasks;
+  return p.pt_tasks < sm_count / 2 || best.ks > 1 ? p.pt_tasks : sm_count / 2;
+}
+
+void pair_describe(LinearParams p, int sm_count, const int* max_clusters, sdq_diag_plan_t* out, sdq_diag_task_t* tasks, int64_t cap)
+{
+  const PairPlan best = pair_best(p.M, p.N, p.K, p.out_n, p.b32 != 0, p.dense != 0, sm_count, max_clusters);
+  out->ctas = 2 * best.ks * pair_apply(p, best, sm_count);
+  out->form = best.form; out->cluster = 2 * best.ks; out->ksplit = best.ks; out->tasks = best.tasks; out->doubles = best.doubles; out->halves = best.split;
+  out->alternate = best.acc2; out->token_tile = p.n_tile;
+  for (int64_t i = 0; tasks && i < best.tasks && i < cap; ++i) {
+    const PairTask t = best.form == PAIR_TWO ? pair_task<PAIR_TWO>(p, (int)i) : pair_task<PAIR_FLEX>(p, (int)i);
+    tasks[i] = {0, t.u0, t.nu, pair_group0(p, t.mt), pair_group0(p, t.mt + 1)};
+  }
+}
+
+cudaError_t launch_linear_pair(LinearParams p, bool f32_out, DeviceInfo* d, cudaStream_t stream)
+{
+  const PairPlan best = pair_best(p.M, p.N, p.K, p.out_n, p.b32 != 0, p.dense != 0, d->sm_count, pair_max_clusters(d));
+  const int pairs = pair_apply(p, best, d->sm_count);
+  std::atomic<uint32_t>* attr_mask = &d->pair_attr;
   const int v = (f32_out ? 4 : 0) | (p.dense ? 2 : (p.b32 ? 1 : 0));
   switch (v) {
     case 0: return launch_one<false, false, false>(p, best.form, pairs, stream, attr_mask);

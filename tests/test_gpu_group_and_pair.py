@@ -76,13 +76,13 @@ def test_group_call_matches_oracle(shapes, Ms, out_n, share_x):
 
 @pytest.mark.parametrize("shapes,M,cfg_args", [
     ([(9600, 1024)], 3, (1, so.GRAN_PAIR, 64, 0)),                       # one item each for 75 CTAs: nothing to split
-    ([(11008, 1024), (8192, 1536)], 16, (1, so.GRAN_PAIR, 64, 0)),       # 150 items: a round and two left over, K differs
-    ([(4352, 1280)] * 5, 20, (1, so.GRAN_PAIR, 64, 0)),                  # 170 items of five units: uneven parts, 32-token tile
-    ([(11008, 1024), (8192, 1024)], 5, (1, so.GRAN_PAIR, 64, 0, 0, 1)),  # int8: the parts are added as integers
+    ([(11008, 1024), (8192, 1536)], 16, (1, so.GRAN_PAIR, 64, 0)),       # 150 items: a round and two left over, too short to be split; K differs
+    ([(4352, 1280)] * 5, 20, (1, so.GRAN_PAIR, 64, 0)),                  # 170 items of five units, 32-token tile
+    ([(11008, 1024), (8192, 1024)], 5, (1, so.GRAN_PAIR, 64, 0, 0, 1)),  # int8
     ([(11008, 1024), (8448, 1024)], 7, (0, so.GRAN_PAIR, 64, 0)),        # no outlier part
 ])
 def test_group_items_left_over_after_whole_rounds(shapes, M, cfg_args):
-    """left-over items share a cluster's CTAs along K: every layer's last row tiles and a few others against the oracle, the
+    """items left over after whole rounds, of short K: every layer's last row tiles and a few others against the oracle, the
     fused-quantizer call bit for bit"""
     m, cfg, Ws, Xs, ps, xqs = _layers(shapes, [M] * len(shapes), cfg_args, 4300)
     y32, y16 = m.sdq_linear_group(xqs, ps, f32=True), m.sdq_linear_group(xqs, ps)
@@ -102,8 +102,35 @@ def test_group_items_left_over_after_whole_rounds(shapes, M, cfg_args):
 
 @pytest.mark.parametrize("M,N,K,out_n", [(1, 4096, 4096, 1), (17, 4224, 1024, 1), (32, 8448, 2048, 1), (3, 128, 1280, 1), (9, 16640, 1024, 0)])
 def test_single_layers_on_the_grouped_kernel(M, N, K, out_n):
-    """few-token calls that the grouped kernel takes: one, two and four CTAs per row tile, a tile count just above the clusters"""
+    """few-token calls that the grouped kernel takes: whole row tiles and split ones"""
     run_case(M, N, K, 4400 + M, out_n=out_n, check_rows=None if N <= 4224 else (N - 256, N))
+
+
+@pytest.mark.parametrize("shapes,M,cfg_args", [
+    ([(11008, 4096)] * 2, 16, (1, so.GRAN_PAIR, 64, 0)),                 # two CTAs per left-over item
+    ([(4352, 4352)] * 5, 20, (1, so.GRAN_PAIR, 64, 0)),                  # 17 units: uneven parts, 32-token tile
+    ([(11008, 3072), (8192, 3328)], 7, (1, so.GRAN_PAIR, 64, 0)),        # four CTAs per left-over item, K differs, 13 units
+    ([(11008, 3072), (8192, 3328)], 7, (1, so.GRAN_PAIR, 64, 0, 0, 1)),  # int8: the parts are added as integers
+    ([(11008, 3072), (8192, 3328)], 7, (0, so.GRAN_PAIR, 64, 0)),        # no outlier part
+    ([(8192, 8192)], 5, (1, so.GRAN_PAIR, 64, 0)),                       # two CTAs per item, no whole rounds (a single call takes the same form)
+    ([(19072, 4096)], 3, (1, so.GRAN_PAIR, 64, 0)),                      # 149 items: one shared by four CTAs behind a round
+])
+def test_group_items_split_over_clusters(shapes, M, cfg_args):
+    """left-over items share a cluster's CTAs along K (tests/test_plans.py says which do): the first and last row tiles and some in
+    between against the oracle; the same bits again"""
+    m, cfg, Ws, Xs, ps, xqs = _layers(shapes, [M] * len(shapes), cfg_args, 4350)
+    y32, y16, again = m.sdq_linear_group(xqs, ps, f32=True), m.sdq_linear_group(xqs, ps), m.sdq_linear_group(xqs, ps, f32=True)
+    assert m.device_status() == 0
+    oc = so.Config(*cfg_args)
+    for i, (W, X, a, b, c) in enumerate(zip(Ws, Xs, y32, y16, again)):
+        N = W.shape[0]
+        rows = sorted({0, 1, 127, 128, N // 2 + 5, N - 385, N - 300, N - 257, N - 160, N - 129, N - 128, N - 97, N - 64, N - 33, N - 1})
+        yref = so.linear(so.quantize_act(sdq_synth.bf16_bits(X), oc), so.decompose(sdq_synth.bf16_bits(W[rows]), oc))
+        d, tol = y_close(a[:, rows].cpu().numpy(), yref)
+        assert (d <= tol).all(), (i, d.max(), (d / tol).max())
+        assert torch.equal(b, a.to(torch.bfloat16)) and torch.equal(a, c)
+    if len(shapes) == 1:
+        assert torch.equal(m.sdq_linear(xqs[0], ps[0], f32=True), y32[0])
 
 
 def test_group_call_runs_twice_in_a_row_and_inside_a_graph():
@@ -191,7 +218,7 @@ def test_cta_pair_many_token_kernel(M, N, K, out_n, block, gran, rule, rows):
     (300, 384, 2048, (1, so.GRAN_PAIR, 32, 2)),       # K over four pairs, E4M3 scales, an odd number of row tiles
     (200, 384, 1536, (1, so.GRAN_DENSE, 32, 0)),      # K over four pairs, dense inliers
     (100, 4096, 2048, (1, so.GRAN_PAIR, 64, 0)),      # up to 128 tokens on pairs
-    (64, 2176, 4096, (2, so.GRAN_PAIR, 64, 0)),
+    (64, 2176, 4096, (2, so.GRAN_PAIR, 64, 0)),       # too narrow for that: the few-token kernel
     (130, 128, 256, (0, so.GRAN_PAIR, 64, 0)),        # a single stage, half a unit
 ])
 def test_cta_pair_task_forms(M, N, K, cfg_args):
