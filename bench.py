@@ -737,7 +737,7 @@ def measure_model(sdq, dev, peaks, token_counts=(1, 16, 128, 1024, 8192)):
         e = entry(time_graph(lambda: model(False), reps=3 if M >= 1024 else 10))
         if M <= 16:
             e["grouped_qkv_and_gate_up"] = entry(time_graph(lambda: model(True), reps=10))
-            e["grouped_with_fused_quantizer"] = entry(time_graph(lambda: model(True, True), reps=10))
+            e["grouped_from_bf16_activations"] = entry(time_graph(lambda: model(True, True), reps=10))
         c5["M%d" % M] = e
         assert sdq.device_status() == 0
     return c5, layers

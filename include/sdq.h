@@ -229,7 +229,8 @@ sdq_status_t sdq_quantize_act(const void* X_bf16, int64_t M, int64_t K, int64_t 
 sdq_status_t sdq_act_export(const sdq_act_t* Xq, const sdq_act_canonical_t* out, void* stream);
 
 /* The decomposed product of Section 5.1, O = O_o + O_i, both sparse products accumulated in fp32 (in one accumulator; few
- * tokens may take the grouped kernel of sdq_linear_group, which adds the two at the end): Y[m][n] = sum_k A_i[m][k] W_i[n][k] + sum_k A_o[m][k] W_o[n][k].
+ * tokens may take the grouped kernel of sdq_linear_group, which adds the two at the end):
+ * Y[m][n] = sum_k A_i[m][k] W_i[n][k] + sum_k A_o[m][k] W_o[n][k].
  *   Xq, P (host descriptors; K and cfg must agree); Y (device) [M][ldy] bf16 (round to nearest even
  *   of the fp32 accumulator); ldy >= N elements, ldy % 8 == 0.  Asynchronous on `stream`.
  *   The kernel is enqueued with programmatic stream serialization: it may begin (set-up, reading the packed

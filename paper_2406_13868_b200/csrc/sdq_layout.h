@@ -27,8 +27,8 @@
 //     the outliers in the form the method states them (one 8-bit code + one 3-bit position per S-Vector of 8 and
 //     outlier, 12 of the 11 algorithmic bits): row r, S-Vector g (0..15 inside the 128-K stage), outlier t: code byte at
 //     r * 16 out_n + g * out_n + t; position (0..7) in nibble (g * out_n + t) & 1 of byte
-//     2048 out_n + r * 8 out_n + (g * out_n + t) / 2.  Few-token calls stream this section instead of WO and rebuild
-//     the 2:4 form in shared memory; the exporter reads it.
+//     2048 out_n + r * 8 out_n + (g * out_n + t) / 2.  The grouped few-token kernel streams this section instead of WO
+//     and rebuilds the 2:4 form in tensor memory; the exporter reads it.
 //   sections row scale exponents [N] i32, inlier row-factor exponents [N] i32 (two-level scaling with E4M3 Q-Vector
 //   scales; zeros otherwise); element-wise 2:4 inliers with one scale per 32 K are stored like dense inliers, plus their
 //   kept indices [N][K/4] u8 for the exporter

@@ -497,7 +497,9 @@ extern "C" sdq_status_t sdq_workspace_size(int64_t M, int64_t N, int64_t K, cons
 }
 
 // The grouped kernel carries the primary format: up to 32 tokens, pair-wise 4:8 inliers, one E8M0 scale per 64 K, at most one
-// outlier per S-Vector, and K >= 1024: an item then spans enough units that the per-item barriers never run two phases apart.
+// outlier per S-Vector, and K >= 1024, the range it is tested and measured in.  (Its per-item barriers ask for no minimum: an item's
+// scale atoms are not overwritten before `acc_full` of it, nor its accumulators before `acc_empty`, so that the last, shared item of a
+// CTA may be a single unit.)
 static bool group_format(const sdq_config_t& c, int64_t K) {
   return c.in_gran == SDQ_GRAN_PAIR && c.in_block == 64 && c.scale_rule != SDQ_SCALE_UE4M3 && c.out_n <= 1 && K >= 4 * K2;
 }

@@ -23,12 +23,12 @@ struct LinearParams {
   int release;           // 1: ring slots are reused (producer waits on `empty`, MMA issuer commits to it)
   int tmem_cols;         // TMEM columns to allocate (128, 256 or 512)
   int meta_col;          // first TMEM column of the metadata / scale buffers
-  int b32;               // 1: one inlier / activation scale per 32 K (kind::mxf4nvf4 .block16), runtime geometry only
+  int b32;               // 1: one inlier / activation scale per 32 K (kind::mxf4nvf4 .block16)
   // two-level scaling (E4M3 Q-Vector scale codes): the accumulator of row n and token m is in units of 2^(tw[n] + tx[m]);
   // the epilogue multiplies that factor back in.  tw == nullptr: not in use.
   const int32_t* tw;     // [N] exponents of the rows' inlier factors (packed weights)
   const int32_t* tx;     // [tokens] exponents of the tokens' 8-bit scales (quantized activations)
-  int dense;             // 1: dense inliers (no Stage 1): 4 dense kind::mxf4 MMAs of 64 K per stage, runtime geometry only
+  int dense;             // 1: dense inliers (no Stage 1): 4 dense kind::mxf4 MMAs of 64 K per stage
   // CTA-pair kernel: a task is one token tile and one or two row units (a unit = 256 weight rows = 128 per CTA).  Token tile i
   // of pt_mtiles covers the 32-token groups [i G / pt_mtiles, (i + 1) G / pt_mtiles) of the G there are; n_tile is the widest.
   int pt_units, pt_mtiles, pt_groups;

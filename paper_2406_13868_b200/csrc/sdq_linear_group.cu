@@ -4,7 +4,7 @@
 // With a handful of tokens a layer is a stream of its packed weights through the tensor core, and one launch per
 // layer costs more than the stream itself (set-up, the dependency on the previous grid, the split-K reduction).  Here
 // the work items (layer, 128-row tile) of all layers of the call are dealt out round-robin over one CTA per SM; a CTA
-// runs its items back to back through one shared-memory ring, so the weights of the next item are already landing
+// runs its items back to back through its shared-memory rings, so the weights of the next item are already landing
 // while the current one is multiplied and stored.  Items left over after the whole rounds -- or all, when there are fewer than
 // SMs -- have their K range split over the CTAs of a cluster, which add their parts through distributed shared memory.
 //

@@ -1,8 +1,8 @@
 // Native half of the Python binding: the calls a program makes for every batch of activations (quantize, linear, grouped
-// linear) or for every weight matrix (decompose, compact, channel norm), marshalled without ctypes.  Each function takes the arguments of its namesake in __init__.py, does what that
-// does -- allocate what was not supplied, look up the current stream, call the C-ABI, raise SdqError -- and returns None
-// where an argument is not what such a call has in the ordinary case (a CPU tensor, another type, another shape); the Python
-// function then goes its own way, which checks and reports.
+// linear) or for every weight matrix (decompose, compact, channel norm), marshalled without ctypes.  Each function takes the
+// arguments of its namesake in __init__.py, does what that does -- allocate what was not supplied, look up the current stream,
+// call the C-ABI, raise SdqError -- and returns None where an argument is not what such a call has in the ordinary case (a CPU
+// tensor, another type, another shape); the Python function then goes its own way, which checks and reports.
 //
 // Why it exists: the kernels of a one-token layer take ~11 us, and the same two calls through ctypes took the host 25 us,
 // most of it argument conversion, torch.empty and the stream look-up from Python.
