@@ -588,7 +588,7 @@ struct PairPlan { int form, T, mt, acc2, doubles, split, tasks, ks; double us; }
 // measurements (4096 x 4096 to 16384 x 4096, 130 to 8192 tokens): a stage of one unit takes 0.158 (the chain of barrier test
 // and issue) or 10.5 ns per KB that an SM stages (12.5 with every SM busy, 11.8 with compile-time geometry), one of two units 0.10 + 0.00188 T (the tensor pipe at the clock it keeps
 // under load) or 13.5 ns per KB; a call 4.2 and 0.02 per pair it uses; a task ends with a drain of its accumulator that the next one waits for unless the accumulator alternates.
-static bool pair_plan(int groups, int mt, int units, int T1, int T2, bool dbl, uint32_t wib, bool s32, int pairs, const int* max_clusters, PairPlan* out)
+static bool pair_plan(int groups, int mt, int units, int T1, int T2, bool dbl, uint32_t wib, bool s32, bool dense, int pairs, const int* max_clusters, PairPlan* out)
 {
   PairPlan q;
   const int T = 32 * ((groups + mt - 1) / mt), cols = s32 ? (int)PairGeom<true, false>::COLS : (int)PairGeom<false, false>::COLS;
@@ -601,7 +601,11 @@ static bool pair_plan(int groups, int mt, int units, int T1, int T2, bool dbl, u
   const double s1i = kb1 * (wib + avgT * 64.0), s1o = kb1 * (WO_BYTES + avgT * 64.0), m2 = 0.10 + 0.00188 * avgT;
   const double c1 = T2 * (s1i > 0.158 ? s1i : 0.158) + T1 * (s1o > 0.158 ? s1o : 0.158) + (q.acc2 ? 0.3 : 1.0);
   const double s2i = 0.0135e-3 * (2 * wib + avgT * 64.0), s2o = 0.0135e-3 * (2 * WO_BYTES + avgT * 64.0);
-  const double c2 = T2 * (s2i > m2 ? s2i : m2) + T1 * (s2o > m2 ? s2o : m2) + 1.0;
+  // dense inliers: a stage has twice the MMAs, 2.0 times as long under load, 1.7 times in a call of one round, which is over before
+  // the clock falls.  (Priced like the sparse ones, calls of several rounds took two-unit tasks where one-unit tasks are faster: 4096 x
+  // 4096 -> 11008 199 us against 182, 4096 x 16384 -> 4096 306 against 277; one round, 1500 x 11008 -> 4096: 77 us against 83)
+  const double m2i = dense ? ((units / 2) * mt > pairs ? 2.0 : 1.7) * m2 : m2;
+  const double c2 = T2 * (s2i > m2i ? s2i : m2i) + T1 * (s2o > m2 ? s2o : m2) + 1.0;
   q.doubles = q.split = 0;
   double us;
   if (!dbl) {
@@ -641,7 +645,7 @@ static PairPlan pair_best(int64_t M, int64_t N, int64_t K, int out_n, bool b32, 
   const int mt0 = (groups + 7) / 8, mt1 = groups <= 32 ? groups : 2 * mt0;
   for (int mt = mt0; mt <= mt1; ++mt)
     for (int d = 0; d < 2; ++d)
-      if (pair_plan(groups, mt, units, out_n ? (int)(K / K1) : 0, (int)(K / K2), d != 0, dense ? 17408u : (b32 ? 11264u : 10752u), b32 || dense, sm_count / 2,
+      if (pair_plan(groups, mt, units, out_n ? (int)(K / K1) : 0, (int)(K / K2), d != 0, dense ? 17408u : (b32 ? 11264u : 10752u), b32 || dense, dense, sm_count / 2,
                     max_clusters, &q) && (best.us < 0 || q.us < best.us))
         best = q;
   return best;

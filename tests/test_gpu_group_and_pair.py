@@ -215,6 +215,7 @@ def test_cta_pair_many_token_kernel(M, N, K, out_n, block, gran, rule, rows):
     (2901, 3200, 2048, (2, so.GRAN_PAIR, 32, 1)),     # the same with one scale per 32 K, two outliers per 8
     (4001, 2304, 2048, (1, so.GRAN_PAIR, 32, 2)),     # E4M3 scales, one-unit tasks of 256 tokens
     (4001, 1664, 2048, (1, so.GRAN_DENSE, 32, 0)),    # one-unit tasks with alternating accumulators, dense inliers
+    (2048, 2560, 1280, (1, so.GRAN_DENSE, 32, 0)),    # two-unit tasks, one round, dense inliers
     (300, 384, 2048, (1, so.GRAN_PAIR, 32, 2)),       # K over four pairs, E4M3 scales, an odd number of row tiles
     (200, 384, 1536, (1, so.GRAN_DENSE, 32, 0)),      # K over four pairs, dense inliers
     (100, 4096, 2048, (1, so.GRAN_PAIR, 64, 0)),      # up to 128 tokens on pairs

@@ -102,6 +102,11 @@ FORMS = [
     (2901, 3200, 2048, B32, dict(kernel=PAIRS, form=TWO)),
     (4001, 2304, 2048, UE, dict(kernel=PAIRS, form=FULL)),
     (4001, 1664, 2048, DENSE, dict(kernel=PAIRS, form=FLEX, alternate=True, split=False)),
+    (4096, 11008, 4096, DENSE, dict(kernel=PAIRS, form=FULL)),          # dense inliers, several rounds: one-unit tasks are faster
+    (4096, 4096, 16384, DENSE, dict(kernel=PAIRS, form=FULL)),
+    (1500, 16384, 4096, m.Config(1, m.gran_keep(7), 32), dict(kernel=PAIRS, form=FULL)),
+    (1500, 4096, 11008, DENSE, dict(kernel=PAIRS, form=TWO)),           # ... one round: two-unit tasks are
+    (2048, 2560, 1280, DENSE, dict(kernel=PAIRS, form=TWO)),
     (300, 384, 2048, UE, dict(kernel=PAIRS, form=FLEX, split=True)),
     (200, 384, 1536, DENSE, dict(kernel=PAIRS, form=FLEX, split=True)),
     (100, 4096, 2048, PAIR, dict(kernel=PAIRS, form=FLEX, split=True)),
