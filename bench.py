@@ -277,8 +277,8 @@ def run_ours(args):
     roofline = {"kernel": "sdq_linear_pair_kernel", "bound": "tensor", "achieved": gemm_tf, "peak": mixed_peak, "unit": "TFLOP/s",
                 "frac": gemm_tf / mixed_peak,
                 # dram__bytes_read.sum + dram__bytes_write.sum of one captured launch of the gate / up shape
-                # (profiles/sdq_linear_pair_kernel_prefill_M2048_N11008_K4096.md); the down shape was not captured
-                "traffic": 84.1e6, "traffic_unit": "bytes per launch (gate/up shape)",
+                # (profiles/kernels_current.md); the down shape was not captured
+                "traffic": 91.1e6, "traffic_unit": "bytes per launch (gate/up shape)",
                 "peak_basis": "%s bf16 burst %.1f TF/s x 8/3 (sparse FP4 at 8x + sparse FP8 at 4x per dense-equivalent flop)" % (peaks["source"], peaks["bf16"]),
                 "avg_launch_ms": gemm_ms / gemm_n, "launches": gemm_n,
                 # what actually bounds the kernel: bytes staged from L2 into shared memory per launch against the rate that
@@ -353,10 +353,11 @@ def run_ours(args):
 def l2_to_sm(sdq, dev, gemm_launch_ms):
     """The ceiling of the L2 -> shared-memory path measured live with the library's copy-only kernel (every SM keeps 128 to
     220 KB of bulk copies in flight from a 37 MB, L2-resident source; best of four copy shapes, each the best of five
-    launches of ~2 GB), and the fraction of it that the GEMM's staged operand bytes reach.  Staged bytes per launch of the
-    CTA-pair kernel: per CTA and 256 x 256 tile, 16 inlier stages of 28160 B (weight record + own 128 tokens' codes + two
-    scale atoms) + 32 outlier stages of 26624 B + 1536 B of outlier scale atoms = 1.304 MB; x 2 CTAs x 344 tiles = 0.897 GB
-    for the gate / up shape (0.897 GB for the down shape too: 128 tiles of 43 + 86 stages)."""
+    launches of ~2 GB), and the fraction of it that the GEMM's staged operand bytes reach, as a mean over the step's three launches.
+    Staged bytes per launch of the CTA-pair kernel, from its tasks (sdq_diag_linear_plan), each CTA: per inlier stage (256 K) 10752 B per row
+    unit, 64 B per token and 1024 B of scale atoms, per outlier stage (128 K) 10240 B per unit and 64 B per token, once per task 512 B
+    per unit and 1024 B of outlier scale atoms.  Gate / up: 210 tasks of two units and 10 of one, 10 token tiles = 0.715 GB (the profiler counts 0.715);
+    down: 144 tasks of one unit, 9 token tiles = 0.941 GB."""
     sms = torch.cuda.get_device_properties(dev).multi_processor_count
     src = torch.empty(sms * (256 << 10), dtype=torch.uint8, device=dev).fill_(1)
     best = 0.0
@@ -369,7 +370,7 @@ def l2_to_sm(sdq, dev, gemm_launch_ms):
             torch.cuda.synchronize()
             if rep >= 2:
                 best = max(best, moved / (a.elapsed_time(b) * 1e-3) / 1e12)
-    staged = 0.897e9
+    staged = (2 * 0.715e9 + 0.941e9) / 3
     ach = staged / (gemm_launch_ms * 1e-3) / 1e12
     return {"bytes_per_launch": staged, "achieved_TBps": ach, "measured_ceiling_TBps": best, "frac": ach / best,
             "ceiling_basis": "copy-only kernel of this library (sdq_diag_l2_copy), all SMs, best of 3 x 64 KB, 6 x 32 KB, 13 x 16 KB and 15 x 14 KB bulk copies in flight per SM, L2-resident source"}
