@@ -12,7 +12,9 @@
 // over two passes to 138), DRAM is at 30 %.  11008 x 4096, 1:8 + pair-wise 4:8: 189 us as one kernel with a CTA per row and a
 // thread per S-Vector scattering bytes -> 20 + 42 us with the row scales in a launch of their own -> 49 us -> 42 us with the
 // pairs picked by two minima and two maxima instead of six comparisons and the choices kept from the first pass.  4096 x 11008,
-// 1:8 + 6:8 with channel weights: 98 us choosing in both passes -> 67.
+// 1:8 + 6:8 with channel weights: 98 us choosing in both passes -> 67.  Loops of four S-Vectors (first pass) and of one Q-Vector
+// (second) instead of 16 and 4 in a row, each warp starting on its own part of the tile, the first arrival relaxed: 43.6 -> 43.0 and
+// 68.2 -> 66.0, without channel weights 53.7 -> 46.6; 16384 x 4096 with E4M3 scales 70.5 -> 64.4.
 #include <cstring>
 #include <type_traits>
 #include <mutex>
@@ -194,6 +196,10 @@ __device__ __forceinline__ uint32_t dropped_set(int (&k)[8], int o0, int o1, int
   return m;
 }
 
+// the next 16 bits of eight bytes, the next word of four: after four of them the first is the lowest
+__device__ __forceinline__ void queue16(uint32_t (&q)[2], uint32_t v) { q[0] = prmt(q[0], q[1], 0x5432u); q[1] = prmt(q[1], v, 0x5432u); }
+__device__ __forceinline__ void queue32(uint32_t (&q)[4], uint32_t v) { q[0] = q[1]; q[1] = q[2]; q[2] = q[3]; q[3] = v; }
+
 struct PackParams {
   const __nv_bfloat16* W;
   int64_t N, K, ldw;
@@ -333,8 +339,9 @@ pack_kernel(const PackParams p, const BlobHeader hdr)
   const int T1 = (int)(p.K / K1), T2 = T1 / 2;
   const int cx = (int)((p.K + PK_K - 1) / PK_K), rank = (int)(blockIdx.x % (uint32_t)cx);   // FUSED: a cluster is the cx CTAs of these rows
   const bool first_rows = blockIdx.x < (uint32_t)cx;
-  // (waited for before the first store into another CTA's shared memory: every CTA of the cluster has started by then)
-  if constexpr (FUSED) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  // (waited for before the first store into another CTA's shared memory: every CTA of the cluster has started by then; there is
+  // nothing to release yet, and a releasing arrival is a memory barrier for every warp)
+  if constexpr (FUSED) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
   const int64_t n_first = (int64_t)(blockIdx.x / (uint32_t)cx) * PK_ROWS;
   {
     // 256 threads x 16 B = the 4096 B of one row per round
@@ -354,7 +361,7 @@ pack_kernel(const PackParams p, const BlobHeader hdr)
   const int64_t n = n_first + row;
   uint8_t* mine = tile + row * PK_PITCH + ch * 256;
   const float* colw = WGT ? p.colw + (int64_t)kc * K1 : nullptr;
-  __syncthreads();
+  __syncwarp();                                          // (a warp has loaded what its own threads read)
 
   // ---- first pass: the choices, the row's largest outlier (and inlier), non-finite check.
   // Pair-wise: everything is chosen here and the S-Vector's 16 bytes in the tile become what is left to encode, the two pairs that
@@ -369,31 +376,39 @@ pack_kernel(const PackParams p, const BlobHeader hdr)
   if constexpr (CHOSEN) {
     const bool look_at_all = WGT || OUTN == 0 || p.order_mask;    // for non-finite values: otherwise they are outliers
     if (on) {
+#pragma unroll 1
+      for (int t = 0; t < 4; ++t) {                      // four S-Vectors a trip
+        uint32_t n_o0 = 0, n_o1 = 0, n_nib = 0, n_gone = 0;
 #pragma unroll
-      for (int i = 0; i < 16; ++i) {
-        uint4* at = reinterpret_cast<uint4*>(mine) + i;
-        const uint4 v = *at;
-        uint32_t r[4] = {v.x, v.y, v.z, v.w};
-        const float* c = WGT ? colw + 8 * i : nullptr;
-        int o0, o1;
-        float f0, f1;
-        if (look_at_all) all2 = max_magnitudes(all2, r);
-        if constexpr (!DENSE) {
-          uint32_t w0, w1, nibble;
-          choose_pairs<WGT, OUTN>(p, r, c, o0, o1, f0, f1, w0, w1, nibble);
-          if (p.ue) imax = max_abs2(max_abs2(imax, w0), w1);
-          *at = make_uint4(w0, w1, __float_as_uint(f0), __float_as_uint(f1));
-          c_nib[i >> 3] |= nibble << (4 * (i & 7));
-        } else {
-          int k[8];
-          rank_keys<WGT>(r, c, k);
-          pick_outliers<WGT, OUTN>(k, p.order_mask, p.sv4 != 0, o0, o1);
-          f0 = OUTN > 0 ? pick_value(r, o0) : 0.0f;
-          f1 = OUTN > 1 ? pick_value(r, o1) : 0.0f;
-          c_gone[i >> 2] |= dropped_set<WGT, OUTN>(k, o0, o1, p.keep_in, p.sv4 || p.elem, p.order_mask) << (8 * (i & 3));
+        for (int i = 0; i < 4; ++i) {
+          uint4* at = reinterpret_cast<uint4*>(mine) + 4 * t + i;
+          const uint4 v = *at;
+          uint32_t r[4] = {v.x, v.y, v.z, v.w};
+          const float* c = WGT ? colw + 8 * (4 * t + i) : nullptr;
+          int o0, o1;
+          float f0, f1;
+          if (look_at_all) all2 = max_magnitudes(all2, r);
+          if constexpr (!DENSE) {
+            uint32_t w0, w1, nibble;
+            choose_pairs<WGT, OUTN>(p, r, c, o0, o1, f0, f1, w0, w1, nibble);
+            if (p.ue) imax = max_abs2(max_abs2(imax, w0), w1);
+            *at = make_uint4(w0, w1, __float_as_uint(f0), __float_as_uint(f1));
+            n_nib |= nibble << (4 * i);
+          } else {
+            int k[8];
+            rank_keys<WGT>(r, c, k);
+            pick_outliers<WGT, OUTN>(k, p.order_mask, p.sv4 != 0, o0, o1);
+            f0 = OUTN > 0 ? pick_value(r, o0) : 0.0f;
+            f1 = OUTN > 1 ? pick_value(r, o1) : 0.0f;
+            n_gone |= dropped_set<WGT, OUTN>(k, o0, o1, p.keep_in, p.sv4 || p.elem, p.order_mask) << (8 * i);
+          }
+          if constexpr (OUTN > 0) { omax = max(omax, magnitude(f0)); n_o0 |= (uint32_t)o0 << (4 * i); }
+          if constexpr (OUTN > 1) { omax = max(omax, magnitude(f1)); n_o1 |= (uint32_t)o1 << (4 * i); }
         }
-        if constexpr (OUTN > 0) { omax = max(omax, magnitude(f0)); c_o0[i >> 3] |= (uint32_t)o0 << (4 * (i & 7)); }
-        if constexpr (OUTN > 1) { omax = max(omax, magnitude(f1)); c_o1[i >> 3] |= (uint32_t)o1 << (4 * (i & 7)); }
+        queue16(c_nib, n_nib);
+        queue16(c_o0, n_o0);
+        queue16(c_o1, n_o1);
+        queue32(c_gone, n_gone);
       }
     }
   }
@@ -458,11 +473,17 @@ pack_kernel(const PackParams p, const BlobHeader hdr)
 
   uint32_t in_word[2][2];                                // pair-wise inliers: the 64-K half's codes, two S-Vectors per word
   uint32_t sc = 0;                                       // scale bytes of the 128 K
-  uint32_t codes[4], sels[4], metas[4];                  // outlier bytes of the 128 K
+  uint32_t codes[4] = {0, 0, 0, 0}, sels[4] = {0, 0, 0, 0}, metas[4] = {0, 0, 0, 0};   // outlier bytes of the 128 K
   uint32_t kept[16];                                     // pair-wise inliers of a Q-Vector of 64 K, outlier positions zeroed
   uint32_t qmax2 = 0;                                    // packed running maximum of the Q-Vector
+  // (rolled up, like the first pass: as straight-line code the two took a fifth of the warps' time in waits for instructions)
+  constexpr int TRIP = DENSE ? 1 : 2;                    // blocks a trip (pair-wise: a Q-Vector of 64 K)
+#pragma unroll 1
+  for (int b0 = 0; b0 < 4; b0 += TRIP) {
+   [[maybe_unused]] const uint32_t w_o0 = b0 < 2 ? c_o0[0] : c_o0[1], w_o1 = b0 < 2 ? c_o1[0] : c_o1[1];
 #pragma unroll
-  for (int b = 0; b < 4; ++b) {                          // blocks of 4 S-Vectors (32 K)
+   for (int bi = 0; bi < TRIP; ++bi) {                   // blocks of 4 S-Vectors (32 K)
+    const int b = b0 + bi, odd = DENSE ? b & 1 : bi;
     uint32_t ocode[4], ocode1[4], opos[4], opos1[4];
     uint32_t dense_codes[4], dval[16];
     [[maybe_unused]] uint32_t emeta[2] = {0, 0};
@@ -470,12 +491,11 @@ pack_kernel(const PackParams p, const BlobHeader hdr)
     for (int i = 0; i < 4; ++i) {
       const uint4 v = *reinterpret_cast<const uint4*>(mine + (4 * b + i) * 16);
       uint32_t x[4] = {v.x, v.y, v.z, v.w};
-      const int sv = 4 * b + i;
       [[maybe_unused]] int k[8];
       int o0, o1;
       if constexpr (CHOSEN) {
-        o0 = (int)((c_o0[sv >> 3] >> (4 * (sv & 7))) & 7u);
-        o1 = (int)((c_o1[sv >> 3] >> (4 * (sv & 7))) & 7u);
+        o0 = (int)((w_o0 >> (16 * odd + 4 * i)) & 7u);
+        o1 = (int)((w_o1 >> (16 * odd + 4 * i)) & 7u);
       } else {
         rank_keys<false>(x, nullptr, k);
         pick_outliers<false, OUTN>(k, p.order_mask, p.sv4 != 0, o0, o1);
@@ -492,12 +512,12 @@ pack_kernel(const PackParams p, const BlobHeader hdr)
         opos1[i] = (uint32_t)o1;
       }
       if constexpr (!DENSE) {
-        kept[2 * (4 * (b & 1) + i)] = x[0];
-        kept[2 * (4 * (b & 1) + i) + 1] = x[1];
+        kept[2 * (4 * odd + i)] = x[0];
+        kept[2 * (4 * odd + i) + 1] = x[1];
         qmax2 = max_abs2(max_abs2(qmax2, x[0]), x[1]);
       } else {
         uint32_t gone;
-        if constexpr (CHOSEN) gone = (c_gone[b] >> (8 * i)) & 255u;
+        if constexpr (CHOSEN) gone = (c_gone[0] >> (8 * i)) & 255u;
         else gone = dropped_set<false, OUTN>(k, o0, o1, p.keep_in, p.sv4 || p.elem, p.order_mask);
         zero_set(x, gone);
         qmax2 = max_magnitudes(qmax2, x);
@@ -529,17 +549,17 @@ pack_kernel(const PackParams p, const BlobHeader hdr)
       }
       if (p.elem) *reinterpret_cast<uint2*>(p.blob + p.off.emeta + (size_t)n * (size_t)(p.K / 4) + (kc * 16 + 4 * b) * 2) = make_uint2(emeta[0], emeta[1]);
       // 16 code bytes per 32 K: K-block (64 K) 2 h + b / 2 of the record, chunk b & 1
-      *reinterpret_cast<uint4*>(wi + (2 * h + (b >> 1)) * 4096 + core + (b & 1) * 128) = make_uint4(dense_codes[0], dense_codes[1], dense_codes[2], dense_codes[3]);
+      *reinterpret_cast<uint4*>(wi + (2 * h + (b >> 1)) * 4096 + core + odd * 128) = make_uint4(dense_codes[0], dense_codes[1], dense_codes[2], dense_codes[3]);
       sc |= c << (8 * b);
       qmax2 = 0;
-    } else if ((b & 1) || b32) {
+    } else if (odd || b32) {
       // a Q-Vector is complete: 64 K (both blocks of the half) or 32 K (this one)
       const uint32_t key = larger_half(qmax2);
       const uint32_t c = p.ue ? ue4m3_scale_code(bf16_bits_to_float(key) * pow2_neg(tw), key != 0) : e8m0_scale_code_bf16(key, p.ceil_rule != 0);
       const float inv = p.ue ? ue4m3_scale_inverse(max(c, 1u)) : pow2_inv_e8m0(c);
 #pragma unroll
       for (int hb = 0; hb < 2; ++hb) {                   // 32-K block of the half
-        if (hb != (b & 1) && b32) continue;              // (one scale per 64 K: both now)
+        if (hb != odd && b32) continue;              // (one scale per 64 K: both now)
 #pragma unroll
         for (int i = 0; i < 2; ++i) {                    // two S-Vectors per code word
           float f[8];
@@ -564,7 +584,7 @@ pack_kernel(const PackParams p, const BlobHeader hdr)
       qmax2 = 0;
     }
     if constexpr (!DENSE) {
-      if (b & 1) {
+      if (odd) {
         // 16 code bytes per 64 K (K-block h, chunk b / 2)
         *reinterpret_cast<uint4*>(wi + h * 4096 + core + (b >> 1) * 128) = make_uint4(in_word[0][0], in_word[0][1], in_word[1][0], in_word[1][1]);
       }
@@ -576,12 +596,12 @@ pack_kernel(const PackParams p, const BlobHeader hdr)
       // per S-Vector: position ps (0..7) sits in group of 4 number ps >> 2 at p = ps & 3, whose slots are (p, 3), the value
       // first, or (0, 3), the value second, when p = 3; the other group has slots (0, 1).  Metadata bytes and byte shifts
       // come from 8-entry tables looked up by byte-permutes, the four position nibbles being the selector.
-      codes[b] = ocode[0] | (ocode[1] << 8) | (ocode[2] << 16) | (ocode[3] << 24);
-      const uint32_t sel = CHOSEN ? (c_o0[b >> 1] >> (16 * (b & 1))) & 0xFFFFu : opos[0] | (opos[1] << 4) | (opos[2] << 8) | (opos[3] << 12);
+      queue32(codes, ocode[0] | (ocode[1] << 8) | (ocode[2] << 16) | (ocode[3] << 24));
+      const uint32_t sel = CHOSEN ? (w_o0 >> (16 * odd)) & 0xFFFFu : opos[0] | (opos[1] << 4) | (opos[2] << 8) | (opos[3] << 12);
       const uint32_t sh = __byte_perm(0x08000000u, 0x18101010u, sel);
-      metas[b] = __byte_perm(0x4C4E4D4Cu, 0xC4E4D4C4u, sel);
-      sels[b] = sel;
-      *reinterpret_cast<uint4*>(wo + (b >> 1) * 4096 + core + (b & 1) * 128) =
+      queue32(metas, __byte_perm(0x4C4E4D4Cu, 0xC4E4D4C4u, sel));
+      queue32(sels, sel);
+      *reinterpret_cast<uint4*>(wo + (b >> 1) * 4096 + core + odd * 128) =
           make_uint4(ocode[0] << (sh & 31u), ocode[1] << ((sh >> 8) & 31u), ocode[2] << ((sh >> 16) & 31u), ocode[3] << (sh >> 24));
     } else if constexpr (OUTN == 2) {
       uint32_t st[4], meta = 0;
@@ -603,13 +623,15 @@ pack_kernel(const PackParams p, const BlobHeader hdr)
           meta |= m << (8 * i + 4 * q);
         }
       }
-      *reinterpret_cast<uint4*>(wo + (b >> 1) * 4096 + core + (b & 1) * 128) = make_uint4(st[0], st[1], st[2], st[3]);
-      metas[b] = meta;
+      *reinterpret_cast<uint4*>(wo + (b >> 1) * 4096 + core + odd * 128) = make_uint4(st[0], st[1], st[2], st[3]);
+      queue32(metas, meta);
       *reinterpret_cast<uint2*>(wc + r * 32 + 8 * b) =
           make_uint2(ocode[0] | (ocode1[0] << 8) | (ocode[1] << 16) | (ocode1[1] << 24), ocode[2] | (ocode1[2] << 8) | (ocode[3] << 16) | (ocode1[3] << 24));
       *reinterpret_cast<uint32_t*>(wc + 2 * WC_CODE_BYTES + r * 16 + 4 * b) =
           opos[0] | (opos1[0] << 4) | (opos[1] << 8) | (opos1[1] << 12) | (opos[2] << 16) | (opos1[2] << 20) | (opos[3] << 24) | (opos1[3] << 28);
     }
+   }
+   if constexpr (DENSE && CHOSEN) queue32(c_gone, 0u);
   }
   if constexpr (!DENSE) *reinterpret_cast<uint2*>(wi + A_IN_BYTES + r * 16 + h * 8) = make_uint2(c_nib[0], c_nib[1]);
   if constexpr (OUTN > 0) *reinterpret_cast<uint4*>(wo + A_OUT_BYTES + r * 16) = make_uint4(metas[0], metas[1], metas[2], metas[3]);
