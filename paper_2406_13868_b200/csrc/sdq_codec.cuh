@@ -100,6 +100,16 @@ __device__ __forceinline__ float ue4m3_scale_inverse(uint32_t c) {
   return __fdividef(1.0f, __half2float(__half(h)));
 }
 
+// two packed bf16 times a power of two (the bits of a bf16), as floats, in one instruction each (unpacking and multiplying take
+// three a pair more: 2048 x 11008 18.5 -> 18.0 us).  Rounded once, as the fp32 product is; the sum's -0 keeps the sign of zeros
+__device__ __forceinline__ void scaled2(uint32_t x, uint32_t s, float& lo, float& hi) {
+  asm("{\n.reg .b16 l, h, t;\n"
+      "mov.b32 {l, h}, %2;\n"
+      "cvt.u16.u32 t, %3;\n"
+      "fma.rn.f32.bf16 %0, l, t, %4;\n"
+      "fma.rn.f32.bf16 %1, h, t, %4;\n}"
+      : "=f"(lo), "=f"(hi) : "r"(x), "r"(s), "f"(-0.0f));
+}
 // two floats -> two E2M1 codes in one byte (x in the low nibble)
 __device__ __forceinline__ uint32_t e2m1x2(float x, float y) {
   return (uint32_t)__nv_cvt_float2_to_fp4x2(make_float2(x, y), __NV_E2M1, cudaRoundNearest);

@@ -11,11 +11,11 @@
 // then a 4-lane shuffle, a token's four scales are one word, and every store instruction of codes writes whole 128-byte
 // lines (8 tokens x 16 B per core matrix).  Codes come from the hardware E2M1 / E4M3 converters.
 //
-// Bound by DRAM traffic and the conversion instructions: 2048 x 11008 at 3.9 TB/s of algorithmic bytes (20.2 us; a warp
-// per scattered 64-K Q-Vector with byte stores of scales: 24.7), 8192 x 4096 at 5.0 TB/s (23.5 us; 31.6), one token 2.3 us
-// (4.6), most of it the launch.  E4M3 scales and int8 codes multiply by a reciprocal instead of dividing
-// every element (see sdq_codec.cuh): 4096 x 16384 with E4M3 scales 91 -> 60.0 us, int8 2048 x 4096 15.0 -> 12.3, one int8
-// token 14.1 -> 3.0 (zeros took the division's slow path).
+// Bound by DRAM traffic and the conversion instructions: 2048 x 11008 at 4.4 TB/s of algorithmic bytes (18.0 us), 8192 x 11008 at
+// 5.4 TB/s (58.3), 8192 x 4096 at 5.5 (21.5), one token 2.1 us, most of it the launch.  Against releasing cluster arrivals, no
+// fetching ahead and an unpacking in front of every multiplication: 20.1, 66.0, 23.5 us; 4096 x 16384 with E4M3 scales, where 64
+// registers also let a fourth CTA onto the SM, 60.1 -> 45.7.  E4M3 scales and int8 codes multiply by a reciprocal instead of
+// dividing every element (see sdq_codec.cuh): one int8 token 14.1 -> 3.0 us (zeros took the division's slow path).
 #include "sdq_codec.cuh"
 #include "sdq_internal.h"
 #include "sdq_layout.h"
@@ -88,6 +88,7 @@ __device__ __forceinline__ void qa_encode(const QaUnit<NQ>& u, int first, float 
                                           uint8_t* __restrict__ buf, const ActOffsets& off) {
   const int e = fp8_scale_exp(ramax);
   const float s8 = pow2_neg(e);
+  const uint32_t s8x = (uint32_t)(127 - e) << 7;         // as bf16
   const bool i8 = cfg.out_fmt == SDQ_OUT_INT8;           // A_o in int8: fp32 token scale amax / 127
   const Int8Coder k8 = int8_coder(int8_scale(ramax));
   const bool b32 = cfg.in_block == 32;                   // one scale per 32 K: a Q-Vector is a lane pair
@@ -98,24 +99,21 @@ __device__ __forceinline__ void qa_encode(const QaUnit<NQ>& u, int first, float 
   for (int i = 0; i < NQ; ++i) {
     const int iq = first + i;
     const uint32_t r[8] = {u.raw[i][0].x, u.raw[i][0].y, u.raw[i][0].z, u.raw[i][0].w, u.raw[i][1].x, u.raw[i][1].y, u.raw[i][1].z, u.raw[i][1].w};
-    float v[16];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      v[2 * j] = __uint_as_float(r[j] << 16);
-      v[2 * j + 1] = __uint_as_float(r[j] & 0xFFFF0000u);
-    }
     uint32_t bm = u.qmax[i];
     bm = max(bm, __shfl_xor_sync(0xffffffffu, bm, 1));
     if (!b32) bm = max(bm, __shfl_xor_sync(0xffffffffu, bm, 2));
     uint32_t q4[2] = {0, 0}, q8[4] = {0, 0, 0, 0};
+    float v8[16];                                        // in units of the token's 8-bit scale
+#pragma unroll
+    for (int j = 0; j < 8; ++j) scaled2(r[j], s8x, v8[2 * j], v8[2 * j + 1]);
     if constexpr (!UE) {
       c[i] = e8m0_scale_code_bf16(bm, cfg.scale_rule == SDQ_SCALE_CEIL_NOSAT);
-      const float s4 = pow2_inv_e8m0(c[i]);
+      const uint32_t s4x = (254u - c[i]) << 7;
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         float f[8];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) f[j] = v[8 * h + j] * s4;
+        for (int j = 0; j < 4; ++j) scaled2(r[4 * h + j], s4x, f[2 * j], f[2 * j + 1]);
         q4[h] = e2m1x8(f);
       }
     } else {
@@ -127,17 +125,18 @@ __device__ __forceinline__ void qa_encode(const QaUnit<NQ>& u, int first, float 
         for (int h = 0; h < 2; ++h) {
           float f[8];
 #pragma unroll
-          for (int j = 0; j < 8; ++j) f[j] = small_quotient(v[8 * h + j] * s8, inv);
+          for (int j = 0; j < 8; ++j) f[j] = small_quotient(v8[8 * h + j], inv);
           q4[h] = e2m1x8(f);
         }
       }
     }
     if (!i8) {
 #pragma unroll
-      for (int j = 0; j < 4; ++j) q8[j] = e4m3x4(v[4 * j] * s8, v[4 * j + 1] * s8, v[4 * j + 2] * s8, v[4 * j + 3] * s8);
+      for (int j = 0; j < 4; ++j) q8[j] = e4m3x4(v8[4 * j], v8[4 * j + 1], v8[4 * j + 2], v8[4 * j + 3]);
     } else {
 #pragma unroll
-      for (int j = 0; j < 8; ++j) q8[j >> 1] |= (int8_code(v[2 * j], k8) | (int8_code(v[2 * j + 1], k8) << 8)) << (16 * (j & 1));
+      for (int j = 0; j < 8; ++j)
+        q8[j >> 1] |= (int8_code(__uint_as_float(r[j] << 16), k8) | (int8_code(__uint_as_float(r[j] & 0xFFFF0000u), k8) << 8)) << (16 * (j & 1));
     }
     if (live) {
       // 4-bit codes: bytes 32 i + 8 l of the token's 128; 8-bit codes: bytes 64 (i & 1) + 16 l of the 128-K record i / 2
@@ -241,9 +240,9 @@ quant_act_kernel(const __nv_bfloat16* __restrict__ X, int64_t M, int64_t K, int6
 // memory, and the codes are produced from the registers.  The two-launch path stays for rows longer than a cluster of
 // eight CTAs holds (K > 16384).
 template <bool UE, int NQ>
-__global__ void __launch_bounds__(NQ == 4 ? QA_THREADS : 512, NQ == 4 ? (UE ? 3 : 4) : 1)
+__global__ void __launch_bounds__(NQ == 4 ? QA_THREADS : 512, NQ == 4 ? 4 : 1)
 quant_act_fused_kernel(const __nv_bfloat16* __restrict__ X, int64_t M, int64_t K, int64_t ldx, sdq_config_t cfg, uint8_t* __restrict__ buf,
-                       ActOffsets off, uint32_t* __restrict__ flags, int early_next)
+                       ActOffsets off, uint32_t* __restrict__ flags, int early_next, int ahead)
 {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int t = lane >> 2, l = lane & 3;                 // token within the group of 8, quarter of the Q-Vector
@@ -257,8 +256,9 @@ quant_act_fused_kernel(const __nv_bfloat16* __restrict__ X, int64_t M, int64_t K
     ptx::fence_barrier_init();
     ptx::mbar_expect_tx(&s_bar, cx * 8u * 4u);
   }
-  // (waited for before the first push: by then, behind the loads, every CTA's barrier has long been set up)
-  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  // (waited for before the first push: by then, behind the loads, every CTA's barrier has long been set up.  The fence has released the
+  // barrier's set-up, nothing else was written: as a releasing arrival every warp stood in a memory barrier here, 9 % of the kernel)
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
   // launched with programmatic stream serialization: X may still be being written by the previous kernel.  The next launch of
   // the stream is let in behind that wait: a linear kernel reads packed weights before its own, and those may be what the
   // kernel in front of this one writes.  Before it only in calls that want the packed weights complete
@@ -272,6 +272,12 @@ quant_act_fused_kernel(const __nv_bfloat16* __restrict__ X, int64_t M, int64_t K
   QaUnit<NQ> u;
   qa_load(u, X + m * ldx + (int64_t)q * 64 + l * 16, live && on);
   float amax = bf16_bits_to_float(qa_maxima(u));
+  // The CTAs of a wave load together and encode together, so while this one encodes, the piece that the CTA taking its place will load
+  // comes from DRAM into L2 (8192 x 11008 61.5 -> 58.3 us, 2048 x 4096, less than a wave, the same; half or one and a half waves ahead no better)
+  if constexpr (NQ == 4) {
+    const int64_t m2 = ((int64_t)blockIdx.y + ahead) * 8 + tid, k = (int64_t)rank * QA_CHUNK;
+    if (ahead && tid < 8 && m2 < M) ptx::bulk_prefetch_l2(X + m2 * ldx + k, 2u * (uint32_t)(K - k < QA_CHUNK ? K - k : QA_CHUNK));
+  }
   amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, 1));
   amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, 2));
   if (l == 0) s_warp[warp][t] = amax;
@@ -381,7 +387,8 @@ sdq_status_t sdq::quantize_act(const void* X, int64_t M, int64_t K, int64_t ldx,
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     lc.attrs = attr;
     lc.numAttrs = 2;
-    auto go = [&](auto kern) { return cudaLaunchKernelEx(&lc, kern, Xb, M, K, ldx, *cfg, bufp, off, flags, (int)early_next); };
+    const int ahead = nq == 4 ? 4 * dinfo->sm_count / (int)cx : 0;   // token groups whose CTAs run at once (four CTAs per SM)
+    auto go = [&](auto kern) { return cudaLaunchKernelEx(&lc, kern, Xb, M, K, ldx, *cfg, bufp, off, flags, (int)early_next, ahead); };
     const cudaError_t le = nq == 4   ? (ue ? go(quant_act_fused_kernel<true, 4>) : go(quant_act_fused_kernel<false, 4>))
                            : nq == 2 ? (ue ? go(quant_act_fused_kernel<true, 2>) : go(quant_act_fused_kernel<false, 2>))
                                      : (ue ? go(quant_act_fused_kernel<true, 1>) : go(quant_act_fused_kernel<false, 1>));
