@@ -136,8 +136,13 @@ sdq_linear_pair_kernel(const __grid_constant__ LinearParams p)
   const int my_tasks = p.pt_tasks > pair ? (p.pt_tasks - pair + n_pairs - 1) / n_pairs : 0;
   const int total = my_tasks * S;                                  // stages of this CTA, numbered through its tasks
 
-  if (tid == 0) ptx::griddep_launch_dependents();
-  if (tid == 0) {
+  // Set-up.  The producers need nothing but this CTA's barriers for the ring's first lap, so they start on those while tensor memory
+  // is being allocated and the other CTAs of the cluster are waited for (by everybody else, before anything remote).  Only warp 1 has
+  // something to release to them (chains of calls, everybody behind one barrier before -> now: 40 x 4096 -> 4096 9.56 -> 9.33 us, 500 x
+  // 4096 -> 4096 14.93 -> 14.65, 1000 17.28 -> 16.7, 300 x 4096 -> 11008 21.65 -> 21.2; 130 x 16384 -> 4096 20.38 -> 20.50).
+  const bool producer = warp == 0 || warp == 2 || warp == 3;
+  if (warp == 1 && lane == 0) {
+    ptx::griddep_launch_dependents();
     *timed_out = 0u;
     for (uint32_t s = 0; s < NSLOT; ++s) {
       ptx::mbar_init(&full[s], rank == 0 ? 3 : 2);
@@ -146,15 +151,27 @@ sdq_linear_pair_kernel(const __grid_constant__ LinearParams p)
     for (int a = 0; a < 2; ++a) { ptx::mbar_init(&acc_full[a], 1); ptx::mbar_init(&acc_empty[a], 32); }
     ptx::fence_barrier_init();
   }
-  if (warp == 1) ptx::tmem_alloc_pair(tmem_slot, 512);
-  ptx::tc_fence_before();
-  __syncthreads();
-  ptx::cluster_sync();                                             // both CTAs' barriers exist before any remote arrival
-  ptx::tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
+  __syncwarp();
+  uint32_t tmem = 0;
+  if (producer) {
+    ptx::named_bar_sync(5, 128);
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+  } else {
+    if (warp == 1) {                                               // (its barriers are set up: the producers go on)
+      ptx::named_bar_arrive(5, 128);
+      ptx::tmem_alloc_pair(tmem_slot, 512);
+    }
+    ptx::tc_fence_before();
+    ptx::named_bar_sync(6, PAIR_THREADS - 96);
+    if (warp == 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    else asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");   // both CTAs' barriers and tensor memory exist before anything remote
+    ptx::tc_fence_after();
+    tmem = *tmem_slot;
+  }
   const uint32_t meta = tmem + (FORM == PAIR_TWO || acc2 ? 2u * TMAX : TMAX);   // metadata and scales follow the accumulator columns
 
-  if (warp == 0 || warp == 2 || warp == 3) {
+  if (producer) {
     if (lane < 2) {
       // ---------------- producers (both CTAs): role 0 = own weight records, 1 = own activation codes, 2 = scale atoms.
       // Ring slots are released in pairs, so lanes 0 and 1 of the warp run the loop in lockstep, lane l filling the slots of
@@ -245,6 +262,8 @@ sdq_linear_pair_kernel(const __grid_constant__ LinearParams p)
       }
       if (!ok) atomicOr(&p.flags[FLAG_TIMEOUT], 1u);
     }
+    __syncwarp();
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
   } else if (warp == 1 && rank == 1) {
     if (lane < 2) {
       // ---------------- odd CTA: forward "my part of the slot has landed" to the leader's barrier (lane l: slots of parity l)

@@ -339,6 +339,10 @@ __device__ __forceinline__ float4 ld_cluster_f32x4(uint32_t raddr) {
 __device__ __forceinline__ void named_bar_sync(uint32_t id, uint32_t threads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
+// this warp's arrival on a named barrier that others wait on
+__device__ __forceinline__ void named_bar_arrive(uint32_t id, uint32_t threads) {
+  asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
 // the same barrier; true on all of its threads if `v` is true on any
 __device__ __forceinline__ bool named_bar_any(uint32_t id, uint32_t nthreads, bool v) {
   uint32_t r;
