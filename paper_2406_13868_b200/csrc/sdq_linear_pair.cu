@@ -50,7 +50,8 @@ namespace sdq {
 constexpr int PAIR_THREADS = 640;            // 20 warps
 constexpr int PAIR_MAX_SLOTS = 12;
 constexpr int PAIR_STG = 4096;               // transpose buffer: 4 groups x 4 tokens x 128 features bf16
-constexpr int PAIR_TAIL = PAIR_STG + (2 * PAIR_MAX_SLOTS + 4) * 8 + 16 + 128;   // + barriers + alignment slack
+constexpr int PAIR_BARS = 14;                // full barriers, and as many for the releases: two geometries of a ring have 14 slots at most
+constexpr int PAIR_TAIL = PAIR_STG + (2 * PAIR_BARS + 4) * 8 + 16 + 128;   // + barriers + alignment slack
 
 // Geometry of a launch.  TWO: tasks of two units (and one), FULL: of one unit with token tiles of up to 256, both with the
 // ring's and tensor memory's geometry known at compile time (the issue loop pays for every runtime parameter: 474 against
@@ -74,6 +75,22 @@ __host__ __device__ constexpr uint32_t pair_slot_bytes(uint32_t wib, bool s32, i
 __host__ __device__ constexpr int pair_slots(uint32_t slot) {      // released two at a time: an even number
   const int n = (int)((232448u - PAIR_TAIL) / slot) / 2 * 2;
   return n < PAIR_MAX_SLOTS ? n : PAIR_MAX_SLOTS;
+}
+
+// Dense inliers: an inlier weight record has 17 KB, an outlier record 10, so slots that hold the former leave a third of the ring
+// unused in the outlier stages, two thirds of the task, while the bytes in flight are what bounds it.  With one task per pair (DUAL) the
+// outlier stages use the ring in another geometry: | outlier record, row-scale atom | x units | codes | two token-scale atoms |, six
+// slots instead of four (two units x 192 tokens), eight instead of six (one unit x 256).  The first stage in such a slot waits for the
+// inlier slots that had its bytes.  1500 x 11008 -> 4096, 1:8 + 6:8: 71.5 -> 61.9 us, 1500 x 4096 -> 4096 29.7 -> 26.3, 300 x 8704 -> 10880 53.7
+// -> 46.3.  With several tasks per pair the ring would have to turn back for each: 8192 x 2560 -> 2560 57 -> 63, long K the same (the clock
+// is lower there and the tensor pipe the bound).  From K = 2048 on, where the turn costs less than it gives: K 2048 19.15 -> 17.98, 1024
+// 14.15 -> 14.02, 1280 15.2 -> 15.6, 768 13.0 -> 13.3 (1500 tokens).
+__host__ __device__ constexpr uint32_t pair_out_slot_bytes(int units, int T) {
+  return (uint32_t)units * (WO_BYTES + SF_ATOM_BYTES) + (uint32_t)T * 64u + 2u * SF_ATOM_BYTES;
+}
+__host__ __device__ constexpr uint32_t pair_ring_bytes(uint32_t slot, int nslot, bool dual, int units, int T) {
+  const uint32_t i = slot * (uint32_t)nslot, o = dual ? pair_out_slot_bytes(units, T) * (uint32_t)pair_slots(pair_out_slot_bytes(units, T)) : 0u;
+  return i > o ? i : o;
 }
 
 struct PairTask { int u0, nu, mt; };
@@ -102,7 +119,7 @@ __host__ __device__ __forceinline__ PairTask pair_task(const LinearParams& p, in
 // first 32-token group of token tile `mt`
 __host__ __device__ __forceinline__ int pair_group0(const LinearParams& p, int mt) { return (int)((int64_t)mt * p.pt_groups / p.pt_mtiles); }
 
-template <bool F32_OUT, bool B32, bool DENSE, int FORM>
+template <bool F32_OUT, bool B32, bool DENSE, int FORM, bool DUAL>
 __global__ void __maxnreg__(96)
 sdq_linear_pair_kernel(const __grid_constant__ LinearParams p)
 {
@@ -117,14 +134,22 @@ sdq_linear_pair_kernel(const __grid_constant__ LinearParams p)
   const uint32_t TMAX = FORM == PAIR_FLEX ? (uint32_t)p.n_tile : FIXED_T, SLOT = FORM == PAIR_FLEX ? (uint32_t)p.slot_bytes : FIXED_SLOT;
   const uint32_t NSLOT = FORM == PAIR_FLEX ? (uint32_t)p.nslot : (uint32_t)pair_slots(FIXED_SLOT), SL_SF = SL_B + TMAX * 64u;
   const bool acc2 = FORM == PAIR_FLEX && p.pt_acc2;
-  uint8_t* stg_base = sm + NSLOT * SLOT;
+  // the ring of the outlier stages: the same one, or (DUAL) the second geometry
+  static_assert(!DUAL || (DENSE && FORM != PAIR_FLEX));
+  constexpr int UNITS = FORM == PAIR_TWO ? 2 : 1;
+  constexpr uint32_t O_UNIT = DUAL ? WO_BYTES + SF_ATOM_BYTES : G::WIB;     // from one unit's record to the next
+  constexpr uint32_t O_FIXED = pair_out_slot_bytes(UNITS, (int)FIXED_T);
+  const uint32_t O_SLOT = DUAL ? O_FIXED : SLOT, O_NSLOT = DUAL ? (uint32_t)pair_slots(O_FIXED) : NSLOT;
+  const uint32_t O_B = DUAL ? UNITS * O_UNIT : SL_B, O_SF = O_B + TMAX * 64u;
+  uint8_t* stg_base = sm + (FORM == PAIR_FLEX ? NSLOT * SLOT : pair_ring_bytes(FIXED_SLOT, pair_slots(FIXED_SLOT), DUAL, UNITS, (int)FIXED_T));
   uint64_t* full = reinterpret_cast<uint64_t*>(stg_base + PAIR_STG);   // the producers' parts of slot s have landed (leader: + the peer's)
-  uint64_t* empty = full + PAIR_MAX_SLOTS;                         // [s / 2]: the MMAs that read slots s and s ^ 1 have completed
-  uint64_t* acc_full = empty + PAIR_MAX_SLOTS;                     // [2]
+  uint64_t* empty = full + PAIR_BARS;                              // [s / 2]: the MMAs that read slots s and s ^ 1 have completed
+  uint64_t* acc_full = empty + PAIR_BARS;                          // [2]
   uint64_t* acc_empty = acc_full + 2;                              // [2] leader: all epilogue warps of the pair have drained the accumulator
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 2);
   volatile uint32_t* timed_out = tmem_slot + 1;                    // an epilogue group's wait gave up
 
+  uint64_t *full_o = DUAL ? full + NSLOT : full, *empty_o = DUAL ? empty + NSLOT / 2 : empty;   // of the outlier stages' ring
   const uint32_t crank = ptx::cluster_ctarank(), rank = crank & 1u, lead = crank & ~1u;   // rank 0 = leader of the pair
   const int ks = FORM == PAIR_FLEX ? p.pt_ks : 1, split = (int)(crank >> 1);   // pairs that share the K range of a task
   const int pair = (int)blockIdx.x / (2 * ks), n_pairs = (int)gridDim.x / (2 * ks);
@@ -144,7 +169,7 @@ sdq_linear_pair_kernel(const __grid_constant__ LinearParams p)
   if (warp == 1 && lane == 0) {
     ptx::griddep_launch_dependents();
     *timed_out = 0u;
-    for (uint32_t s = 0; s < NSLOT; ++s) {
+    for (uint32_t s = 0; s < NSLOT + (DUAL ? O_NSLOT : 0u); ++s) {
       ptx::mbar_init(&full[s], rank == 0 ? 3 : 2);
       if (!(s & 1)) ptx::mbar_init(&empty[s >> 1], 1);
     }
@@ -182,6 +207,35 @@ sdq_linear_pair_kernel(const __grid_constant__ LinearParams p)
       // the first.
       bool ok = true;
       auto produce = [&](auto on_task, auto on_stage) {
+        if constexpr (DUAL) {
+          // n stages in N slots of SZ bytes; both lanes wait for every pair of slots, also where an odd number leaves the second one empty
+          auto stages = [&](int k0, int n, uint32_t N, uint32_t SZ, uint64_t* fl, uint64_t* em, auto first_lap) {
+            uint32_t s = lane;
+            bool ready = false;
+            for (uint32_t g = 0; (int)(2 * g) < n && ok; ++g) {
+              if (g < N / 2) ok = first_lap(s >> 1);
+              else if (!ready) ok = ptx::mbar_wait(&em[s >> 1], ((g / (N / 2)) & 1u) ^ 1u);
+              if (!ok) break;
+              if ((int)(2 * g + lane) < n) on_stage(k0 + (int)(2 * g + lane), sm + (size_t)s * SZ, &fl[s]);
+              s += 2;
+              if (s >= N) s -= N;
+              ready = g + 1 >= N / 2 && ptx::mbar_test(&em[s >> 1], (((g + 1) / (N / 2)) & 1u) ^ 1u);
+            }
+            ok = __all_sync(3u, ok);       // (together again behind an odd number: lanes that run apart take twice as long a trip, 62 -> 72 us)
+          };
+          on_task(pair_task<FORM>(p, pair));
+          stages(0, NI, NSLOT, SLOT, full, empty, [](uint32_t) { return true; });
+          if (ok)
+            stages(NI, S - NI, O_NSLOT, O_SLOT, full_o, empty_o, [&](uint32_t e) {
+              // the pairs of inlier slots with bytes of this pair, of `used` uses in all: the last use of each
+              const uint32_t used = (uint32_t)(NI + 1) / 2, y1 = min((2 * (e + 1) * O_SLOT - 1) / (2 * SLOT), NSLOT / 2 - 1);
+              bool free = true;
+              for (uint32_t y = e * O_SLOT / SLOT; y <= y1 && free; ++y)
+                if (used > y) free = ptx::mbar_wait(&empty[y], ((used - 1 - y) / (NSLOT / 2)) & 1u);
+              return free;
+            });
+          return;
+        }
         uint32_t s = lane, wrapped = 0, ph = 0;
         int tseq = 0, k = (int)lane, cur = -1;                               // this lane's stage: task number in the CTA's sequence, stage in the task
         while (k >= S) { k -= S; ++tseq; }
@@ -225,10 +279,10 @@ sdq_linear_pair_kernel(const __grid_constant__ LinearParams p)
             const bool first_o = k == NI;
             ptx::mbar_expect_tx(bar, (two ? 2u : 1u) * (WO_BYTES + (first_o ? SF_ATOM_BYTES : 0u)));
             ptx::bulk_g2s(st, wo0 + off, WO_BYTES, bar);
-            if (two) ptx::bulk_g2s(st + G::WIB, wo1 + off, WO_BYTES, bar);
+            if (two) ptx::bulk_g2s(st + O_UNIT, wo1 + off, WO_BYTES, bar);
             if (first_o) {
               ptx::bulk_g2s(st + WO_BYTES, sf0, SF_ATOM_BYTES, bar);
-              if (two) ptx::bulk_g2s(st + G::WIB + WO_BYTES, sf1, SF_ATOM_BYTES, bar);
+              if (two) ptx::bulk_g2s(st + O_UNIT + WO_BYTES, sf1, SF_ATOM_BYTES, bar);
             }
           }
         });
@@ -251,12 +305,13 @@ sdq_linear_pair_kernel(const __grid_constant__ LinearParams p)
           if (codes) {
             const uint32_t bytes = own + (inl ? have * NA * SF_ATOM_BYTES : (first_o ? have * SF_ATOM_BYTES : 0u));
             if (bytes) ptx::mbar_expect_tx(bar, bytes); else ptx::mbar_arrive(bar);
-            if (own) ptx::bulk_g2s(st + SL_B, inl ? xi + (size_t)k * p.aoff.xi_stride : xo + (size_t)(k - NI) * p.aoff.xo_stride, own, bar);
+            if (own) ptx::bulk_g2s(st + (inl ? SL_B : O_B), inl ? xi + (size_t)k * p.aoff.xi_stride : xo + (size_t)(k - NI) * p.aoff.xo_stride, own, bar);
           } else if (inl || first_o) {
             const uint8_t* src = inl ? xi + (size_t)k * p.aoff.xi_stride : sf;
             const uint32_t nb = inl ? NA * SF_ATOM_BYTES : SF_ATOM_BYTES;
-            ptx::bulk_g2s(st + SL_SF, src, nb, bar);
-            if (have == 2) ptx::bulk_g2s(st + SL_SF + nb, src + 4 * nb, nb, bar);
+            uint8_t* dst = st + (inl ? SL_SF : O_SF);
+            ptx::bulk_g2s(dst, src, nb, bar);
+            if (have == 2) ptx::bulk_g2s(dst + nb, src + 4 * nb, nb, bar);
           }
         });
       }
@@ -269,12 +324,17 @@ sdq_linear_pair_kernel(const __grid_constant__ LinearParams p)
       // ---------------- odd CTA: forward "my part of the slot has landed" to the leader's barrier (lane l: slots of parity l)
       bool ok = true;
       uint32_t s = lane, ph = 0;
-      for (int i = (int)lane; i < total; i += 2) {
-        if (!(ok = ptx::mbar_wait(&full[s], ph))) break;
-        ptx::mbar_arrive_remote(&full[s], lead);
-        s += 2;
-        if (s >= NSLOT) { s -= NSLOT; ph ^= 1; }
-      }
+      auto forward = [&](int n, uint64_t* fl, uint32_t N) {
+        for (int i = (int)lane; i < n; i += 2) {
+          if (!(ok = ptx::mbar_wait(&fl[s], ph))) break;
+          ptx::mbar_arrive_remote(&fl[s], lead);
+          s += 2;
+          if (s >= N) { s -= N; ph ^= 1; }
+        }
+      };
+      forward(DUAL ? NI : total, full, NSLOT);
+      if (DUAL) ok = __all_sync(3u, ok);
+      if (DUAL && ok) { s = lane; ph = 0; forward(S - NI, full_o, O_NSLOT); }
       if (!ok) atomicOr(&p.flags[FLAG_TIMEOUT], 1u);
     }
   } else if (warp == 1) {
@@ -289,10 +349,11 @@ sdq_linear_pair_kernel(const __grid_constant__ LinearParams p)
     bool ok = true;
     const uint32_t smb = ptx::smem_u32(sm);
     uint32_t s = 0, ph = 0, par = 0;                                // ring slot, its lap parity, parity of the TMEM set
-    const uint64_t d_a = ptx::smem_desc(smb, 128, 256), d_b = ptx::smem_desc(smb + SL_B, 128, 1024);
-    const uint64_t d_cp = ptx::smem_desc(smb, 0, 128), d_sf = ptx::smem_desc(smb + SL_SF, 0, 128);   // copies to TMEM: weight record, scale atoms
+    const uint64_t d_a = ptx::smem_desc(smb, 128, 256), d_b = ptx::smem_desc(smb + SL_B, 128, 1024), d_bo = ptx::smem_desc(smb + O_B, 128, 1024);
+    const uint64_t d_cp = ptx::smem_desc(smb, 0, 128), d_sf = ptx::smem_desc(smb + SL_SF, 0, 128), d_sfo = ptx::smem_desc(smb + O_SF, 0, 128);   // copies to TMEM
     constexpr uint32_t wib16 = G::WIB >> 4, atom16 = SF_ATOM_BYTES >> 4;
-    const uint32_t slot16 = SLOT >> 4;
+    const uint32_t slot16 = SLOT >> 4, o_slot16 = O_SLOT >> 4;
+    constexpr uint32_t o_unit16 = O_UNIT >> 4;
     const uint32_t sfo = meta + 2u * G::SET;                        // outlier scales of the task: SFA_out 2 x 4 | SFB_out 8
     uint32_t tcount = 0;
     for (int task = pair; task < p.pt_tasks && ok; task += n_pairs, ++tcount) {
@@ -308,15 +369,17 @@ sdq_linear_pair_kernel(const __grid_constant__ LinearParams p)
       const uint32_t ab = acc2 ? tcount & 1u : 0u, use = acc2 ? tcount >> 1 : tcount;
       const uint32_t acc0 = tmem + ab * TMAX, acc1 = acc0 + TMAX;
       // instructions of the stages k .. k + n - 1 of the task in ring slots s ..., by one elected lane
-      auto issue = [&](auto units, int k, int n) {
+      // (`stages`: bit 0 inlier, bit 1 outlier ones; DUAL: a run is all the one or all the other, compiled for its ring)
+      auto issue = [&](auto units, auto stages, int k, int n) {
         constexpr int NU = decltype(units)::value;
+        constexpr bool INL = decltype(stages)::value & 1, OUTL = decltype(stages)::value & 2, outl = !INL;
         uint32_t ss = s, pp = par;
         for (int kk = k; kk < k + n; ++kk) {
-          const uint64_t so = (uint64_t)(ss * slot16);
+          const uint64_t so = (uint64_t)(ss * (outl ? o_slot16 : slot16));
           const uint32_t mb = meta + (pp ? G::SET : 0u);
           pp ^= 1u;
           const uint32_t acc = kk ? 1u : 0u;   // the first MMA of the task overwrites the accumulator
-          if (kk < NI) {
+          if (INL && (!OUTL || kk < NI)) {
             // scale words of the tokens: K-block kb, 128 tokens a at SFB + 8 kb + 4 a, staged as [128 tokens][K-block]
             ptx::tc2_cp_32x128b_warpx4(mb + G::SFB, d_sf + so);
             if constexpr (S32) ptx::tc2_cp_32x128b_warpx4(mb + G::SFB + 8, d_sf + so + atom16);
@@ -349,32 +412,35 @@ sdq_linear_pair_kernel(const __grid_constant__ LinearParams p)
           } else {
             if (kk == NI) {
               ptx::tc2_cp_32x128b_warpx4(sfo, d_cp + so + (WO_BYTES >> 4));
-              if constexpr (NU == 2) ptx::tc2_cp_32x128b_warpx4(sfo + 4, d_cp + so + wib16 + (WO_BYTES >> 4));
-              ptx::tc2_cp_32x128b_warpx4(sfo + 8, d_sf + so);
-              if (wide) ptx::tc2_cp_32x128b_warpx4(sfo + 12, d_sf + so + atom16);
+              if constexpr (NU == 2) ptx::tc2_cp_32x128b_warpx4(sfo + 4, d_cp + so + o_unit16 + (WO_BYTES >> 4));
+              ptx::tc2_cp_32x128b_warpx4(sfo + 8, d_sfo + so);
+              if (wide) ptx::tc2_cp_32x128b_warpx4(sfo + 12, d_sfo + so + atom16);
             }
 #pragma unroll
             for (int u = 0; u < NU; ++u) {
-              const uint64_t wo = so + (u ? wib16 : 0u);
+              const uint64_t wo = so + (u ? o_unit16 : 0u);
               const uint32_t e = mb + (u ? 4u : 0u), d = u ? acc1 : acc0, sfa = sfo + (u ? 4u : 0u);
               ptx::tc2_cp_128x128b(e, d_cp + wo + (A_OUT_BYTES >> 4));
-              ptx::mma2_sp_mxf8(d, d_a + wo, d_b + so, id8, e, sfa, sfo + 8, acc);
-              ptx::mma2_sp_mxf8(d, d_a + wo + (4096 >> 4), d_b + so + (512 >> 4), id8, e + 2, sfa, sfo + 8, 1u);
+              ptx::mma2_sp_mxf8(d, d_a + wo, d_bo + so, id8, e, sfa, sfo + 8, acc);
+              ptx::mma2_sp_mxf8(d, d_a + wo + (4096 >> 4), d_bo + so + (512 >> 4), id8, e + 2, sfa, sfo + 8, 1u);
             }
           }
-          if (ss & 1) ptx::tc2_commit_both(&empty[ss >> 1], both);     // slots ss - 1 and ss may be refilled (both CTAs)
+          // slots ss - 1 and ss may be refilled (both CTAs); DUAL: also the last one of an odd number of inlier stages
+          if ((ss & 1) || (DUAL && kk == NI - 1)) ptx::tc2_commit_both(outl ? &empty_o[ss >> 1] : &empty[ss >> 1], both);
           if (kk == S - 1) ptx::tc2_commit_both(&acc_full[ab], both);  // the task's accumulator is complete (both CTAs)
-          if (++ss == NSLOT) ss = 0;
+          if (++ss == (outl ? O_NSLOT : NSLOT)) ss = 0;
         }
       };
       int k = 0;
       while (k < S) {
         // lane i: has slot s + i (the i-th next stage of this task) landed in both CTAs?
-        const uint32_t idx = s + lane, sl = idx >= NSLOT ? idx - NSLOT : idx;
-        const bool r = (int)lane < min(4, S - k) && ptx::mbar_test(&full[sl], idx >= NSLOT ? ph ^ 1 : ph);
+        const bool outl = DUAL && k >= NI;
+        uint64_t* cf = outl ? full_o : full;
+        const uint32_t N = outl ? O_NSLOT : NSLOT, idx = s + lane, sl = idx >= N ? idx - N : idx;
+        const bool r = (int)lane < min(4, (DUAL && !outl ? NI : S) - k) && ptx::mbar_test(&cf[sl], idx >= N ? ph ^ 1 : ph);
         const int n = __ffs(~__ballot_sync(0xffffffffu, r)) - 1;    // length of the run of ready slots
         if (n == 0) {   // nothing yet: wait for the next slot, then look again (its neighbours tend to land with it)
-          ok = __all_sync(0xffffffffu, ptx::mbar_wait(&full[s], ph));
+          ok = __all_sync(0xffffffffu, ptx::mbar_wait(&cf[s], ph));
           if (!ok) break;
           continue;
         }
@@ -384,14 +450,20 @@ sdq_linear_pair_kernel(const __grid_constant__ LinearParams p)
         }
         ptx::tc_fence_after();
         if (ptx::elect_one()) {
-          if (FORM == PAIR_TWO && nu == 2) issue(std::integral_constant<int, FORM == PAIR_TWO ? 2 : 1>{}, k, n);
-          else issue(std::integral_constant<int, 1>{}, k, n);
+          auto run = [&](auto units) {
+            if constexpr (!DUAL) issue(units, std::integral_constant<int, 3>{}, k, n);
+            else if (!outl) issue(units, std::integral_constant<int, 1>{}, k, n);
+            else issue(units, std::integral_constant<int, 2>{}, k, n);
+          };
+          if (FORM == PAIR_TWO && nu == 2) run(std::integral_constant<int, FORM == PAIR_TWO ? 2 : 1>{});
+          else run(std::integral_constant<int, 1>{});
         }
         __syncwarp();
         k += n;
         par ^= (uint32_t)n & 1u;
         s += (uint32_t)n;
-        if (s >= NSLOT) { s -= NSLOT; ph ^= 1; }
+        if (s >= N) { s -= N; ph ^= 1; }
+        if (DUAL && k == NI) s = ph = 0;
       }
     }
     // (a kernel whose stage count is odd leaves its last slot unreleased: nobody waits for it)
@@ -566,11 +638,11 @@ sdq_linear_pair_kernel(const __grid_constant__ LinearParams p)
   if (warp == 1) ptx::tmem_dealloc_pair(tmem, 512);
 }
 
-template <bool F32_OUT, bool B32, bool DENSE, int FORM>
+template <bool F32_OUT, bool B32, bool DENSE, int FORM, bool DUAL = false>
 static cudaError_t launch_form(const LinearParams& p, int pairs, cudaStream_t stream, std::atomic<uint32_t>* attr_mask)
 {
-  auto kern = sdq_linear_pair_kernel<F32_OUT, B32, DENSE, FORM>;
-  const uint32_t bit = 1u << (((F32_OUT ? 3 : 0) + (DENSE ? 2 : (B32 ? 1 : 0))) * 3 + FORM);
+  auto kern = sdq_linear_pair_kernel<F32_OUT, B32, DENSE, FORM, DUAL>;
+  const uint32_t bit = 1u << (DUAL ? 18 + (F32_OUT ? 2 : 0) + FORM : ((F32_OUT ? 3 : 0) + (DENSE ? 2 : (B32 ? 1 : 0))) * 3 + FORM);
   if (!(*attr_mask & bit)) {     // once per device and instantiation
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
     if (e != cudaSuccess) return e;
@@ -579,7 +651,7 @@ static cudaError_t launch_form(const LinearParams& p, int pairs, cudaStream_t st
   cudaLaunchConfig_t lc = {};
   lc.gridDim = dim3((unsigned)(2 * p.pt_ks * pairs));
   lc.blockDim = dim3(PAIR_THREADS);
-  lc.dynamicSmemBytes = (size_t)p.nslot * (size_t)p.slot_bytes + PAIR_TAIL;
+  lc.dynamicSmemBytes = (size_t)p.ring_bytes + PAIR_TAIL;
   lc.stream = stream;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -595,6 +667,10 @@ static cudaError_t launch_form(const LinearParams& p, int pairs, cudaStream_t st
 template <bool F32_OUT, bool B32, bool DENSE>
 static cudaError_t launch_one(const LinearParams& p, int form, int pairs, cudaStream_t stream, std::atomic<uint32_t>* attr_mask)
 {
+  if constexpr (DENSE)
+    if (p.pt_dual)
+      return form == PAIR_TWO ? launch_form<F32_OUT, B32, DENSE, PAIR_TWO, true>(p, pairs, stream, attr_mask)
+                              : launch_form<F32_OUT, B32, DENSE, PAIR_FULL, true>(p, pairs, stream, attr_mask);
   if (form == PAIR_TWO) return launch_form<F32_OUT, B32, DENSE, PAIR_TWO>(p, pairs, stream, attr_mask);
   if (form == PAIR_FULL) return launch_form<F32_OUT, B32, DENSE, PAIR_FULL>(p, pairs, stream, attr_mask);
   return launch_form<F32_OUT, B32, DENSE, PAIR_FLEX>(p, pairs, stream, attr_mask);
@@ -677,7 +753,7 @@ const int* pair_max_clusters(DeviceInfo* d)
   static std::mutex filling;
   if (!d->clusters_known) {
     std::lock_guard<std::mutex> lock(filling);
-    auto kern = sdq_linear_pair_kernel<false, false, false, PAIR_FLEX>;
+    auto kern = sdq_linear_pair_kernel<false, false, false, PAIR_FLEX, false>;
     for (int k = 2; k <= 4 && !d->clusters_known; ++k) {
       cudaLaunchConfig_t lc = {};
       lc.gridDim = dim3((unsigned)(2 * k));
@@ -702,6 +778,9 @@ const int* pair_max_clusters(DeviceInfo* d)
 double pair_kernel_us(int64_t M, int64_t N, int64_t K, int out_n, bool b32, bool dense, int sm_count, const int* max_clusters)
 { return pair_best(M, N, K, out_n, b32, dense, sm_count, max_clusters).us; }
 
+static bool pair_dual(const LinearParams& p, int form, int pairs) {
+  return p.dense && p.out_n > 0 && form != PAIR_FLEX && p.pt_tasks <= pairs && p.K >= 8 * K2;
+}
 // the plan's numbers into the launch parameters (p.M, N, K and the format are there); returns the pairs to launch
 static int pair_apply(LinearParams& p, const PairPlan& best, int sm_count)
 {
@@ -712,6 +791,8 @@ static int pair_apply(LinearParams& p, const PairPlan& best, int sm_count)
   p.pt_doubles = best.doubles; p.pt_split = best.split; p.pt_tasks = best.tasks; p.pt_acc2 = best.acc2; p.pt_ks = best.ks;
   p.slot_bytes = (int)pair_slot_bytes(p.dense ? 17408u : (p.b32 ? 11264u : 10752u), s32, best.form == PAIR_TWO ? 2 : 1, T);
   p.nslot = pair_slots((uint32_t)p.slot_bytes);
+  p.pt_dual = pair_dual(p, best.form, sm_count / 2);
+  p.ring_bytes = (int)pair_ring_bytes((uint32_t)p.slot_bytes, p.nslot, p.pt_dual != 0, best.form == PAIR_TWO ? 2 : 1, T);
   return p.pt_tasks < sm_count / 2 || best.ks > 1 ? p.pt_tasks : sm_count / 2;
 }
 

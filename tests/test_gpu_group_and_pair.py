@@ -828,3 +828,28 @@ def test_group_x_needs_no_memory():
     with pytest.raises(m.SdqError) as e:
         m.sdq_linear_group_x(big, ps)
     assert e.value.code == 4
+
+
+@pytest.mark.parametrize("M,N,K,out_n,gran", [
+    (600, 5120, 2048, 1, so.GRAN_DENSE),      # one-unit tasks, an even number of inlier stages, each slot used once or twice
+    (600, 5120, 2304, 1, so.gran_keep(7)),    # an odd number: the last pair of inlier slots is half used
+    (2900, 1152, 2816, 2, so.GRAN_DENSE),     # an odd number of row tiles, two outliers per S-Vector
+    (1100, 4096, 2304, 1, so.gran_keep(7)),   # two-unit tasks, odd
+    (1300, 3200, 2048, 1, so.GRAN_DENSE),     # two-unit tasks and the odd unit of every token tile, even
+    (4001, 1152, 3072, 1, so.GRAN_ELEM),      # the same, half of the last unit is padding
+])
+def test_outlier_stages_in_a_ring_geometry_of_their_own(M, N, K, out_n, gran):
+    """dense inliers, one task per pair of CTAs: sampled tokens against the oracle, bf16 = RNE of the fp32 result, the same bits again"""
+    m = sdq()
+    cfg = m.Config(out_n, gran, 32, 0)
+    W, X = sdq_synth.make_weight(N, K, 71), sdq_synth.make_act(M, K, 72)
+    p, xq = m.sdq_decompose(W.cuda(), cfg), m.sdq_quantize_act(X.cuda(), cfg)
+    y = m.sdq_linear(xq, p, f32=True)
+    y16, again = m.sdq_linear(xq, p), m.sdq_linear(xq, p, f32=True)
+    assert m.device_status() == 0
+    assert torch.equal(y16, y.to(torch.bfloat16)) and torch.equal(y, again)
+    toks = sorted({0, 95, 96, 191, 192, 255, 256, M // 2, M - 33, M - 1})
+    oc = ocfg(out_n, 0, 32, gran)
+    yref = so.linear(so.quantize_act(sdq_synth.bf16_bits(X[toks]), oc), so.decompose(sdq_synth.bf16_bits(W), oc))
+    d, tol = y_close(y[toks].cpu().numpy(), yref)
+    assert (d <= tol).all(), (d.max(), (d / tol).max())
