@@ -707,8 +707,14 @@ static bool pair_plan(int groups, int mt, int units, int T1, int T2, bool dbl, u
     q.tasks = units * mt;
     us = c1 * ((q.tasks + pairs - 1) / pairs);
     // few tasks: as many pairs to each as the clusters that fit the GPU allow (a reduction costs 1 us + 10 ns a token)
-    for (int k = 2; k <= 4 && q.acc2; ++k)
-      if (q.tasks <= max_clusters[k] && k <= T2 && c1 / k + 1.0 + 0.01 * avgT < us) { us = c1 / k + 1.0 + 0.01 * avgT; q.ks = k; }
+    // (tiles too wide for alternating accumulators are split over two pairs at most, 2.0: with few tokens to a CTA's stages the codes' bytes
+    // count as much as the weights', and tiles of 256 tokens stage a quarter less than twice as many of 128: 500 x 4096 -> 4096 14.73 ->
+    // 14.20 us, 512 x 8192 -> 4096 23.3 -> 19.3, with E4M3 scales 442 x 8704 -> 4096 25.3 -> 20.4; over three pairs 256 x 4096 -> 4096
+    // would go from 12.1 to 13.7.  Adding two items of a reduction at a time was slower by 1 to 5 %)
+    for (int k = 2; k <= (q.acc2 ? 4 : 2); ++k) {
+      const double red = q.acc2 ? 1.0 + 0.01 * avgT : 2.0;
+      if (q.tasks <= max_clusters[k] && k <= T2 && c1 / k + red < us) { us = c1 / k + red; q.ks = k; q.form = PAIR_FLEX; }
+    }
   } else {
     const int D = (units / 2) * mt, odd = (units & 1) * mt;
     const int full = D / pairs * pairs, left = D - full;

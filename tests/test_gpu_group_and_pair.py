@@ -853,3 +853,12 @@ def test_outlier_stages_in_a_ring_geometry_of_their_own(M, N, K, out_n, gran):
     yref = so.linear(so.quantize_act(sdq_synth.bf16_bits(X[toks]), oc), so.decompose(sdq_synth.bf16_bits(W), oc))
     d, tol = y_close(y[toks].cpu().numpy(), yref)
     assert (d <= tol).all(), (d.max(), (d / tol).max())
+
+
+@pytest.mark.parametrize("M,N,K,cfg_args", [
+    (497, 3968, 4096, (1, so.GRAN_PAIR, 64, 0)),      # two tiles of 256 tokens, odd row tiles
+    (450, 3840, 4352, (1, so.GRAN_PAIR, 32, 2)),      # E4M3 scales, K in unequal halves
+    (512, 4096, 4096, (1, so.GRAN_DENSE, 32, 0)),
+])
+def test_wide_tiles_with_k_over_two_pairs(M, N, K, cfg_args):
+    test_cta_pair_task_forms(M, N, K, cfg_args)

@@ -177,3 +177,16 @@ def test_the_device_at_hand_takes_the_same_forms():
         plan, segs = group_plan(M, shapes, here)
         runs(plan, want)
         cover_group(plan, segs, shapes)
+
+
+def test_wide_tiles_are_split_over_two_pairs_at_most():
+    """tiles of more tokens than an alternating accumulator has room for: K over one pair or two, in the form without alternation"""
+    on, seen = machine(*B200), set()
+    for M, N, K, cfg in [(500, 4096, 4096, PAIR), (470, 3840, 5120, PAIR), (512, 4096, 8192, UE), (500, 4096, 4096, DENSE), (500, 2048, 4096, PAIR), (8192, 1024, 1024, PAIR),
+                         (500, 4096, 2048, PAIR), (256, 4096, 4096, PAIR), (1000, 2048, 4096, PAIR), (250, 8192, 4096, PAIR)]:
+        plan, tasks = linear_plan(M, N, K, cfg, on)
+        cover_pairs(plan, tasks, M, N)
+        seen.add((plan.token_tile > 224, plan.ksplit))
+        if plan.ksplit > 1 and plan.token_tile > 224:
+            assert plan.ksplit == 2 and not plan.alternate and plan.tasks <= B200[1][0]
+    assert (True, 2) in seen and (False, 1) in seen
