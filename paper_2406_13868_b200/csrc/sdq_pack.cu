@@ -13,8 +13,9 @@
 // thread per S-Vector scattering bytes -> 20 + 42 us with the row scales in a launch of their own -> 49 us -> 42 us with the
 // pairs picked by two minima and two maxima instead of six comparisons and the choices kept from the first pass.  4096 x 11008,
 // 1:8 + 6:8 with channel weights: 98 us choosing in both passes -> 67.  Loops of four S-Vectors (first pass) and of one Q-Vector
-// (second) instead of 16 and 4 in a row, each warp starting on its own part of the tile, the first arrival relaxed: 43.6 -> 43.0 and
-// 68.2 -> 66.0, without channel weights 53.7 -> 46.6; 16384 x 4096 with E4M3 scales 70.5 -> 64.4.
+// (second) instead of 16 and 4 in a row, each warp starting on its own part of the tile, the rows' maxima exchanged by counted stores
+// instead of a cluster barrier, whole calls: 4096 x 11008 78.5 -> 74.9, without channel weights 64.4 -> 55.8; 16384 x 4096 with E4M3 scales
+// 79.8 -> 74.7; 11008 x 4096 56.0 -> 55.6 (kernel 43.6 -> 43; with the cluster barrier and the loops only, 1 us more).
 #include <cstring>
 #include <type_traits>
 #include <mutex>
@@ -24,6 +25,7 @@
 #include "sdq_internal.h"
 #include "sdq_layout.h"
 #include "sdq_plain.h"
+#include "sdq_ptx.cuh"
 
 namespace sdq {
 
@@ -209,6 +211,7 @@ struct PackParams {
   uint32_t* nonfinite;         // host-visible word, set to 1 when a weight (or channel weight) is not finite
   int out_n, keep_in, order_mask;
   int sv4, elem, ue, i8, b32, ceil_rule;
+  uint32_t* flags;             // sticky status words of the device
 };
 
 // outlier scale of a row from its largest outlier: exponent, or the bit pattern of the fp32 scale amax / 127 (int8)
@@ -335,13 +338,21 @@ pack_kernel(const PackParams p, const BlobHeader hdr)
   extern __shared__ __align__(16) uint8_t tile[];
   __shared__ uint32_t s_part[2][PK_ROWS][PK_ROWS + 1];   // [outliers / inliers][row][128-K chunk]: largest magnitudes
   __shared__ uint32_t s_all[2][8][PK_ROWS];              // [outliers / inliers][cluster rank][row], pushed by their owners
+  __shared__ uint64_t s_bar;                             // ... all of which have arrived
   const uint32_t tid = threadIdx.x;
   const int T1 = (int)(p.K / K1), T2 = T1 / 2;
   const int cx = (int)((p.K + PK_K - 1) / PK_K), rank = (int)(blockIdx.x % (uint32_t)cx);   // FUSED: a cluster is the cx CTAs of these rows
   const bool first_rows = blockIdx.x < (uint32_t)cx;
-  // (waited for before the first store into another CTA's shared memory: every CTA of the cluster has started by then; there is
-  // nothing to release yet, and a releasing arrival is a memory barrier for every warp)
-  if constexpr (FUSED) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+  // (waited for before the first store into another CTA's shared memory: every CTA of the cluster has started by then; the fence
+  // releases the barrier's set-up, and a releasing arrival would be a memory barrier for every warp)
+  if constexpr (FUSED) {
+    if (tid == 0) {
+      ptx::mbar_init(&s_bar, 1);
+      ptx::fence_barrier_init();
+      ptx::mbar_expect_tx(&s_bar, (uint32_t)cx * 2u * PK_ROWS * 4u);
+    }
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+  }
   const int64_t n_first = (int64_t)(blockIdx.x / (uint32_t)cx) * PK_ROWS;
   {
     // 256 threads x 16 B = the 4096 B of one row per round
@@ -440,15 +451,12 @@ pack_kernel(const PackParams p, const BlobHeader hdr)
       uint32_t m = 0;
 #pragma unroll
       for (int c = 0; c < 16; ++c) m = max(m, s_part[which][r][c]);
-      const uint32_t mine_at = (uint32_t)__cvta_generic_to_shared(&s_all[which][rank][r]);
-      for (uint32_t peer = 0; peer < (uint32_t)cx; ++peer) {
-        uint32_t ra;
-        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(mine_at), "r"(peer));
-        asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(ra), "r"(m) : "memory");
-      }
+      const uint32_t mine_at = ptx::smem_u32(&s_all[which][rank][r]), bar = ptx::smem_u32(&s_bar);
+      for (uint32_t peer = 0; peer < (uint32_t)cx; ++peer) ptx::st_async_u32(ptx::mapa_u32(mine_at, peer), m, ptx::mapa_u32(bar, peer));
     }
-    // every push is visible after this barrier, and nobody touches another CTA's memory afterwards
-    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    // counted stores, as in the activation quantizer: a CTA waits for what it needs and for nothing else, and does not leave before all
+    // pushes to it have arrived
+    if (!ptx::mbar_wait_cluster(&s_bar, 0) && (tid & 31u) == 0) atomicOr(&p.flags[FLAG_TIMEOUT], 1u);
     omax = imax = 0;
     for (int c = 0; c < cx; ++c) { omax = max(omax, s_all[0][c][row]); imax = max(imax, s_all[1][c][row]); }
     if (rank == 0 && ch == 0) store_row_scale(p, n, omax, imax);
@@ -882,12 +890,13 @@ extern "C" sdq_status_t sdq_decompose_metric(const void* W, int64_t N, int64_t K
   uint32_t* report = g_report.take();
   if (!report) return SDQ_ERR_CUDA;
   uint32_t* report_dev = nullptr;
-  bool ok = cudaHostGetDevicePointer((void**)&report_dev, report, 0) == cudaSuccess;
+  bool ok = cudaHostGetDevicePointer((void**)&report_dev, report, 0) == cudaSuccess && device_flags();
   if (ok && tc) {
     PackParams p;
     p.W = (const __nv_bfloat16*)W; p.N = N; p.K = K; p.ldw = ldw; p.colw = col_weight;
     p.blob = (uint8_t*)packed_buf; p.off = off; p.nonfinite = report_dev;
     p.out_n = cfg->out_n;
+    p.flags = device_flags();
     p.sv4 = cfg->in_gran == SDQ_GRAN_3OF4;          // S-Vectors of 4: one outlier and two inliers per 4
     p.elem = cfg->in_gran == SDQ_GRAN_ELEM;         // element-wise 2:4: the 2 most significant non-outliers of every 4
     // dense family: inliers kept per group (8 - out_n without Stage 1; groups of 4: 3 minus the outlier, or 2 for 2:4)
