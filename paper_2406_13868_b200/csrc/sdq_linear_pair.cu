@@ -162,32 +162,33 @@ sdq_linear_pair_kernel(const __grid_constant__ LinearParams p)
   const int total = my_tasks * S;                                  // stages of this CTA, numbered through its tasks
 
   // Set-up.  The producers need nothing but this CTA's barriers for the ring's first lap, so they start on those while tensor memory
-  // is being allocated and the other CTAs of the cluster are waited for (by everybody else, before anything remote).  Only warp 1 has
-  // something to release to them (chains of calls, everybody behind one barrier before -> now: 40 x 4096 -> 4096 9.56 -> 9.33 us, 500 x
-  // 4096 -> 4096 14.93 -> 14.65, 1000 17.28 -> 16.7, 300 x 4096 -> 11008 21.65 -> 21.2; 130 x 16384 -> 4096 20.38 -> 20.50).
+  // is being allocated and the other CTAs of the cluster are waited for (by everybody else, before anything remote).  The fence behind
+  // the barriers releases them; only warp 1's allocation has to be released besides.  Chains of calls, everybody behind one barrier before ->
+  // now: 40 x 4096 -> 4096 9.56 -> 9.08 us, 500 x 4096 -> 4096 14.73 -> 13.9, 1000 17.28 -> 16.4, 130 x 16384 -> 4096 20.38 -> 20.05.
   const bool producer = warp == 0 || warp == 2 || warp == 3;
-  if (warp == 1 && lane == 0) {
-    ptx::griddep_launch_dependents();
-    *timed_out = 0u;
-    for (uint32_t s = 0; s < NSLOT + (DUAL ? O_NSLOT : 0u); ++s) {
-      ptx::mbar_init(&full[s], rank == 0 ? 3 : 2);
-      if (!(s & 1)) ptx::mbar_init(&empty[s >> 1], 1);
+  if (warp == 0) {
+    if (lane < NSLOT + (DUAL ? O_NSLOT : 0u)) {
+      ptx::mbar_init(&full[lane], rank == 0 ? 3 : 2);
+      if (!(lane & 1)) ptx::mbar_init(&empty[lane >> 1], 1);
+    } else if (lane >= 30) {
+      ptx::mbar_init(&acc_full[lane - 30], 1);
+      ptx::mbar_init(&acc_empty[lane - 30], 32);
+    } else if (lane == 29) {
+      ptx::griddep_launch_dependents();
+      *timed_out = 0u;
     }
-    for (int a = 0; a < 2; ++a) { ptx::mbar_init(&acc_full[a], 1); ptx::mbar_init(&acc_empty[a], 32); }
     ptx::fence_barrier_init();
   }
   __syncwarp();
   uint32_t tmem = 0;
   if (producer) {
-    ptx::named_bar_sync(5, 128);
+    if (warp == 0) ptx::named_bar_arrive(6, PAIR_THREADS - 64);
+    ptx::named_bar_sync(5, 96);
     asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
   } else {
-    if (warp == 1) {                                               // (its barriers are set up: the producers go on)
-      ptx::named_bar_arrive(5, 128);
-      ptx::tmem_alloc_pair(tmem_slot, 512);
-    }
+    if (warp == 1) ptx::tmem_alloc_pair(tmem_slot, 512);
     ptx::tc_fence_before();
-    ptx::named_bar_sync(6, PAIR_THREADS - 96);
+    ptx::named_bar_sync(6, PAIR_THREADS - 64);
     if (warp == 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
     else asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");   // both CTAs' barriers and tensor memory exist before anything remote
@@ -254,7 +255,7 @@ sdq_linear_pair_kernel(const __grid_constant__ LinearParams p)
       if (warp == 0) {
         // weight records of the one or two units
         const uint8_t *wi0 = nullptr, *wi1 = nullptr, *wo0 = nullptr, *wo1 = nullptr, *sf0 = nullptr, *sf1 = nullptr;
-        uint32_t nu = 1;
+        uint32_t nu = 1, early = NSLOT / 4;     // pairs of slots filled before the previous kernel has ended
         produce([&](const PairTask& t) {
           nu = (uint32_t)t.nu;
           // (an odd number of row tiles: the last unit's second half repeats the last tile and is not stored)
@@ -268,6 +269,9 @@ sdq_linear_pair_kernel(const __grid_constant__ LinearParams p)
             sf1 = p.w + p.poff.sfa_out + (size_t)rt1 * SF_ATOM_BYTES;
           }
         }, [&](int k, uint8_t* st, uint64_t* bar) {
+          // half a lap of weights is under way when the activations come; the other half would only stand in the way of what the previous
+          // kernel, as a rule the quantizer, still has to load
+          if (early-- == 0) ptx::griddep_wait();
           const bool two = FORM == PAIR_TWO && nu == 2;
           if (k < NI) {
             const uint32_t off = (uint32_t)k * G::WIB;
