@@ -35,7 +35,6 @@ struct LinearParams {
   int pt_doubles, pt_split;       // the first tasks, of two units; of the one-unit tasks behind them, the first pt_split are halves of two-unit ones
   int pt_tasks;                   // all tasks
   int pt_ks;                      // pairs that share the K range of a task, in a cluster of 2 pt_ks CTAs (then one task per cluster)
-  int pt_dual;                    // 1: the outlier stages use the ring in a geometry of their own (dense inliers, one task per pair)
   int pt_acc2;                    // 1: the accumulator alternates between two sets of columns (one-unit tasks only)
   int ksplit;            // CTAs sharing the K range of one row tile (1 = no split)
   int cluster_ks;        // > 1: those CTAs form a cluster and reduce through distributed shared memory

@@ -642,6 +642,9 @@ sdq_linear_pair_kernel(const __grid_constant__ LinearParams p)
   if (warp == 1) ptx::tmem_dealloc_pair(tmem, 512);
 }
 
+static bool pair_dual(const LinearParams& p, int form, int pairs) {
+  return p.dense && p.out_n > 0 && form != PAIR_FLEX && p.pt_tasks <= pairs && p.K >= 8 * K2;
+}
 template <bool F32_OUT, bool B32, bool DENSE, int FORM, bool DUAL = false>
 static cudaError_t launch_form(const LinearParams& p, int pairs, cudaStream_t stream, std::atomic<uint32_t>* attr_mask)
 {
@@ -672,7 +675,7 @@ template <bool F32_OUT, bool B32, bool DENSE>
 static cudaError_t launch_one(const LinearParams& p, int form, int pairs, cudaStream_t stream, std::atomic<uint32_t>* attr_mask)
 {
   if constexpr (DENSE)
-    if (p.pt_dual)
+    if (pair_dual(p, form, pairs))
       return form == PAIR_TWO ? launch_form<F32_OUT, B32, DENSE, PAIR_TWO, true>(p, pairs, stream, attr_mask)
                               : launch_form<F32_OUT, B32, DENSE, PAIR_FULL, true>(p, pairs, stream, attr_mask);
   if (form == PAIR_TWO) return launch_form<F32_OUT, B32, DENSE, PAIR_TWO>(p, pairs, stream, attr_mask);
@@ -788,9 +791,6 @@ const int* pair_max_clusters(DeviceInfo* d)
 double pair_kernel_us(int64_t M, int64_t N, int64_t K, int out_n, bool b32, bool dense, int sm_count, const int* max_clusters)
 { return pair_best(M, N, K, out_n, b32, dense, sm_count, max_clusters).us; }
 
-static bool pair_dual(const LinearParams& p, int form, int pairs) {
-  return p.dense && p.out_n > 0 && form != PAIR_FLEX && p.pt_tasks <= pairs && p.K >= 8 * K2;
-}
 // the plan's numbers into the launch parameters (p.M, N, K and the format are there); returns the pairs to launch
 static int pair_apply(LinearParams& p, const PairPlan& best, int sm_count)
 {
@@ -801,8 +801,7 @@ static int pair_apply(LinearParams& p, const PairPlan& best, int sm_count)
   p.pt_doubles = best.doubles; p.pt_split = best.split; p.pt_tasks = best.tasks; p.pt_acc2 = best.acc2; p.pt_ks = best.ks;
   p.slot_bytes = (int)pair_slot_bytes(p.dense ? 17408u : (p.b32 ? 11264u : 10752u), s32, best.form == PAIR_TWO ? 2 : 1, T);
   p.nslot = pair_slots((uint32_t)p.slot_bytes);
-  p.pt_dual = pair_dual(p, best.form, sm_count / 2);
-  p.ring_bytes = (int)pair_ring_bytes((uint32_t)p.slot_bytes, p.nslot, p.pt_dual != 0, best.form == PAIR_TWO ? 2 : 1, T);
+  p.ring_bytes = (int)pair_ring_bytes((uint32_t)p.slot_bytes, p.nslot, pair_dual(p, best.form, sm_count / 2), best.form == PAIR_TWO ? 2 : 1, T);
   return p.pt_tasks < sm_count / 2 || best.ks > 1 ? p.pt_tasks : sm_count / 2;
 }
 
