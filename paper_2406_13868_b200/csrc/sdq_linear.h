@@ -19,7 +19,7 @@ struct LinearParams {
   int n_tile;            // few tokens: 16, 32, 64 or 128, the one token tile; pairs: tokens of the widest tile
   int total_tiles;       // (N / 128) * ksplit
   int nslot, slot_bytes; // shared-memory ring geometry (depends on n_tile)
-  int ring_bytes;        // nslot * slot_bytes; the transpose buffer and the barriers follow
+  int ring_bytes;        // nslot * slot_bytes (pairs: or what the outlier stages' own slots take, if more); the transpose buffer and the barriers follow
   int release;           // 1: ring slots are reused (producer waits on `empty`, MMA issuer commits to it)
   int tmem_cols;         // TMEM columns to allocate (128, 256 or 512)
   int meta_col;          // first TMEM column of the metadata / scale buffers

@@ -18,7 +18,7 @@
 //
 // Sustained (0.3 s of calls), one unit x 256 tokens before -> now: 2048 x 4096 -> 11008 80.2 -> 77.5 us, 8192 x 11008 -> 4096
 // 278 -> 259 us, with E4M3 scales 4096 x 16384 -> 4096 265 -> 232 us, dense inliers 1500 x 11008 -> 4096 90 -> 78 us; K over
-// several pairs 130 x 16384 -> 4096 27 -> 21 us, 400 x 16384 -> 1024 35 -> 17 us; 500 x 4096 -> 4096 21.1 -> 14.3 us.
+// several pairs 130 x 16384 -> 4096 27 -> 21 us, 400 x 16384 -> 1024 35 -> 17 us; 500 x 4096 -> 4096 21.1 -> 13.9 us.
 //
 // Few tasks (narrow matrices, few tokens): a task is one chain of stages at ~0.16 us each however few tokens it has, so its K
 // range is split over 2 to 4 pairs of a larger cluster; their fp32 partial tiles meet in shared memory and every CTA adds
@@ -55,7 +55,7 @@ constexpr int PAIR_TAIL = PAIR_STG + (2 * PAIR_BARS + 4) * 8 + 16 + 128;   // + 
 
 // Geometry of a launch.  TWO: tasks of two units (and one), FULL: of one unit with token tiles of up to 256, both with the
 // ring's and tensor memory's geometry known at compile time (the issue loop pays for every runtime parameter: 474 against
-// 427 cycles per stage of two 256-token MMAs); FLEX: one unit, narrower tiles, geometry from the launch parameters.
+// 427 cycles per stage of two 256-token MMAs); FLEX: one unit, narrower tiles or K split, geometry from the launch parameters.
 enum { PAIR_TWO = 0, PAIR_FULL = 1, PAIR_FLEX = 2 };
 
 template <bool B32, bool DENSE>
@@ -167,6 +167,7 @@ sdq_linear_pair_kernel(const __grid_constant__ LinearParams p)
   // now: 40 x 4096 -> 4096 9.56 -> 9.08 us, 500 x 4096 -> 4096 14.73 -> 13.9, 1000 17.28 -> 16.4, 130 x 16384 -> 4096 20.38 -> 20.05.
   const bool producer = warp == 0 || warp == 2 || warp == 3;
   if (warp == 0) {
+    if (lane == 0) ptx::griddep_launch_dependents();   // (first of all: behind the barriers' set-up a pass of 100 tokens took 17.82 instead of 17.72 us)
     if (lane < NSLOT + (DUAL ? O_NSLOT : 0u)) {
       ptx::mbar_init(&full[lane], rank == 0 ? 3 : 2);
       if (!(lane & 1)) ptx::mbar_init(&empty[lane >> 1], 1);
@@ -174,7 +175,6 @@ sdq_linear_pair_kernel(const __grid_constant__ LinearParams p)
       ptx::mbar_init(&acc_full[lane - 30], 1);
       ptx::mbar_init(&acc_empty[lane - 30], 32);
     } else if (lane == 29) {
-      ptx::griddep_launch_dependents();
       *timed_out = 0u;
     }
     ptx::fence_barrier_init();
