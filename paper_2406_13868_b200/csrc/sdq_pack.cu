@@ -455,8 +455,12 @@ pack_kernel(const PackParams p, const BlobHeader hdr)
       for (uint32_t peer = 0; peer < (uint32_t)cx; ++peer) ptx::st_async_u32(ptx::mapa_u32(mine_at, peer), m, ptx::mapa_u32(bar, peer));
     }
     // counted stores, as in the activation quantizer: a CTA waits for what it needs and for nothing else, and does not leave before all
-    // pushes to it have arrived
-    if (!ptx::mbar_wait_cluster(&s_bar, 0) && (tid & 31u) == 0) atomicOr(&p.flags[FLAG_TIMEOUT], 1u);
+    // pushes to it have arrived.  Where the wait gives up, peers may still push: this CTA stays until they have, or have given up as well
+    if (!ptx::mbar_wait_cluster(&s_bar, 0)) {
+      atomicOr(&p.flags[FLAG_TIMEOUT], 1u);
+      ptx::cluster_wait_for_others();
+      (void)ptx::mbar_wait_cluster(&s_bar, 0);             // (what was sent last is still on its way)
+    }
     omax = imax = 0;
     for (int c = 0; c < cx; ++c) { omax = max(omax, s_all[0][c][row]); imax = max(imax, s_all[1][c][row]); }
     if (rank == 0 && ch == 0) store_row_scale(p, n, omax, imax);

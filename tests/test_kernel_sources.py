@@ -45,6 +45,13 @@ def test_no_remote_shared_memory_before_the_cluster_has_started(name):
             assert started and started.start() < first
 
 
+def test_a_packer_whose_wait_gives_up_stays_for_its_peers():
+    """peers may still store into the shared memory of a thread block that gave up: it waits for them before it can leave"""
+    body = {n: b for _, n, b in kernels()}["pack_kernel"]
+    gave_up = re.search(r"if \(!ptx::mbar_wait_cluster\(&s_bar, 0\)\) \{([^{}]*)\}", body)
+    assert gave_up and re.search(r"ptx::cluster_wait_for_others\(\);\s*\(void\)ptx::mbar_wait_cluster\(&s_bar, 0\);", gave_up.group(1))
+
+
 def test_packed_weights_are_ordered_behind_the_kernels_in_front():
     """a quantizer lets the next launch in (which may read packed weights at once) only behind its own wait for the previous
     one, and the grouped kernel copies nothing before its wait -- but in the calls that want the weights complete"""
