@@ -36,7 +36,7 @@ typedef enum {
   SDQ_ERR_BUFFER_TOO_SMALL = 5, /* caller buffer smaller than the matching *_size query      */
   SDQ_ERR_NONFINITE = 6,        /* Inf/NaN weight (or bad channel weight) seen by sdq_decompose */
   SDQ_ERR_CUDA = 7,             /* a CUDA runtime call failed (launch error etc.)            */
-  SDQ_ERR_TIMEOUT = 8           /* a bounded device-side wait gave up (sticky device status) */
+  SDQ_ERR_TIMEOUT = 8           /* a bounded device-side wait gave up (sticky device status; sdq_decompose returns it) */
 } sdq_status_t;
 
 enum { SDQ_GRAN_PAIR = 0, SDQ_GRAN_ELEM = 1, SDQ_GRAN_DENSE = 2 }; /* inlier pattern            */
@@ -159,7 +159,7 @@ sdq_status_t sdq_packed_size(int64_t N, int64_t K, const sdq_config_t* cfg, size
  *   W (device) [N][ldw] bf16, ldw >= K elements; packed_buf (device) >= *bytes of sdq_packed_size;
  *   out (host) receives the descriptor.  Enqueues on `stream`, then synchronises that stream once
  *   to read back the non-finite flag.  Errors: INVALID_ARG, SHAPE, ALIGNMENT, BUFFER_TOO_SMALL,
- *   NONFINITE (buffer contents undefined), CUDA. */
+ *   NONFINITE and TIMEOUT (buffer contents undefined), CUDA. */
 sdq_status_t sdq_decompose(const void* W_bf16, int64_t N, int64_t K, int64_t ldw, const sdq_config_t* cfg,
                            void* packed_buf, size_t packed_bytes, sdq_packed_t* out, void* stream);
 

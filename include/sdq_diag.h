@@ -25,11 +25,18 @@ sdq_status_t sdq_diag_l2_copy(const void* src, size_t src_bytes, int slot_bytes,
 
 
 /* Self-test of the failure detection: every device-side wait of the library is bounded and reports through the sticky
- * status word instead of hanging.  This enqueues a one-thread kernel that waits, for at most `polls` polls (1 .. 4096),
+ * status word (packing: through its return value) instead of hanging.  This enqueues a one-thread kernel that waits, for at most `polls` polls (1 .. 4096),
  * on a shared-memory barrier that nothing ever completes; the wait gives up, the kernel sets the status word and
  * returns.  sdq_device_status(stream) then returns SDQ_ERR_TIMEOUT once (and clears it).  Nothing traps, nothing hangs,
  * the context stays usable.  Asynchronous on `stream`.  Errors: SHAPE (polls out of range), CUDA. */
 sdq_status_t sdq_diag_wait_timeout(int polls, void* stream);
+
+/* The same of a packing call, which waits for its kernel and so reports by itself: sdq_decompose whose kernel gives its wait for the
+ * rows' maxima no polls at all (K <= 16384 and a configuration that sdq_linear accepts; others have no wait).  The thread blocks give
+ * up, wait for what their peers still send them, and the call returns SDQ_ERR_TIMEOUT (SDQ_ERR_NONFINITE comes first); what
+ * packed_buf then holds is not to be used.  Nothing is left behind for later calls.  Errors: as sdq_decompose. */
+sdq_status_t sdq_diag_decompose_timeout(const void* W, int64_t N, int64_t K, int64_t ldw, const sdq_config_t* cfg, void* packed_buf,
+                                        size_t packed_bytes, sdq_packed_t* out, void* stream);
 
 /* What a call would run, decided by the functions that decide it in the call itself; nothing is launched.
  *   sm_count > 0: for a GPU of that many SMs, of which max_clusters[k] (k = 2, 3, 4; NULL: none) clusters of 2 k thread blocks, one

@@ -70,7 +70,7 @@ class _ActCanon(ctypes.Structure):
 
 EXPORTS = ["sdq_packed_size", "sdq_decompose", "sdq_decompose_metric", "sdq_channel_norm", "sdq_packed_export", "sdq_packed_attach", "sdq_packed_compact_size", "sdq_packed_compact", "sdq_act_size", "sdq_quantize_act", "sdq_act_export",
            "sdq_linear", "sdq_linear_f32", "sdq_workspace_size", "sdq_workspace_init", "sdq_linear_ws", "sdq_linear_f32_ws", "sdq_linear_noalloc",
-           "sdq_linear_group", "sdq_linear_group_f32", "sdq_linear_group_x", "sdq_linear_group_x_f32", "sdq_linear_group_x_ws", "sdq_linear_group_x_f32_ws", "sdq_diag_l2_copy", "sdq_diag_wait_timeout", "sdq_diag_linear_plan", "sdq_diag_group_plan", "sdq_device_status", "sdq_status_string"]
+           "sdq_linear_group", "sdq_linear_group_f32", "sdq_linear_group_x", "sdq_linear_group_x_f32", "sdq_linear_group_x_ws", "sdq_linear_group_x_f32_ws", "sdq_diag_l2_copy", "sdq_diag_wait_timeout", "sdq_diag_decompose_timeout", "sdq_diag_linear_plan", "sdq_diag_group_plan", "sdq_device_status", "sdq_status_string"]
 
 _lib = None
 
@@ -92,6 +92,7 @@ def lib() -> ctypes.CDLL:
         L.sdq_packed_export.argtypes = [ctypes.POINTER(_Packed), ctypes.POINTER(_Canon), vp]
         L.sdq_packed_attach.argtypes = [vp, sz, ctypes.POINTER(_Packed), vp]
         L.sdq_diag_wait_timeout.argtypes = [ctypes.c_int, vp]
+        L.sdq_diag_decompose_timeout.argtypes = L.sdq_decompose.argtypes
         L.sdq_act_size.argtypes = [i64, i64, ctypes.POINTER(Config), ctypes.POINTER(sz)]
         L.sdq_quantize_act.argtypes = [vp, i64, i64, i64, ctypes.POINTER(Config), vp, sz, ctypes.POINTER(_Act), vp]
         L.sdq_act_export.argtypes = [ctypes.POINTER(_Act), ctypes.POINTER(_ActCanon), vp]

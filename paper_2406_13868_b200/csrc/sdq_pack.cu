@@ -21,6 +21,7 @@
 #include <mutex>
 #include <condition_variable>
 
+#include "../../include/sdq_diag.h"
 #include "sdq_codec.cuh"
 #include "sdq_internal.h"
 #include "sdq_layout.h"
@@ -209,6 +210,8 @@ struct PackParams {
   uint8_t* blob;
   PackedOffsets off;
   uint32_t* nonfinite;         // host-visible word, set to 1 when a weight (or channel weight) is not finite
+  uint32_t* gave_up;           // ... when a wait for the rows' maxima gave up
+  uint32_t polls;              // ... which it does after that many
   int out_n, keep_in, order_mask;
   int sv4, elem, ue, i8, b32, ceil_rule;
   uint32_t* flags;             // sticky status words of the device
@@ -456,8 +459,8 @@ pack_kernel(const PackParams p, const BlobHeader hdr)
     }
     // counted stores, as in the activation quantizer: a CTA waits for what it needs and for nothing else, and does not leave before all
     // pushes to it have arrived.  Where the wait gives up, peers may still push: this CTA stays until they have, or have given up as well
-    if (!ptx::mbar_wait_cluster(&s_bar, 0)) {
-      atomicOr(&p.flags[FLAG_TIMEOUT], 1u);
+    if (!ptx::mbar_wait_cluster(&s_bar, 0, p.polls)) {
+      *reinterpret_cast<volatile uint32_t*>(p.gave_up) = 1u;
       ptx::cluster_wait_for_others();
       (void)ptx::mbar_wait_cluster(&s_bar, 0);             // (what was sent last is still on its way)
     }
@@ -687,31 +690,31 @@ static void launch_pack(const PackParams& p, const BlobHeader& hdr, cudaStream_t
   go(pack_kernel<DENSE, WGT, OUTN, false>, 0);
 }
 
-// One host-visible word per call in flight, where the kernels report a non-finite weight: a page of pinned memory, taken
-// once per process and kept; a call holds its word until its stream has been synchronised, so calls of other threads and
-// streams never share one.  More calls at once than words wait for one to be given back.
+// Host-visible words of a call in flight, where the kernels report a non-finite weight and a wait that gave up: a page of pinned
+// memory, taken once per process and kept; a call holds its words until its stream has been synchronised, so calls of other threads
+// and streams never share any.  More calls at once than there are words for wait for some to be given back.
 class ReportWords {
  public:
   uint32_t* take() {
     std::unique_lock<std::mutex> lock(m_);
     if (!base_) {
       void* ptr = nullptr;
-      if (cudaHostAlloc(&ptr, COUNT * sizeof(uint32_t), cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) return nullptr;
+      if (cudaHostAlloc(&ptr, COUNT * WORDS * sizeof(uint32_t), cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) return nullptr;
       base_ = (uint32_t*)ptr;
       for (int i = 0; i < COUNT; ++i) free_[i] = i;
       n_free_ = COUNT;
     }
     cv_.wait(lock, [this] { return n_free_ > 0; });
-    uint32_t* w = base_ + free_[--n_free_];
-    *reinterpret_cast<volatile uint32_t*>(w) = 0u;
+    uint32_t* w = base_ + free_[--n_free_] * WORDS;
+    for (int i = 0; i < WORDS; ++i) reinterpret_cast<volatile uint32_t*>(w)[i] = 0u;
     return w;
   }
   void give_back(uint32_t* w) {
-    { std::lock_guard<std::mutex> lock(m_); free_[n_free_++] = (int)(w - base_); }
+    { std::lock_guard<std::mutex> lock(m_); free_[n_free_++] = (int)(w - base_) / WORDS; }
     cv_.notify_one();
   }
  private:
-  static constexpr int COUNT = 64;
+  static constexpr int COUNT = 64, WORDS = 2;
   std::mutex m_;
   std::condition_variable cv_;
   uint32_t* base_ = nullptr;
@@ -856,13 +859,9 @@ extern "C" sdq_status_t sdq_packed_size(int64_t N, int64_t K, const sdq_config_t
   return SDQ_OK;
 }
 
-extern "C" sdq_status_t sdq_decompose(const void* W, int64_t N, int64_t K, int64_t ldw, const sdq_config_t* cfg, void* packed_buf,
-                                      size_t packed_bytes, sdq_packed_t* out, void* stream)
-{ return sdq_decompose_metric(W, N, K, ldw, cfg, nullptr, packed_buf, packed_bytes, out, stream); }
-
-extern "C" sdq_status_t sdq_decompose_metric(const void* W, int64_t N, int64_t K, int64_t ldw, const sdq_config_t* cfg,
-                                             const float* col_weight, void* packed_buf, size_t packed_bytes, sdq_packed_t* out,
-                                             void* stream)
+// polls: what a wait inside the kernel is given
+static sdq_status_t decompose(const void* W, int64_t N, int64_t K, int64_t ldw, const sdq_config_t* cfg, const float* col_weight, void* packed_buf,
+                              size_t packed_bytes, sdq_packed_t* out, void* stream, uint32_t polls = 1u << 22)
 {
   if (!W || !packed_buf || !out || !cfg_ok(cfg)) return SDQ_ERR_INVALID_ARG;
   if (cfg_unsupported(cfg)) return SDQ_ERR_UNSUPPORTED;
@@ -898,7 +897,7 @@ extern "C" sdq_status_t sdq_decompose_metric(const void* W, int64_t N, int64_t K
   if (ok && tc) {
     PackParams p;
     p.W = (const __nv_bfloat16*)W; p.N = N; p.K = K; p.ldw = ldw; p.colw = col_weight;
-    p.blob = (uint8_t*)packed_buf; p.off = off; p.nonfinite = report_dev;
+    p.blob = (uint8_t*)packed_buf; p.off = off; p.nonfinite = report_dev; p.gave_up = report_dev + 1; p.polls = polls;
     p.out_n = cfg->out_n;
     p.flags = device_flags();
     p.sv4 = cfg->in_gran == SDQ_GRAN_3OF4;          // S-Vectors of 4: one outlier and two inliers per 4
@@ -929,11 +928,24 @@ extern "C" sdq_status_t sdq_decompose_metric(const void* W, int64_t N, int64_t K
   }
   ok = (cudaGetLastError() == cudaSuccess) && ok;
   ok = (cudaStreamSynchronize(st) == cudaSuccess) && ok;      // also before the word goes back: no kernel writes it afterwards
-  const uint32_t nonfinite = *reinterpret_cast<volatile uint32_t*>(report);
+  const uint32_t nonfinite = reinterpret_cast<volatile uint32_t*>(report)[0], gave_up = reinterpret_cast<volatile uint32_t*>(report)[1];
   g_report.give_back(report);
   if (!ok) return SDQ_ERR_CUDA;
-  return nonfinite ? SDQ_ERR_NONFINITE : SDQ_OK;
+  return nonfinite ? SDQ_ERR_NONFINITE : (gave_up ? SDQ_ERR_TIMEOUT : SDQ_OK);
 }
+
+extern "C" sdq_status_t sdq_decompose(const void* W, int64_t N, int64_t K, int64_t ldw, const sdq_config_t* cfg, void* packed_buf,
+                                      size_t packed_bytes, sdq_packed_t* out, void* stream)
+{ return decompose(W, N, K, ldw, cfg, nullptr, packed_buf, packed_bytes, out, stream); }
+
+extern "C" sdq_status_t sdq_decompose_metric(const void* W, int64_t N, int64_t K, int64_t ldw, const sdq_config_t* cfg,
+                                             const float* col_weight, void* packed_buf, size_t packed_bytes, sdq_packed_t* out,
+                                             void* stream)
+{ return decompose(W, N, K, ldw, cfg, col_weight, packed_buf, packed_bytes, out, stream); }
+
+extern "C" sdq_status_t sdq_diag_decompose_timeout(const void* W, int64_t N, int64_t K, int64_t ldw, const sdq_config_t* cfg, void* packed_buf,
+                                                   size_t packed_bytes, sdq_packed_t* out, void* stream)
+{ return decompose(W, N, K, ldw, cfg, nullptr, packed_buf, packed_bytes, out, stream, 0); }
 
 extern "C" sdq_status_t sdq_packed_attach(const void* dev, size_t bytes, sdq_packed_t* out, void* stream)
 {

@@ -406,6 +406,25 @@ def test_a_bounded_wait_that_runs_out_sets_the_sticky_status_and_the_context_sta
     assert (d <= tol).all()
 
 
+@pytest.mark.parametrize("N,K,cfg_args,waits", [
+    (128, 256, (1, so.GRAN_PAIR, 64, 0), True),          # a thread block that waits for itself
+    (256, 4352, (1, so.GRAN_DENSE, 32, 0), True),        # three of them, the last with little to do
+    (4096, 16384, (2, so.GRAN_PAIR, 32, 2), True),       # eight, in several rounds
+    (128, 16640, (1, so.GRAN_PAIR, 64, 0), False),       # longer rows: row scales in a launch of their own, no wait
+    (128, 256, (1, so.GRAN_ELEM, 64, 0), False),         # the layout that is packed only
+])
+def test_a_packing_call_whose_wait_gives_up_returns_the_timeout(N, K, cfg_args, waits):
+    m = sdq()
+    cfg = m.Config(*cfg_args)
+    W = sdq_synth.make_weight(N, K, 4822).cuda()
+    buf, d = torch.zeros(m.packed_size(N, K, cfg)[0], dtype=torch.uint8, device="cuda"), m._Packed()
+    want = m.sdq_decompose(W, cfg, buf.clone()).buf
+    st = m.lib().sdq_diag_decompose_timeout(W.data_ptr(), N, K, W.stride(0), ctypes.byref(cfg), buf.data_ptr(), buf.numel(), ctypes.byref(d), m._stream())
+    assert st == (8 if waits else 0)
+    assert m.device_status() == 0                              # the call's own report, not the device's word
+    assert torch.equal(m.sdq_decompose(W, cfg, torch.zeros_like(want)).buf, want)
+
+
 # ---------------------------------------------------------------------------------------------------------------------
 # int8 outlier operands (Section 5.1: W_o and A_o in int8; the evaluation's "1:8int8" configurations)
 
