@@ -214,7 +214,6 @@ struct PackParams {
   uint32_t polls;              // ... which it does after that many
   int out_n, keep_in, order_mask;
   int sv4, elem, ue, i8, b32, ceil_rule;
-  uint32_t* flags;             // sticky status words of the device
 };
 
 // outlier scale of a row from its largest outlier: exponent, or the bit pattern of the fp32 scale amax / 127 (int8)
@@ -893,13 +892,12 @@ static sdq_status_t decompose(const void* W, int64_t N, int64_t K, int64_t ldw, 
   uint32_t* report = g_report.take();
   if (!report) return SDQ_ERR_CUDA;
   uint32_t* report_dev = nullptr;
-  bool ok = cudaHostGetDevicePointer((void**)&report_dev, report, 0) == cudaSuccess && device_flags();
+  bool ok = cudaHostGetDevicePointer((void**)&report_dev, report, 0) == cudaSuccess;
   if (ok && tc) {
     PackParams p;
     p.W = (const __nv_bfloat16*)W; p.N = N; p.K = K; p.ldw = ldw; p.colw = col_weight;
     p.blob = (uint8_t*)packed_buf; p.off = off; p.nonfinite = report_dev; p.gave_up = report_dev + 1; p.polls = polls;
     p.out_n = cfg->out_n;
-    p.flags = device_flags();
     p.sv4 = cfg->in_gran == SDQ_GRAN_3OF4;          // S-Vectors of 4: one outlier and two inliers per 4
     p.elem = cfg->in_gran == SDQ_GRAN_ELEM;         // element-wise 2:4: the 2 most significant non-outliers of every 4
     // dense family: inliers kept per group (8 - out_n without Stage 1; groups of 4: 3 minus the outlier, or 2 for 2:4)

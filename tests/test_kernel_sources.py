@@ -57,6 +57,12 @@ def test_a_packer_whose_wait_gives_up_stays_for_its_peers_and_says_so():
     assert re.search(r"give_back\(report\);[^{}]*gave_up \? SDQ_ERR_TIMEOUT", host[:host.index("\n}\n")])
 
 
+def test_packing_does_not_depend_on_the_device_s_status_word():
+    """a packing call reports through words of its own; the plain layout's has no wait at all"""
+    for f in ("sdq_pack.cu", "sdq_plain.cu"):
+        assert "device_flags" not in open(os.path.join(CSRC, f)).read()
+
+
 def test_packed_weights_are_ordered_behind_the_kernels_in_front():
     """a quantizer lets the next launch in (which may read packed weights at once) only behind its own wait for the previous
     one, and the grouped kernel copies nothing before its wait -- but in the calls that want the weights complete"""
