@@ -16,6 +16,8 @@
 // fetching ahead and an unpacking in front of every multiplication: 20.1, 66.0, 23.5 us; 4096 x 16384 with E4M3 scales, where 64
 // registers also let a fourth CTA onto the SM, 60.1 -> 45.7.  E4M3 scales and int8 codes multiply by a reciprocal instead of
 // dividing every element (see sdq_codec.cuh): one int8 token 14.1 -> 3.0 us (zeros took the division's slow path).
+// Products that only one of the 8-bit forms needs are formed in its branch: in front of it, int8 calls paid for E4M3's (8192 x 4096,
+// back to back, 45.6 -> 42.7 us; before scaled2 43.9) and everybody for their registers (8192 x 2048 10.2 -> 9.9, 2048 x 11008 15.9 -> 15.2).
 #include "sdq_codec.cuh"
 #include "sdq_internal.h"
 #include "sdq_layout.h"
@@ -103,9 +105,11 @@ __device__ __forceinline__ void qa_encode(const QaUnit<NQ>& u, int first, float 
     bm = max(bm, __shfl_xor_sync(0xffffffffu, bm, 1));
     if (!b32) bm = max(bm, __shfl_xor_sync(0xffffffffu, bm, 2));
     uint32_t q4[2] = {0, 0}, q8[4] = {0, 0, 0, 0};
-    float v8[16];                                        // in units of the token's 8-bit scale
+    [[maybe_unused]] float v8[16];                       // in units of the token's 8-bit scale
+    if constexpr (UE) {
 #pragma unroll
-    for (int j = 0; j < 8; ++j) scaled2(r[j], s8x, v8[2 * j], v8[2 * j + 1]);
+      for (int j = 0; j < 8; ++j) scaled2(r[j], s8x, v8[2 * j], v8[2 * j + 1]);
+    }
     if constexpr (!UE) {
       c[i] = e8m0_scale_code_bf16(bm, cfg.scale_rule == SDQ_SCALE_CEIL_NOSAT);
       const uint32_t s4x = (254u - c[i]) << 7;
@@ -132,7 +136,13 @@ __device__ __forceinline__ void qa_encode(const QaUnit<NQ>& u, int first, float 
     }
     if (!i8) {
 #pragma unroll
-      for (int j = 0; j < 4; ++j) q8[j] = e4m3x4(v8[4 * j], v8[4 * j + 1], v8[4 * j + 2], v8[4 * j + 3]);
+      for (int j = 0; j < 4; ++j) {
+        if constexpr (!UE) {                             // (here, since int8 has no use for them)
+          scaled2(r[2 * j], s8x, v8[4 * j], v8[4 * j + 1]);
+          scaled2(r[2 * j + 1], s8x, v8[4 * j + 2], v8[4 * j + 3]);
+        }
+        q8[j] = e4m3x4(v8[4 * j], v8[4 * j + 1], v8[4 * j + 2], v8[4 * j + 3]);
+      }
     } else {
 #pragma unroll
       for (int j = 0; j < 8; ++j)
