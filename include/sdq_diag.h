@@ -62,6 +62,11 @@ typedef struct {
 typedef struct { int32_t layer, row, rows, begin, end; } sdq_diag_task_t;
 sdq_status_t sdq_diag_linear_plan(int64_t M, int64_t N, int64_t K, const sdq_config_t* cfg, int workspace, int sm_count,
                                   const int* max_clusters, sdq_diag_plan_t* out, sdq_diag_task_t* tasks, int64_t cap);
+/* The shared-memory ring that the CTA pairs of such a call stage their operands in, by stage kind; all zero where the call runs another kernel.
+ * out_slots and out_slot_bytes differ from slots and slot_bytes where the outlier stages have a geometry of their own.  Errors as above. */
+typedef struct { int32_t slots, slot_bytes, out_slots, out_slot_bytes, bytes; } sdq_diag_rings_t;
+sdq_status_t sdq_diag_linear_rings(int64_t M, int64_t N, int64_t K, const sdq_config_t* cfg, int sm_count, const int* max_clusters,
+                                   sdq_diag_rings_t* out);
 sdq_status_t sdq_diag_group_plan(int n, int64_t M, const int64_t* N, const int64_t* K, int sm_count, const int* max_clusters,
                                  sdq_diag_plan_t* out, sdq_diag_task_t* segs, int64_t cap);
 

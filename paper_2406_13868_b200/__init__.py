@@ -70,7 +70,7 @@ class _ActCanon(ctypes.Structure):
 
 EXPORTS = ["sdq_packed_size", "sdq_decompose", "sdq_decompose_metric", "sdq_channel_norm", "sdq_packed_export", "sdq_packed_attach", "sdq_packed_compact_size", "sdq_packed_compact", "sdq_act_size", "sdq_quantize_act", "sdq_act_export",
            "sdq_linear", "sdq_linear_f32", "sdq_workspace_size", "sdq_workspace_init", "sdq_linear_ws", "sdq_linear_f32_ws", "sdq_linear_noalloc",
-           "sdq_linear_group", "sdq_linear_group_f32", "sdq_linear_group_x", "sdq_linear_group_x_f32", "sdq_linear_group_x_ws", "sdq_linear_group_x_f32_ws", "sdq_diag_l2_copy", "sdq_diag_wait_timeout", "sdq_diag_decompose_timeout", "sdq_diag_linear_plan", "sdq_diag_group_plan", "sdq_device_status", "sdq_status_string"]
+           "sdq_linear_group", "sdq_linear_group_f32", "sdq_linear_group_x", "sdq_linear_group_x_f32", "sdq_linear_group_x_ws", "sdq_linear_group_x_f32_ws", "sdq_diag_l2_copy", "sdq_diag_wait_timeout", "sdq_diag_decompose_timeout", "sdq_diag_linear_plan", "sdq_diag_linear_rings", "sdq_diag_group_plan", "sdq_device_status", "sdq_status_string"]
 
 _lib = None
 

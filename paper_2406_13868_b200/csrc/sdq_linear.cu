@@ -830,6 +830,12 @@ static bool diag_machine(int& sm_count, const int*& max_clusters) {
   return true;
 }
 
+static LinearParams pair_params(int64_t M, int64_t N, int64_t K, const sdq_config_t& cfg) {
+  LinearParams p = {};
+  p.M = M; p.N = N; p.K = K; p.out_n = cfg.out_n; p.b32 = cfg.in_block == 32; p.dense = is_dense_layout(cfg);
+  return p;
+}
+
 extern "C" sdq_status_t sdq_diag_linear_plan(int64_t M, int64_t N, int64_t K, const sdq_config_t* cfg, int workspace, int sm_count,
                                              const int* max_clusters, sdq_diag_plan_t* out, sdq_diag_task_t* tasks, int64_t cap)
 {
@@ -841,12 +847,22 @@ extern "C" sdq_status_t sdq_diag_linear_plan(int64_t M, int64_t N, int64_t K, co
   const LinearRoute r = linear_route(M, N, K, *cfg, workspace != 0, sm_count, max_clusters);
   out->kernel = r.kernel;
   if (r.kernel == SDQ_DIAG_FEW) { out->ksplit = r.ksplit; out->cluster = r.cluster_ks; out->token_tile = n_tile_for(M); }
-  if (r.kernel == SDQ_DIAG_PAIRS) {
-    LinearParams p = {};
-    p.M = M; p.N = N; p.K = K; p.out_n = cfg->out_n; p.b32 = cfg->in_block == 32; p.dense = is_dense_layout(*cfg);
-    pair_describe(p, sm_count, max_clusters, out, tasks, cap);
-  }
+  if (r.kernel == SDQ_DIAG_PAIRS) pair_describe(pair_params(M, N, K, *cfg), sm_count, max_clusters, out, tasks, cap);
   if (r.kernel == SDQ_DIAG_GROUP) return sdq_diag_group_plan(1, M, &N, &K, sm_count, max_clusters, out, tasks, cap);
+  return SDQ_OK;
+}
+
+extern "C" sdq_status_t sdq_diag_linear_rings(int64_t M, int64_t N, int64_t K, const sdq_config_t* cfg, int sm_count, const int* max_clusters,
+                                              sdq_diag_rings_t* out)
+{
+  sdq_diag_plan_t plan;
+  if (!out) return SDQ_ERR_INVALID_ARG;
+  const sdq_status_t st = sdq_diag_linear_plan(M, N, K, cfg, 0, sm_count, max_clusters, &plan, nullptr, 0);
+  if (st != SDQ_OK) return st;
+  *out = sdq_diag_rings_t{};
+  if (plan.kernel != SDQ_DIAG_PAIRS) return SDQ_OK;
+  if (!diag_machine(sm_count, max_clusters)) return SDQ_ERR_CUDA;
+  pair_describe_rings(pair_params(M, N, K, *cfg), sm_count, max_clusters, out);
   return SDQ_OK;
 }
 

@@ -36,6 +36,7 @@ struct LinearParams {
   int pt_tasks;                   // all tasks
   int pt_ks;                      // pairs that share the K range of a task, in a cluster of 2 pt_ks CTAs (then one task per cluster)
   int pt_acc2;                    // 1: the accumulator alternates between two sets of columns (one-unit tasks only)
+  int pt_dual;                    // 1: the outlier stages' ring has a geometry of its own
   int ksplit;            // CTAs sharing the K range of one row tile (1 = no split)
   int cluster_ks;        // > 1: those CTAs form a cluster and reduce through distributed shared memory
   uint32_t* ws_counter;  // split-K workspace: arrival counters [row tile], zero between calls
@@ -83,6 +84,7 @@ double pair_kernel_us(int64_t M, int64_t N, int64_t K, int out_n, bool b32, bool
 // clusters of k pairs of CTAs, one CTA per SM, that run at once on the current device: entries 2..4
 const int* pair_max_clusters(DeviceInfo* d);
 // what sdq_diag_linear_plan and sdq_diag_group_plan report (the parameters as for a launch, pointers unset)
+void pair_describe_rings(LinearParams p, int sm_count, const int* max_clusters, sdq_diag_rings_t* out);
 void pair_describe(LinearParams p, int sm_count, const int* max_clusters, sdq_diag_plan_t* out, sdq_diag_task_t* tasks, int64_t cap);
 void group_describe(GroupParams p, int sm_count, const int* max_clusters, sdq_diag_plan_t* out, sdq_diag_task_t* segs, int64_t cap);
 cudaError_t launch_linear_pair(LinearParams p, bool f32_out, DeviceInfo* d, cudaStream_t stream);

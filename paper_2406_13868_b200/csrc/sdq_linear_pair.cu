@@ -82,9 +82,12 @@ __host__ __device__ constexpr int pair_slots(uint32_t slot) {      // released t
 // outlier stages use the ring in another geometry: | outlier record, row-scale atom | x units | codes | two token-scale atoms |, six
 // slots instead of four (two units x 192 tokens), eight instead of six (one unit x 256).  The first stage in such a slot waits for the
 // inlier slots that had its bytes.  1500 x 11008 -> 4096, 1:8 + 6:8: 71.5 -> 61.9 us, 1500 x 4096 -> 4096 29.7 -> 26.3, 300 x 8704 -> 10880 53.7
-// -> 46.3.  With several tasks per pair the ring would have to turn back for each: 8192 x 2560 -> 2560 57 -> 63, long K the same (the clock
-// is lower there and the tensor pipe the bound).  From K = 2048 on, where the turn costs less than it gives: K 2048 19.15 -> 17.98, 1024
-// 14.15 -> 14.02, 1280 15.2 -> 15.6, 768 13.0 -> 13.3 (1500 tokens).
+// -> 46.3 (chains of calls, burst clocks).  With several tasks per pair the ring would have to turn back for each: 8192 x 2560 -> 2560 57 ->
+// 63, long K the same (the clock is lower there and the tensor pipe the bound).  A turn costs about 1.2 us, the slots give what the task's
+// length makes of them.  Two-unit tasks, of four slots that were too few, from K = 2048 on: 360 x 2048 -> 14592 19.8 -> 18.4, 329 x 2304 -> 11392 18.0
+// -> 17.4; below, 1500 tokens, 1024 14.15 -> 14.02, 1280 15.2 -> 15.6.  One-unit tasks, of six that nearly did, from K = 6144 on: 692 x 6144 ->
+// 4864 24.9 -> 23.9, 512 x 7168 -> 6528 30.9 -> 28.8, 498 x 7936 -> 6912 35.9 -> 35.0; below, 387 x 2048 -> 8192 12.7 -> 13.8, 423 x 3584 -> 6272
+// 17.1 -> 18.2, 243 x 4864 -> 9728 22.5 -> 23.0, 604 x 5376 -> 4864 21.4 -> 21.7.
 __host__ __device__ constexpr uint32_t pair_out_slot_bytes(int units, int T) {
   return (uint32_t)units * (WO_BYTES + SF_ATOM_BYTES) + (uint32_t)T * 64u + 2u * SF_ATOM_BYTES;
 }
@@ -136,9 +139,11 @@ sdq_linear_pair_kernel(const __grid_constant__ LinearParams p)
   const bool acc2 = FORM == PAIR_FLEX && p.pt_acc2;
   // the ring of the outlier stages: the same one, or (DUAL) the second geometry
   static_assert(!DUAL || (DENSE && FORM != PAIR_FLEX));
+  static_assert(PAIR_MAX_SLOTS <= PAIR_BARS && PAIR_BARS <= 29);   // (lanes 29 to 31 of the warp that sets the barriers up have others)
   constexpr int UNITS = FORM == PAIR_TWO ? 2 : 1;
   constexpr uint32_t O_UNIT = DUAL ? WO_BYTES + SF_ATOM_BYTES : G::WIB;     // from one unit's record to the next
   constexpr uint32_t O_FIXED = pair_out_slot_bytes(UNITS, (int)FIXED_T);
+  static_assert(!DUAL || pair_slots(FIXED_SLOT) + pair_slots(O_FIXED) <= PAIR_BARS);
   const uint32_t O_SLOT = DUAL ? O_FIXED : SLOT, O_NSLOT = DUAL ? (uint32_t)pair_slots(O_FIXED) : NSLOT;
   const uint32_t O_B = DUAL ? UNITS * O_UNIT : SL_B, O_SF = O_B + TMAX * 64u;
   uint8_t* stg_base = sm + (FORM == PAIR_FLEX ? NSLOT * SLOT : pair_ring_bytes(FIXED_SLOT, pair_slots(FIXED_SLOT), DUAL, UNITS, (int)FIXED_T));
@@ -642,9 +647,6 @@ sdq_linear_pair_kernel(const __grid_constant__ LinearParams p)
   if (warp == 1) ptx::tmem_dealloc_pair(tmem, 512);
 }
 
-static bool pair_dual(const LinearParams& p, int form, int pairs) {
-  return p.dense && p.out_n > 0 && form != PAIR_FLEX && p.pt_tasks <= pairs && p.K >= 8 * K2;
-}
 template <bool F32_OUT, bool B32, bool DENSE, int FORM, bool DUAL = false>
 static cudaError_t launch_form(const LinearParams& p, int pairs, cudaStream_t stream, std::atomic<uint32_t>* attr_mask)
 {
@@ -675,7 +677,7 @@ template <bool F32_OUT, bool B32, bool DENSE>
 static cudaError_t launch_one(const LinearParams& p, int form, int pairs, cudaStream_t stream, std::atomic<uint32_t>* attr_mask)
 {
   if constexpr (DENSE)
-    if (pair_dual(p, form, pairs))
+    if (p.pt_dual)
       return form == PAIR_TWO ? launch_form<F32_OUT, B32, DENSE, PAIR_TWO, true>(p, pairs, stream, attr_mask)
                               : launch_form<F32_OUT, B32, DENSE, PAIR_FULL, true>(p, pairs, stream, attr_mask);
   if (form == PAIR_TWO) return launch_form<F32_OUT, B32, DENSE, PAIR_TWO>(p, pairs, stream, attr_mask);
@@ -791,6 +793,11 @@ const int* pair_max_clusters(DeviceInfo* d)
 double pair_kernel_us(int64_t M, int64_t N, int64_t K, int out_n, bool b32, bool dense, int sm_count, const int* max_clusters)
 { return pair_best(M, N, K, out_n, b32, dense, sm_count, max_clusters).us; }
 
+// do the outlier stages of a call have a ring geometry of their own (see pair_out_slot_bytes)?
+static bool pair_dual(const LinearParams& p, const PairPlan& best, int pairs) {
+  return p.dense && p.out_n > 0 && best.form != PAIR_FLEX && best.tasks <= pairs && p.K >= (best.form == PAIR_TWO ? 8 : 24) * K2;
+}
+
 // the plan's numbers into the launch parameters (p.M, N, K and the format are there); returns the pairs to launch
 static int pair_apply(LinearParams& p, const PairPlan& best, int sm_count)
 {
@@ -801,7 +808,8 @@ static int pair_apply(LinearParams& p, const PairPlan& best, int sm_count)
   p.pt_doubles = best.doubles; p.pt_split = best.split; p.pt_tasks = best.tasks; p.pt_acc2 = best.acc2; p.pt_ks = best.ks;
   p.slot_bytes = (int)pair_slot_bytes(p.dense ? 17408u : (p.b32 ? 11264u : 10752u), s32, best.form == PAIR_TWO ? 2 : 1, T);
   p.nslot = pair_slots((uint32_t)p.slot_bytes);
-  p.ring_bytes = (int)pair_ring_bytes((uint32_t)p.slot_bytes, p.nslot, pair_dual(p, best.form, sm_count / 2), best.form == PAIR_TWO ? 2 : 1, T);
+  p.pt_dual = pair_dual(p, best, sm_count / 2);
+  p.ring_bytes = (int)pair_ring_bytes((uint32_t)p.slot_bytes, p.nslot, p.pt_dual != 0, best.form == PAIR_TWO ? 2 : 1, T);
   return p.pt_tasks < sm_count / 2 || best.ks > 1 ? p.pt_tasks : sm_count / 2;
 }
 
@@ -815,6 +823,16 @@ void pair_describe(LinearParams p, int sm_count, const int* max_clusters, sdq_di
     const PairTask t = best.form == PAIR_TWO ? pair_task<PAIR_TWO>(p, (int)i) : pair_task<PAIR_FLEX>(p, (int)i);
     tasks[i] = {0, t.u0, t.nu, pair_group0(p, t.mt), pair_group0(p, t.mt + 1)};
   }
+}
+
+void pair_describe_rings(LinearParams p, int sm_count, const int* max_clusters, sdq_diag_rings_t* out)
+{
+  const PairPlan best = pair_best(p.M, p.N, p.K, p.out_n, p.b32 != 0, p.dense != 0, sm_count, max_clusters);
+  (void)pair_apply(p, best, sm_count);
+  const uint32_t o = pair_out_slot_bytes(best.form == PAIR_TWO ? 2 : 1, p.n_tile);
+  out->slots = p.nslot; out->slot_bytes = p.slot_bytes;
+  out->out_slots = p.pt_dual ? pair_slots(o) : p.nslot; out->out_slot_bytes = p.pt_dual ? (int)o : p.slot_bytes;
+  out->bytes = p.ring_bytes;
 }
 
 cudaError_t launch_linear_pair(LinearParams p, bool f32_out, DeviceInfo* d, cudaStream_t stream)

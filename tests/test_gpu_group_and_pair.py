@@ -9,6 +9,7 @@ import torch
 import sdq_synth
 from oracle import sdq_oracle as so
 from tests.test_gpu_parity import ocfg, run_case, sdq, y_close
+from tests.test_plans import linear_plan, linear_rings
 
 pytestmark = pytest.mark.gpu
 
@@ -849,25 +850,32 @@ def test_group_x_needs_no_memory():
     assert e.value.code == 4
 
 
-@pytest.mark.parametrize("M,N,K,out_n,gran", [
-    (600, 5120, 2048, 1, so.GRAN_DENSE),      # one-unit tasks, an even number of inlier stages, each slot used once or twice
-    (600, 5120, 2304, 1, so.gran_keep(7)),    # an odd number: the last pair of inlier slots is half used
-    (2900, 1152, 2816, 2, so.GRAN_DENSE),     # an odd number of row tiles, two outliers per S-Vector
-    (1100, 4096, 2304, 1, so.gran_keep(7)),   # two-unit tasks, odd
-    (1300, 3200, 2048, 1, so.GRAN_DENSE),     # two-unit tasks and the odd unit of every token tile, even
-    (4001, 1152, 3072, 1, so.GRAN_ELEM),      # the same, half of the last unit is padding
+@pytest.mark.parametrize("M,N,K,out_n,gran,own", [
+    (600, 5120, 6144, 1, so.GRAN_DENSE, True),        # one-unit tasks, an even number of inlier stages
+    (600, 5120, 6400, 1, so.gran_keep(7), True),      # an odd number: the last pair of inlier slots is half used
+    (2900, 1152, 6912, 2, so.GRAN_DENSE, True),       # an odd number of row tiles, two outliers per S-Vector
+    (1100, 4096, 2304, 1, so.gran_keep(7), True),     # two-unit tasks, odd
+    (1300, 3200, 2048, 1, so.GRAN_DENSE, True),       # two-unit tasks and the odd unit of every token tile, even
+    (4001, 1152, 3072, 1, so.GRAN_ELEM, True),        # the same, half of the last unit is padding
+    (600, 5120, 2048, 1, so.GRAN_DENSE, False),       # one-unit tasks of few stages keep one geometry
+    (600, 5120, 2304, 1, so.gran_keep(7), False),
+    (2900, 1152, 2816, 2, so.GRAN_DENSE, False),
 ])
-def test_outlier_stages_in_a_ring_geometry_of_their_own(M, N, K, out_n, gran):
-    """dense inliers, one task per pair of CTAs: sampled tokens against the oracle, bf16 = RNE of the fp32 result, the same bits again"""
+def test_outlier_stages_in_a_ring_geometry_of_their_own(M, N, K, out_n, gran, own):
+    """dense inliers, one task per pair of CTAs: sampled tokens of every token tile against the oracle, bf16 = RNE of the fp32 result, the same bits again"""
     m = sdq()
     cfg = m.Config(out_n, gran, 32, 0)
+    here = (ctypes.c_int(0), None)
+    rings, tasks = linear_rings(M, N, K, cfg, here), linear_plan(M, N, K, cfg, here)[1]
+    assert (rings.out_slots > rings.slots) == own
     W, X = sdq_synth.make_weight(N, K, 71), sdq_synth.make_act(M, K, 72)
     p, xq = m.sdq_decompose(W.cuda(), cfg), m.sdq_quantize_act(X.cuda(), cfg)
     y = m.sdq_linear(xq, p, f32=True)
     y16, again = m.sdq_linear(xq, p), m.sdq_linear(xq, p, f32=True)
     assert m.device_status() == 0
     assert torch.equal(y16, y.to(torch.bfloat16)) and torch.equal(y, again)
-    toks = sorted({0, 95, 96, 191, 192, 255, 256, M // 2, M - 33, M - 1})
+    tiles = {(32 * g0, min(32 * g1, M)) for g0, g1 in tasks[:, 3:5]}       # the first, a middle and the last token of each
+    toks = sorted({t for a, b in tiles for t in (a, (a + b) // 2, b - 1)})
     oc = ocfg(out_n, 0, 32, gran)
     yref = so.linear(so.quantize_act(sdq_synth.bf16_bits(X[toks]), oc), so.decompose(sdq_synth.bf16_bits(W), oc))
     d, tol = y_close(y[toks].cpu().numpy(), yref)

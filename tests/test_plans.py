@@ -41,6 +41,17 @@ def group_plan(M, shapes, on):
     return plan, segs[:plan.tasks]
 
 
+class Rings(ctypes.Structure):
+    _fields_ = [(n, ctypes.c_int32) for n in ("slots", "slot_bytes", "out_slots", "out_slot_bytes", "bytes")]
+
+
+def linear_rings(M, N, K, cfg, on):
+    m.build()
+    r = Rings()
+    assert m.lib().sdq_diag_linear_rings(i64(M), i64(N), i64(K), ctypes.byref(cfg), *on, ctypes.byref(r)) == 0
+    return r
+
+
 def cover_pairs(plan, tasks, M, N):
     units, groups = -(-N // 256), -(-M // 32)
     seen = np.zeros((units, groups), np.int32)
@@ -134,6 +145,28 @@ GROUPS = [
 ]
 
 
+# dense inliers, one task per pair of CTAs -> form, do the outlier stages have a ring geometry of their own (slots: inliers', outliers')
+KEEP7, DENSE2, ELEM = m.Config(1, m.gran_keep(7), 32), m.Config(2, m.GRAN_DENSE, 32), m.Config(1, m.GRAN_ELEM, 32)
+RINGS = [
+    (600, 5120, 6144, DENSE, FULL, (6, 8)),
+    (600, 5120, 6400, KEEP7, FULL, (6, 8)),
+    (2900, 1152, 6912, DENSE2, FULL, (6, 8)),
+    (1100, 4096, 2304, KEEP7, TWO, (4, 6)),
+    (1300, 3200, 2048, DENSE, TWO, (4, 6)),
+    (4001, 1152, 3072, ELEM, TWO, (4, 6)),
+    (1500, 4096, 11008, KEEP7, TWO, (4, 6)),
+    # one-unit tasks with few stages, several tasks per pair, less than eight inlier stages, no outliers
+    (600, 5120, 2048, DENSE, FULL, (6, 6)),
+    (600, 5120, 2304, KEEP7, FULL, (6, 6)),
+    (2900, 1152, 2816, DENSE2, FULL, (6, 6)),
+    (387, 8192, 2048, ELEM, FULL, (6, 6)),
+    (423, 6272, 3584, DENSE, FULL, (6, 6)),
+    (4096, 4096, 16384, DENSE, FULL, (6, 6)),
+    (2048, 2560, 1280, DENSE, TWO, (4, 4)),
+    (600, 8192, 11008, m.Config(0, m.GRAN_DENSE, 32), TWO, (4, 4)),
+]
+
+
 def runs(plan, want):
     for name, value in want.items():
         got = plan.ksplit > 1 if name == "split" else getattr(plan, name)
@@ -143,6 +176,16 @@ def runs(plan, want):
 @pytest.mark.parametrize("M,N,K,cfg,want", FORMS)
 def test_shapes_take_the_forms_they_are_tested_for(M, N, K, cfg, want):
     runs(linear_plan(M, N, K, cfg, machine(*B200))[0], want)
+
+
+@pytest.mark.parametrize("M,N,K,cfg,form,slots", RINGS)
+def test_ring_geometries(M, N, K, cfg, form, slots):
+    on = machine(*B200)
+    r = linear_rings(M, N, K, cfg, on)
+    runs(linear_plan(M, N, K, cfg, on)[0], dict(kernel=PAIRS, form=form))
+    assert (r.slots, r.out_slots) == slots
+    assert r.bytes == max(r.slots * r.slot_bytes, r.out_slots * r.out_slot_bytes) <= 227 * 1024
+    assert (r.out_slot_bytes < r.slot_bytes) == (r.out_slots > r.slots)
 
 
 @pytest.mark.parametrize("M,shapes,want", GROUPS)
@@ -173,6 +216,10 @@ def test_the_device_at_hand_takes_the_same_forms():
     for M, N, K, cfg, want in FORMS:
         plan, tasks = linear_plan(M, N, K, cfg, here)
         runs(plan, want)
+    for M, N, K, cfg, form, slots in RINGS:
+        r = linear_rings(M, N, K, cfg, here)
+        runs(linear_plan(M, N, K, cfg, here)[0], dict(kernel=PAIRS, form=form))
+        assert (r.slots, r.out_slots) == slots
     for M, shapes, want in GROUPS:
         plan, segs = group_plan(M, shapes, here)
         runs(plan, want)
