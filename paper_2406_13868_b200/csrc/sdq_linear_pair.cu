@@ -688,17 +688,20 @@ static cudaError_t launch_one(const LinearParams& p, int form, int pairs, cudaSt
 // How a call is cut into tasks: token tiles, one or two units per task, pairs per task (K split).
 struct PairPlan { int form, T, mt, acc2, doubles, split, tasks, ks; double us; };
 
-// The plan for `mt` token tiles with one- or two-unit tasks; false if tensor memory does not hold it.  Times in us, fitted to
-// measurements (4096 x 4096 to 16384 x 4096, 130 to 8192 tokens): a stage of one unit takes 0.158 (the chain of barrier test
+// The plan for `mt` token tiles with one-unit tasks, two-unit tasks or K over two pairs in tiles too wide to alternate; false if tensor
+// memory does not hold it or there is none.  Times in us, fitted to measurements (4096 x 4096 to 16384 x 4096, 130 to 8192 tokens): a stage of one unit takes 0.158 (the chain of barrier test
 // and issue) or 10.5 ns per KB that an SM stages (12.5 with every SM busy, 11.8 with compile-time geometry), one of two units 0.10 + 0.00188 T (the tensor pipe at the clock it keeps
 // under load) or 13.5 ns per KB; a call 4.2 and 0.02 per pair it uses; a task ends with a drain of its accumulator that the next one waits for unless the accumulator alternates.
-static bool pair_plan(int groups, int mt, int units, int T1, int T2, bool dbl, uint32_t wib, bool s32, bool dense, int pairs, const int* max_clusters, PairPlan* out)
+enum { PLAN_ONE, PLAN_TWO, PLAN_WIDE, PLAN_KINDS };
+static bool pair_plan(int groups, int mt, int units, int T1, int T2, int kind, uint32_t wib, bool s32, bool dense, int pairs, const int* max_clusters, PairPlan* out)
 {
+  const bool dbl = kind == PLAN_TWO;
   PairPlan q;
   const int T = 32 * ((groups + mt - 1) / mt), cols = s32 ? (int)PairGeom<true, false>::COLS : (int)PairGeom<false, false>::COLS;
   q.T = T; q.mt = mt; q.ks = 1;
   if (T > pair_tmax(dbl ? PAIR_TWO : PAIR_FULL, s32)) return false;
   q.acc2 = !dbl && 2 * T + cols <= 512;
+  if (kind == PLAN_WIDE && (q.acc2 || units * mt > max_clusters[2] || T2 < 2)) return false;
   q.form = dbl ? PAIR_TWO : (q.acc2 ? PAIR_FLEX : PAIR_FULL);
   const double avgT = 32.0 * groups / mt;
   const double kb1 = !dbl && units * mt < pairs ? 0.0105e-3 : (q.acc2 ? 0.0125e-3 : 0.0118e-3);
@@ -720,10 +723,13 @@ static bool pair_plan(int groups, int mt, int units, int T1, int T2, bool dbl, u
     // count as much as the weights', and tiles of 256 tokens stage a quarter less than twice as many of 128: 500 x 4096 -> 4096 14.73 ->
     // 14.20 us, 512 x 8192 -> 4096 23.3 -> 19.3, with E4M3 scales 442 x 8704 -> 4096 25.3 -> 20.4; over three pairs 256 x 4096 -> 4096
     // would go from 12.1 to 13.7.  Adding two items of a reduction at a time was slower by 1 to 5 %)
-    for (int k = 2; k <= (q.acc2 ? 4 : 2); ++k) {
-      const double red = q.acc2 ? 1.0 + 0.01 * avgT : 2.0;
-      if (q.tasks <= max_clusters[k] && k <= T2 && c1 / k + red < us) { us = c1 / k + red; q.ks = k; q.form = PAIR_FLEX; }
+    if (kind == PLAN_WIDE) {
+      if (c1 / 2 + 2.0 >= us) return false;
+      us = c1 / 2 + 2.0; q.ks = 2; q.form = PAIR_FLEX;
     }
+    const double red = 1.0 + 0.01 * avgT;
+    for (int k = 2; k <= 4 && q.acc2; ++k)
+      if (q.tasks <= max_clusters[k] && k <= T2 && c1 / k + red < us) { us = c1 / k + red; q.ks = k; }
   } else {
     const int D = (units / 2) * mt, odd = (units & 1) * mt;
     const int full = D / pairs * pairs, left = D - full;
@@ -749,16 +755,23 @@ static bool pair_plan(int groups, int mt, int units, int T1, int T2, bool dbl, u
 static PairPlan pair_best(int64_t M, int64_t N, int64_t K, int out_n, bool b32, bool dense, int sm_count, const int* max_clusters)
 {
   const int units = (int)((N + 2 * TILE_ROWS - 1) / (2 * TILE_ROWS)), groups = (int)((M + 31) / 32);
-  PairPlan best, q;
-  best.us = -1.0;
+  PairPlan best, wide, q;
+  best.us = wide.us = -1.0;
   // from tiles of 256 tokens down to tiles of 128, or of 32 where the call is small (up to 1024 tokens)
   const int mt0 = (groups + 7) / 8, mt1 = groups <= 32 ? groups : 2 * mt0;
   for (int mt = mt0; mt <= mt1; ++mt)
-    for (int d = 0; d < 2; ++d)
-      if (pair_plan(groups, mt, units, out_n ? (int)(K / K1) : 0, (int)(K / K2), d != 0, dense ? 17408u : (b32 ? 11264u : 10752u), b32 || dense, dense, sm_count / 2,
-                    max_clusters, &q) && (best.us < 0 || q.us < best.us))
-        best = q;
-  return best;
+    for (int kind = 0; kind < PLAN_KINDS; ++kind) {
+      if (!pair_plan(groups, mt, units, out_n ? (int)(K / K1) : 0, (int)(K / K2), kind, dense ? 17408u : (b32 ? 11264u : 10752u), b32 || dense, dense, sm_count / 2,
+                     max_clusters, &q)) continue;
+      PairPlan& b = kind == PLAN_WIDE ? wide : best;
+      if (b.us < 0 || q.us < b.us) b = q;
+    }
+  // Dense inliers: alternating tiles of 128 tokens and more take 0.4 to 0.9 us less than their price, and without outliers, where all of a
+  // task's stages are of the kind that is priced too high, 1 to 2.  Chosen by price alone, wide tiles made 252 x 7168 -> 7808 without outliers
+  // 13.5 us instead of 12.0, 236 x 11520 -> 4864 15.6 instead of 14.6, with them 1259 x 2560 -> 1024 11.8 instead of 11.3.  What they still win: 919 x 5888
+  // -> 1920 19.2 -> 17.6, 211 x 9216 -> 7424 28.3 -> 22.8, against tiles of 96 tokens 450 x 4608 -> 2944 15.8 -> 15.0
+  const double margin = !dense || best.form != PAIR_FLEX ? 0.0 : (!out_n ? 1.5 : (best.T > 96 ? 0.6 : 0.0));
+  return wide.us >= 0 && (best.us < 0 || wide.us + margin < best.us) ? wide : best;
 }
 
 // largest grids, in clusters of 4, 6 and 8 CTAs with one CTA per SM, that run at once on the current device: [pairs per cluster]

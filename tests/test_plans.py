@@ -237,3 +237,25 @@ def test_wide_tiles_are_split_over_two_pairs_at_most():
         if plan.ksplit > 1 and plan.token_tile > 224:
             assert plan.ksplit == 2 and not plan.alternate and plan.tasks <= B200[1][0]
     assert (True, 2) in seen and (False, 1) in seen
+
+
+@pytest.mark.parametrize("M,N,K,cfg,wide", [
+    (240, 6528, 7680, m.Config(0, m.GRAN_DENSE, 32), False),
+    (1068, 1408, 7424, m.Config(0, m.GRAN_DENSE, 32), False),
+    (1259, 1024, 2560, KEEP7, False),
+    (1711, 1024, 2816, DENSE, False),
+    (1264, 1536, 3328, DENSE2, False),
+    (211, 5376, 14336, m.Config(0, m.GRAN_DENSE, 32), True),
+    (252, 7808, 7168, m.Config(0, m.GRAN_DENSE, 32), False),
+    (236, 4864, 11520, m.Config(0, m.GRAN_DENSE, 32), False),
+    (1118, 1280, 4608, ELEM, False),
+    (450, 2944, 4608, DENSE, True),
+    (919, 1920, 5888, DENSE, True),
+    (211, 7424, 9216, ELEM, True),
+    (1249, 1280, 3584, UE, True),
+    (500, 4096, 4096, PAIR, True),
+])
+def test_which_wide_tiles_are_split(M, N, K, cfg, wide):
+    """dense inliers: narrower tiles, with alternating accumulators, where these are the faster"""
+    plan, _ = linear_plan(M, N, K, cfg, machine(*B200))
+    assert (plan.ksplit == 2 and not plan.alternate) == wide
