@@ -384,12 +384,17 @@ pack_kernel(const PackParams p, const BlobHeader hdr)
   // collected (4096 x 11008, 1:8 + 6:8: 67 and 98).  Dense by magnitude: the outliers, if the most significant, hold the row's
   // largest magnitude, this pass has nothing to choose and leaves it to the second.
   constexpr bool CHOSEN = !DENSE || WGT;
+  // trips of either pass' loop in a row: one, since straight-line code waits for instructions; four where the row scales come from a launch
+  // of their own, the inliers are pair-wise and the choices, made by magnitude or of two outliers or none, short (28672 x 8192, all in
+  // a row, rolled -> so: 1:8 250 -> 248 us, E4M3 scales without outliers 189 -> 183, 2:8 with channel weights 607 -> 589; the others would lose: 1:8 + 6:8
+  // 236 -> 259, 1:8 with channel weights 361 -> 370)
+  constexpr int UNROLL = FUSED || DENSE || (WGT && OUTN == 1) ? 1 : 4;
   [[maybe_unused]] uint32_t c_o0[2] = {0, 0}, c_o1[2] = {0, 0}, c_nib[2] = {0, 0}, c_gone[4] = {0, 0, 0, 0};
   uint32_t all2 = 0, omax = 0, imax = 0, bad = 0;        // all2, imax: packed running maxima
   if constexpr (CHOSEN) {
     const bool look_at_all = WGT || OUTN == 0 || p.order_mask;    // for non-finite values: otherwise they are outliers
     if (on) {
-#pragma unroll 1
+#pragma unroll (UNROLL)
       for (int t = 0; t < 4; ++t) {                      // four S-Vectors a trip
         uint32_t n_o0 = 0, n_o1 = 0, n_nib = 0, n_gone = 0;
 #pragma unroll
@@ -490,9 +495,9 @@ pack_kernel(const PackParams p, const BlobHeader hdr)
   uint32_t codes[4] = {0, 0, 0, 0}, sels[4] = {0, 0, 0, 0}, metas[4] = {0, 0, 0, 0};   // outlier bytes of the 128 K
   uint32_t kept[16];                                     // pair-wise inliers of a Q-Vector of 64 K, outlier positions zeroed
   uint32_t qmax2 = 0;                                    // packed running maximum of the Q-Vector
-  // (rolled up, like the first pass: as straight-line code the two took a fifth of the warps' time in waits for instructions)
+  // (like the first pass: as straight-line code the two took a fifth of the warps' time in waits for instructions)
   constexpr int TRIP = DENSE ? 1 : 2;                    // blocks a trip (pair-wise: a Q-Vector of 64 K)
-#pragma unroll 1
+#pragma unroll (UNROLL)
   for (int b0 = 0; b0 < 4; b0 += TRIP) {
    [[maybe_unused]] const uint32_t w_o0 = b0 < 2 ? c_o0[0] : c_o0[1], w_o1 = b0 < 2 ? c_o1[0] : c_o1[1];
 #pragma unroll
