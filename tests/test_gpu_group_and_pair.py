@@ -886,6 +886,10 @@ def test_outlier_stages_in_a_ring_geometry_of_their_own(M, N, K, out_n, gran, ow
     (497, 3968, 4096, (1, so.GRAN_PAIR, 64, 0)),      # two tiles of 256 tokens, odd row tiles
     (450, 3840, 4352, (1, so.GRAN_PAIR, 32, 2)),      # E4M3 scales, K in unequal halves
     (512, 4096, 4096, (1, so.GRAN_DENSE, 32, 0)),
+    (213, 6656, 5632, (1, so.GRAN_DENSE, 32, 0)),     # one tile of 224: too wide to alternate where a scale covers 32 K
+    (220, 5120, 5120, (1, so.GRAN_PAIR, 32, 2)),
 ])
 def test_wide_tiles_with_k_over_two_pairs(M, N, K, cfg_args):
+    plan = linear_plan(M, N, K, sdq().Config(*cfg_args), (ctypes.c_int(0), None))[0]
+    assert plan.ksplit == 2 and not plan.alternate
     test_cta_pair_task_forms(M, N, K, cfg_args)

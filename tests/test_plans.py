@@ -64,6 +64,7 @@ def cover_pairs(plan, tasks, M, N):
         assert plan.doubles == plan.halves == 0
     if plan.ksplit > 1:                                   # one task per cluster, all clusters at once
         assert plan.form == FLEX and plan.ctas == plan.cluster * plan.tasks and plan.cluster == 2 * plan.ksplit
+        assert plan.alternate or plan.ksplit == 2         # tiles too wide to alternate are shared by two pairs at most
 
 
 def cover_group(plan, segs, shapes):
@@ -124,6 +125,11 @@ FORMS = [
     (64, 2176, 4096, m.Config(2), dict(kernel=FEW, split=True)),
     (130, 128, 256, NONE, dict(kernel=PAIRS, form=FLEX, split=False)),
     (3371, 2688, 2048, UE, dict(kernel=PAIRS, form=TWO)),
+    (497, 3968, 4096, PAIR, dict(kernel=PAIRS, form=FLEX, split=True, ksplit=2, alternate=False, token_tile=256)),
+    (450, 3840, 4352, UE, dict(kernel=PAIRS, form=FLEX, split=True, ksplit=2, alternate=False, token_tile=256)),
+    (512, 4096, 4096, DENSE, dict(kernel=PAIRS, form=FLEX, split=True, ksplit=2, alternate=False, token_tile=256)),
+    (213, 6656, 5632, DENSE, dict(kernel=PAIRS, form=FLEX, split=True, ksplit=2, alternate=False, token_tile=224)),
+    (220, 5120, 5120, UE, dict(kernel=PAIRS, form=FLEX, split=True, ksplit=2, alternate=False, token_tile=224)),
     (1, 4096, 4096, PAIR, dict(kernel=GROUP, split=True, rounds=False)),
     (17, 4224, 4096, PAIR, dict(kernel=GROUP, split=True, rounds=False)),
     (5, 8192, 8192, PAIR, dict(kernel=GROUP, split=True, rounds=False)),
