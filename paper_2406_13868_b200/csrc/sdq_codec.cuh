@@ -101,7 +101,7 @@ __device__ __forceinline__ float ue4m3_scale_inverse(uint32_t c) {
 }
 
 // two packed bf16 times a power of two (the bits of a bf16), as floats, in one instruction each (unpacking and multiplying take
-// three a pair more: 2048 x 11008 18.5 -> 18.0 us).  Rounded once, as the fp32 product is; the sum's -0 keeps the sign of zeros
+// two a pair more: 2048 x 11008 18.5 -> 18.0 us).  Rounded once, as the fp32 product is; the sum's -0 keeps the sign of zeros
 __device__ __forceinline__ void scaled2(uint32_t x, uint32_t s, float& lo, float& hi) {
   asm("{\n.reg .b16 l, h, t;\n"
       "mov.b32 {l, h}, %2;\n"

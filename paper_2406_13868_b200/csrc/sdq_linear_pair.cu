@@ -18,7 +18,8 @@
 //
 // Sustained (0.3 s of calls), one unit x 256 tokens before -> now: 2048 x 4096 -> 11008 80.2 -> 77.5 us, 8192 x 11008 -> 4096
 // 278 -> 259 us, with E4M3 scales 4096 x 16384 -> 4096 265 -> 232 us, dense inliers 1500 x 11008 -> 4096 90 -> 78 us; K over
-// several pairs 130 x 16384 -> 4096 27 -> 21 us, 400 x 16384 -> 1024 35 -> 17 us; 500 x 4096 -> 4096 21.1 -> 13.9 us.
+// several pairs 130 x 16384 -> 4096 27 -> 21 us, 400 x 16384 -> 1024 35 -> 17 us.  A chain of calls at burst clocks: 500 x 4096 -> 4096 21.1 ->
+// 13.9 us (K over pairs 14.9, wide tiles of it too 14.3, the set-up below 13.9).
 //
 // Few tasks (narrow matrices, few tokens): a task is one chain of stages at ~0.16 us each however few tokens it has, so its K
 // range is split over 2 to 4 pairs of a larger cluster; their fp32 partial tiles meet in shared memory and every CTA adds
@@ -168,8 +169,9 @@ sdq_linear_pair_kernel(const __grid_constant__ LinearParams p)
 
   // Set-up.  The producers need nothing but this CTA's barriers for the ring's first lap, so they start on those while tensor memory
   // is being allocated and the other CTAs of the cluster are waited for (by everybody else, before anything remote).  The fence behind
-  // the barriers releases them; only warp 1's allocation has to be released besides.  Chains of calls, everybody behind one barrier before ->
-  // now: 40 x 4096 -> 4096 9.56 -> 9.08 us, 500 x 4096 -> 4096 14.73 -> 13.9, 1000 17.28 -> 16.4, 130 x 16384 -> 4096 20.38 -> 20.05.
+  // the barriers releases them; only warp 1's allocation has to be released besides.  Everybody behind one barrier -> so, chains of calls at
+  // burst clocks: 40 x 4096 -> 4096 9.48 -> 9.15 us, 500 14.3 -> 13.9, 1000 17.06 -> 16.80, 100 x 4096 -> 11008 14.47 -> 14.24; with a quantizer in front of each
+  // 11.3 -> 11.1, 18.2 -> 18.0, 21.8 -> 21.3, but 16.56 -> 16.65: 60 to 230 tokens against 43 units lose half a percent
   const bool producer = warp == 0 || warp == 2 || warp == 3;
   if (warp == 0) {
     if (lane == 0) ptx::griddep_launch_dependents();   // (first of all: behind the barriers' set-up a pass of 100 tokens took 17.82 instead of 17.72 us)
@@ -275,7 +277,9 @@ sdq_linear_pair_kernel(const __grid_constant__ LinearParams p)
           }
         }, [&](int k, uint8_t* st, uint64_t* bar) {
           // half a lap of weights is under way when the activations come; the other half would only stand in the way of what the previous
-          // kernel, as a rule the quantizer, still has to load
+          // kernel, as a rule the quantizer, still has to load.  No weights / half a lap / a lap / no limit, behind a quantizer: 150 x 4096 -> 16384
+          // 19.01, 18.96, 19.07, 19.15 us, 300 x 4096 -> 11008 23.8, 23.6, 24.0, 23.4, 1000 x 11008 -> 4096 53.4, 52.8, 53.3, 52.7; behind a product: 60 x
+          // 4096 -> 11008 13.47, 13.48, 13.56, 13.56, 260 19.38, 19.15, 19.09, 19.05, 1000 x 4096 -> 4096 16.90, 16.80, 16.80, 16.67
           if (early-- == 0) ptx::griddep_wait();
           const bool two = FORM == PAIR_TWO && nu == 2;
           if (k < NI) {

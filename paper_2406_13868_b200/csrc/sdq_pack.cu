@@ -9,7 +9,7 @@
 // through distributed shared memory.  Longer rows: `row_scale_kernel` finds it and the same kernel follows without clusters.
 //
 // What bounds it: the integer pipe (selections on packed keys instead of index loops took it from ~350 instructions per S-Vector
-// over two passes to 138), DRAM is at 30 %.  11008 x 4096, 1:8 + pair-wise 4:8: 189 us as one kernel with a CTA per row and a
+// over two passes to some 140), DRAM is at 30 %.  11008 x 4096, 1:8 + pair-wise 4:8: 189 us as one kernel with a CTA per row and a
 // thread per S-Vector scattering bytes -> 20 + 42 us with the row scales in a launch of their own -> 49 us -> 42 us with the
 // pairs picked by two minima and two maxima instead of six comparisons and the choices kept from the first pass.  4096 x 11008,
 // 1:8 + 6:8 with channel weights: 98 us choosing in both passes -> 67.  Loops of four S-Vectors (first pass) and of one Q-Vector
@@ -499,158 +499,158 @@ pack_kernel(const PackParams p, const BlobHeader hdr)
   constexpr int TRIP = DENSE ? 1 : 2;                    // blocks a trip (pair-wise: a Q-Vector of 64 K)
 #pragma unroll (UNROLL)
   for (int b0 = 0; b0 < 4; b0 += TRIP) {
-   [[maybe_unused]] const uint32_t w_o0 = b0 < 2 ? c_o0[0] : c_o0[1], w_o1 = b0 < 2 ? c_o1[0] : c_o1[1];
+    [[maybe_unused]] const uint32_t w_o0 = b0 < 2 ? c_o0[0] : c_o0[1], w_o1 = b0 < 2 ? c_o1[0] : c_o1[1];
 #pragma unroll
-   for (int bi = 0; bi < TRIP; ++bi) {                   // blocks of 4 S-Vectors (32 K)
-    const int b = b0 + bi, odd = DENSE ? b & 1 : bi;
-    uint32_t ocode[4], ocode1[4], opos[4], opos1[4];
-    uint32_t dense_codes[4], dval[16];
-    [[maybe_unused]] uint32_t emeta[2] = {0, 0};
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const uint4 v = *reinterpret_cast<const uint4*>(mine + (4 * b + i) * 16);
-      uint32_t x[4] = {v.x, v.y, v.z, v.w};
-      [[maybe_unused]] int k[8];
-      int o0, o1;
-      if constexpr (CHOSEN) {
-        o0 = (int)((w_o0 >> (16 * odd + 4 * i)) & 7u);
-        o1 = (int)((w_o1 >> (16 * odd + 4 * i)) & 7u);
-      } else {
-        rank_keys<false>(x, nullptr, k);
-        pick_outliers<false, OUTN>(k, p.order_mask, p.sv4 != 0, o0, o1);
-      }
-      // Stage 3, outliers: E4M3 codes of w / 2^e, or int8 codes of w / s
-      if constexpr (OUTN > 0) {
-        const float f = DENSE ? pick_value(x, o0) : __uint_as_float(x[2]);
-        ocode[i] = !DENSE && p.i8 ? int8_code(f, __int_as_float(e)) : e4m3x1(f * s8);
-        opos[i] = (uint32_t)o0;
-      }
-      if constexpr (OUTN > 1) {
-        const float f = DENSE ? pick_value(x, o1) : __uint_as_float(x[3]);
-        ocode1[i] = !DENSE && p.i8 ? int8_code(f, __int_as_float(e)) : e4m3x1(f * s8);
-        opos1[i] = (uint32_t)o1;
-      }
-      if constexpr (!DENSE) {
-        kept[2 * (4 * odd + i)] = x[0];
-        kept[2 * (4 * odd + i) + 1] = x[1];
-        qmax2 = max_abs2(max_abs2(qmax2, x[0]), x[1]);
-      } else {
-        uint32_t gone;
-        if constexpr (CHOSEN) gone = (c_gone[0] >> (8 * i)) & 255u;
-        else gone = dropped_set<false, OUTN>(k, o0, o1, p.keep_in, p.sv4 || p.elem, p.order_mask);
-        zero_set(x, gone);
-        qmax2 = max_magnitudes(qmax2, x);
-#pragma unroll
-        for (int j = 0; j < 4; ++j) dval[4 * i + j] = x[j];
-        if (p.elem) {
-          // the kept indices (two ascending 2-bit values per group of 4) are only needed by the exporter.  Exactly two of a
-          // group's four bits are set: the nibble that such a set stands for, looked up
-          const uint32_t lo = (~gone) & 15u, hi = (~gone >> 4) & 15u;
-          const uint32_t ml = ((lo & 8u) ? 0x000E0DC0u : 0x09804000u) >> (4 * (lo & 7u)), mh = ((hi & 8u) ? 0x000E0DC0u : 0x09804000u) >> (4 * (hi & 7u));
-          emeta[i >> 1] |= ((ml & 15u) | ((mh & 15u) << 8)) << (16 * (i & 1));
-        }
-      }
-    }
-
-    // ---- Stage 3, inliers
-    if constexpr (DENSE) {
-      const uint32_t c = e8m0_scale_code_bf16(larger_half(qmax2), p.ceil_rule != 0);
-      const float inv = pow2_inv_e8m0(c);
+    for (int bi = 0; bi < TRIP; ++bi) {                   // blocks of 4 S-Vectors (32 K)
+      const int b = b0 + bi, odd = DENSE ? b & 1 : bi;
+      uint32_t ocode[4], ocode1[4], opos[4], opos1[4];
+      uint32_t dense_codes[4], dval[16];
+      [[maybe_unused]] uint32_t emeta[2] = {0, 0};
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        float f[8];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          f[2 * j] = __uint_as_float(dval[4 * i + j] << 16) * inv;
-          f[2 * j + 1] = __uint_as_float(dval[4 * i + j] & 0xFFFF0000u) * inv;
+        const uint4 v = *reinterpret_cast<const uint4*>(mine + (4 * b + i) * 16);
+        uint32_t x[4] = {v.x, v.y, v.z, v.w};
+        [[maybe_unused]] int k[8];
+        int o0, o1;
+        if constexpr (CHOSEN) {
+          o0 = (int)((w_o0 >> (16 * odd + 4 * i)) & 7u);
+          o1 = (int)((w_o1 >> (16 * odd + 4 * i)) & 7u);
+        } else {
+          rank_keys<false>(x, nullptr, k);
+          pick_outliers<false, OUTN>(k, p.order_mask, p.sv4 != 0, o0, o1);
         }
-        dense_codes[i] = e2m1x8(f);
+        // Stage 3, outliers: E4M3 codes of w / 2^e, or int8 codes of w / s
+        if constexpr (OUTN > 0) {
+          const float f = DENSE ? pick_value(x, o0) : __uint_as_float(x[2]);
+          ocode[i] = !DENSE && p.i8 ? int8_code(f, __int_as_float(e)) : e4m3x1(f * s8);
+          opos[i] = (uint32_t)o0;
+        }
+        if constexpr (OUTN > 1) {
+          const float f = DENSE ? pick_value(x, o1) : __uint_as_float(x[3]);
+          ocode1[i] = !DENSE && p.i8 ? int8_code(f, __int_as_float(e)) : e4m3x1(f * s8);
+          opos1[i] = (uint32_t)o1;
+        }
+        if constexpr (!DENSE) {
+          kept[2 * (4 * odd + i)] = x[0];
+          kept[2 * (4 * odd + i) + 1] = x[1];
+          qmax2 = max_abs2(max_abs2(qmax2, x[0]), x[1]);
+        } else {
+          uint32_t gone;
+          if constexpr (CHOSEN) gone = (c_gone[0] >> (8 * i)) & 255u;
+          else gone = dropped_set<false, OUTN>(k, o0, o1, p.keep_in, p.sv4 || p.elem, p.order_mask);
+          zero_set(x, gone);
+          qmax2 = max_magnitudes(qmax2, x);
+#pragma unroll
+          for (int j = 0; j < 4; ++j) dval[4 * i + j] = x[j];
+          if (p.elem) {
+            // the kept indices (two ascending 2-bit values per group of 4) are only needed by the exporter.  Exactly two of a
+            // group's four bits are set: the nibble that such a set stands for, looked up
+            const uint32_t lo = (~gone) & 15u, hi = (~gone >> 4) & 15u;
+            const uint32_t ml = ((lo & 8u) ? 0x000E0DC0u : 0x09804000u) >> (4 * (lo & 7u)), mh = ((hi & 8u) ? 0x000E0DC0u : 0x09804000u) >> (4 * (hi & 7u));
+            emeta[i >> 1] |= ((ml & 15u) | ((mh & 15u) << 8)) << (16 * (i & 1));
+          }
+        }
       }
-      if (p.elem) *reinterpret_cast<uint2*>(p.blob + p.off.emeta + (size_t)n * (size_t)(p.K / 4) + (kc * 16 + 4 * b) * 2) = make_uint2(emeta[0], emeta[1]);
-      // 16 code bytes per 32 K: K-block (64 K) 2 h + b / 2 of the record, chunk b & 1
-      *reinterpret_cast<uint4*>(wi + (2 * h + (b >> 1)) * 4096 + core + odd * 128) = make_uint4(dense_codes[0], dense_codes[1], dense_codes[2], dense_codes[3]);
-      sc |= c << (8 * b);
-      qmax2 = 0;
-    } else if (odd || b32) {
-      // a Q-Vector is complete: 64 K (both blocks of the half) or 32 K (this one)
-      const uint32_t key = larger_half(qmax2);
-      const uint32_t c = p.ue ? ue4m3_scale_code(bf16_bits_to_float(key) * pow2_neg(tw), key != 0) : e8m0_scale_code_bf16(key, p.ceil_rule != 0);
-      const float inv = p.ue ? ue4m3_scale_inverse(max(c, 1u)) : pow2_inv_e8m0(c);
+
+      // ---- Stage 3, inliers
+      if constexpr (DENSE) {
+        const uint32_t c = e8m0_scale_code_bf16(larger_half(qmax2), p.ceil_rule != 0);
+        const float inv = pow2_inv_e8m0(c);
 #pragma unroll
-      for (int hb = 0; hb < 2; ++hb) {                   // 32-K block of the half
-        if (hb != odd && b32) continue;              // (one scale per 64 K: both now)
-#pragma unroll
-        for (int i = 0; i < 2; ++i) {                    // two S-Vectors per code word
+        for (int i = 0; i < 4; ++i) {
           float f[8];
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
-            const uint32_t w = kept[8 * hb + 4 * i + j];
-            const float lo = __uint_as_float(w << 16), hi = __uint_as_float(w & 0xFFFF0000u);
-            if (p.ue) {
-              // (an outlier's position stays +0; the quotient of a dropped one is +0 as well)
-              f[2 * j] = small_quotient(lo * pow2_neg(tw), inv);
-              f[2 * j + 1] = small_quotient(hi * pow2_neg(tw), inv);
-            } else {
-              f[2 * j] = lo * inv;
-              f[2 * j + 1] = hi * inv;
-            }
+            f[2 * j] = __uint_as_float(dval[4 * i + j] << 16) * inv;
+            f[2 * j + 1] = __uint_as_float(dval[4 * i + j] & 0xFFFF0000u) * inv;
           }
-          in_word[hb][i] = p.ue && c == 0 ? 0u : e2m1x8(f);
+          dense_codes[i] = e2m1x8(f);
+        }
+        if (p.elem) *reinterpret_cast<uint2*>(p.blob + p.off.emeta + (size_t)n * (size_t)(p.K / 4) + (kc * 16 + 4 * b) * 2) = make_uint2(emeta[0], emeta[1]);
+        // 16 code bytes per 32 K: K-block (64 K) 2 h + b / 2 of the record, chunk b & 1
+        *reinterpret_cast<uint4*>(wi + (2 * h + (b >> 1)) * 4096 + core + odd * 128) = make_uint4(dense_codes[0], dense_codes[1], dense_codes[2], dense_codes[3]);
+        sc |= c << (8 * b);
+        qmax2 = 0;
+      } else if (odd || b32) {
+        // a Q-Vector is complete: 64 K (both blocks of the half) or 32 K (this one)
+        const uint32_t key = larger_half(qmax2);
+        const uint32_t c = p.ue ? ue4m3_scale_code(bf16_bits_to_float(key) * pow2_neg(tw), key != 0) : e8m0_scale_code_bf16(key, p.ceil_rule != 0);
+        const float inv = p.ue ? ue4m3_scale_inverse(max(c, 1u)) : pow2_inv_e8m0(c);
+#pragma unroll
+        for (int hb = 0; hb < 2; ++hb) {                   // 32-K block of the half
+          if (hb != odd && b32) continue;              // (one scale per 64 K: both now)
+#pragma unroll
+          for (int i = 0; i < 2; ++i) {                    // two S-Vectors per code word
+            float f[8];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              const uint32_t w = kept[8 * hb + 4 * i + j];
+              const float lo = __uint_as_float(w << 16), hi = __uint_as_float(w & 0xFFFF0000u);
+              if (p.ue) {
+                // (an outlier's position stays +0; the quotient of a dropped one is +0 as well)
+                f[2 * j] = small_quotient(lo * pow2_neg(tw), inv);
+                f[2 * j + 1] = small_quotient(hi * pow2_neg(tw), inv);
+              } else {
+                f[2 * j] = lo * inv;
+                f[2 * j + 1] = hi * inv;
+              }
+            }
+            in_word[hb][i] = p.ue && c == 0 ? 0u : e2m1x8(f);
+          }
+        }
+        if (b32) { sc |= c << (8 * b); }
+        else sc |= c << (8 * (b >> 1));
+        qmax2 = 0;
+      }
+      if constexpr (!DENSE) {
+        if (odd) {
+          // 16 code bytes per 64 K (K-block h, chunk b / 2)
+          *reinterpret_cast<uint4*>(wi + h * 4096 + core + (b >> 1) * 128) = make_uint4(in_word[0][0], in_word[0][1], in_word[1][0], in_word[1][1]);
         }
       }
-      if (b32) { sc |= c << (8 * b); }
-      else sc |= c << (8 * (b >> 1));
-      qmax2 = 0;
-    }
-    if constexpr (!DENSE) {
-      if (odd) {
-        // 16 code bytes per 64 K (K-block h, chunk b / 2)
-        *reinterpret_cast<uint4*>(wi + h * 4096 + core + (b >> 1) * 128) = make_uint4(in_word[0][0], in_word[0][1], in_word[1][0], in_word[1][1]);
-      }
-    }
 
-    // ---- outliers of the 4 S-Vectors: compact record, and the 2:4 embedding the sparse FP8 path consumes (per 4 K two
-    // ascending slot indices, unused slots hold +0)
-    if constexpr (OUTN == 1) {
-      // per S-Vector: position ps (0..7) sits in group of 4 number ps >> 2 at p = ps & 3, whose slots are (p, 3), the value
-      // first, or (0, 3), the value second, when p = 3; the other group has slots (0, 1).  Metadata bytes and byte shifts
-      // come from 8-entry tables looked up by byte-permutes, the four position nibbles being the selector.
-      queue32(codes, ocode[0] | (ocode[1] << 8) | (ocode[2] << 16) | (ocode[3] << 24));
-      const uint32_t sel = CHOSEN ? (w_o0 >> (16 * odd)) & 0xFFFFu : opos[0] | (opos[1] << 4) | (opos[2] << 8) | (opos[3] << 12);
-      const uint32_t sh = __byte_perm(0x08000000u, 0x18101010u, sel);
-      queue32(metas, __byte_perm(0x4C4E4D4Cu, 0xC4E4D4C4u, sel));
-      queue32(sels, sel);
-      *reinterpret_cast<uint4*>(wo + (b >> 1) * 4096 + core + odd * 128) =
-          make_uint4(ocode[0] << (sh & 31u), ocode[1] << ((sh >> 8) & 31u), ocode[2] << ((sh >> 16) & 31u), ocode[3] << (sh >> 24));
-    } else if constexpr (OUTN == 2) {
-      uint32_t st[4], meta = 0;
+      // ---- outliers of the 4 S-Vectors: compact record, and the 2:4 embedding the sparse FP8 path consumes (per 4 K two
+      // ascending slot indices, unused slots hold +0)
+      if constexpr (OUTN == 1) {
+        // per S-Vector: position ps (0..7) sits in group of 4 number ps >> 2 at p = ps & 3, whose slots are (p, 3), the value
+        // first, or (0, 3), the value second, when p = 3; the other group has slots (0, 1).  Metadata bytes and byte shifts
+        // come from 8-entry tables looked up by byte-permutes, the four position nibbles being the selector.
+        queue32(codes, ocode[0] | (ocode[1] << 8) | (ocode[2] << 16) | (ocode[3] << 24));
+        const uint32_t sel = CHOSEN ? (w_o0 >> (16 * odd)) & 0xFFFFu : opos[0] | (opos[1] << 4) | (opos[2] << 8) | (opos[3] << 12);
+        const uint32_t sh = __byte_perm(0x08000000u, 0x18101010u, sel);
+        queue32(metas, __byte_perm(0x4C4E4D4Cu, 0xC4E4D4C4u, sel));
+        queue32(sels, sel);
+        *reinterpret_cast<uint4*>(wo + (b >> 1) * 4096 + core + odd * 128) =
+            make_uint4(ocode[0] << (sh & 31u), ocode[1] << ((sh >> 8) & 31u), ocode[2] << ((sh >> 16) & 31u), ocode[3] << (sh >> 24));
+      } else if constexpr (OUTN == 2) {
+        uint32_t st[4], meta = 0;
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int o0 = (int)opos[i], o1 = (int)opos1[i];
-        st[i] = 0;
+        for (int i = 0; i < 4; ++i) {
+          const int o0 = (int)opos[i], o1 = (int)opos1[i];
+          st[i] = 0;
 #pragma unroll
-        for (int q = 0; q < 2; ++q) {
-          const bool in0 = (o0 >> 2) == q, in1 = (o1 >> 2) == q;
-          uint32_t s, m;
-          if (in0 && in1) { s = ocode[i] | (ocode1[i] << 8); m = (uint32_t)((o0 & 3) | ((o1 & 3) << 2)); }
-          else if (in0 || in1) {
-            const uint32_t pp = (uint32_t)((in0 ? o0 : o1) & 3), cc = in0 ? ocode[i] : ocode1[i];
-            s = pp == 3u ? cc << 8 : cc;
-            m = (pp == 3u ? 0u : pp) | 12u;
-          } else { s = 0; m = 4u; }
-          st[i] |= s << (16 * q);
-          meta |= m << (8 * i + 4 * q);
+          for (int q = 0; q < 2; ++q) {
+            const bool in0 = (o0 >> 2) == q, in1 = (o1 >> 2) == q;
+            uint32_t s, m;
+            if (in0 && in1) { s = ocode[i] | (ocode1[i] << 8); m = (uint32_t)((o0 & 3) | ((o1 & 3) << 2)); }
+            else if (in0 || in1) {
+              const uint32_t pp = (uint32_t)((in0 ? o0 : o1) & 3), cc = in0 ? ocode[i] : ocode1[i];
+              s = pp == 3u ? cc << 8 : cc;
+              m = (pp == 3u ? 0u : pp) | 12u;
+            } else { s = 0; m = 4u; }
+            st[i] |= s << (16 * q);
+            meta |= m << (8 * i + 4 * q);
+          }
         }
+        *reinterpret_cast<uint4*>(wo + (b >> 1) * 4096 + core + odd * 128) = make_uint4(st[0], st[1], st[2], st[3]);
+        queue32(metas, meta);
+        *reinterpret_cast<uint2*>(wc + r * 32 + 8 * b) =
+            make_uint2(ocode[0] | (ocode1[0] << 8) | (ocode[1] << 16) | (ocode1[1] << 24), ocode[2] | (ocode1[2] << 8) | (ocode[3] << 16) | (ocode1[3] << 24));
+        *reinterpret_cast<uint32_t*>(wc + 2 * WC_CODE_BYTES + r * 16 + 4 * b) =
+            opos[0] | (opos1[0] << 4) | (opos[1] << 8) | (opos1[1] << 12) | (opos[2] << 16) | (opos1[2] << 20) | (opos[3] << 24) | (opos1[3] << 28);
       }
-      *reinterpret_cast<uint4*>(wo + (b >> 1) * 4096 + core + odd * 128) = make_uint4(st[0], st[1], st[2], st[3]);
-      queue32(metas, meta);
-      *reinterpret_cast<uint2*>(wc + r * 32 + 8 * b) =
-          make_uint2(ocode[0] | (ocode1[0] << 8) | (ocode[1] << 16) | (ocode1[1] << 24), ocode[2] | (ocode1[2] << 8) | (ocode[3] << 16) | (ocode1[3] << 24));
-      *reinterpret_cast<uint32_t*>(wc + 2 * WC_CODE_BYTES + r * 16 + 4 * b) =
-          opos[0] | (opos1[0] << 4) | (opos[1] << 8) | (opos1[1] << 12) | (opos[2] << 16) | (opos1[2] << 20) | (opos[3] << 24) | (opos1[3] << 28);
     }
-   }
-   if constexpr (DENSE && CHOSEN) queue32(c_gone, 0u);
+    if constexpr (DENSE && CHOSEN) queue32(c_gone, 0u);    // (the next trip's sets of dropped positions to the front)
   }
   if constexpr (!DENSE) *reinterpret_cast<uint2*>(wi + A_IN_BYTES + r * 16 + h * 8) = make_uint2(c_nib[0], c_nib[1]);
   if constexpr (OUTN > 0) *reinterpret_cast<uint4*>(wo + A_OUT_BYTES + r * 16) = make_uint4(metas[0], metas[1], metas[2], metas[3]);
