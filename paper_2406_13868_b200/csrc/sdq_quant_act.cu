@@ -304,8 +304,13 @@ quant_act_fused_kernel(const __nv_bfloat16* __restrict__ X, int64_t M, int64_t K
     for (int w = 0; w < warps; ++w) a = fmaxf(a, s_warp[w][tok]);
     ptx::st_async_u32(ptx::mapa_u32(ptx::smem_u32(&s_all[rank][tok]), peer), __float_as_uint(a), ptx::mapa_u32(ptx::smem_u32(&s_bar), peer));
   }
-  // no CTA leaves before all pushes to it have arrived, and its own go to CTAs that wait for them
-  if (!ptx::mbar_wait_cluster(&s_bar, 0) && lane == 0) atomicOr(&flags[FLAG_TIMEOUT], 1u);
+  // no CTA leaves before all pushes to it have arrived, and its own go to CTAs that wait for them.  Where the wait gives up, peers may still
+  // push: this CTA stays until they have, or have given up as well
+  if (!ptx::mbar_wait_cluster(&s_bar, 0)) {
+    atomicOr(&flags[FLAG_TIMEOUT], 1u);
+    ptx::cluster_wait_for_others();
+    (void)ptx::mbar_wait_cluster(&s_bar, 0);               // (what was sent last is still on its way)
+  }
   float ramax = 0.0f;
   for (uint32_t c = 0; c < cx; ++c) ramax = fmaxf(ramax, s_all[c][t]);
   if (live && rank == 0 && warp == 0) qa_token_scale<UE>(ramax, m, (uint32_t)l, cfg, buf, off);
