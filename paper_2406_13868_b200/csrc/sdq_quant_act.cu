@@ -11,11 +11,11 @@
 // then a 4-lane shuffle, a token's four scales are one word, and every store instruction of codes writes whole 128-byte
 // lines (8 tokens x 16 B per core matrix).  Codes come from the hardware E2M1 / E4M3 converters.
 //
-// Bound by DRAM traffic and the conversion instructions: 2048 x 11008 at 4.4 TB/s of algorithmic bytes (18.0 us), 8192 x 11008 at
-// 5.4 TB/s (58.3), 8192 x 4096 at 5.5 (21.5), one token 2.1 us, most of it the launch.  Against releasing cluster arrivals, no
-// fetching ahead and an unpacking in front of every multiplication: 20.1, 66.0, 23.5 us; 4096 x 16384 with E4M3 scales, where 64
-// registers also let a fourth CTA onto the SM, 60.1 -> 45.7.  E4M3 scales and int8 codes multiply by a reciprocal instead of
-// dividing every element (see sdq_codec.cuh): one int8 token 14.1 -> 3.0 us (zeros took the division's slow path).
+// Bound by DRAM traffic and the conversion instructions: 2048 x 11008 at 4.7 TB/s of algorithmic bytes (16.9 us), 8192 x 11008 at
+// 5.6 TB/s (56.7), 8192 x 4096 at 5.7 (20.7), one token 2.1 us, most of it the launch.  In steps: with releasing cluster arrivals, no
+// fetching ahead and an unpacking in front of every multiplication 20.1, 66.0, 23.5 us, without these 18.0, 58.3, 21.5; 4096 x 16384 with
+// E4M3 scales, where 64 registers also let a fourth CTA onto the SM, 60.1 -> 45.7.  E4M3 scales and int8 codes multiply by a reciprocal
+// instead of dividing every element (see sdq_codec.cuh): one int8 token 14.1 -> 3.0 us (zeros took the division's slow path).
 // Products that only one of the 8-bit forms needs are formed in its branch: in front of it, int8 calls paid for E4M3's (8192 x 4096,
 // back to back, 45.6 -> 42.7 us; before scaled2 43.9) and everybody for their registers (8192 x 2048 10.2 -> 9.9, 2048 x 11008 15.9 -> 15.2).
 #include "sdq_codec.cuh"
