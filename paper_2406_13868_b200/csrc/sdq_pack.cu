@@ -463,7 +463,7 @@ pack_kernel(const PackParams p, const BlobHeader hdr)
     }
     // counted stores, as in the activation quantizer: a CTA waits for what it needs and for nothing else, and does not leave before all
     // pushes to it have arrived.  Where the wait gives up, peers may still push: this CTA stays until they have, or have given up as well
-    if (!ptx::mbar_wait_cluster(&s_bar, 0, p.polls)) {
+    if (__any_sync(0xffffffffu, !ptx::mbar_wait_cluster(&s_bar, 0, p.polls))) {
       *reinterpret_cast<volatile uint32_t*>(p.gave_up) = 1u;
       ptx::cluster_wait_for_others();
       (void)ptx::mbar_wait_cluster(&s_bar, 0);             // (what was sent last is still on its way)

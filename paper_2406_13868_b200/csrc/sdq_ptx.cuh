@@ -299,10 +299,10 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity
   }
   return false;
 }
-// for threads whose wait on the cluster's other CTAs gave up (the kernel's first cluster barrier lies behind them): returns when every
+// for warps whose wait on the cluster's other CTAs gave up (the kernel's first cluster barrier lies behind them; all lanes): returns when every
 // other thread of the cluster has come here too or has exited
 __device__ __forceinline__ void cluster_wait_for_others() {
-  asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 __device__ __forceinline__ bool mbar_test_cluster(uint64_t* bar, uint32_t parity) {
   uint32_t ok;

@@ -305,9 +305,9 @@ quant_act_fused_kernel(const __nv_bfloat16* __restrict__ X, int64_t M, int64_t K
     ptx::st_async_u32(ptx::mapa_u32(ptx::smem_u32(&s_all[rank][tok]), peer), __float_as_uint(a), ptx::mapa_u32(ptx::smem_u32(&s_bar), peer));
   }
   // no CTA leaves before all pushes to it have arrived, and its own go to CTAs that wait for them.  Where the wait gives up, peers may still
-  // push: this CTA stays until they have, or have given up as well
-  if (!ptx::mbar_wait_cluster(&s_bar, 0)) {
-    atomicOr(&flags[FLAG_TIMEOUT], 1u);
+  // push: this CTA stays until they have, or have given up as well.  (Decided by the warp: by each thread, every call paid 0.1 us)
+  if (__any_sync(0xffffffffu, !ptx::mbar_wait_cluster(&s_bar, 0))) {
+    if (lane == 0) atomicOr(&flags[FLAG_TIMEOUT], 1u);
     ptx::cluster_wait_for_others();
     (void)ptx::mbar_wait_cluster(&s_bar, 0);               // (what was sent last is still on its way)
   }

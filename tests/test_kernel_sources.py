@@ -49,7 +49,7 @@ def test_no_remote_shared_memory_before_the_cluster_has_started(name):
 def test_a_thread_block_whose_wait_gives_up_stays_for_its_peers(name):
     """peers may still store into the shared memory of a thread block that gave up: it waits for them before it can leave"""
     body = {n: b for _, n, b in kernels()}[name]
-    gave_up = re.search(r"if \(!ptx::mbar_wait_cluster\(&s_bar, 0[^()]*\)\) \{([^{}]*)\}", body)
+    gave_up = re.search(r"if \(__any_sync\(0xffffffffu, !ptx::mbar_wait_cluster\(&s_bar, 0[^()]*\)\)\) \{([^{}]*)\}", body)
     assert gave_up and re.search(r"= 1u;|atomicOr\(&flags\[FLAG_TIMEOUT\], 1u\);", gave_up.group(1))
     assert re.search(r"ptx::cluster_wait_for_others\(\);\s*\(void\)ptx::mbar_wait_cluster\(&s_bar, 0\);", gave_up.group(1))
 
@@ -57,7 +57,7 @@ def test_a_thread_block_whose_wait_gives_up_stays_for_its_peers(name):
 def test_a_packing_call_whose_wait_gave_up_returns_the_timeout():
     """it reads its kernel's report back anyway"""
     body = {n: b for _, n, b in kernels()}["pack_kernel"]
-    assert re.search(r"if \(!ptx::mbar_wait_cluster\(&s_bar, 0[^()]*\)\) \{[^{}]*\(p.gave_up\) = 1u;", body)
+    assert re.search(r"if \(__any_sync\(0xffffffffu, !ptx::mbar_wait_cluster\(&s_bar, 0[^()]*\)\)\) \{[^{}]*\(p.gave_up\) = 1u;", body)
     src = open(os.path.join(CSRC, "sdq_pack.cu")).read()
     host = src[src.index("static sdq_status_t decompose("):]
     assert re.search(r"give_back\(report\);[^{}]*gave_up \? SDQ_ERR_TIMEOUT", host[:host.index("\n}\n")])
